@@ -206,17 +206,17 @@ extern "C" int lfc_plan_inject_fault(lfc_plan P, int fault) {
     if (!P || fault < 0 || fault > LFC_FAULT_SORT_WITHHOLD) return LFC_ERR_INVALID_ARG;
     // the device word is read by the next suffix sort that runs on the GPU
     // (a call's or a replayed batch's); the withholding tile clears it
-    CK(cudaMemsetAsync(P->ws.act_total + kSortFaultWord, fault ? 1 : 0, sizeof(int32_t), P->stream));
+    CK(cudaMemsetAsync(P->ws.act_total + kRsFault, fault ? 1 : 0, sizeof(int32_t), P->stream));
     return LFC_OK;
 }
 
 extern "C" int lfc_plan_device_status(lfc_plan P) {
     if (!P) return LFC_ERR_INVALID_ARG;
     int32_t st = 0;
-    CK(cudaMemcpyAsync(&st, P->ws.act_total + kSortStickyWord, sizeof(int32_t), cudaMemcpyDeviceToHost, P->stream));
+    CK(cudaMemcpyAsync(&st, P->ws.act_total + kRsSticky, sizeof(int32_t), cudaMemcpyDeviceToHost, P->stream));
     CK(cudaStreamSynchronize(P->stream));
     if (st == 0) return LFC_OK;
-    CK(cudaMemsetAsync(P->ws.act_total + kSortStickyWord, 0, sizeof(int32_t), P->stream));
+    CK(cudaMemsetAsync(P->ws.act_total + kRsSticky, 0, sizeof(int32_t), P->stream));
     CK(cudaStreamSynchronize(P->stream));
     return st == LFC_ERR_TIMEOUT ? fail(P, LFC_ERR_TIMEOUT, "a bounded device wait gave up") : fail(P, LFC_ERR_CUDA, "device status");
 }
@@ -252,7 +252,7 @@ extern "C" int lfc_plan_block_capacity(lfc_plan P) { return P ? P->block_cap : 0
 
 static void free_ws(Workspace &w) {
     void *ptrs[] = {w.hist, w.summ, w.chain_first, w.scores, w.choice, w.jframes, w.cand, w.l2tab, w.stream, w.blocks, w.bstate,
-                    w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.val2, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.tileaux, w.bwt,
+                    w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.bcode, w.bcount, w.bcursor, w.bstart, w.bitems, w.bflag, w.tileaux, w.bwt,
                     w.mtfidx, w.mtflists, w.mtfrec, w.mtfreclen, w.sym, w.freq, w.rfreq, w.sel, w.lens, w.codes, w.packed, w.cstream, w.masks, w.class_ids,
                     w.act_total, w.block_dst, w.frame_crc, w.crc_part, w.crc_part2, w.chunk_desc, w.dec_tt,
                     w.hx_frames, w.hx_prev, w.hx_out, w.hx_choice, w.hx_sizes};
@@ -346,13 +346,19 @@ extern "C" int lfc_plan_create(const lfc_config *cfg, void *cuda_stream, lfc_pla
     AL(act, (size_t)BC * kBlockCap);
     AL(act2, (size_t)BC * kBlockCap);
     AL(val, (size_t)BC * kBlockCap);
-    AL(val2, (size_t)BC * kBlockCap);
     AL(keys, (size_t)BC * kBlockCap);
     AL(keys2, (size_t)BC * kBlockCap);
     ws.lbstat_words = (size_t)BC * kTilesPerBlock * 256;
     AL(lbstat, 2 * ws.lbstat_words);
     AL(dhist, (size_t)BC * 8 * 256);
     AL(segbig, (size_t)BC);
+    AL(bcode, (size_t)BC);
+    AL(bcount, (size_t)BC * kBuckets);
+    AL(bcursor, (size_t)BC * kBuckets);
+    AL(bstart, (size_t)BC * kBucketRow);
+    ws.bitems_cap = (size_t)BC * kBuckets;
+    AL(bitems, kRsBucketClasses * ws.bitems_cap);
+    AL(bflag, (size_t)BC);
     AL(tileaux, (size_t)BC * kTilesPerBlock * 4);
     AL(bwt, (size_t)BC * kBlockCap);
     AL(mtfidx, (size_t)BC * kBlockCap);

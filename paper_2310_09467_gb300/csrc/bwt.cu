@@ -3,34 +3,26 @@
 // public bzip2 format).
 //
 // BWT = sort of all cyclic rotations, ties between identical rotations by
-// start index. Two phases over all blocks of a pass at once. Every element
-// carries its sort key. A radix pass is one persistent kernel whose CTAs
-// take 4096-element tiles from a device work queue, tile-major over the
-// blocks so that a block has only a few tiles in flight: a CTA reads its tile's
-// (key, element) pairs coalesced, ranks them by digit in shared memory,
-// publishes the tile's digit counts and adds up the counts of the block's
-// earlier tiles as they are published (decoupled look-back: a tile only waits
-// on tiles taken from the queue before it, every wait bounded by a cycle
-// budget), then writes each digit's run of the tile contiguously. The
-// block's digit totals for every pass come from the kernel that builds the
-// keys, so a pass needs no separate histogram or scan launch.
-//  1. Keys = the first 8 bytes of each rotation (big-endian), built from
-//     sequential reads; 8 stable LSD passes of 8-bit digits.
+// start index, over all blocks of a pass at once. The bucket sort of
+// bwt_bucket.cu finishes almost every block; this file has what is left for
+// the blocks it flags (repetitive data):
+//  1. kFlagOver blocks (a bucket too large for shared memory): their words
+//     (44 key bits above the 20-bit start) take 8 stable LSD passes of 8-bit
+//     digits. A radix pass is one persistent kernel whose CTAs take
+//     4096-element tiles from a device work queue, tile-major over the blocks
+//     so that a block has only a few tiles in flight: a CTA reads its tile's
+//     words coalesced, ranks them by digit in shared memory, publishes the
+//     tile's digit counts and adds up the counts of the block's earlier tiles
+//     as they are published (decoupled look-back: a tile only waits on tiles
+//     taken from the queue before it, every wait bounded by a cycle budget),
+//     then writes each digit's run of the tile contiguously.
 //  2. Prefix doubling on the groups still tied: rank[i] = head position of
 //     i's group in the suffix array; each round keys the tied elements by
-//     (rank[i] << 20 | rank[i + h]) (m < 2^20), sorts them with 5 stable LSD
-//     passes, splits groups, and doubles h. Here an element is one 64-bit
-//     word, the 40-bit key above the element (20 bits), and the passes sort
-//     bits 20..59 only. Groups left when h >= m hold identical rotations,
-//     already in start-index order (every pass is stable and the first starts
-//     from the identity).
+//     (rank[i] << 20 | rank[i + h]) (m < 2^20), sorts them, splits groups,
+//     and doubles h, from the bytes that every group left tied shares. Groups left when h >= m hold identical rotations, already in
+//     start-index order (the words hold the start below the key).
 #include <algorithm>
 #include <climits>
-#include <utility>
-
-#ifndef LFC_PHASE1_BYTES
-#define LFC_PHASE1_BYTES 8
-#endif
 
 #include "lfc_common.cuh"
 
@@ -238,28 +230,17 @@ cudaError_t launch_rle1(lfc_plan P, int nblocks, const BlockDesc *d_blocks) {
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------ sort keys
+// ------------------------------------------------------------ sort state
+// Blocks that the bucket sort (bwt_bucket.cu) finished take no part here:
+// phase 1 (MODE 0) runs on flagged blocks, a round on their tied elements.
 template <int MODE>
-__device__ __forceinline__ int sort_count(const BlockState &s, int h) {
-    if (MODE == 0) return s.m;
+__device__ __forceinline__ int sort_count(const BlockState &s, int h, int flagged) {
+    if (MODE == 0) return flagged ? s.m : 0;
     return h < s.m ? s.n_act : 0;
 }
 
 template <int MODE>
-__device__ __forceinline__ int round_h(const int32_t *rs) { return MODE == 0 ? 0 : rs[2]; }
-
-// Sort state in device memory (rs): tied elements after a round, their
-// per-block maximum, the shift h, the round number; the abort word (nonzero
-// once a bounded wait has given up in this suffix sort: every later sort
-// kernel returns at once), the fault-injection word (test hook), the two work
-// queues of the radix passes (by pass parity), the work items of the current
-// pass, the sticky status (kept until the host reads it), and from
-// kRsTileOff on the per-block prefix of tile counts (nblocks + 1 entries).
-enum : int {
-    kRsTied = 0, kRsTiedMax = 1, kRsH = 2, kRsRound = 3, kRsAbort = 4, kRsFault = kSortFaultWord, kRsQueue = 6,
-    kRsItems = 8, kRsSticky = kSortStickyWord, kRsTileOff = 16
-};
-static_assert(kRsTileOff == kSortCtlHead, "sort control layout");
+__device__ __forceinline__ int round_h(const int32_t *rs) { return MODE == 0 ? 0 : rs[kRsH]; }
 
 // Look-back status word of one digit of one tile: bits 30-31 a flag, bits
 // 0-29 a count (at most kBlockCap < 2^30).
@@ -313,69 +294,17 @@ __global__ void zero_u32_kernel(uint32_t *p, size_t n) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = 0;
 }
 
-// Phase 1 keys: K[v] = bytes v .. v + 7 (cyclic) big-endian, element v.
-// Phase 1 sorts the first kPhase1Bytes bytes of every rotation; they sit in
-// the top bytes of the 64-bit key, so passes 8 - kPhase1Bytes .. 7 carry them.
-constexpr int kPhase1Bytes = LFC_PHASE1_BYTES;
-
-// Also adds the tile's bytes to the block's byte histogram and clears the
-// tile's look-back status words in both status arrays (the first pass reads
-// array 0 and clears array 1 for the second, and so on). Over all rotations
-// of a block, the digit of every pass (one byte of each rotation's prefix)
-// takes each byte position of the block exactly once, so the digit totals
-// of all 8 passes equal the block's byte histogram: one histogram serves
-// every pass.
-__global__ void __launch_bounds__(kSortThreads) key8_kernel(const BlockState *__restrict__ st,
-                                                            const uint8_t *__restrict__ rle_all,
-                                                            uint64_t *__restrict__ K_all, int32_t *__restrict__ V_all,
-                                                            uint32_t *__restrict__ dhist_all, uint32_t *__restrict__ lb_all,
-                                                            size_t lb_array_words) {
-    __shared__ uint8_t sb[kTile + 8];
-    __shared__ uint32_t hst[1][256];
-    const int b = blockIdx.y, tile = blockIdx.x;
-    const int m = st[b].m;
-    const int t0 = tile * kTile;
-    if (t0 >= m) return;
-    const int cnt = min(kTile, m - t0);
-    const uint8_t *rle = rle_all + (size_t)b * kBlockCap;
-    for (int i = threadIdx.x; i < cnt + 7; i += kSortThreads) sb[i] = rle[(t0 + i) % m];
-    hst[0][threadIdx.x] = 0;
-    uint32_t *lbt = lb_all + (size_t)b * kLbBlockWords + (size_t)tile * 256;
-    lbt[threadIdx.x] = 0;
-    lbt[lb_array_words + threadIdx.x] = 0;
-    __syncthreads();
-    uint64_t *K = K_all + (size_t)b * kBlockCap;
-    int32_t *V = V_all + (size_t)b * kBlockCap;
-    for (int r = 0; r < kPerThread; r++) {
-        const int kl = r * kSortThreads + threadIdx.x;
-        const bool ok = kl < cnt;
-        uint64_t key = 0;
-        if (ok) {
-#pragma unroll
-            for (int q = 0; q < kPhase1Bytes; q++) key = (key << 8) | sb[kl + q];
-            key <<= 8 * (8 - kPhase1Bytes);
-            K[t0 + kl] = key;
-            V[t0 + kl] = t0 + kl;
-        }
-        tile_digits<1>((uint64_t)sb[kl], ok, 0, hst);  // the tile's own byte
-    }
-    __syncthreads();
-    flush_digits<1>(hst, dhist_all + (size_t)b * kSweepPasses * 256);
-}
-
 // Round words of the tied elements: rank[v] << 40 | rank[(v + h) mod m] << 20 | v.
-constexpr uint64_t kElemMask = (1u << 20) - 1u;
-
 __global__ void __launch_bounds__(kSortThreads) key40_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
                                                              const int32_t *__restrict__ V_all, const int32_t *__restrict__ rank_all,
                                                              uint64_t *__restrict__ K_all, int32_t *__restrict__ big) {
     if (rs[kRsAbort]) return;
     const int b = blockIdx.y, tile = blockIdx.x;
-    const int h = rs[2];
+    const int h = rs[kRsH];
     const BlockState s = st[b];
-    const int n = sort_count<1>(s, h);
-    if (tile * kTile >= n) return;
+    const int n = sort_count<1>(s, h, 0);
     if (tile == 0 && threadIdx.x == 0) big[b] = 0;  // set again by the segmented sort if a group is too large
+    if (tile * kTile >= n) return;
     const size_t bo = (size_t)b * kBlockCap;
     // all elements first, then all rank gathers (independent loads in flight together)
     int vv[kPerThread];
@@ -395,27 +324,36 @@ __global__ void __launch_bounds__(kSortThreads) key40_kernel(const int32_t *__re
     }
 }
 
-// Digit totals of the 5 round passes, for the blocks the segmented sort
-// flagged (the only ones that take the radix passes).
-__global__ void __launch_bounds__(kSortThreads) round_digits_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
+// Digit totals of the radix passes and clear look-back words, for the blocks
+// that take them: MODE 0 the blocks flagged kFlagOver (8 passes over all 64
+// bits of their words), MODE 1 the blocks the segmented sort flagged in this
+// round (5 passes over bits 20..59).
+template <int MODE>
+__global__ void __launch_bounds__(kSortThreads) sweep_digits_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
                                                                     const uint64_t *__restrict__ K_all, uint32_t *__restrict__ dhist_all,
-                                                                    const int32_t *__restrict__ big) {
-    __shared__ uint32_t hst[5][256];
+                                                                    const int32_t *__restrict__ which, uint32_t *__restrict__ lb_all,
+                                                                    size_t lb_array_words) {
+    constexpr int NP = MODE == 0 ? 8 : 5;
+    __shared__ uint32_t hst[NP][256];
     if (rs[kRsAbort]) return;
     const int b = blockIdx.y, tile = blockIdx.x;
-    if (!big[b]) return;
-    const int n = sort_count<1>(st[b], rs[2]);
+    const bool take = MODE == 0 ? (which[b] & kFlagOver) != 0 : which[b] != 0;
+    if (!take) return;
+    const int n = sort_count<MODE>(st[b], round_h<MODE>(rs), 1);
     if (tile * kTile >= n) return;
-    for (int i = threadIdx.x; i < 5 * 256; i += kSortThreads) (&hst[0][0])[i] = 0;
+    uint32_t *lbt = lb_all + (size_t)b * kLbBlockWords + (size_t)tile * 256;
+    lbt[threadIdx.x] = 0;
+    lbt[lb_array_words + threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < NP * 256; i += kSortThreads) (&hst[0][0])[i] = 0;
     __syncthreads();
     const uint64_t *K = K_all + (size_t)b * kBlockCap;
     for (int r = 0; r < kPerThread; r++) {
         const int k = tile * kTile + r * kSortThreads + threadIdx.x;
         const bool ok = k < n;
-        tile_digits<5>(ok ? K[k] : 0ull, ok, 20, hst);
+        tile_digits<NP>(ok ? K[k] : 0ull, ok, MODE == 0 ? 0 : 20, hst);
     }
     __syncthreads();
-    flush_digits<5>(hst, dhist_all + (size_t)b * kSweepPasses * 256);
+    flush_digits<NP>(hst, dhist_all + (size_t)b * kSweepPasses * 256);
 }
 
 // Work items of the radix passes of a phase or round, tile-major: item i is
@@ -424,36 +362,20 @@ __global__ void __launch_bounds__(kSortThreads) round_digits_kernel(const int32_
 // finished (a look-back then stops within a few steps). Per block its tile
 // count ceil(n_b / kTile) goes to rs[kRsTileOff + b]; rs[kRsItems] = the
 // largest count x nblocks (items past a block's last tile are skipped); both
-// work queues start empty. One CTA.
-// In a round (MODE 1) only the blocks flagged by the segmented sort (a group
-// longer than its window) take the radix passes. In phase 1 (MODE 0) it also
-// writes row 1 of every block's digit totals: the exclusive prefix of row 0
-// (the byte histogram), i.e. the block's elements with a smaller digit, the
-// same for every pass and tile.
+// work queues start empty. One CTA. Only the blocks of sweep_digits_kernel
+// have tiles.
 template <int MODE>
 __global__ void __launch_bounds__(1024) sort_items_kernel(int32_t *__restrict__ rs, const BlockState *__restrict__ st, int nblocks,
-                                                          const int32_t *__restrict__ big, uint32_t *__restrict__ dhist_all) {
+                                                          const int32_t *__restrict__ which) {
     __shared__ int smax;
-    if (MODE == 0) {
-        const int lane = threadIdx.x & 31;
-        for (int bb = threadIdx.x >> 5; bb < nblocks; bb += blockDim.x >> 5) {
-            uint32_t *row = dhist_all + (size_t)bb * kSweepPasses * 256;
-            uint32_t c[8], t = 0;
-#pragma unroll
-            for (int i = 0; i < 8; i++) { c[i] = row[lane * 8 + i]; t += c[i]; }
-            uint32_t x = warp_incl_sum(t) - t;
-#pragma unroll
-            for (int i = 0; i < 8; i++) { row[256 + lane * 8 + i] = x; x += c[i]; }
-        }
-    }
     const bool abort = rs[kRsAbort] != 0;
     const int h = round_h<MODE>(rs);
     if (threadIdx.x == 0) smax = 0;
     __syncthreads();
     int mx = 0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        const bool take = !abort && (MODE == 0 || big[b] != 0);
-        const int t = take ? (sort_count<MODE>(st[b], h) + kTile - 1) / kTile : 0;
+        const bool take = !abort && (MODE == 0 ? (which[b] & kFlagOver) != 0 : which[b] != 0);
+        const int t = take ? (sort_count<MODE>(st[b], h, 1) + kTile - 1) / kTile : 0;
         rs[kRsTileOff + b] = t;
         mx = max(mx, t);
     }
@@ -463,6 +385,24 @@ __global__ void __launch_bounds__(1024) sort_items_kernel(int32_t *__restrict__ 
         rs[kRsItems] = smax * nblocks;
         rs[kRsQueue] = 0;
         rs[kRsQueue + 1] = 0;
+    }
+}
+
+// After the radix passes of the kFlagOver blocks: suffix array with the
+// non-head mark (an element whose key equals its predecessor's) in bit 31.
+__global__ void __launch_bounds__(kSortThreads) over_heads_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
+                                                                  const uint64_t *__restrict__ K_all, const int32_t *__restrict__ bflag,
+                                                                  int32_t *__restrict__ sa_all) {
+    const int b = blockIdx.y;
+    if (rs[kRsAbort] || !(bflag[b] & kFlagOver)) return;
+    const int m = st[b].m;
+    const uint64_t *K = K_all + (size_t)b * kBlockCap;
+    for (int r = 0; r < kPerThread; r++) {
+        const int k = blockIdx.x * kTile + r * kSortThreads + threadIdx.x;
+        if (k >= m) return;
+        const uint64_t w = K[k];
+        const bool tied = k > 0 && (K[k - 1] >> 20) == (w >> 20);
+        sa_all[(size_t)b * kBlockCap + k] = (int32_t)(w & kElemMask) | (tied ? (int32_t)0x80000000 : 0);
     }
 }
 
@@ -505,8 +445,8 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const int32_t *__r
     __shared__ int s_last[kSegCap / 32], s_first[kSegCap / 32], s_scan[33];
     if (rs[kRsAbort]) return;
     const int b = blockIdx.y, tile = blockIdx.x;
-    const int h = rs[2];
-    const int n = sort_count<1>(st[b], h);
+    const int h = rs[kRsH];
+    const int n = sort_count<1>(st[b], h, 0);
     const int t0 = tile * kTile;
     if (t0 >= n) return;
     const size_t bo = (size_t)b * kBlockCap;
@@ -621,12 +561,13 @@ __global__ void __launch_bounds__(kSegThreads) segsort_kernel(const int32_t *__r
     }
 }
 
-// Digit position of a pass: phase 1 sorts all 64 key bits, a round bits 20..59.
+// Digit position of a pass: phase 1 sorts all 64 bits of the words, a round bits 20..59.
 template <int MODE>
 __device__ __forceinline__ int digit_shift(int pass) { return (MODE == 0 ? 0 : 20) + 8 * pass; }
 
-// One stable LSD pass of (key, element) pairs (MODE 0) or round words (MODE
-// 1, the element rides in the word) over every block of the pass.
+// One stable LSD pass of words over every block that takes the passes
+// (MODE 0 kFlagOver blocks, MODE 1 a round's blocks with a group too long for
+// the segmented sort).
 // Persistent: CTAs take tiles from the pass's work queue until it is empty
 // (tile-major order, see sort_items_kernel).
 // Per tile: warp w ranks elements [w*512, (w+1)*512) of the tile 32 at a
@@ -635,10 +576,8 @@ __device__ __forceinline__ int digit_shift(int pass) { return (MODE == 0 ? 0 : 2
 // c[d] (flag "aggregate"; tile 0: "inclusive"), adds the published counts of
 // the block's earlier tiles back to the nearest "inclusive" one, publishes
 // its own inclusive count, and the run of digit d starts at (elements of the
-// block with a smaller digit: in phase 1 the offsets sort_items_kernel
-// derived from the block's byte histogram, in a round a scan of the pass's
-// digit totals) + (elements of digit d in earlier tiles). A CTA takes its
-// next work item while it sorts the current one. Tiles are placed in shared memory in digit
+// block with a smaller digit, a scan of the pass's digit totals) + (elements
+// of digit d in earlier tiles). Tiles are placed in shared memory in digit
 // order and each digit's run is written with consecutive threads on
 // consecutive addresses.
 // A tile waits only on tiles taken from the queue before it, which are held
@@ -648,24 +587,20 @@ __device__ __forceinline__ int digit_shift(int pass) { return (MODE == 0 ? 0 : 2
 // Status words of the pass live in array par = pass parity; each tile clears
 // its words in the other array for the next pass (which runs on the same or
 // fewer tiles of every block).
-constexpr size_t kScatterSmem = (size_t)kTile * 12 + (size_t)(kSortThreads / 32) * 256 * 4 + 2 * 256 * 4;
-// MODE 1 moves the words alone (Vin / Vout unused)
-constexpr size_t kScatterSmem1 = (size_t)kTile * 8 + (size_t)(kSortThreads / 32) * 256 * 4 + 2 * 256 * 4;
+constexpr size_t kScatterSmem = (size_t)kTile * 8 + (size_t)(kSortThreads / 32) * 256 * 4 + 2 * 256 * 4;
 constexpr int kSweepCtasPerSm = 3;
+constexpr int kLbBatch = 8;  // tiles read per look-back step
 
 template <int MODE>
 __global__ void __launch_bounds__(kSortThreads, kSweepCtasPerSm)
 radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockState *__restrict__ st,
-                   const uint64_t *__restrict__ Kin_all, const int32_t *__restrict__ Vin_all,
-                   uint64_t *__restrict__ Kout_all, int32_t *__restrict__ Vout_all,
+                   const uint64_t *__restrict__ Kin_all, uint64_t *__restrict__ Kout_all,
                    const uint32_t *__restrict__ dhist_all, uint32_t *__restrict__ lb_all, size_t lb_array_words,
                    long long budget) {
     constexpr int NW = kSortThreads / 32;
     extern __shared__ __align__(16) uint8_t smem[];
     uint64_t *sK = reinterpret_cast<uint64_t *>(smem);           // [kTile]
-    int32_t *sV = reinterpret_cast<int32_t *>(sK + kTile);        // [kTile], MODE 0
-    uint32_t *wcnt = reinterpret_cast<uint32_t *>(MODE == 0 ? reinterpret_cast<uint8_t *>(sV + kTile)
-                                                            : reinterpret_cast<uint8_t *>(sK + kTile));  // [NW][256]
+    uint32_t *wcnt = reinterpret_cast<uint32_t *>(sK + kTile);    // [NW][256]
     uint32_t *loff = wcnt + NW * 256;                             // [256] tile-local start of a digit
     uint32_t *gbase = loff + 256;                                 // [256] global start of the tile's run
     __shared__ uint32_t sh[33];
@@ -680,16 +615,13 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, d = threadIdx.x;
     const int shift = digit_shift<MODE>(pass);
     const uint32_t lt = lanemask_lt(), gt = lanemask_gt();
-    // the next work item is taken while the current one is sorted (its ticket
-    // is larger, so every tile still only waits on tiles taken before it)
-    int nxt = 0;
-    if (threadIdx.x == 0) nxt = atomicAdd(queue, 1);
     for (;;) {
+        // a tile is taken when its CTA can start on it: one taken ahead would
+        // keep the block's later tiles waiting for the CTA's current one
         if (threadIdx.x == 0) {
-            s_item = nxt;
+            s_item = atomicAdd(queue, 1);
             s_abort = ld_volatile_i32(rs + kRsAbort);
             s_fault = ld_volatile_i32(rs + kRsFault);
-            nxt = atomicAdd(queue, 1);
         }
         for (int i = threadIdx.x; i < NW * 256; i += kSortThreads) wcnt[i] = 0;
         __syncthreads();
@@ -700,21 +632,16 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
             __syncthreads();
             continue;
         }
-        const int n = sort_count<MODE>(st[b], h);
+        const int n = sort_count<MODE>(st[b], h, 1);
         const size_t bo = (size_t)b * kBlockCap;
-        // phase 1: the block's elements with a smaller digit (row 1, see sort_items_kernel)
-        const uint32_t below1 = MODE == 0 ? dhist_all[((size_t)b * kSweepPasses + 1) * 256 + d] : 0u;
         const uint64_t *Kin = Kin_all + bo;
-        const int32_t *Vin = Vin_all + bo;
         uint64_t keys[kPerThread];
-        int32_t vals[kPerThread];
         uint32_t rnk[kPerThread];
 #pragma unroll
         for (int r = 0; r < kPerThread; r++) {
             const int k = tile * kTile + w * 512 + r * 32 + lane;
             const bool ok = k < n;
             keys[r] = ok ? Kin[k] : 0;
-            vals[r] = (MODE == 0 && ok) ? Vin[k] : 0;
             const uint32_t dg = (uint32_t)(keys[r] >> shift) & 255u;
             const uint32_t mm = __match_any_sync(LFC_FULL, ok ? dg : 256u + lane);
             uint32_t before = 0;
@@ -740,16 +667,25 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
         uint32_t excl = 0;
         bool gave_up = false;
         if (tile > 0) {
+            // kLbBatch tiles back per step: their words are independent loads
             const long long t0 = clock64();
             int tp = tile - 1;
-            for (;;) {
-                const uint32_t sv = ld_status(lbb + (size_t)tp * 256 + d);
-                if (sv & (kLbAgg | kLbIncl)) {
-                    excl += sv & kLbCount;
-                    if ((sv & kLbIncl) || tp == 0) break;
-                    tp--;
-                    continue;
+            bool found = false;
+            while (!found && !gave_up) {
+                uint32_t sv[kLbBatch];
+#pragma unroll
+                for (int i = 0; i < kLbBatch; i++) sv[i] = tp - i >= 0 ? ld_status(lbb + (size_t)(tp - i) * 256 + d) : 0u;
+                int taken = 0;
+#pragma unroll
+                for (int i = 0; i < kLbBatch; i++) {
+                    if (found || taken != i || !(sv[i] & (kLbAgg | kLbIncl))) continue;
+                    excl += sv[i] & kLbCount;
+                    taken = i + 1;
+                    found = (sv[i] & kLbIncl) || tp - i == 0;
                 }
+                if (found) break;
+                tp -= taken;
+                if (taken) continue;
                 if (ld_volatile_i32(rs + kRsAbort)) { gave_up = true; break; }
                 if (clock64() - t0 > budget) {
                     gave_up = true;
@@ -762,9 +698,8 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
             if (!gave_up) st_status(lbb + (size_t)tile * 256 + d, kLbIncl | (excl + cnt_d));
         }
         lb_next[(size_t)b * kLbBlockWords + (size_t)tile * 256 + d] = 0;
-        const uint32_t below = MODE == 0 ? below1
-                                         : block_excl_sum<uint32_t>(dhist_all[((size_t)b * kSweepPasses + pass) * 256 + d],
-                                                                    sh, nullptr);  // block elements with a smaller digit
+        const uint32_t below = block_excl_sum<uint32_t>(dhist_all[((size_t)b * kSweepPasses + pass) * 256 + d], sh,
+                                                        nullptr);  // block elements with a smaller digit
         gbase[d] = below + excl;
         if (withhold && d == 0) atomicExch(rs + kRsFault, 0);  // the fault fires once
         if (__syncthreads_or(gave_up)) break;
@@ -774,12 +709,10 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
             const uint32_t dg = (uint32_t)(keys[r] >> shift) & 255u;
             const uint32_t pos = loff[dg] + wcnt[w * 256 + dg] + rnk[r];
             sK[pos] = keys[r];
-            if (MODE == 0) sV[pos] = vals[r];
         }
         __syncthreads();
         const int cnt = min(kTile, n - tile * kTile);
         uint64_t *Kout = Kout_all + bo;
-        int32_t *Vout = Vout_all + bo;
 #pragma unroll 4
         for (int r = 0; r < kPerThread; r++) {
             const int j = r * kSortThreads + threadIdx.x;
@@ -788,7 +721,6 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
                 const uint32_t dg = (uint32_t)(key >> shift) & 255u;
                 const uint32_t g = gbase[dg] + ((uint32_t)j - loff[dg]);
                 Kout[g] = key;
-                if (MODE == 0) Vout[g] = sV[j];
             }
         }
         __syncthreads();
@@ -796,45 +728,47 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
 }
 
 // ---------------------------------------------------------- group heads
-// Head flags come from neighbouring keys of the sorted (key, element) list:
-// the 8-byte prefixes after phase 1, the 40-bit round keys after a round.
+// Head flags: after phase 1 (MODE 0, flagged blocks) bit 31 of the suffix
+// array is set on the elements that are not heads; after a round they come
+// from neighbouring round words.
 // Pass A: per tile, the largest head position and the number of elements
 // that stay tied. Head flags go to flags[] for pass B.
 template <int MODE>
 __global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
-                                                                  const uint64_t *__restrict__ keys_all, const int32_t *__restrict__ actA,
-                                                                  const int32_t *__restrict__ actB,
+                                                                  const int32_t *__restrict__ bflag,
+                                                                  const uint64_t *__restrict__ keys_all, const int32_t *__restrict__ sa_all,
+                                                                  const int32_t *__restrict__ actA, const int32_t *__restrict__ actB,
                                                                   uint8_t *__restrict__ flags_all, int32_t *__restrict__ aux_all) {
     if (rs[kRsAbort]) return;
     const int b = blockIdx.y, tile = blockIdx.x;
     const int h = round_h<MODE>(rs);
     const BlockState s = st[b];
-    const int n = sort_count<MODE>(s, h);
+    const int n = sort_count<MODE>(s, h, bflag[b]);
     if (tile * kTile >= n) return;
     const uint64_t *K = keys_all + (size_t)b * kBlockCap;
-    const int32_t *act = ((MODE == 1 && (rs[3] & 1)) ? actB : actA) + (size_t)b * kBlockCap;
+    const int32_t *sa = sa_all + (size_t)b * kBlockCap;
+    const int32_t *act = ((MODE == 1 && (rs[kRsRound] & 1)) ? actB : actA) + (size_t)b * kBlockCap;
     uint8_t *flags = flags_all + (size_t)b * kBlockCap;
     const int k0 = tile * kTile + threadIdx.x * kPerThread;
     int hmax = -1, tied = 0;
-    const int ks = MODE == 0 ? 0 : 20;  // round words carry the element below the key
-    if (k0 + kPerThread <= n) {  // full run: 16-byte loads of the keys, one 16-byte store of the flags
+    if (MODE == 1 && k0 + kPerThread <= n) {  // full run: 16-byte loads of the words, one 16-byte store of the flags
         uint64_t kk[kPerThread];
         const ulonglong2 *K2 = reinterpret_cast<const ulonglong2 *>(K + k0);
 #pragma unroll
         for (int q = 0; q < kPerThread / 2; q++) {
             const ulonglong2 v = K2[q];
-            kk[2 * q] = v.x >> ks;
-            kk[2 * q + 1] = v.y >> ks;
+            kk[2 * q] = v.x >> 20;
+            kk[2 * q + 1] = v.y >> 20;
         }
-        const bool last_head = k0 + kPerThread >= n || (K[k0 + kPerThread] >> ks) != kk[kPerThread - 1];
-        bool curhead = (k0 == 0) || kk[0] != (K[k0 - (k0 > 0)] >> ks);
+        const bool last_head = k0 + kPerThread >= n || (K[k0 + kPerThread] >> 20) != kk[kPerThread - 1];
+        bool curhead = (k0 == 0) || kk[0] != (K[k0 - (k0 > 0)] >> 20);
         uint32_t fl[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int q = 0; q < kPerThread; q++) {
             const bool nexthead = q + 1 < kPerThread ? kk[q + 1] != kk[q] : last_head;
             if (curhead) {
                 fl[q >> 2] |= 1u << (8 * (q & 3));
-                hmax = MODE == 0 ? k0 + q : act[k0 + q];
+                hmax = act[k0 + q];
             }
             tied += !(curhead && nexthead);
             curhead = nexthead;
@@ -842,21 +776,12 @@ __global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(const int32_t 
         *reinterpret_cast<uint4 *>(flags + k0) = make_uint4(fl[0], fl[1], fl[2], fl[3]);
     } else if (k0 < n) {
         const int k1 = min(n, k0 + kPerThread);
-        uint64_t prevk = k0 > 0 ? K[k0 - 1] >> ks : 0;
-        uint64_t cur = K[k0] >> ks;
-        bool curhead = (k0 == 0) || cur != prevk;
         for (int k = k0; k < k1; k++) {
-            bool nexthead = true;
-            uint64_t nk = 0;
-            if (k + 1 < n) {
-                nk = K[k + 1] >> ks;
-                nexthead = nk != cur;
-            }
-            flags[k] = (uint8_t)curhead;
-            if (curhead) hmax = MODE == 0 ? k : act[k];
-            tied += !(curhead && nexthead);
-            cur = nk;
-            curhead = nexthead;
+            const bool cur = MODE == 0 ? sa[k] >= 0 : (k == 0 || (K[k] >> 20) != (K[k - 1] >> 20));
+            const bool nxt = k + 1 >= n || (MODE == 0 ? sa[k + 1] >= 0 : (K[k + 1] >> 20) != (K[k] >> 20));
+            flags[k] = (uint8_t)cur;
+            if (cur) hmax = MODE == 0 ? k : act[k];
+            tied += !(cur && nxt);
         }
     }
     int mine = hmax;  // last head position among this thread's elements
@@ -877,14 +802,15 @@ __global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(const int32_t 
 // Pass across tiles of a block: exclusive max of head positions, exclusive
 // sum of tied counts, total tied count of the block.
 template <int MODE>
-__global__ void __launch_bounds__(256) heads_scan_kernel(int32_t *__restrict__ rs, BlockState *__restrict__ st, int32_t *__restrict__ aux_all) {
+__global__ void __launch_bounds__(256) heads_scan_kernel(int32_t *__restrict__ rs, BlockState *__restrict__ st,
+                                                         const int32_t *__restrict__ bflag, int32_t *__restrict__ aux_all) {
     __shared__ int32_t shm[33];
     __shared__ int32_t shs[33];
     if (rs[kRsAbort]) return;
     const int b = blockIdx.x;
     const int h = round_h<MODE>(rs);
     int32_t *counters = rs;
-    const int n = sort_count<MODE>(st[b], h);
+    const int n = sort_count<MODE>(st[b], h, bflag[b]);
     int32_t *aux = aux_all + (size_t)b * kTilesPerBlock * 4;
     const int nt = (n + kTile - 1) / kTile;
     // nt <= 220 < 256: one tile per thread
@@ -913,7 +839,7 @@ __device__ __forceinline__ int pad32(int i) { return i + (i >> 5); }  // conflic
 
 template <int MODE>
 __global__ void __launch_bounds__(kSortThreads) heads_apply_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
-                                                                   const int32_t *__restrict__ sorted_all, const uint64_t *__restrict__ words_all,
+                                                                   const int32_t *__restrict__ bflag, const uint64_t *__restrict__ words_all,
                                                                    int32_t *__restrict__ actA,
                                                                    int32_t *__restrict__ actB,
                                                                    const uint8_t *__restrict__ flags_all, const int32_t *__restrict__ aux_all,
@@ -928,14 +854,13 @@ __global__ void __launch_bounds__(kSortThreads) heads_apply_kernel(const int32_t
     const int h = round_h<MODE>(rs);
     // round r reads list A (r even) or B (r odd) and writes the other; the
     // initial pass (MODE 0) writes A, which round 0 reads
-    const bool odd = MODE == 1 && (rs[3] & 1);
+    const bool odd = MODE == 1 && (rs[kRsRound] & 1);
     const int32_t *act_all = odd ? actB : actA;
     int32_t *act_out_all = MODE == 0 ? actA : (odd ? actA : actB);
     const BlockState s = st[b];
-    const int n = sort_count<MODE>(s, h);
+    const int n = sort_count<MODE>(s, h, bflag[b]);
     if (tile * kTile >= n) return;
     const size_t bo = (size_t)b * kBlockCap;
-    const int32_t *sorted = sorted_all + bo;   // MODE 0: the suffix array
     const uint64_t *words = words_all + bo;    // MODE 1: sorted round words
     const int32_t *act = act_all + bo;
     const uint8_t *flags = flags_all + bo;
@@ -1009,9 +934,9 @@ __global__ void __launch_bounds__(kSortThreads) heads_apply_kernel(const int32_t
     for (int j = threadIdx.x; j < cnt; j += kSortThreads) {
         const int k = t0 + j;
         const int pos = MODE == 0 ? k : act[k];
-        const int32_t v = MODE == 0 ? sorted[k] : (int32_t)(words[k] & kElemMask);
+        const int32_t v = MODE == 0 ? (sa[k] & 0x7FFFFFFF) : (int32_t)(words[k] & kElemMask);
         rank[v] = s_head[pad32(j)];
-        if (MODE == 1 || sorted != sa) sa[pos] = v;
+        sa[pos] = v;
         const int o = s_off[pad32(j)];
         if (o >= 0) {
             act_out[o] = pos;
@@ -1025,34 +950,45 @@ __global__ void commit_round_kernel(BlockState *st, int nblocks) {
     if (b < nblocks) { st[b].n_act = st[b].n_act_next; st[b].n_act_next = 0; }
 }
 
-__global__ void round_start_kernel(int32_t *rs, int first) {
-    rs[0] = 0;
-    rs[1] = 0;
-    if (first) { rs[2] = kPhase1Bytes; rs[3] = 0; }
+__global__ void round_start_kernel(int32_t *rs) {
+    rs[kRsTied] = 0;
+    rs[kRsTiedMax] = 0;
+}
+
+// Inside a graph: which of the conditional nodes run. The blocks' flags
+// decide on the LSD passes and the group heads; their tied elements on the
+// first round.
+__global__ void flags_cond_kernel(const int32_t *rs, cudaGraphConditionalHandle over, cudaGraphConditionalHandle flagged) {
+    cudaGraphSetConditional(over, rs[kRsOver] > 0 ? 1u : 0u);
+    cudaGraphSetConditional(flagged, rs[kRsFlagged] > 0 ? 1u : 0u);
+}
+__global__ void rounds_cond_kernel(const int32_t *rs, int max_m, cudaGraphConditionalHandle rounds) {
+    cudaGraphSetConditional(rounds, (rs[kRsAbort] == 0 && rs[kRsTied] > 0 && rs[kRsH] < max_m) ? 1u : 0u);
 }
 
 // End of a doubling round: double h; inside a graph, continue the WHILE node
 // while tied elements remain, h is below the largest block length and no
 // wait has given up.
 __global__ void round_end_kernel(int32_t *rs, int max_m, cudaGraphConditionalHandle cond, int set_cond) {
-    rs[2] *= 2;
-    rs[3] += 1;
-    if (set_cond) cudaGraphSetConditional(cond, (rs[kRsAbort] == 0 && rs[0] > 0 && rs[2] < max_m) ? 1u : 0u);
+    rs[kRsH] *= 2;
+    rs[kRsRound] += 1;
+    if (set_cond) cudaGraphSetConditional(cond, (rs[kRsAbort] == 0 && rs[kRsTied] > 0 && rs[kRsH] < max_m) ? 1u : 0u);
 }
 
-// L[j] = block[(SA[j] - 1) mod m]; origPtr = j with SA[j] = 0; bytes in use.
+// Bytes in use, and for flagged blocks L[j] = block[(SA[j] - 1) mod m] and
+// origPtr = j with SA[j] = 0 (the bucket sort has written both for the others).
 // Each CTA also writes the MTF summary of its 4096-byte segment of L: the
 // distinct bytes ordered by last occurrence, latest first. Thread = 16
 // consecutive positions; the last position of each byte value comes from one
 // shared-memory max per distinct value of a thread's run; each value is then
 // marked at its last position and the marks are compacted from the top.
-// After an aborted sort the suffix array is incomplete: the kernel then
-// takes the identity order instead, so that every later stage still reads
+// After an aborted sort a flagged block's suffix array is incomplete: the
+// kernel then takes the identity order instead, so that every later stage still reads
 // in-range values (the call reports LFC_ERR_TIMEOUT and its output is void).
 __global__ void __launch_bounds__(kSortThreads) bwt_output_kernel(BlockState *__restrict__ st, const int32_t *__restrict__ sa_all,
                                                                   const uint8_t *__restrict__ rle_all, uint8_t *__restrict__ L_all,
                                                                   uint8_t *__restrict__ rec_all, int32_t *__restrict__ reclen_all,
-                                                                  const int32_t *__restrict__ rs) {
+                                                                  const int32_t *__restrict__ rs, const int32_t *__restrict__ bflag) {
     __shared__ int32_t lastpos[256];
     __shared__ uint16_t mark[kTile];  // value + 1 at its last position, 0 elsewhere
     __shared__ int sh[33];
@@ -1066,40 +1002,24 @@ __global__ void __launch_bounds__(kSortThreads) bwt_output_kernel(BlockState *__
     const int jl = (int)threadIdx.x * kPerThread;  // tile-local start of the thread's run
     const int j0 = tile * kTile + jl;
     uint8_t c[kPerThread];
-    int32_t sv[kPerThread];
-    if (rs[kRsAbort]) {
+    if (!bflag[b]) {
+        if (j0 + kPerThread <= m) {
+            *reinterpret_cast<uint4 *>(c) = *reinterpret_cast<const uint4 *>(L_all + bo + j0);
+        } else {
 #pragma unroll
-        for (int q = 0; q < kPerThread; q++) sv[q] = j0 + q < m ? j0 + q : -1;
-    } else if (j0 + kPerThread <= m) {  // full run: the suffix array by 16-byte loads
-#pragma unroll
-        for (int q = 0; q < kPerThread; q += 4) {
-            const int4 s4 = *reinterpret_cast<const int4 *>(sa_all + bo + j0 + q);
-            sv[q] = s4.x; sv[q + 1] = s4.y; sv[q + 2] = s4.z; sv[q + 3] = s4.w;
+            for (int q = 0; q < kPerThread; q++) c[q] = j0 + q < m ? L_all[bo + j0 + q] : 0;
         }
     } else {
+        const bool identity = rs[kRsAbort] != 0;
 #pragma unroll
-        for (int q = 0; q < kPerThread; q++) sv[q] = j0 + q < m ? sa_all[bo + j0 + q] : -1;
-    }
-#pragma unroll
-    for (int q = 0; q < kPerThread; q++) {
-        const int v = sv[q];
-        c[q] = 0;
-        if (v >= 0) {
+        for (int q = 0; q < kPerThread; q++) {
+            c[q] = 0;
+            if (j0 + q >= m) continue;
+            const int v = identity ? j0 + q : sa_all[bo + j0 + q];
             c[q] = rle_all[bo + (v == 0 ? m - 1 : v - 1)];
             if (v == 0) st[b].orig_ptr = j0 + q;
+            L_all[bo + j0 + q] = c[q];
         }
-    }
-    if (j0 + kPerThread <= m) {
-        uint32_t pk[4];
-#pragma unroll
-        for (int w = 0; w < 4; w++)
-            pk[w] = (uint32_t)c[4 * w] | ((uint32_t)c[4 * w + 1] << 8) | ((uint32_t)c[4 * w + 2] << 16) |
-                    ((uint32_t)c[4 * w + 3] << 24);
-        *reinterpret_cast<uint4 *>(L_all + bo + j0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    } else {
-#pragma unroll
-        for (int q = 0; q < kPerThread; q++)
-            if (j0 + q < m) L_all[bo + j0 + q] = c[q];
     }
 #pragma unroll
     for (int q = kPerThread - 1; q >= 0; q--) {  // last occurrence in the run first
@@ -1154,12 +1074,10 @@ cudaError_t launch_copy_bwt(lfc_plan P, int nblocks, uint8_t *d_L, size_t stride
 }
 
 template <int MODE>
-static void sweep_pass(lfc_plan P, cudaStream_t st, int nblocks, int ctas, int pass, const uint64_t *kin, const int32_t *vin,
-                       uint64_t *kout, int32_t *vout) {
+static void sweep_pass(lfc_plan P, cudaStream_t st, int nblocks, int ctas, int pass, const uint64_t *kin, uint64_t *kout) {
     Workspace &ws = P->ws;
-    radix_sweep_kernel<MODE><<<ctas, kSortThreads, MODE == 0 ? kScatterSmem : kScatterSmem1, st>>>(
-        pass, nblocks, ws.act_total, ws.bstate, kin, vin, kout, vout, ws.dhist, ws.lbstat, ws.lbstat_words,
-        P->wait_cycles);
+    radix_sweep_kernel<MODE><<<ctas, kSortThreads, kScatterSmem, st>>>(
+        pass, nblocks, ws.act_total, ws.bstate, kin, kout, ws.dhist, ws.lbstat, ws.lbstat_words, P->wait_cycles);
     count_launches(P, 1);
 }
 
@@ -1169,12 +1087,43 @@ static int sweep_ctas(lfc_plan P, int nblocks, int tiles) {
     return (int)std::max<long long>(1, std::min(items, cap));
 }
 
+// The LSD passes of the kFlagOver blocks: keys2 -> keys -> ... -> keys2.
+static void bwt_over(lfc_plan P, cudaStream_t st, int nblocks, int tiles) {
+    Workspace &ws = P->ws;
+    const size_t nd = (size_t)nblocks * kSweepPasses * 256;
+    const dim3 grid(tiles, nblocks);
+    zero_u32_kernel<<<(unsigned)std::min<size_t>(64, (nd + 255) / 256), 256, 0, st>>>(ws.dhist, nd);
+    sweep_digits_kernel<0><<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys2, ws.dhist, ws.bflag, ws.lbstat,
+                                                          ws.lbstat_words);
+    sort_items_kernel<0><<<1, 1024, 0, st>>>(ws.act_total, ws.bstate, nblocks, ws.bflag);
+    const int ctas = sweep_ctas(P, nblocks, tiles);
+    for (int pass = 0; pass < 8; pass++) {
+        if (pass & 1) sweep_pass<0>(P, st, nblocks, ctas, pass, ws.keys, ws.keys2);
+        else sweep_pass<0>(P, st, nblocks, ctas, pass, ws.keys2, ws.keys);
+    }
+    over_heads_kernel<<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys2, ws.bflag, ws.sa);
+    count_launches(P, 4);
+}
+
+// Group heads, ranks and the tied elements of the flagged blocks.
+static void bwt_heads(lfc_plan P, cudaStream_t st, int nblocks, int tiles) {
+    Workspace &ws = P->ws;
+    const dim3 grid(tiles, nblocks);
+    heads_tile_kernel<0><<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.keys2, ws.sa, ws.act, ws.act2,
+                                                        ws.bwt, ws.tileaux);
+    heads_scan_kernel<0><<<nblocks, 256, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.tileaux);
+    heads_apply_kernel<0><<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.keys2, ws.act, ws.act2, ws.bwt,
+                                                         ws.tileaux, ws.rank, ws.sa, ws.val);
+    commit_round_kernel<<<(nblocks + 255) / 256, 256, 0, st>>>(ws.bstate, nblocks);
+    count_launches(P, 4);
+}
+
 // One prefix-doubling round over the tied elements (h and the parity of the
 // active lists come from the round state in device memory).
 static void bwt_round(lfc_plan P, cudaStream_t st, int nblocks, int tiles, int max_m, cudaGraphConditionalHandle cond,
                       int set_cond) {
     Workspace &ws = P->ws;
-    round_start_kernel<<<1, 1, 0, st>>>(ws.act_total, 0);
+    round_start_kernel<<<1, 1, 0, st>>>(ws.act_total);
     const size_t nd = (size_t)nblocks * kSweepPasses * 256;
     zero_u32_kernel<<<(unsigned)std::min<size_t>(64, (nd + 255) / 256), 256, 0, st>>>(ws.dhist, nd);
     dim3 g1(tiles, nblocks);
@@ -1183,22 +1132,51 @@ static void bwt_round(lfc_plan P, cudaStream_t st, int nblocks, int tiles, int m
     // longer group are flagged and take the 5 LSD passes over bits 20..59 of
     // the words instead: keys -> keys2 -> ... -> keys2
     segsort_kernel<<<g1, kSegThreads, kSegSmem, st>>>(ws.act_total, ws.bstate, ws.keys, ws.keys2, ws.segbig);
-    round_digits_kernel<<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys, ws.dhist, ws.segbig);
-    sort_items_kernel<1><<<1, 1024, 0, st>>>(ws.act_total, ws.bstate, nblocks, ws.segbig, nullptr);
+    sweep_digits_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys, ws.dhist, ws.segbig, ws.lbstat,
+                                                        ws.lbstat_words);
+    sort_items_kernel<1><<<1, 1024, 0, st>>>(ws.act_total, ws.bstate, nblocks, ws.segbig);
     count_launches(P, 6);
     const int ctas = sweep_ctas(P, nblocks, tiles);
     for (int pass = 0; pass < 5; pass++) {
-        if (pass & 1) sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys2, nullptr, ws.keys, nullptr);
-        else sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys, nullptr, ws.keys2, nullptr);
+        if (pass & 1) sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys2, ws.keys);
+        else sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys, ws.keys2);
     }
-    heads_tile_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys2, ws.act, ws.act2, ws.bwt,
-                                                      ws.tileaux);
-    heads_scan_kernel<1><<<nblocks, 256, 0, st>>>(ws.act_total, ws.bstate, ws.tileaux);
-    heads_apply_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, nullptr, ws.keys2, ws.act, ws.act2,
-                                                       ws.bwt, ws.tileaux, ws.rank, ws.sa, ws.val);
+    heads_tile_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.keys2, ws.sa, ws.act, ws.act2,
+                                                      ws.bwt, ws.tileaux);
+    heads_scan_kernel<1><<<nblocks, 256, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.tileaux);
+    heads_apply_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.keys2, ws.act, ws.act2, ws.bwt,
+                                                       ws.tileaux, ws.rank, ws.sa, ws.val);
     commit_round_kernel<<<(nblocks + 255) / 256, 256, 0, st>>>(ws.bstate, nblocks);
     round_end_kernel<<<1, 1, 0, st>>>(ws.act_total, max_m, cond, set_cond);
     count_launches(P, 5);
+}
+
+// Adds a conditional node behind the capture's current end and starts the
+// capture of its body on the plan's auxiliary stream.
+static cudaError_t begin_cond(lfc_plan P, cudaStream_t s, cudaGraphConditionalHandle handle, cudaGraphConditionalNodeType type,
+                              cudaGraphNode_t *node, cudaGraph_t *body) {
+    cudaStreamCaptureStatus cap;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edata = nullptr;
+    size_t ndeps = 0;
+    cudaGraph_t cg = nullptr;
+    unsigned long long cid = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &cap, &cid, &cg, &deps, &edata, &ndeps);
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams np = {};
+    np.type = cudaGraphNodeTypeConditional;
+    np.conditional.handle = handle;
+    np.conditional.type = type;
+    np.conditional.size = 1;
+    e = cudaGraphAddNode(node, cg, deps, edata, ndeps, &np);
+    if (e != cudaSuccess) return e;
+    *body = np.conditional.phGraph_out[0];
+    return cudaStreamBeginCaptureToGraph(P->aux_stream, *body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
+}
+static cudaError_t end_cond(lfc_plan P, cudaStream_t s, cudaGraphNode_t *node, cudaGraph_t *body) {
+    cudaError_t e = cudaStreamEndCapture(P->aux_stream, body);
+    if (e != cudaSuccess) return e;
+    return cudaStreamUpdateCaptureDependencies(s, node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
 cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m) {
@@ -1213,95 +1191,74 @@ cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m) {
     const bool graph = cap == cudaStreamCaptureStatusActive;
     e = cudaFuncSetAttribute(radix_sweep_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(radix_sweep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem1);
+        e = cudaFuncSetAttribute(radix_sweep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(segsort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSegSmem);
+    if (e == cudaSuccess) e = launch_bucket_sort(P, nblocks, max_m, graph);
     if (e != cudaSuccess) return e;
-    // a new suffix sort: no wait has given up yet (outside graphs the sticky
-    // status is reported by this call, so it starts clear as well)
-    e = cudaMemsetAsync(ws.act_total + kRsAbort, 0, sizeof(int32_t), s);
-    if (e == cudaSuccess && !graph) e = cudaMemsetAsync(ws.act_total + kRsSticky, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess) return e;
-    // phase 1: prefix keys and the digit totals of all passes, then 8 LSD
-    // passes (keys, sa) -> (keys2, sa2) -> ... -> (keys, sa)
-    stage_begin(P, LFC_STAGE_BWT_KEYS);
-    dim3 grid(tiles, nblocks);
-    const size_t nd = (size_t)nblocks * kSweepPasses * 256;
-    zero_u32_kernel<<<(unsigned)std::min<size_t>(64, (nd + 255) / 256), 256, 0, s>>>(ws.dhist, nd);
-    key8_kernel<<<grid, kSortThreads, 0, s>>>(ws.bstate, ws.rle, ws.keys, ws.sa, ws.dhist, ws.lbstat, ws.lbstat_words);
-    sort_items_kernel<0><<<1, 1024, 0, s>>>(ws.act_total, ws.bstate, nblocks, nullptr, ws.dhist);
-    count_launches(P, 3);
-    uint64_t *kin = ws.keys, *kout = ws.keys2;
-    int32_t *vin = ws.sa, *vout = ws.sa2;
-    stage_end(P, LFC_STAGE_BWT_KEYS);
-    stage_begin(P, LFC_STAGE_BWT_SORT8);
-    const int ctas = sweep_ctas(P, nblocks, tiles);
-    for (int pass = 8 - kPhase1Bytes; pass < 8; pass++) {
-        sweep_pass<0>(P, s, nblocks, ctas, pass, kin, vin, kout, vout);
-        std::swap(kin, kout);
-        std::swap(vin, vout);
-    }
-    stage_end(P, LFC_STAGE_BWT_SORT8);  // sorted keys / suffix array now in kin / vin
     stage_begin(P, LFC_STAGE_BWT_REFINE);
-    round_start_kernel<<<1, 1, 0, s>>>(ws.act_total, 1);
-    heads_tile_kernel<0><<<grid, kSortThreads, 0, s>>>(ws.act_total, ws.bstate, kin, ws.sa, ws.sa, ws.bwt, ws.tileaux);
-    heads_scan_kernel<0><<<nblocks, 256, 0, s>>>(ws.act_total, ws.bstate, ws.tileaux);
-    heads_apply_kernel<0><<<grid, kSortThreads, 0, s>>>(ws.act_total, ws.bstate, vin, nullptr, ws.act, ws.act2,
-                                                        ws.bwt, ws.tileaux, ws.rank, ws.sa, ws.val);
-    commit_round_kernel<<<(nblocks + 255) / 256, 256, 0, s>>>(ws.bstate, nblocks);
-    count_launches(P, 5);
     P->bwt_calls++;
     if (graph) {
-        // rounds as a WHILE node: the body is one round, its last kernel
-        // decides whether another round runs
+        // what the flagged blocks need as conditional nodes: the LSD passes,
+        // the group heads, and the rounds as a WHILE node whose body is one
+        // round, its last kernel deciding whether another one runs
+        cudaGraph_t cg = nullptr;
+        unsigned long long cid = 0;
         const cudaGraphNode_t *deps = nullptr;
         const cudaGraphEdgeData *edata = nullptr;
         size_t ndeps = 0;
-        cudaGraph_t cg = nullptr;
-        unsigned long long cid = 0;
         e = cudaStreamGetCaptureInfo(s, &cap, &cid, &cg, &deps, &edata, &ndeps);
+        cudaGraphConditionalHandle over, flagged, rounds;
+        if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&over, cg, 0, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&flagged, cg, 0, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&rounds, cg, 0, cudaGraphCondAssignDefault);
         if (e != cudaSuccess) return e;
-        cudaGraphConditionalHandle cond;
-        e = cudaGraphConditionalHandleCreate(&cond, cg, 1, cudaGraphCondAssignDefault);
-        if (e != cudaSuccess) return e;
-        cudaGraphNodeParams np = {};
-        np.type = cudaGraphNodeTypeConditional;
-        np.conditional.handle = cond;
-        np.conditional.type = cudaGraphCondTypeWhile;
-        np.conditional.size = 1;
         cudaGraphNode_t node;
-        e = cudaGraphAddNode(&node, cg, deps, edata, ndeps, &np);
+        cudaGraph_t body;
+        flags_cond_kernel<<<1, 1, 0, s>>>(ws.act_total, over, flagged);
+        e = begin_cond(P, s, over, cudaGraphCondTypeIf, &node, &body);
         if (e != cudaSuccess) return e;
-        cudaGraph_t body = np.conditional.phGraph_out[0];
-        e = cudaStreamBeginCaptureToGraph(P->aux_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
+        bwt_over(P, P->aux_stream, nblocks, tiles);
+        e = end_cond(P, s, &node, &body);
+        if (e == cudaSuccess) e = begin_cond(P, s, flagged, cudaGraphCondTypeIf, &node, &body);
         if (e != cudaSuccess) return e;
-        bwt_round(P, P->aux_stream, nblocks, kTilesPerBlock, max_m, cond, 1);
-        e = cudaStreamEndCapture(P->aux_stream, &body);
+        bwt_heads(P, P->aux_stream, nblocks, tiles);
+        e = end_cond(P, s, &node, &body);
         if (e != cudaSuccess) return e;
-        e = cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+        rounds_cond_kernel<<<1, 1, 0, s>>>(ws.act_total, max_m, rounds);
+        e = begin_cond(P, s, rounds, cudaGraphCondTypeWhile, &node, &body);
         if (e != cudaSuccess) return e;
+        bwt_round(P, P->aux_stream, nblocks, tiles, max_m, rounds, 1);
+        e = end_cond(P, s, &node, &body);
+        if (e != cudaSuccess) return e;
+        count_launches(P, 2);
     } else {
-        e = cudaMemcpyAsync(ws.h_act_total, ws.act_total, kSortCtlHead * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+        const int32_t *h = ws.h_act_total;
+        auto read_state = [&]() {
+            cudaError_t r = cudaMemcpyAsync(ws.h_act_total, ws.act_total, kSortCtlHead * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+            return r == cudaSuccess ? cudaStreamSynchronize(s) : r;
+        };
+        e = read_state();
         if (e != cudaSuccess) return e;
-        e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return e;
-        int round = 0;
-        for (int h = kPhase1Bytes; ws.h_act_total[kRsAbort] == 0 && ws.h_act_total[0] > 0 && h < max_m; h *= 2, round++) {
-            P->bwt_rounds++;
-            P->bwt_tied_total += ws.h_act_total[0];
-            if (round < 32) P->bwt_round_tied[round] += ws.h_act_total[0];
-            const int t1 = (ws.h_act_total[1] + kTile - 1) / kTile;
-            bwt_round(P, s, nblocks, t1, max_m, cudaGraphConditionalHandle{}, 0);
-            e = cudaMemcpyAsync(ws.h_act_total, ws.act_total, kSortCtlHead * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+        if (h[kRsFlagged] > 0) {
+            if (h[kRsOver] > 0) bwt_over(P, s, nblocks, tiles);
+            bwt_heads(P, s, nblocks, tiles);
+            e = read_state();
             if (e != cudaSuccess) return e;
-            e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess) return e;
+            for (int round = 0; h[kRsAbort] == 0 && h[kRsTied] > 0 && h[kRsH] < max_m; round++) {
+                P->bwt_rounds++;
+                P->bwt_tied_total += h[kRsTied];
+                if (round < 32) P->bwt_round_tied[round] += h[kRsTied];
+                bwt_round(P, s, nblocks, (h[kRsTiedMax] + kTile - 1) / kTile, max_m, cudaGraphConditionalHandle{}, 0);
+                e = read_state();
+                if (e != cudaSuccess) return e;
+            }
+            if (h[kRsAbort] != 0) P->bwt_timed_out = true;
         }
-        if (ws.h_act_total[kRsAbort] != 0) P->bwt_timed_out = true;
     }
     stage_end(P, LFC_STAGE_BWT_REFINE);
     stage_begin(P, LFC_STAGE_BWT_OUT);
-    bwt_output_kernel<<<grid, kSortThreads, 0, s>>>(ws.bstate, ws.sa, ws.rle, ws.bwt, ws.mtfrec, ws.mtfreclen,
-                                                     ws.act_total);
+    bwt_output_kernel<<<dim3(tiles, nblocks), kSortThreads, 0, s>>>(ws.bstate, ws.sa, ws.rle, ws.bwt, ws.mtfrec, ws.mtfreclen,
+                                                                    ws.act_total, ws.bflag);
     stage_end(P, LFC_STAGE_BWT_OUT);
     count_launches(P, 1);
     return cudaGetLastError();

@@ -25,11 +25,42 @@ constexpr int kMaxGroups = 6;
 constexpr int kMaxSelectors = 18002;
 constexpr int kHistBins = 65536;
 constexpr int kMaxCand = 104;                        // candidates per frame: 26 default ids x 2 byte layouts x 2 (temporal)
-constexpr int kSortCtlHead = 16;                     // sort state words before the per-block tile offsets
-constexpr int kSortFaultWord = 5;                    // sort state word of the fault-injection test hook
-constexpr int kSortStickyWord = 9;                   // sort state word kept until lfc_plan_device_status reads it
+
+// Sort state in device memory (rs): tied elements after a round, their
+// per-block maximum, the shift h, the round number; the abort word (nonzero
+// once a bounded wait has given up in this suffix sort: every later sort
+// kernel returns at once), the fault-injection word (test hook), the two work
+// queues of the radix passes (by pass parity), the work items of the current
+// pass, the sticky status (kept until the host reads it), the blocks the
+// bucket sort flagged and those with kFlagOver, the queues and item counts of
+// the bucket classes, the tied groups (short, long), and from kRsTileOff on the per-block tile counts.
+enum : int {
+    kRsTied = 0, kRsTiedMax = 1, kRsH = 2, kRsRound = 3, kRsAbort = 4, kRsFault = 5, kRsQueue = 6, kRsItems = 8,
+    kRsSticky = 9, kRsFlagged = 10, kRsOver = 11, kRsBucketQueue = 12, kRsBucketClasses = 3,
+    kRsBucketItems = kRsBucketQueue + kRsBucketClasses, kRsTies = kRsBucketItems + kRsBucketClasses,
+    kRsTiesLong = kRsTies + 1, kRsTileOff = kRsTiesLong + 1
+};
+constexpr int kSortCtlHead = kRsTileOff;             // sort state words before the per-block tile counts
+constexpr int kFlagTied = 1, kFlagOver = 2;          // block flags of the bucket sort (bwt_bucket.cu)
+constexpr uint64_t kElemMask = (1u << 20) - 1u;      // rotation start in a sort word, below its key
+constexpr int kCodeMax = 12;                         // longest code of the order-preserving byte code
+constexpr int kKeyBits = 44;                         // code bits in a sort word
+constexpr int kMinDepth = kKeyBits / kCodeMax;       // bytes that rotations with equal keys share at least
+constexpr int kBuckets = 1408;                       // most buckets of a block
+constexpr int kBucketRow = kBuckets + 8;             // bucket starts of a block (one more than buckets)
 
 #define LFC_FULL 0xffffffffu
+
+// One block's byte codes (length << 12 | code; after a zero byte, after
+// another byte, first byte of a key), the first bucket of every 12-bit key
+// prefix, and the 16-bit key prefix where each bucket starts.
+struct BwtCode {
+    uint16_t code[3 * 256];
+    uint16_t base12[4104];  // 4097 used
+    uint16_t split[kBuckets];
+    int32_t nb, pad[3];
+};
+static_assert(sizeof(BwtCode) % 16 == 0, "BwtCode rows stay 16-byte aligned");
 
 // ------------------------------------------------------------ warp helpers
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
@@ -200,13 +231,19 @@ struct Workspace {
     int32_t *act = nullptr;        // active SA positions
     int32_t *act2 = nullptr;
     int32_t *val = nullptr;        // SA values of the active elements
-    int32_t *val2 = nullptr;
-    uint64_t *keys = nullptr;      // sort keys riding with sa / val, block_cap * kBlockCap
+    uint64_t *keys = nullptr;      // sort words, block_cap * kBlockCap
     uint64_t *keys2 = nullptr;
     uint32_t *lbstat = nullptr;    // radix look-back status, 2 arrays of block_cap * kTilesPerBlock * 256
     size_t lbstat_words = 0;       // words of one of those arrays
     uint32_t *dhist = nullptr;     // per block and radix pass: digit totals, block_cap * 8 * 256
     int32_t *segbig = nullptr;     // per block: a doubling round has a group longer than the segmented sort's window
+    BwtCode *bcode = nullptr;      // bucket sort: byte code and splitters per block
+    uint32_t *bcount = nullptr;    // rotations per bucket, block_cap * kBuckets
+    uint32_t *bcursor = nullptr;   // scatter cursors, same shape
+    uint32_t *bstart = nullptr;    // bucket starts, block_cap * kBucketRow
+    uint32_t *bitems = nullptr;    // bucket work lists, one of bitems_cap entries per size class
+    size_t bitems_cap = 0;
+    int32_t *bflag = nullptr;      // kFlag* per block
     int32_t *tileaux = nullptr;    // block_cap * kTilesPerBlock * 4
     uint8_t *bwt = nullptr;        // L column
     uint8_t *mtfidx = nullptr;
@@ -328,6 +365,8 @@ cudaError_t launch_range_crc(lfc_plan P, const uint8_t *const *h_ptr, const int6
 // bwt.cu
 cudaError_t launch_rle1(lfc_plan P, int nblocks, const BlockDesc *d_blocks);
 cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m);
+// bwt_bucket.cu: sorts every block's rotations, writes last columns; flags the blocks it could not finish
+cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph);
 cudaError_t launch_copy_bwt(lfc_plan P, int nblocks, uint8_t *d_L, size_t stride, uint32_t *d_len, uint32_t *d_orig);
 
 // mtf_huff.cu
