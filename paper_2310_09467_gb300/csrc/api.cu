@@ -12,6 +12,9 @@ using namespace lfc;
 namespace {
 
 constexpr int kJudgeFramesCap = 16;
+// the decoder never reads a stream past its 18002 selectors, six tables and
+// 18002 groups of 50 codes of at most 20 bits
+constexpr int64_t kMaxStreamRead = 3000000;
 constexpr int kDefaultWaitMs = 1000;  // bounded device waits give up after this long
 
 int fail(lfc_plan P, int code, const std::string &what, cudaError_t e = cudaSuccess) {
@@ -1084,7 +1087,7 @@ extern "C" int lfc_decompress(lfc_plan P, const uint8_t *const *h_in, const uint
             for (int k = 0; k < H.nb; k++) {
                 DecBlockHost d;
                 d.src = h_in[f1] + off;
-                d.src_len = H.sizes[k];
+                d.src_len = std::min<int64_t>(H.sizes[k], kMaxStreamRead);
                 d.dst = ws.stream + (size_t)(f1 - f0) * ws.stream_slot + (size_t)k * H.bb;
                 d.expect = (int32_t)std::min<int64_t>(H.bb, nbytes - (int64_t)k * H.bb);
                 d.pad = 0;
@@ -1094,26 +1097,44 @@ extern "C" int lfc_decompress(lfc_plan P, const uint8_t *const *h_in, const uint
             f1++;
         }
         if (f1 - f0 > P->cfg.max_frames) return fail(P, LFC_ERR_INVALID_ARG, "too many frames");
+        // block table | CRC run over the blocks' outputs | frames | CRC run over the frames
         const int nb = (int)blocks.size();
-        CK(cudaMemcpyAsync(ws.chunk_desc, blocks.data(), sizeof(DecBlockHost) * nb, cudaMemcpyHostToDevice, P->stream));
-        CK(launch_bzip2_decode(P, ws.chunk_desc, nb, d_status));
+        Arena A;
+        const size_t off_blocks = A.put(blocks.data(), sizeof(DecBlockHost) * nb);
+        std::vector<const uint8_t *> bptr(nb), outp;
+        std::vector<int64_t> blen(nb), outl;
+        for (int k = 0; k < nb; k++) {
+            bptr[k] = blocks[k].dst;
+            blen[k] = blocks[k].expect;
+        }
+        CrcRun bcrc, fcrc;
+        const size_t off_bcrc = A.reserve(crc_table_bytes(crc_count_chunks(blen.data(), nb), nb));
+        crc_build_tables(bptr.data(), blen.data(), nb, A.host.data() + off_bcrc, &bcrc);
+        std::vector<InvFrame> inv;
+        int32_t *E = ws.rank;  // a frame's scratch field: at most half its blocks' bytes in elements
+        for (int i = f0; i < f1; i++) {
+            const Hdr &H = hd[i];
+            const uint16_t *Z = reinterpret_cast<const uint16_t *>(ws.stream + (size_t)(i - f0) * ws.stream_slot);
+            inv.push_back(InvFrame{Z, (H.id & 0x80) ? h_prev[i] : nullptr, h_out[i], E, H.W, H.H, H.p, H.id});
+            E += (size_t)H.W * H.H;
+            outp.push_back(reinterpret_cast<const uint8_t *>(h_out[i]));
+            outl.push_back(2LL * H.W * H.H);
+        }
+        const size_t off_inv = A.put(inv.data(), sizeof(InvFrame) * inv.size());
+        const size_t off_fcrc = A.reserve(crc_table_bytes(crc_count_chunks(outl.data(), f1 - f0), f1 - f0));
+        crc_build_tables(outp.data(), outl.data(), f1 - f0, A.host.data() + off_fcrc, &fcrc);
+        const int ra = stage_arena(P, A);
+        if (ra) return ra;
+        const uint8_t *d_arena = reinterpret_cast<const uint8_t *>(ws.chunk_desc);
+        CK(launch_bzip2_decode(P, blocks.data(), d_arena + off_blocks, nb, d_arena + off_bcrc, bcrc, d_status));
         std::vector<int32_t> st(nb);
         CK(cudaMemcpyAsync(st.data(), d_status, 4 * (size_t)nb, cudaMemcpyDeviceToHost, P->stream));
         CK(cudaStreamSynchronize(P->stream));
         for (int k = 0; k < nb; k++) {
             if (st[k] != 0) return fail(P, LFC_ERR_CORRUPT, "bzip2 block failed to decode (code " + std::to_string(st[k]) + ")");
         }
-        std::vector<const uint8_t *> outp;
-        std::vector<int64_t> outl;
-        for (int i = f0; i < f1; i++) {
-            const Hdr &H = hd[i];
-            const uint16_t *Z = reinterpret_cast<const uint16_t *>(ws.stream + (size_t)(i - f0) * ws.stream_slot);
-            const uint16_t *pv = (H.id & 0x80) ? h_prev[i] : nullptr;
-            CK(launch_inverse_predict(P, Z, pv, h_out[i], ws.rank, H.W, H.H, H.p, H.id));
-            outp.push_back(reinterpret_cast<const uint8_t *>(h_out[i]));
-            outl.push_back(2LL * H.W * H.H);
-        }
-        CK(launch_range_crc(P, outp.data(), outl.data(), f1 - f0, ws.frame_crc));
+        CK(launch_inverse_predict(P, inv.data(), reinterpret_cast<const InvFrame *>(d_arena + off_inv), f1 - f0));
+        CK(launch_crc(P, d_arena + off_fcrc, fcrc, ws.frame_crc, 1));
         std::vector<uint32_t> crc(f1 - f0);
         CK(cudaMemcpyAsync(crc.data(), ws.frame_crc, 4 * (size_t)(f1 - f0), cudaMemcpyDeviceToHost, P->stream));
         CK(cudaStreamSynchronize(P->stream));

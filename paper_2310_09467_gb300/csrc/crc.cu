@@ -186,30 +186,4 @@ cudaError_t launch_crc(lfc_plan P, const uint8_t *d_tables, const CrcRun &run, u
     return cudaGetLastError();
 }
 
-// Immediate form: stage the tables in the plan's descriptor buffer first.
-static cudaError_t run_ranges(lfc_plan P, const uint8_t *const *ptr, const int64_t *len, int n, uint32_t *out,
-                              int out_stride_words) {
-    const int nchunks = crc_count_chunks(len, n);
-    std::vector<uint8_t> blob(crc_table_bytes(nchunks, n));
-    CrcRun run;
-    crc_build_tables(ptr, len, n, blob.data(), &run);
-    if (blob.size() > P->ws.chunk_desc_bytes) return cudaErrorInvalidValue;
-    uint8_t *d = reinterpret_cast<uint8_t *>(P->ws.chunk_desc);
-    cudaError_t e = cudaMemcpyAsync(d, blob.data(), blob.size(), cudaMemcpyHostToDevice, P->stream);
-    if (e != cudaSuccess) return e;  // pageable source: staged before the call returns
-    return launch_crc(P, d, run, out, out_stride_words);
-}
-
-cudaError_t launch_block_crc(lfc_plan P, const BlockDesc *h_blocks, int nblocks, BlockState *d_state) {
-    std::vector<const uint8_t *> ptr(nblocks);
-    std::vector<int64_t> len(nblocks);
-    for (int b = 0; b < nblocks; b++) { ptr[b] = h_blocks[b].src; len[b] = h_blocks[b].len; }
-    static_assert(sizeof(BlockState) % 4 == 0, "BlockState words");
-    return run_ranges(P, ptr.data(), len.data(), nblocks, &d_state[0].crc, (int)(sizeof(BlockState) / 4));
-}
-
-cudaError_t launch_range_crc(lfc_plan P, const uint8_t *const *h_ptr, const int64_t *h_len, int n, uint32_t *d_out) {
-    return run_ranges(P, h_ptr, h_len, n, d_out, 1);
-}
-
 }  // namespace lfc

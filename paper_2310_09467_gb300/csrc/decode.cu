@@ -1,43 +1,42 @@
 // decode.cu -- decompression (Fig. 2b: unpack the header, bzip2-decode every
 // block, then the inverse predictor chosen by the header's id).
 //
-// One CTA per bzip2 stream. Every read of the coded stream is checked
-// against its length and every write against its buffer, so corrupt input
-// ends in an error flag, never an out-of-bounds access.
-//  1. thread 0: headers and tables; the CTA: Huffman lookup tables (a
-//     symbol per 10-bit prefix; whole-code counts and lengths per 12-bit
-//     prefix); thread 0 walks the groups of 50 codes for their bit offsets
-//     (EOB lies in the last group, as an encoder writes one selector per
-//     group it uses: a stream with more selectors is rejected as corrupt);
-//     every thread decodes whole groups into the symbol array; inverse
-//     RUNA/RUNB and MTF by 32 segments (each segment's moves permute list
-//     positions whatever the list holds: permutations first, then the lists
-//     at the segment starts in order, then every segment decoded) -> the BWT
-//     last column L;
-//  2. the CTA: LF mapping T[j] = C[L[j]] + rank of j among equal bytes (a
-//     stable counting sort of L with per-warp counters);
-//  3. 1024 walkers invert the BWT: each starts at its own row (walker 0 at
-//     origPtr), follows T until it meets another walker's start row, the
-//     pieces are chained from walker 0, and every walker re-walks its piece
-//     writing bytes from the end of the block backwards;
-//  4. the CTA: inverse RLE1 from sync points (one piece per thread), then
-//     CRC-32/BZIP2 of the output vs the stored block CRC.
+// Every step of a block is spread over many CTAs, so that one frame's few
+// blocks fill the GPU as well as a batch does. Every read of the coded stream
+// is checked against its length and every write against its buffer, so
+// corrupt input ends in an error flag, never an out-of-bounds access.
+//  1. Header (a CTA per block): selectors from the positions of the zero bits
+//     of their unary codes (a scan), their move-to-front as a scan over
+//     permutations of six tables; code lengths and lookup tables.
+//  2. Group offsets. A group is 50 codes of one table, so where it ends
+//     follows from where it starts. For every bit position and every table
+//     the length of 50 codes from there is computed in parallel (lengths of
+//     2, 4, 8 and 16 codes by doubling, in shared memory); then one thread
+//     per block only adds up a looked-up length per group (EOB lies in the
+//     last group, as an encoder writes one selector per group it uses: a
+//     stream with more selectors is rejected as corrupt).
+//  3. Every group's symbols, a thread per group.
+//  4. Inverse RUNA/RUNB and MTF by kSegs segments, a thread each with its
+//     256-byte list in shared memory: a segment's moves permute list
+//     positions whatever the list holds, so the permutations and output
+//     lengths come first, the segment-start lists and offsets are chained,
+//     and every segment is decoded from its list -> the BWT last column L.
+//  5. LF mapping by a stable counting sort over tiles; a word per row holds
+//     the next row and the row's byte.
+//  6. Inverse BWT: a walker per kWalkStep rows (and one at the origin) follows
+//     the rows until it meets another walker's start; the pieces are ranked
+//     along their list by pointer doubling; every walker writes its piece.
+//  7. Inverse RLE1 by tiles from sync points; block CRCs (crc.cu).
 #include <climits>
 
 #include "lfc_common.cuh"
 
 namespace lfc {
 
-constexpr int kDecThreads = 1024;
-constexpr int kWalkers = kDecThreads;
-constexpr uint32_t kPolyD = 0x04C11DB7u;
-
 enum : int32_t {
     DEC_OK = 0, DEC_BAD_MAGIC = 1, DEC_TRUNC = 2, DEC_BAD_TABLE = 3, DEC_BAD_DATA = 4,
     DEC_OVERFLOW = 5, DEC_BAD_ORIG = 6, DEC_BAD_LEN = 7, DEC_BAD_CRC = 8, DEC_BAD_WALK = 9
 };
-
-constexpr int kDecWarps = kDecThreads / 32;       // MTF segments per block
 
 struct DecBlock {
     const uint8_t *src;   // one standalone bzip2 stream
@@ -46,6 +45,40 @@ struct DecBlock {
     int32_t expect;       // decoded length the container promises
     int32_t pad;
 };
+
+// What the header says of a block, and how far its decoding has come.
+struct DecMeta {
+    int32_t status, block_max, orig, n_in_use, alpha, n_groups, n_sel;
+    int32_t group, bit;   // next group and its bit offset (group chase)
+    int32_t nsym;         // symbols up to and including EOB
+    int32_t m;            // bytes of the last column
+    uint32_t stored_crc, crc;
+    int32_t pad[7];
+};
+static_assert(sizeof(DecMeta) == sizeof(BlockState), "the decoder's block records live in the coder's");
+
+constexpr int kJBits = 13;  // prefix bits of the length table
+struct DecTab {
+    uint16_t jlut[kMaxGroups][1 << kJBits];  // bits of the first code | bits of the first two << 5 (0: do not fit)
+    uint16_t lut[kMaxGroups][1 << 10];       // symbol << 5 | code length, 0: longer code
+    int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];
+    uint16_t perm[kMaxGroups][kMaxAlpha];    // symbols by code
+    uint8_t seq_to_unseq[256];
+};
+static_assert(sizeof(DecTab) <= sizeof(int32_t) * kBlockCap, "tables fit a block's slot");
+
+// 32 bits from bit position `bit` on (MSB first), zeros past the end.
+__device__ __forceinline__ uint32_t stream_bits32(const uint8_t *p, int64_t nbytes, int64_t bit) {
+    const int64_t a = bit >> 3;
+    uint64_t w = 0;
+    if (a + 5 <= nbytes) {
+#pragma unroll
+        for (int i = 0; i < 5; i++) w = (w << 8) | __ldg(p + a + i);
+    } else {
+        for (int i = 0; i < 5; i++) w = (w << 8) | (a + i < nbytes ? __ldg(p + a + i) : 0u);
+    }
+    return (uint32_t)(w >> (8 - (int)(bit & 7)));
+}
 
 // MSB-first bit reader over a bounded byte string: up to 64 bits buffered
 // left-aligned, each byte loaded once. get(k) (k <= 32) past the end sets
@@ -64,6 +97,13 @@ struct BitReader {
         bcnt = 0;
         err = false;
     }
+    __device__ void seek(int64_t bit) {
+        next = bit >> 3;
+        buf = 0;
+        bcnt = 0;
+        skip((int)(bit & 7));
+    }
+    __device__ __forceinline__ int64_t tell() const { return next * 8 - bcnt; }
     // Called with fewer bits buffered than a read needs (at most 32): 32
     // more bits from four independent loads (one memory latency, not four);
     // the last bytes of the string one by one
@@ -98,137 +138,54 @@ struct BitReader {
     }
 };
 
-__device__ __forceinline__ uint32_t gf_mul(uint32_t a, uint32_t b) {
-    uint32_t r = 0;
-    for (int i = 31; i >= 0; i--) {
-        r = (r & 0x80000000u) ? (r << 1) ^ kPolyD : (r << 1);
-        if ((b >> i) & 1u) r ^= a;
-    }
-    return r;
-}
-__device__ __forceinline__ uint32_t xpow8(uint64_t k) {
-    uint32_t r = 1u, b = 0x100u;
-    while (k) {
-        if (k & 1) r = gf_mul(r, b);
-        b = gf_mul(b, b);
-        k >>= 1;
-    }
-    return r;
-}
-
-struct DecShared {
-    uint32_t crc_tab[256];
-    uint32_t warp_cnt[kDecThreads / 32][256];
-    uint32_t C[256];
-    int32_t walk_next[kWalkers];
-    int32_t walk_len[kWalkers];
-    int64_t walk_pos[kWalkers];
-    uint8_t seq_to_unseq[256];
-    uint8_t mtf[256];
-    uint8_t sel_list[8];
-    uint8_t len[6][258];
-    int32_t first[6][22], count[6][22], pidx[6][22];
-    uint16_t perm[6][258];
-    uint16_t lut[6][1 << 10];  // next 10 bits -> (symbol << 5) | code length, 0: longer code
-    uint16_t mlut[6][1 << 12]; // next 12 bits -> (codes << 5) | their bits: the whole codes (at most 4) in them, 0: the first is longer
-    BitReader br;              // the header reader, handed from the parse to the decode loop
-    int32_t alpha, block_max;
-    uint32_t red[32];
-    int32_t status, nblock, orig, n_in_use, n_groups, n_sel, out_len;
-    uint32_t stored_crc;
-    int32_t nsym, ngroups_used;            // Huffman symbols up to EOB, groups holding them
-    int32_t seg_start[kDecWarps];          // MTF segment of warp w: [seg_start[w], next start)
-    int32_t seg_len[kDecWarps], seg_off[kDecWarps];  // its output bytes and their offset in L
-    int32_t seg_status[kDecWarps];
-    uint8_t seg_perm[kDecWarps][256];      // where the segment's MTF moves take each list position
-    uint8_t seg_list[kDecWarps][256];      // the list at the segment's start
-    int32_t scan_sh[33];        // block scan scratch
-};
-
-// BitReader whose next 4 bytes are loaded one refill ahead, so a refill
-// does not wait for memory (for the one thread that walks all groups).
-struct AheadReader : BitReader {
-    uint32_t pf;  // bytes next .. next + 3, big-endian (when next + 4 <= nbytes)
-    __device__ __forceinline__ uint32_t load4(int64_t at) const {
-        return ((uint32_t)__ldg(p + at) << 24) | ((uint32_t)__ldg(p + at + 1) << 16) |
-               ((uint32_t)__ldg(p + at + 2) << 8) | (uint32_t)__ldg(p + at + 3);
-    }
-    __device__ void start(const BitReader &r) {
-        *static_cast<BitReader *>(this) = r;
-        pf = next + 4 <= nbytes ? load4(next) : 0u;
-    }
-    __device__ __forceinline__ void refill() {
-        if (bcnt <= 32 && next + 4 <= nbytes) {
-            buf |= (uint64_t)pf << (32 - bcnt);
-            bcnt += 32;
-            next += 4;
-            pf = next + 4 <= nbytes ? load4(next) : 0u;  // used at the next refill
-            return;
-        }
-        while (bcnt <= 56 && next < nbytes) {
-            buf |= (uint64_t)__ldg(p + next++) << (56 - bcnt);
-            bcnt += 8;
-        }
-    }
-    __device__ __forceinline__ uint32_t peek(int k) {
-        if (bcnt < k) refill();
-        return (uint32_t)(buf >> (64 - k));
-    }
-    __device__ __forceinline__ bool skip(int k) {
-        if (bcnt < k) refill();
-        if (bcnt < k) { err = true; bcnt = 0; buf = 0; return false; }
-        buf <<= k;
-        bcnt -= k;
-        return true;
-    }
-    __device__ __forceinline__ uint32_t get(int k) {
-        const uint32_t v = peek(k);
-        return skip(k) ? v : 0u;
-    }
-};
-
 // One Huffman symbol with table t: the 10-bit lookup, else the canonical
 // search from 11 bits; -1 for a code that is not in the table or a stream
 // that ends first (br.err).
-template <class Reader>
-__device__ __forceinline__ int huff_symbol(Reader &br, const DecShared &S, int t) {
-    const uint32_t e = S.lut[t][br.peek(10)];
+__device__ __forceinline__ int huff_symbol(BitReader &br, const uint16_t *lut, const DecTab &T, int t) {
+    const uint32_t e = lut[br.peek(10)];
     if (e) return br.skip(e & 31) ? (int)(e >> 5) : -1;
     int32_t c = (int32_t)br.peek(10);
     if (!br.skip(10)) return -1;
     for (int l = 11; l <= 20; l++) {
         c = (c << 1) | (int32_t)br.get(1);
         if (br.err) return -1;
-        const uint32_t d = (uint32_t)(c - S.first[t][l]);
-        if (d < (uint32_t)S.count[t][l]) return S.perm[t][S.pidx[t][l] + (int)d];
+        const uint32_t d = (uint32_t)(c - T.first[t][l]);
+        if (d < (uint32_t)T.count[t][l]) return T.perm[t][T.pidx[t][l] + (int)d];
     }
     return -1;
 }
 
-// Workspace per block: sel (kMaxSelectors bytes), L (kBlockCap), T (int32
-// kBlockCap), rowmark (int32 kBlockCap, walker id or -1), blk (kBlockCap).
-// 64 registers at most, so that a CTA of kDecThreads = 1024 fits an SM.
-__global__ void __maxnreg__(64) bzip2_decode_kernel(const DecBlock *__restrict__ blocks, int32_t *__restrict__ status,
-                                                                   uint8_t *__restrict__ sel_all, uint8_t *__restrict__ L_all,
-                                                                   int32_t *__restrict__ T_all, int32_t *__restrict__ mark_all,
-                                                                   uint8_t *__restrict__ blk_all) {
-    extern __shared__ __align__(16) uint8_t smraw[];
-    DecShared &S = *reinterpret_cast<DecShared *>(smraw);
-    const int b = blockIdx.x;
+// ------------------------------------------------------------- 1. header
+constexpr int kHdrThreads = 512;
+
+// Lists of six tables as nibbles, entry k in bits 4k .. 4k + 3.
+constexpr uint32_t kListId = 0x543210u;
+__device__ __forceinline__ uint32_t list_move(uint32_t l, int j) {  // entry j to the front
+    const uint32_t v = (l >> (4 * j)) & 15u, keep = ~0u << (4 * j + 4);
+    return (l & keep) | ((l << 4) & ~keep & ~15u) | v;
+}
+__device__ __forceinline__ uint32_t list_after(uint32_t a, uint32_t b) {  // entry k: a[b[k]]
+    uint32_t r = 0;
+#pragma unroll
+    for (int k = 0; k < kMaxGroups; k++) r |= ((a >> (4 * ((b >> (4 * k)) & 15u))) & 15u) << (4 * k);
+    return r;
+}
+
+__global__ void __launch_bounds__(kHdrThreads) dec_header_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
+                                                                 DecTab *__restrict__ tabs, size_t tab_stride,
+                                                                 uint8_t *__restrict__ sel_all, int32_t *__restrict__ zpos_all) {
+    __shared__ uint8_t len[kMaxGroups][kMaxAlpha];
+    __shared__ int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];
+    __shared__ int sh[33];
+    __shared__ uint32_t wlist[kHdrThreads / 32];
+    __shared__ int s_status, s_alpha, s_ng, s_nsel, s_bit;
+    const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
     const DecBlock D = blocks[b];
+    DecMeta &M = meta[b];
+    DecTab &T = *reinterpret_cast<DecTab *>(reinterpret_cast<uint8_t *>(tabs) + (size_t)b * tab_stride);
     uint8_t *sel = sel_all + (size_t)b * kMaxSelectors;
-    uint8_t *L = L_all + (size_t)b * kBlockCap;
-    int32_t *T = T_all + (size_t)b * kBlockCap;
-    int32_t *mark = mark_all + (size_t)b * kBlockCap;
-    uint8_t *blk = blk_all + (size_t)b * kBlockCap;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < 256; i += blockDim.x) {
-        uint32_t v = (uint32_t)i << 24;
-        for (int k = 0; k < 8; k++) v = (v & 0x80000000u) ? (v << 1) ^ kPolyD : (v << 1);
-        S.crc_tab[i] = v;
-    }
-    if (tid == 0) {
-        S.status = DEC_OK;
+    int32_t *zpos = zpos_all + (size_t)b * kBlockCap;
+    if (t == 0) {
         BitReader br;
         br.init(D.src, D.src_len);
         int st = DEC_OK;
@@ -236,503 +193,959 @@ __global__ void __maxnreg__(64) bzip2_decode_kernel(const DecBlock *__restrict__
             if (br.get(8) != 'B' || br.get(8) != 'Z' || br.get(8) != 'h') { st = DEC_BAD_MAGIC; break; }
             const uint32_t lvl = br.get(8);
             if (lvl < '1' || lvl > '9') { st = DEC_BAD_MAGIC; break; }
-            const int block_max = 100000 * (int)(lvl - '0');
+            M.block_max = 100000 * (int)(lvl - '0');
             if (br.get(24) != 0x314159u || br.get(24) != 0x265359u) { st = DEC_BAD_MAGIC; break; }
-            S.stored_crc = br.get(32);
+            M.stored_crc = br.get(32);
             if (br.get(1) != 0) { st = DEC_BAD_DATA; break; }
-            const int orig = (int)br.get(24);
+            M.orig = (int)br.get(24);
             const uint32_t used16 = br.get(16);
             int niu = 0;
             for (int i = 0; i < 16; i++) {
                 if (!(used16 & (1u << (15 - i)))) continue;
                 const uint32_t bits = br.get(16);
                 for (int j = 0; j < 16; j++)
-                    if (bits & (1u << (15 - j))) S.seq_to_unseq[niu++] = (uint8_t)(i * 16 + j);
+                    if (bits & (1u << (15 - j))) T.seq_to_unseq[niu++] = (uint8_t)(i * 16 + j);
             }
             if (br.err) { st = DEC_TRUNC; break; }
             if (niu == 0) { st = DEC_BAD_TABLE; break; }
-            const int alpha = niu + 2;
-            const int ng = (int)br.get(3);
-            const int nsel = (int)br.get(15);
+            const int ng = (int)br.get(3), nsel = (int)br.get(15);
             if (br.err) { st = DEC_TRUNC; break; }
             if (ng < 2 || ng > 6 || nsel < 1 || nsel > kMaxSelectors) { st = DEC_BAD_TABLE; break; }
-            for (int t = 0; t < ng; t++) S.sel_list[t] = (uint8_t)t;
-            for (int i = 0; i < nsel && st == DEC_OK; i++) {
-                int j = 0;
-                while (br.get(1)) {
-                    if (++j >= ng) { st = DEC_BAD_TABLE; break; }
-                }
-                if (br.err) st = DEC_TRUNC;
-                if (st != DEC_OK) break;
-                const uint8_t v = S.sel_list[j];
-                for (int q = j; q > 0; q--) S.sel_list[q] = S.sel_list[q - 1];
-                S.sel_list[0] = v;
-                sel[i] = v;
-            }
-            if (st != DEC_OK) break;
-            for (int t = 0; t < ng && st == DEC_OK; t++) {
-                int cur = (int)br.get(5);
-                for (int v = 0; v < alpha && st == DEC_OK; v++) {
-                    for (;;) {
-                        if (cur < 1 || cur > 20 || br.err) { st = br.err ? DEC_TRUNC : DEC_BAD_TABLE; break; }
-                        if (!br.get(1)) break;
-                        cur += br.get(1) ? -1 : 1;
-                    }
-                    S.len[t][v] = (uint8_t)cur;
-                }
-            }
-            if (st != DEC_OK) break;
-            // canonical tables: the codes of length l are first[l] ..
-            // first[l] + count[l] - 1, in increasing symbol order
-            for (int t = 0; t < ng; t++) {
-                int np = 0;
-                int32_t code = 0;
-                for (int l = 1; l <= 20; l++) {
-                    S.first[t][l] = code;
-                    S.pidx[t][l] = np;
-                    int cnt = 0;
-                    for (int v = 0; v < alpha; v++)
-                        if (S.len[t][v] == l) { S.perm[t][np++] = (uint16_t)v; cnt++; }
-                    S.count[t][l] = cnt;
-                    code = (code + cnt) << 1;
-                }
-            }
-            S.n_in_use = niu;
-            S.n_groups = ng;
-            S.n_sel = nsel;
-            S.alpha = alpha;
-            S.block_max = block_max;
-            S.orig = orig;
-            S.br = br;
+            M.n_in_use = niu;
+            M.alpha = niu + 2;
+            M.n_groups = ng;
+            M.n_sel = nsel;
+            s_alpha = niu + 2;
+            s_ng = ng;
+            s_nsel = nsel;
+            s_bit = (int)br.tell();
         } while (0);
-        S.status = st;
+        s_status = st;
     }
     __syncthreads();
-    if (S.status != DEC_OK) {
-        if (tid == 0) status[b] = S.status;
+    if (s_status != DEC_OK) {
+        if (t == 0) M.status = s_status;
         return;
     }
-    // lookup tables: entry i of table t decodes the code whose first bits are
-    // i (as 10 bits), if that code is at most 10 bits long
-    for (int q = tid; q < S.n_groups * 1024; q += blockDim.x) {
-        const int t = q >> 10, i = q & 1023;
-        uint16_t e = 0;
-        for (int l = 1; l <= 10; l++) {
-            const uint32_t d = (uint32_t)((int32_t)(i >> (10 - l)) - S.first[t][l]);
-            if (d < (uint32_t)S.count[t][l]) {
-                e = (uint16_t)((S.perm[t][S.pidx[t][l] + (int)d] << 5) | l);
-                break;
-            }
+    const int ng = s_ng, nsel = s_nsel, alpha = s_alpha, bit0 = s_bit;
+    const int64_t nbits = D.src_len * 8;
+    // selector i is a run of ones ended by a zero: zpos[i] = where its zero is
+    int found = 0;
+    for (int64_t base = bit0; found < nsel && base < nbits; base += 32 * kHdrThreads) {
+        const int64_t at = base + 32 * t;
+        uint32_t z = at < nbits ? ~stream_bits32(D.src, D.src_len, at) : 0u;
+        if (at + 32 > nbits && at < nbits) z &= ~0u << (32 - (int)(nbits - at));
+        int total;
+        int i = found + block_excl_sum<int>(__popc(z), sh, &total);
+        while (z && i < nsel) {
+            const int k = __clz(z);
+            zpos[i++] = (int32_t)(at + k);
+            z &= ~(0x80000000u >> k);
         }
-        S.lut[t][i] = e;
-    }
-    // multi-code length tables: how many whole codes the next 12 bits hold
-    // (at most 4) and how many bits they take, for the group walk below
-    for (int q = tid; q < S.n_groups * 4096; q += blockDim.x) {
-        const int t = q >> 12, i = q & 4095;
-        int used = 0, n = 0;
-        while (n < 4) {
-            int l = 1, got = 0;
-            for (; l <= 12 - used; l++) {
-                const uint32_t d = (uint32_t)((int32_t)((i >> (12 - used - l)) & ((1 << l) - 1)) - S.first[t][l]);
-                if (d < (uint32_t)S.count[t][l]) { got = l; break; }
-            }
-            if (!got) break;
-            used += got;
-            n++;
-        }
-        S.mlut[t][i] = (uint16_t)((n << 5) | used);
+        found += total;
     }
     __syncthreads();
-    // ---- 1b. Huffman: thread 0 walks the groups once to find where each
-    // starts in the stream (and where EOB is); then every thread decodes
-    // whole groups from their offsets into the symbol array
-    int32_t *gofs = T;                                  // group bit offsets (T is free until the LF mapping)
-    uint16_t *syms = reinterpret_cast<uint16_t *>(mark);  // symbols in order (mark is free until the walkers)
-    if (tid == 0) {
-        AheadReader br;
-        br.start(S.br);
-        const int nsel = S.n_sel, alpha = S.alpha;
-        int st = DEC_OK, ns = 0, ngu = 0;
-        for (int g = 0; g < nsel && st == DEC_OK; g++) {
-            gofs[g] = (int32_t)(br.next * 8 - br.bcnt);
-            const int t = sel[g];
-            int k = 0;
-            if (g < nsel - 1) {
-                // an encoder writes one selector per group it uses, so EOB is
-                // in the last group and the others hold 50 codes: their
-                // lengths only, several codes per lookup (a misplaced EOB in
-                // a corrupt stream shows up in the group decode or the MTF)
-                const uint16_t *ml = S.mlut[t];
-                while (k < 50) {
-                    if (br.bcnt < 32) br.refill();  // then the whole step needs no other check
-                    const uint32_t e = ml[(uint32_t)(br.buf >> 52)];
-                    const int n = (int)(e >> 5), len = (int)(e & 31);
-                    if (n > 0 && n <= 50 - k && len <= br.bcnt) {
-                        br.buf <<= len;
-                        br.bcnt -= len;
-                        k += n;
-                    } else {
-                        if (huff_symbol(br, S, t) < 0) { st = br.err ? DEC_TRUNC : DEC_BAD_DATA; break; }
-                        k++;
-                    }
-                }
-                continue;
-            }
-            for (; k < 50; k++) {
-                const int sym = huff_symbol(br, S, t);
-                if (sym < 0) { st = br.err ? DEC_TRUNC : DEC_BAD_DATA; break; }
-                if (sym == alpha - 1) break;  // EOB
-            }
-            if (st != DEC_OK) break;
-            if (k < 50) {
-                ns = g * 50 + k + 1;
-                ngu = g + 1;
-                break;
-            }
-            st = DEC_BAD_DATA;  // no EOB
-        }
-        S.nsym = ns;
-        S.ngroups_used = ngu;
-        S.status = st;
-    }
-    __syncthreads();
-    if (S.status != DEC_OK) {
-        if (tid == 0) status[b] = S.status;
+    if (found < nsel) {
+        if (t == 0) M.status = DEC_TRUNC;
         return;
     }
-    {
-        const int ns = S.nsym, ngu = S.ngroups_used;
-        for (int g = tid; g < ngu; g += blockDim.x) {
-            BitReader br;
-            br.init(D.src, D.src_len);
-            const int32_t bo = gofs[g];
-            br.next = bo >> 3;
-            br.skip(bo & 7);
-            const int t = sel[g], cnt = min(50, ns - g * 50);
-            for (int k = 0; k < cnt; k++) syms[g * 50 + k] = (uint16_t)huff_symbol(br, S, t);
-        }
+    // move-to-front over the tables: a stretch of selectors per thread, its
+    // moves as one permutation, a scan over the stretches
+    const int per = (nsel + kHdrThreads - 1) / kHdrThreads;
+    const int a = min(nsel, t * per), e = min(nsel, a + per);
+    uint32_t l = kListId;
+    bool bad = false;
+    for (int i = a; i < e; i++) {
+        const int j = zpos[i] - (i ? zpos[i - 1] : bit0 - 1) - 1;
+        bad |= j >= ng;
+        l = list_move(l, min(j, 5));
     }
-    __syncthreads();
-    // ---- 1c. inverse RUNA/RUNB and MTF by segments. A segment's MTF moves
-    // permute list positions whatever the list holds, so each warp first
-    // finds its segment's permutation and output length (pass 1), warp 0
-    // chains the lists at the segment starts and the output offsets, and
-    // each warp decodes its segment from its own starting list (pass 2).
-    // Segments start right after a symbol that is not a run digit, so no
-    // run is split. The list lives in registers, 8 bytes per lane (lane l
-    // holds positions 8l .. 8l + 7, position 8l + q in byte q of lo for q <
-    // 4, of hi otherwise); moving index j to the front shifts positions
-    // 0 .. j up by one byte and keeps the rest: one byte permute per word.
-    {
-        const int ns = S.nsym, niu = S.n_in_use, alpha = S.alpha, block_max = S.block_max;
-        const int w = tid >> 5, lane = tid & 31;
-        if (lane == 0) {
-            const int per = (ns + kDecWarps - 1) / kDecWarps, s0 = w * per, e0 = min(ns, s0 + per);
-            int p = ns;
-            if (w == 0) {
-                p = 0;
-            } else {
-                for (int q = max(s0, 1); q < e0; q++)
-                    if (syms[q - 1] >= 2) { p = q; break; }
-            }
-            S.seg_start[w] = p;
-        }
-        __syncthreads();
-        const int p0 = S.seg_start[w];
-        int p1 = ns;
-        for (int w2 = w + 1; w2 < kDecWarps; w2++)
-            if (S.seg_start[w2] < ns) { p1 = S.seg_start[w2]; break; }
-        for (int pass = 0; pass < 2; pass++) {
-            int st = DEC_OK;
-            int64_t outc = 0;
-            if (p0 < ns) {
-                uint32_t lo = 0, hi = 0;
-                for (int q = 3; q >= 0; q--) {  // positions (pass 0) or the list at the segment start (pass 1)
-                    const int a = 8 * lane + q, a4 = a + 4;
-                    const uint32_t va = pass ? S.seg_list[w][a] : (uint32_t)a;
-                    const uint32_t va4 = pass ? S.seg_list[w][a4] : (uint32_t)a4;
-                    lo = (lo << 8) | va;
-                    hi = (hi << 8) | va4;
-                }
-                const int64_t off = pass ? S.seg_off[w] : 0;
-                int64_t run = 0, run_w = 1;
-                uint32_t batch = 0;
-                for (int i = p0; i < p1; i++) {
-                    if (((i - p0) & 31) == 0) batch = i + lane < p1 ? syms[i + lane] : 0u;
-                    const int sym = (int)__shfl_sync(LFC_FULL, batch, (i - p0) & 31);
-                    if (sym <= 1) {
-                        run += (int64_t)(sym + 1) * run_w;
-                        run_w <<= 1;
-                        if (run > block_max) { st = DEC_OVERFLOW; break; }
-                        continue;
-                    }
-                    if (run > 0) {
-                        if (pass) {
-                            if (off + outc + run > S.nblock) { st = DEC_OVERFLOW; break; }
-                            const uint8_t v = S.seq_to_unseq[__shfl_sync(LFC_FULL, lo, 0) & 255u];
-                            for (int64_t q = lane; q < run; q += 32) L[off + outc + q] = v;
-                        }
-                        outc += run;
-                        run = 0;
-                        run_w = 1;
-                    }
-                    if (sym == alpha - 1) break;  // EOB
-                    const int j = sym - 1;  // >= 1
-                    if (j >= niu) { st = DEC_BAD_DATA; break; }
-                    const uint32_t holder = __shfl_sync(LFC_FULL, (j & 4) ? hi : lo, j >> 3);
-                    const uint32_t v = (holder >> (8 * (j & 3))) & 255u;
-                    const uint32_t below = __shfl_up_sync(LFC_FULL, hi, 1) >> 24;  // position 8l - 1
-                    const uint32_t slo = (lo << 8) | (lane == 0 ? v : below), shi = __funnelshift_l(lo, hi, 8);
-                    const int cnt = min(8, max(0, j + 1 - 8 * lane));
-                    const int cl = min(cnt, 4), ch = max(cnt - 4, 0);
-                    lo = __byte_perm(slo, lo, 0x7654u - (0x4444u & ((1u << (4 * cl)) - 1u)));
-                    hi = __byte_perm(shi, hi, 0x7654u - (0x4444u & ((1u << (4 * ch)) - 1u)));
-                    if (pass) {
-                        if (off + outc >= S.nblock) { st = DEC_OVERFLOW; break; }
-                        if (lane == 0) L[off + outc] = S.seq_to_unseq[v];
-                    }
-                    outc++;
-                    if (outc > block_max) { st = DEC_OVERFLOW; break; }
-                }
-                if (pass == 0) {  // where the moves took each position
+    uint32_t incl = l;
 #pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        S.seg_perm[w][8 * lane + q] = (uint8_t)(lo >> (8 * q));
-                        S.seg_perm[w][8 * lane + 4 + q] = (uint8_t)(hi >> (8 * q));
-                    }
-                }
-            }
-            if (lane == 0) {
-                S.seg_len[w] = (int32_t)(outc < INT_MAX ? outc : INT_MAX);
-                S.seg_status[w] = st;
-            }
-            __syncthreads();
-            if (pass == 0 && w == 0) {
-                // lists at the segment starts and output offsets, in order
-                int st0 = DEC_OK;
-                for (int q = lane; q < 256; q += 32) S.seg_list[0][q] = (uint8_t)(q < niu ? q : 0);
-                int64_t total = 0;
-                int prev = -1;
-                for (int w2 = 0; w2 < kDecWarps; w2++) {
-                    if (S.seg_start[w2] >= ns) continue;
-                    if (S.seg_status[w2] != DEC_OK) st0 = S.seg_status[w2];
-                    if (prev >= 0) {
-                        __syncwarp();
-                        for (int q = lane; q < 256; q += 32) S.seg_list[w2][q] = S.seg_list[prev][S.seg_perm[prev][q]];
-                    }
-                    if (lane == 0) S.seg_off[w2] = (int32_t)(total < INT_MAX ? total : INT_MAX);
-                    total += S.seg_len[w2];
-                    prev = w2;
-                }
-                if (st0 == DEC_OK && (total > block_max || total > kBlockCap)) st0 = DEC_OVERFLOW;
-                if (st0 == DEC_OK && S.orig >= total) st0 = DEC_BAD_ORIG;
-                if (lane == 0) {
-                    S.status = st0;
-                    S.nblock = (int32_t)(total < INT_MAX ? total : INT_MAX);
-                }
-            }
-            __syncthreads();
-            if (S.status != DEC_OK) break;
-        }
-        if (tid == 0)
-            for (int w2 = 0; w2 < kDecWarps; w2++)
-                if (S.seg_status[w2] != DEC_OK) S.status = S.seg_status[w2];
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(LFC_FULL, incl, o);
+        if (lane >= o) incl = list_after(x, incl);
     }
-    __syncthreads();
-    if (S.status != DEC_OK) {
-        if (tid == 0) status[b] = S.status;
+    if (lane == 31) wlist[w] = incl;
+    if (__syncthreads_or(bad)) {
+        if (t == 0) M.status = DEC_BAD_TABLE;
         return;
     }
-    const int m = S.nblock;
-    // ---- 2. LF mapping: stable counting sort of L with per-warp counters
-    const int w = tid >> 5, lane = tid & 31, NW = kDecThreads / 32;
-    for (int i = lane; i < 256; i += 32) S.warp_cnt[w][i] = 0;
-    __syncwarp();
-    const int per_w = (m + NW - 1) / NW;
-    const int wa = min(m, w * per_w), we = min(m, wa + per_w);
-    for (int base = wa; base < we; base += 32) {
-        const int j = base + lane;
-        const bool ok = j < we;
-        const uint32_t c = ok ? L[j] : 0u;
-        const uint32_t mm = __match_any_sync(LFC_FULL, ok ? c : 256u + lane);
-        if (ok && (mm & lanemask_gt()) == 0) S.warp_cnt[w][c] += __popc(mm);
-        __syncwarp();
+    uint32_t before = __shfl_up_sync(LFC_FULL, incl, 1), cur = kListId;
+    for (int i = 0; i < w; i++) cur = list_after(cur, wlist[i]);
+    if (lane > 0) cur = list_after(cur, before);
+    for (int i = a; i < e; i++) {
+        const int j = zpos[i] - (i ? zpos[i - 1] : bit0 - 1) - 1;
+        cur = list_move(cur, j);
+        sel[i] = (uint8_t)(cur & 15u);
     }
-    __syncthreads();
-    if (tid < 256) {
-        uint32_t acc = 0;
-        for (int ww = 0; ww < NW; ww++) acc += S.warp_cnt[ww][tid];
-        S.C[tid] = acc;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t acc = 0;
-        for (int c = 0; c < 256; c++) { const uint32_t v = S.C[c]; S.C[c] = acc; acc += v; }
-    }
-    __syncthreads();
-    if (tid < 256) {
-        uint32_t acc = S.C[tid];
-        for (int ww = 0; ww < NW; ww++) { const uint32_t v = S.warp_cnt[ww][tid]; S.warp_cnt[ww][tid] = acc; acc += v; }
-    }
-    __syncthreads();
-    for (int base = wa; base < we; base += 32) {
-        const int j = base + lane;
-        const bool ok = j < we;
-        const uint32_t c = ok ? L[j] : 0u;
-        const uint32_t mm = __match_any_sync(LFC_FULL, ok ? c : 256u + lane);
-        uint32_t before = ok ? S.warp_cnt[w][c] : 0u;
-        __syncwarp();
-        if (ok) {
-            T[j] = (int32_t)(before + __popc(mm & lanemask_lt()));
-            if ((mm & lanemask_gt()) == 0) S.warp_cnt[w][c] = before + __popc(mm);
+    // code lengths: 5-bit start, then per symbol steps "10" up / "11" down and a "0"
+    if (t == 0) {
+        BitReader br;
+        br.init(D.src, D.src_len);
+        br.seek((int64_t)zpos[nsel - 1] + 1);
+        int st = DEC_OK;
+        for (int g = 0; g < ng && st == DEC_OK; g++) {
+            int c = (int)br.get(5);
+            for (int v = 0; v < alpha && st == DEC_OK; v++) {
+                for (;;) {
+                    if (br.bcnt < 2) br.refill();
+                    if (c < 1 || c > 20 || br.bcnt < 1) { st = br.bcnt < 1 ? DEC_TRUNC : DEC_BAD_TABLE; break; }
+                    if (!(br.buf >> 63)) {
+                        br.buf <<= 1;
+                        br.bcnt--;
+                        break;
+                    }
+                    if (br.bcnt < 2) { st = DEC_TRUNC; break; }
+                    c += (br.buf >> 62) & 1 ? -1 : 1;
+                    br.buf <<= 2;
+                    br.bcnt -= 2;
+                }
+                len[g][v] = (uint8_t)c;
+            }
         }
-        __syncwarp();
+        if (br.err) st = DEC_TRUNC;
+        s_status = st;
+        s_bit = (int)br.tell();
     }
-    for (int j = tid; j < m; j += blockDim.x) mark[j] = -1;
     __syncthreads();
-    // ---- 3. walkers
-    const int nwk = min(kWalkers, m);
-    int start = -1;
-    if (tid < nwk) {
-        if (tid == 0) {
-            start = S.orig;
-        } else {
-            start = (int)((int64_t)tid * m / nwk);
-            if (start == S.orig) start = -1;  // orig is walker 0's row
+    if (s_status != DEC_OK) {
+        if (t == 0) M.status = s_status;
+        return;
+    }
+    // canonical tables: the codes of length l are first[l] .. first[l] +
+    // count[l] - 1, in increasing symbol order
+    for (int i = t; i < kMaxGroups * 22; i += kHdrThreads) (&count[0][0])[i] = 0;
+    __syncthreads();
+    for (int i = t; i < ng * alpha; i += kHdrThreads) atomicAdd(&count[i / alpha][len[i / alpha][i % alpha]], 1);
+    __syncthreads();
+    if (t < ng) {
+        int32_t code = 0;
+        int np = 0;
+        for (int k = 1; k <= 20; k++) {
+            first[t][k] = code;
+            pidx[t][k] = np;
+            np += count[t][k];
+            code = (code + count[t][k]) << 1;
         }
-        if (start >= 0) mark[start] = tid;
     }
     __syncthreads();
-    if (start >= 0) {
-        int r = start, steps = 0;
-        do {
-            r = T[r];
-            steps++;
-        } while (mark[r] < 0 && steps <= m);
-        S.walk_len[tid] = steps;
-        S.walk_next[tid] = steps <= m ? mark[r] : -1;
-    } else if (tid < kWalkers) {
-        S.walk_len[tid] = 0;
-        S.walk_next[tid] = -1;
+    for (int i = t; i < ng * alpha; i += kHdrThreads) {
+        const int g = i / alpha, v = i - g * alpha, k = len[g][v];
+        int r = 0;
+        for (int x = 0; x < v; x++) r += len[g][x] == k;
+        T.perm[g][pidx[g][k] + r] = (uint16_t)v;
+    }
+    for (int i = t; i < kMaxGroups * 22; i += kHdrThreads) {
+        (&T.first[0][0])[i] = (&first[0][0])[i];
+        (&T.count[0][0])[i] = (&count[0][0])[i];
+        (&T.pidx[0][0])[i] = (&pidx[0][0])[i];
+    }
+    for (int i = t; i < ng << kJBits; i += kHdrThreads) {  // length of the first code of a prefix
+        const int g = i >> kJBits, x = i & ((1 << kJBits) - 1);
+        uint16_t v = 0;
+        for (int k = 1; k <= kJBits; k++)
+            if ((uint32_t)((x >> (kJBits - k)) - first[g][k]) < (uint32_t)count[g][k]) { v = (uint16_t)k; break; }
+        T.jlut[g][x] = v;
     }
     __syncthreads();
-    if (tid == 0) {
-        int k = 0;
-        int64_t pos = 0;
-        int visited = 0;
+    for (int i = t; i < ng << kJBits; i += kHdrThreads) {  // and of the second one, if the prefix holds it
+        const int g = i >> kJBits, x = i & ((1 << kJBits) - 1);
+        const int k = T.jlut[g][x] & 31;
+        if (!k) continue;
+        const int k2 = T.jlut[g][(x << k) & ((1 << kJBits) - 1)] & 31;
+        if (k2 && k + k2 <= kJBits) T.jlut[g][x] = (uint16_t)(k | ((k + k2) << 5));
+    }
+    for (int i = t; i < ng << 10; i += kHdrThreads) {
+        const int g = i >> 10, x = i & 1023;
+        uint16_t v = 0;
+        for (int k = 1; k <= 10; k++) {
+            const uint32_t d = (uint32_t)((x >> (10 - k)) - first[g][k]);
+            if (d < (uint32_t)count[g][k]) { v = (uint16_t)((T.perm[g][pidx[g][k] + (int)d] << 5) | k); break; }
+        }
+        T.lut[g][x] = v;
+    }
+    if (t == 0) {
+        M.group = 0;
+        M.bit = s_bit;
+        M.nsym = 0;
+        M.m = 0;
+        M.status = DEC_OK;
+    }
+}
+
+// ------------------------------------------------------ 2. group offsets
+// Lengths of 50 codes from every bit of a stretch of kJRange bits, for every
+// table: a tile of kJTile bits per CTA with the bits its groups reach into.
+// A tile holds, per bit, the bit a number of codes further (kJSpan: none), so
+// a doubling is one gather: out[i] = in[in[i]]. Bound by issue: about 40
+// instructions per bit and table, two bits per load and store.
+constexpr int kJTile = 8192;
+constexpr int kJHalo = 1024;                  // 50 codes of at most 20 bits
+constexpr int kJSpan = kJTile + kJHalo;
+constexpr int kJRange = (kBlockCap * 4 / 3) / kJTile * kJTile;  // bits per round: three tables fill a slot of 8-byte words
+constexpr int kJThreads = 512;
+static_assert((size_t)kJRange * 3 * 2 <= (size_t)kBlockCap * 8, "three tables of one round fit a key slot");
+
+struct JumpSmem {
+    uint32_t bits[kJSpan / 32 + 4];
+    __align__(16) uint16_t lut[1 << kJBits];
+    __align__(4) uint16_t a[kJSpan + 2], b[kJSpan + 2], c[kJSpan + 2];
+};
+
+// Bits of two codes from bit p of the span, by the canonical tables (codes
+// longer than the lookup prefix); 0 if there are none.
+__device__ __noinline__ int two_codes(const uint32_t *bits, int p, const DecTab &T, int t) {
+    int total = 0;
+    for (int n = 0; n < 2; n++) {
+        const int q = p + total;
+        if (q + 20 > kJSpan + 64) return 0;
+        const uint32_t v = __funnelshift_l(bits[(q >> 5) + 1], bits[q >> 5], q & 31);
+        int l = 1;
+        for (; l <= 20; l++)
+            if ((uint32_t)((int32_t)(v >> (32 - l)) - T.first[t][l]) < (uint32_t)T.count[t][l]) break;
+        if (l > 20) return 0;
+        total += l;
+    }
+    return total;
+}
+
+__global__ void __launch_bounds__(kJThreads) dec_jump_kernel(const DecBlock *__restrict__ blocks, const DecMeta *__restrict__ meta,
+                                                             const DecTab *__restrict__ tabs, size_t tab_stride, int64_t range0,
+                                                             uint64_t *__restrict__ j0_all, uint64_t *__restrict__ j1_all) {
+    extern __shared__ __align__(16) uint8_t smraw[];
+    JumpSmem &S = *reinterpret_cast<JumpSmem *>(smraw);
+    const int b = blockIdx.y, t = threadIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK || M.group >= M.n_sel - 1) return;
+    const DecBlock D = blocks[b];
+    const int64_t nbits = D.src_len * 8;
+    const int64_t w0 = range0 + (int64_t)blockIdx.x * kJTile;
+    if (w0 >= nbits || w0 + kJTile <= M.bit) return;
+    const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
+    for (int i = t; i < kJSpan / 32 + 4; i += kJThreads) S.bits[i] = stream_bits32(D.src, D.src_len, w0 + 32 * i);
+    for (int g = 0; g < M.n_groups; g++) {
+        for (int i = t; i < (1 << kJBits) / 8; i += kJThreads)
+            reinterpret_cast<uint4 *>(S.lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.jlut[g]) + i);
+        __syncthreads();
+        auto two = [&](int i) -> uint32_t {  // the bit two codes after bit i
+            const uint32_t v = __funnelshift_l(S.bits[(i >> 5) + 1], S.bits[i >> 5], i & 31);
+            const uint32_t e = S.lut[v >> (32 - kJBits)];
+            int l = (int)(e >> 5);
+            if (!l) {
+                const int k = (int)(e & 31), q = i + k;
+                const uint32_t v2 = __funnelshift_l(S.bits[(q >> 5) + 1], S.bits[q >> 5], q & 31);
+                const int k2 = k ? (int)(S.lut[v2 >> (32 - kJBits)] & 31u) : 0;
+                l = k2 ? k + k2 : two_codes(S.bits, i, T, g);
+            }
+            return (uint32_t)(l ? min(i + l, kJSpan) : kJSpan);
+        };
+        for (int i = 2 * t; i < kJSpan; i += 2 * kJThreads)
+            *reinterpret_cast<uint32_t *>(&S.a[i]) = two(i) | (two(i + 1) << 16);
+        if (t == 0) S.a[kJSpan] = S.b[kJSpan] = S.c[kJSpan] = (uint16_t)kJSpan;
+        __syncthreads();
+        auto twice = [&](const uint16_t *in, uint16_t *out) {
+#pragma unroll 3
+            for (int i = 2 * t; i < kJSpan; i += 2 * kJThreads) {
+                const uint32_t x = *reinterpret_cast<const uint32_t *>(&in[i]);
+                *reinterpret_cast<uint32_t *>(&out[i]) = (uint32_t)in[x & 0xFFFFu] | ((uint32_t)in[x >> 16] << 16);
+            }
+            __syncthreads();
+        };
+        twice(S.a, S.b);  // 4
+        twice(S.b, S.c);  // 8
+        twice(S.c, S.b);  // 16
+        uint16_t *out = reinterpret_cast<uint16_t *>((g < 3 ? j0_all : j1_all) + (size_t)b * kBlockCap) + (size_t)(g % 3) * kJRange +
+                        (size_t)blockIdx.x * kJTile;
+        auto fifty = [&](uint32_t at16, int i) -> uint32_t {  // 16 + 16 + 16 + 2
+            const uint32_t j = S.a[S.b[S.b[at16]]];
+            return j == (uint32_t)kJSpan ? 0u : j - (uint32_t)i;
+        };
+#pragma unroll 2
+        for (int i = 2 * t; i < kJTile; i += 2 * kJThreads) {
+            const uint32_t x = *reinterpret_cast<const uint32_t *>(&S.b[i]);
+            *reinterpret_cast<uint32_t *>(&out[i]) = fifty(x & 0xFFFFu, i) | (fifty(x >> 16, i + 1) << 16);
+        }
+        __syncthreads();
+    }
+}
+
+// One CTA per block: thread 0 adds up the groups' lengths, the other warps
+// fetch the next window of them. After the last round also the last group,
+// up to EOB.
+constexpr int kChaseThreads = 256;
+constexpr int kChaseWin = 4096;  // bits of a window
+constexpr int kChaseBufs = 3;    // one in use, two on their way
+struct ChaseSmem {
+    __align__(16) uint16_t j[kChaseBufs][kMaxGroups][kChaseWin];
+    uint8_t sel[kMaxSelectors + 14];
+    int64_t p;
+    int g, status;
+};
+static_assert(kJRange % kChaseWin == 0, "a round holds whole windows");
+
+__device__ __forceinline__ void cp_async16(void *smem, const void *g) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(g) : "memory");
+}
+
+__global__ void __launch_bounds__(kChaseThreads) dec_chase_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
+                                                                  const DecTab *__restrict__ tabs, size_t tab_stride, int64_t range0,
+                                                                  const uint64_t *__restrict__ j0_all, const uint64_t *__restrict__ j1_all,
+                                                                  const uint8_t *__restrict__ sel_all, int32_t *__restrict__ gofs_all) {
+    extern __shared__ __align__(16) uint8_t smraw[];
+    ChaseSmem &S = *reinterpret_cast<ChaseSmem *>(smraw);
+    const int b = blockIdx.x, t = threadIdx.x;
+    DecMeta &M = meta[b];
+    if (M.status != DEC_OK || M.group >= M.n_sel) return;
+    const DecBlock D = blocks[b];
+    const int64_t nbits = D.src_len * 8;
+    const int last = M.n_sel - 1, ng = M.n_groups;
+    const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
+    int32_t *gofs = gofs_all + (size_t)b * kBlockCap;
+    for (int i = t; i <= last; i += kChaseThreads) S.sel[i] = sel_all[(size_t)b * kMaxSelectors + i];
+    if (t == 0) {
+        S.p = M.bit;
+        S.g = M.group;
+        S.status = DEC_OK;
+    }
+    __syncthreads();
+    const int64_t range1 = min(nbits, range0 + kJRange);
+    auto fetch = [&](int64_t w, int buf) {  // the window at bit w, by the warps behind the first
+        if (t >= 32 && w < range1) {
+            const size_t o = (size_t)(w - range0);
+            for (int g = 0; g < ng; g++) {
+                const uint16_t *in = reinterpret_cast<const uint16_t *>((g < 3 ? j0_all : j1_all) + (size_t)b * kBlockCap) +
+                                     (size_t)(g % 3) * kJRange + o;
+                for (int q = t - 32; q < kChaseWin / 8; q += kChaseThreads - 32) cp_async16(&S.j[buf][g][8 * q], in + 8 * q);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (S.p < range1 && S.g < last) {
+        int64_t w = range0 + (S.p - range0) / kChaseWin * kChaseWin;
+        fetch(w, 0);
+        fetch(w + kChaseWin, 1);
+        for (int buf = 0; w < range1; w += kChaseWin, buf = buf == kChaseBufs - 1 ? 0 : buf + 1) {
+            bool stop = false;
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncthreads();  // the window is there, and the one before is done with
+            fetch(w + 2 * kChaseWin, buf == 0 ? 2 : buf - 1);
+            if (t == 0) {
+                int g = S.g;
+                int q = (int)(S.p - w);
+                const int32_t base = (int32_t)w;
+                const uint16_t *J = &S.j[buf][0][0];
+                int tb = S.sel[g];
+                while (g < last && q < kChaseWin) {
+                    const int nt = S.sel[g + 1];  // g < last: there is one
+                    int d = J[tb * kChaseWin + q];
+                    gofs[g] = base + q;
+                    if (d == 0) {  // not in the table: decode the group (or find that it cannot be)
+                        BitReader br;
+                        br.init(D.src, D.src_len);
+                        br.seek(w + q);
+                        for (int k = 0; k < 50; k++)
+                            if (huff_symbol(br, T.lut[tb], T, tb) < 0) { S.status = br.err ? DEC_TRUNC : DEC_BAD_DATA; break; }
+                        d = (int)(br.tell() - (w + q));
+                        if (S.status != DEC_OK) { g = last; break; }
+                    }
+                    q += d;
+                    tb = nt;
+                    g++;
+                }
+                S.g = g;
+                S.p = w + q;
+                if (S.p > nbits && S.status == DEC_OK) S.status = DEC_TRUNC;
+                stop = g >= last || S.status != DEC_OK;
+            }
+            if (__syncthreads_or(stop)) break;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    }
+    if (t != 0) return;
+    M.group = S.g;
+    M.bit = (int32_t)S.p;
+    if (S.status == DEC_OK && S.g < last && range1 == nbits) S.status = DEC_TRUNC;
+    if (S.status != DEC_OK) {
+        M.status = S.status;
+        return;
+    }
+    if (S.g != last) return;
+    BitReader br;
+    br.init(D.src, D.src_len);
+    br.seek(S.p);
+    const int tb = S.sel[last], alpha = M.alpha;
+    gofs[last] = (int32_t)S.p;
+    for (int k = 0; k < 50; k++) {
+        const int sym = huff_symbol(br, T.lut[tb], T, tb);
+        if (sym < 0) { M.status = br.err ? DEC_TRUNC : DEC_BAD_DATA; return; }
+        if (sym == alpha - 1) {
+            M.nsym = last * 50 + k + 1;
+            M.group = last + 1;
+            return;
+        }
+    }
+    M.status = DEC_BAD_DATA;  // no EOB
+}
+
+// ---------------------------------------------------------- 3. symbols
+constexpr int kSymGroups = 128;
+
+__global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
+                                                                 const DecTab *__restrict__ tabs, size_t tab_stride,
+                                                                 const uint8_t *__restrict__ sel_all, const int32_t *__restrict__ gofs_all,
+                                                                 uint16_t *__restrict__ sym_all) {
+    __shared__ __align__(16) uint16_t lut[kMaxGroups][1 << 10];
+    __shared__ __align__(16) uint16_t out[kSymGroups * 50];
+    const int b = blockIdx.y, t = threadIdx.x;
+    DecMeta &M = meta[b];
+    if (__syncthreads_or(M.status != DEC_OK)) return;  // one answer for the CTA: another one may set it meanwhile
+    const int g0 = blockIdx.x * kSymGroups, ns = M.nsym, eob = M.alpha - 1;
+    if (g0 * 50 >= ns) return;
+    const DecBlock D = blocks[b];
+    const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
+    for (int i = t; i < M.n_groups * 128; i += kSymGroups)
+        reinterpret_cast<uint4 *>(lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.lut) + i);
+    __syncthreads();
+    const int g = g0 + t;
+    if (g * 50 < ns) {
+        BitReader br;
+        br.init(D.src, D.src_len);
+        br.seek(gofs_all[(size_t)b * kBlockCap + g]);
+        const int tb = sel_all[(size_t)b * kMaxSelectors + g], cnt = min(50, ns - g * 50);
         bool bad = false;
-        for (int i = 0; i < kWalkers; i++) S.walk_pos[i] = -1;
-        while (pos < m) {
-            if (k < 0 || k >= kWalkers || S.walk_pos[k] >= 0 || S.walk_len[k] <= 0) { bad = true; break; }
-            S.walk_pos[k] = pos;
-            pos += S.walk_len[k];
-            visited++;
-            k = S.walk_next[k];
+        for (int k = 0; k < cnt; k++) {
+            const int sym = huff_symbol(br, lut[tb], T, tb);
+            bad |= sym < 0 || (sym == eob) != (g * 50 + k == ns - 1);  // EOB is the last symbol, and only that
+            out[t * 50 + k] = (uint16_t)sym;
         }
-        if (bad || pos != m || k != 0) S.status = DEC_BAD_WALK;
+        if (bad) M.status = DEC_BAD_DATA;
     }
     __syncthreads();
-    if (S.status != DEC_OK) {
-        if (tid == 0) status[b] = S.status;
+    const int n = min(kSymGroups * 50, ns - g0 * 50);
+    uint16_t *sym = sym_all + (size_t)b * (kBlockCap + 64) + g0 * 50;
+    for (int i = t; i < n; i += kSymGroups) sym[i] = out[i];
+}
+
+// ------------------------------------------- 4. inverse RUNA/RUNB and MTF
+// Segments start right after a symbol that is not a run digit, so no run is
+// split: segment s begins at the first such place in its share of the symbols
+// and ends at the first one past it. A thread's list is 32 words of 8 bytes,
+// word i of thread t at [i][t]; moving entry j to the front shifts the words
+// below it by a byte.
+constexpr int kSegThreadsM = 128;
+constexpr int kSegs = 6 * kSegThreadsM;
+
+struct SegInfo {
+    int32_t len, status, off;
+};
+// a block's slot in the segment buffer: permutations, start lists, records
+constexpr size_t kSegPerm = 0, kSegList = (size_t)kSegs * 256, kSegInfo = 2 * (size_t)kSegs * 256;
+static_assert(kSegInfo + kSegs * sizeof(SegInfo) <= sizeof(int32_t) * (size_t)kBlockCap, "segment records fit a block's slot");
+
+// PASS 0: the permutation of list positions and the output length; PASS 1:
+// the output bytes from the segment's starting list.
+template <int PASS>
+__global__ void __launch_bounds__(kSegThreadsM) dec_mtf_kernel(DecMeta *__restrict__ meta, const uint16_t *__restrict__ sym_all,
+                                                               uint8_t *__restrict__ seg_all, uint8_t *__restrict__ L_all) {
+    extern __shared__ __align__(16) uint64_t list_all[];
+    const int b = blockIdx.y, t = threadIdx.x, s = blockIdx.x * kSegThreadsM + t;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    uint64_t *list = list_all + t;  // word i at list[i * kSegThreadsM]
+    uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
+    SegInfo *info = reinterpret_cast<SegInfo *>(slot + kSegInfo) + s;
+    const uint16_t *sym = sym_all + (size_t)b * (kBlockCap + 64);
+    const int ns = M.nsym, niu = M.n_in_use, alpha = M.alpha, block_max = M.block_max;
+    const int per = (ns + kSegs - 1) / kSegs, s0 = min(ns, s * per), e0 = min(ns, s0 + per);
+    int i = s0;
+    if (s > 0)
+        while (i < e0 && sym[i - 1] < 2) i++;
+    if (i >= e0) {  // empty: its symbols belong to the segment before
+        if (PASS == 0) {
+            info->len = 0;
+            info->status = DEC_OK;
+            uint64_t *perm = reinterpret_cast<uint64_t *>(slot + kSegPerm + (size_t)s * 256);
+            for (int k = 0; k < 32; k++) perm[k] = 0x0706050403020100ull + 0x0808080808080808ull * (uint64_t)k;
+        }
         return;
     }
-    if (start >= 0 && S.walk_pos[tid] >= 0) {
-        int r = start;
-        const int64_t p0 = S.walk_pos[tid];
-        for (int s = 0; s < S.walk_len[tid]; s++) {
-            blk[m - 1 - (p0 + s)] = L[r];
-            r = T[r];
+    const uint64_t *start = reinterpret_cast<const uint64_t *>(slot + kSegList + (size_t)s * 256);
+    for (int k = 0; k < 32; k++)
+        list[k * kSegThreadsM] = PASS == 0 ? 0x0706050403020100ull + 0x0808080808080808ull * (uint64_t)k : start[k];
+    uint8_t *L = L_all + (size_t)b * kBlockCap;
+    int out = PASS == 1 ? info->off : 0;
+    const int out0 = out, cap = PASS == 1 ? M.m : block_max;
+    int st = DEC_OK, run = 0, bit = 0;
+    uint64_t acc = 0;  // output bytes of the 8-byte word being filled
+    int acc_n = 0;
+    auto put = [&](uint32_t v) {  // PASS 1; out < cap
+        acc |= (uint64_t)v << (8 * (out & 7));
+        acc_n++;
+        out++;
+        if ((out & 7) == 0) {
+            if (acc_n == 8) *reinterpret_cast<uint64_t *>(L + out - 8) = acc;
+            else
+                for (int k = 8 - acc_n; k < 8; k++) L[out - 8 + k] = (uint8_t)(acc >> (8 * k));
+            acc = 0;
+            acc_n = 0;
         }
-    }
-    __syncthreads();
-    // ---- 4. inverse RLE1, then CRC. A position q is a sync point when
-    // bytes q-2 and q-1 differ and bytes q-5 .. q-2 are not all equal: byte
-    // q-1 is then a literal (a count byte follows four equal literals) that
-    // starts a run, so decoding can start at q from (run 1, last = byte
-    // q-1). Every thread takes the first sync point of its chunk (thread 0:
-    // position 0, fresh) and decodes up to the next thread's: once to count
-    // its output bytes, once to write them at their prefix.
-    {
-        const int nth = blockDim.x;
-        const int ch = max(8, (m + nth - 1) / nth);
-        const int s0 = tid * ch, e0 = min(m, s0 + ch);
-        int p = m;  // this thread's segment start, m: none in its chunk
-        if (s0 < m) {
-            if (tid == 0) {
-                p = 0;
+    };
+    for (; i < ns; i++) {
+        const int x = sym[i];
+        if (i >= e0 && sym[i - 1] >= 2) break;  // the next segment starts here
+        if (x < 2) {
+            if (bit > 20 || (run += (x + 1) << bit) > block_max) { st = DEC_OVERFLOW; break; }
+            bit++;
+            continue;
+        }
+        if (run) {
+            if (run > cap - out) { st = DEC_OVERFLOW; break; }
+            if (PASS == 1) {
+                const uint32_t v = (uint32_t)list[0] & 255u;
+                while (run && (out & 7)) { put(v); run--; }
+                const uint64_t v8 = v * 0x0101010101010101ull;
+                for (; run >= 8; run -= 8, out += 8) *reinterpret_cast<uint64_t *>(L + out) = v8;
+                while (run) { put(v); run--; }
             } else {
-                for (int q = max(s0, 5); q < e0; q++) {
-                    const uint8_t b1 = blk[q - 1], b2 = blk[q - 2];
-                    if (b1 != b2 && !(blk[q - 5] == b2 && blk[q - 4] == b2 && blk[q - 3] == b2)) { p = q; break; }
-                }
+                out += run;
             }
+            run = bit = 0;
         }
-        S.walk_len[tid] = p;
-        __syncthreads();
-        int end = m;  // the next segment start after this one
-        if (p < m)
-            for (int t2 = tid + 1; t2 < nth; t2++)
-                if (S.walk_len[t2] < m) { end = S.walk_len[t2]; break; }
-        int cnt = 0, st = DEC_OK;
-        for (int pass = 0; pass < 2; pass++) {
-            int off = 0;
-            if (pass == 1) {
-                int total = 0;
-                off = block_excl_sum<int>(cnt, S.scan_sh, &total);
-                if (total != D.expect) st = DEC_BAD_LEN;
-                if (__syncthreads_or(st != DEC_OK)) break;
-            }
-            if (p < m) {
-                int o = 0, same = tid == 0 ? 0 : 1, last = tid == 0 ? -1 : (int)blk[p - 1];
-                for (int i = p; i < end; i++) {
-                    const uint8_t v = blk[i];
-                    if (pass) D.dst[off + o] = v;
-                    o++;
-                    same = ((int)v == last) ? same + 1 : 1;
-                    last = v;
-                    if (same == 4) {
-                        if (i + 1 >= m) { st = DEC_BAD_DATA; break; }
-                        const int extra = blk[++i];
-                        if (pass && off + o + extra > D.expect) { st = DEC_BAD_LEN; break; }
-                        if (pass)
-                            for (int q = 0; q < extra; q++) D.dst[off + o + q] = v;
-                        o += extra;
-                        same = 0;
-                        last = -1;
-                    }
-                }
-                cnt = o;
-            }
-            if (__syncthreads_or(st != DEC_OK)) break;
+        if (x == alpha - 1) break;  // EOB
+        const int j = x - 1, k = j >> 3, r = j & 7;
+        if (j >= niu) { st = DEC_BAD_DATA; break; }
+        if (out >= cap) { st = DEC_OVERFLOW; break; }
+        const uint64_t wk = list[k * kSegThreadsM], v = (wk >> (8 * r)) & 255u;
+        uint64_t carry = v;
+        for (int q = 0; q < k; q++) {
+            const uint64_t w = list[q * kSegThreadsM];
+            list[q * kSegThreadsM] = (w << 8) | carry;
+            carry = w >> 56;
         }
-        if (tid == 0) {
-            S.status = DEC_OK;
-            S.out_len = D.expect;
-        }
-        __syncthreads();
-        if (st != DEC_OK) S.status = st;  // any failing thread (benign race: all write an error code)
+        const uint64_t keep = r == 7 ? 0ull : ~0ull << (8 * (r + 1));
+        list[k * kSegThreadsM] = (wk & keep) | (((wk << 8) | carry) & ~keep);
+        if (PASS == 1) put((uint32_t)v); else out++;
     }
-    __syncthreads();
-    if (S.status != DEC_OK) {
-        if (tid == 0) status[b] = S.status;
+    if (PASS == 0) {
+        info->len = out;
+        info->status = st;
+        uint64_t *perm = reinterpret_cast<uint64_t *>(slot + kSegPerm + (size_t)s * 256);
+        for (int k = 0; k < 32; k++) perm[k] = list[k * kSegThreadsM];
+    } else {
+        if (acc_n) {
+            const int o = out & 7;
+            for (int k = o - acc_n; k < o; k++) L[out - o + k] = (uint8_t)(acc >> (8 * k));
+        }
+        if (st != DEC_OK || out - out0 != info->len) meta[b].status = st != DEC_OK ? st : DEC_BAD_DATA;
+    }
+}
+
+// One CTA per block: the list at every segment's start (byte values) and the
+// output offsets.
+__global__ void __launch_bounds__(256) dec_chain_kernel(DecMeta *__restrict__ meta, const DecTab *__restrict__ tabs, size_t tab_stride,
+                                                        uint8_t *__restrict__ seg_all) {
+    constexpr int kAhead = 32, PER = kSegs / 256;
+    __shared__ __align__(16) uint8_t perm[2][kAhead * 256];
+    __shared__ uint8_t list[2][256];
+    __shared__ int sh[33];
+    const int b = blockIdx.x, t = threadIdx.x;
+    DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
+    uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
+    SegInfo *info = reinterpret_cast<SegInfo *>(slot + kSegInfo);
+    const uint4 *in = reinterpret_cast<const uint4 *>(slot + kSegPerm);
+    uint8_t *lists = slot + kSegList;
+    // output offsets
+    int c[PER], sum = 0, st = DEC_OK;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const SegInfo I = info[t * PER + i];
+        c[i] = I.len;
+        sum += min(I.len, kBlockCap);  // at most 768 x 2^20: no overflow
+        if (I.status != DEC_OK) st = I.status;
+    }
+    int total;
+    int off = block_excl_sum<int>(sum, sh, &total);
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        info[t * PER + i].off = off;
+        off += c[i];
+    }
+    const int bad = __syncthreads_or(st != DEC_OK);
+    if (bad || total > M.block_max || total > kBlockCap || M.orig >= total) {
+        if (t == 0) M.status = bad ? DEC_BAD_DATA : M.orig >= total && total <= M.block_max ? DEC_BAD_ORIG : DEC_OVERFLOW;
         return;
     }
-    const int n = S.out_len;
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int a = min(n, tid * per), e = min(n, a + per);
-    uint32_t r = 0;
-    for (int i = a; i < e; i++) r = (r << 8) ^ S.crc_tab[(r >> 24) ^ D.dst[i]];
-    if (e > a) r = gf_mul(r, xpow8((uint64_t)(n - e)));
-    for (int o = 16; o > 0; o >>= 1) r ^= __shfl_xor_sync(LFC_FULL, r, o);
-    if (lane == 0) S.red[w] = r;
+    if (t == 0) M.m = total;
+    list[0][t] = t < M.n_in_use ? T.seq_to_unseq[t] : (uint8_t)0;
+    for (int i = t; i < kAhead * 16; i += 256) reinterpret_cast<uint4 *>(perm[0])[i] = in[i];
     __syncthreads();
-    if (tid == 0) {
-        uint32_t t = 0;
-        for (int i = 0; i < NW; i++) t ^= S.red[i];
-        t ^= gf_mul(0xFFFFFFFFu, xpow8((uint64_t)n));
-        status[b] = (~t == S.stored_crc) ? DEC_OK : DEC_BAD_CRC;
+    for (int s0 = 0; s0 < kSegs; s0 += kAhead) {
+        const int buf = (s0 / kAhead) & 1;
+        if (s0 + kAhead < kSegs)
+            for (int i = t; i < kAhead * 16; i += 256) reinterpret_cast<uint4 *>(perm[buf ^ 1])[i] = in[(s0 + kAhead) * 16 + i];
+        for (int k = 0; k < kAhead; k++) {
+            const uint8_t v = list[k & 1][t];
+            lists[(size_t)(s0 + k) * 256 + t] = v;
+            list[(k & 1) ^ 1][t] = list[k & 1][perm[buf][k * 256 + t]];
+            __syncthreads();
+        }
     }
+}
+
+// -------------------------------------------------------- 5. LF mapping
+// next[j] = C[L[j]] + rank of j among equal bytes; a row's word holds it with
+// the row's byte above (bits 20 .. 27).
+constexpr int kLfThreads = 256;
+
+__global__ void __launch_bounds__(kLfThreads) dec_lf_count_kernel(const DecMeta *__restrict__ meta, const uint8_t *__restrict__ L_all,
+                                                                  uint32_t *__restrict__ hist_all) {
+    __shared__ uint32_t h[256];
+    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK || tile * kTile >= M.m) return;
+    h[t] = 0;
+    __syncthreads();
+    const int a = tile * kTile + 16 * t, m = M.m;
+    const uint8_t *L = L_all + (size_t)b * kBlockCap;
+    if (a + 16 <= m) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(L + a);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 16; k++) atomicAdd(&h[(w[k >> 2] >> (8 * (k & 3))) & 255u], 1u);
+    } else {
+        for (int k = a; k < m; k++) atomicAdd(&h[L[k]], 1u);
+    }
+    __syncthreads();
+    hist_all[(size_t)b * kBlockCap + (size_t)tile * 256 + t] = h[t];
+}
+
+// One CTA per block: per tile and byte, the row of the tile's first such byte.
+__global__ void __launch_bounds__(256) dec_lf_scan_kernel(const DecMeta *__restrict__ meta, uint32_t *__restrict__ hist_all) {
+    __shared__ uint32_t sh[33];
+    const int b = blockIdx.x, t = threadIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    uint32_t *h = hist_all + (size_t)b * kBlockCap;
+    const int nt = (M.m + kTile - 1) / kTile;
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (int i = 0; i < nt; i++) sum += h[i * 256 + t];
+    uint32_t at = block_excl_sum<uint32_t>(sum, sh, nullptr);
+#pragma unroll 8
+    for (int i = 0; i < nt; i++) {
+        const uint32_t c = h[i * 256 + t];
+        h[i * 256 + t] = at;
+        at += c;
+    }
+}
+
+__global__ void __launch_bounds__(kLfThreads) dec_lf_map_kernel(const DecMeta *__restrict__ meta, const uint8_t *__restrict__ L_all,
+                                                                const uint32_t *__restrict__ hist_all, uint32_t *__restrict__ P_all) {
+    constexpr int NW = kLfThreads / 32;
+    __shared__ uint32_t wc[NW][256];
+    __shared__ __align__(16) uint8_t by[kTile];
+    const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK || tile * kTile >= M.m) return;
+    const int cnt = min(kTile, M.m - tile * kTile);
+    const uint8_t *L = L_all + (size_t)b * kBlockCap + (size_t)tile * kTile;
+    reinterpret_cast<uint4 *>(by)[t] = *reinterpret_cast<const uint4 *>(L + 16 * t);  // the slot holds whole tiles
+    for (int i = t; i < NW * 256; i += kLfThreads) (&wc[0][0])[i] = 0;
+    __syncthreads();
+    // warp w: bytes [512 w, 512 w + 512) of the tile, 32 at a time in order
+    uint32_t rk[kTile / kLfThreads];
+#pragma unroll
+    for (int r = 0; r < kTile / kLfThreads; r++) {
+        const int k = w * 512 + r * 32 + lane;
+        const bool ok = k < cnt;
+        const uint32_t c = by[k];
+        const uint32_t mm = __match_any_sync(LFC_FULL, ok ? c : 256u + lane);
+        uint32_t before = 0;
+        if (ok) before = wc[w][c];
+        __syncwarp();
+        if (ok && (mm & lanemask_gt()) == 0) wc[w][c] = before + __popc(mm);
+        __syncwarp();
+        rk[r] = before + __popc(mm & lanemask_lt());
+    }
+    __syncthreads();
+    uint32_t at = hist_all[(size_t)b * kBlockCap + (size_t)tile * 256 + t];
+#pragma unroll
+    for (int i = 0; i < NW; i++) {
+        const uint32_t c = wc[i][t];
+        wc[i][t] = at;
+        at += c;
+    }
+    __syncthreads();
+    uint32_t *P = P_all + (size_t)b * kBlockCap + (size_t)tile * kTile;
+#pragma unroll
+    for (int r = 0; r < kTile / kLfThreads; r++) {
+        const int k = w * 512 + r * 32 + lane;
+        if (k < cnt) P[k] = (wc[w][by[k]] + rk[r]) | ((uint32_t)by[k] << 20);
+    }
+}
+
+// ------------------------------------------------------- 6. inverse BWT
+constexpr int kWalkStep = 64;                             // rows between walkers
+constexpr int kWalkMax = kBlockCap / kWalkStep + 2;       // walkers of a block
+constexpr uint32_t kRowMask = (1u << 20) - 1u;
+// walker records in a block's slot: length, next walker, output position
+constexpr size_t kWalkLen = 0, kWalkNext = kWalkMax, kWalkPos = 2 * (size_t)kWalkMax;
+
+// Walker 0 starts at the origin row, walker k > 0 at row (k - 1) kWalkStep.
+__device__ __forceinline__ int walk_start(int k, int orig) { return k == 0 ? orig : (k - 1) * kWalkStep; }
+
+__global__ void __launch_bounds__(256) dec_walk_kernel(const DecMeta *__restrict__ meta, const uint32_t *__restrict__ P_all,
+                                                       int32_t *__restrict__ rec_all) {
+    const int b = blockIdx.y, k = blockIdx.x * 256 + (int)threadIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    const int m = M.m, orig = M.orig, K = (m + kWalkStep - 1) / kWalkStep + 1;
+    if (k >= K) return;
+    const uint32_t *P = P_all + (size_t)b * kBlockCap;
+    int32_t *rec = rec_all + (size_t)b * kBlockCap;
+    int r = walk_start(k, orig), steps = 0;
+    if (k > 0 && r == orig) {  // walker 0's row
+        rec[kWalkLen + k] = 0;
+        rec[kWalkNext + k] = 0;
+        return;
+    }
+    do {  // the rows form cycles, so a walk ends at its own row at the latest
+        r = (int)(P[r] & kRowMask);
+        steps++;
+    } while (r != orig && (r & (kWalkStep - 1)) != 0);
+    rec[kWalkLen + k] = steps;
+    rec[kWalkNext + k] = r == orig ? 0 : r / kWalkStep + 1;
+}
+
+// One CTA per block: where each walker's piece goes, from its distance to
+// the end of the list (walker 0 first, ended by the return to it).
+struct RankSmem {
+    uint32_t d[2][kWalkMax + 1];
+    uint16_t nx[2][kWalkMax + 1];
+};
+__global__ void __launch_bounds__(1024) dec_rank_kernel(DecMeta *__restrict__ meta, int32_t *__restrict__ rec_all) {
+    extern __shared__ __align__(16) uint8_t smraw[];
+    RankSmem &S = *reinterpret_cast<RankSmem *>(smraw);
+    const int b = blockIdx.x, t = threadIdx.x;
+    DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    const int m = M.m, K = (m + kWalkStep - 1) / kWalkStep + 1;
+    int32_t *rec = rec_all + (size_t)b * kBlockCap;
+    for (int k = t; k <= K; k += 1024) {
+        const int nx = k < K ? rec[kWalkNext + k] : 0;
+        S.d[0][k] = k < K ? (uint32_t)rec[kWalkLen + k] : 0u;
+        S.nx[0][k] = (uint16_t)(k == K || nx == 0 ? K : nx);
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int span = 1; span < K; span <<= 1, cur ^= 1) {
+        for (int k = t; k <= K; k += 1024) {
+            const int nx = S.nx[cur][k];
+            S.d[cur ^ 1][k] = min(S.d[cur][k] + S.d[cur][nx], 1u << 30);  // off the list the sums only have to stay finite
+            S.nx[cur ^ 1][k] = S.nx[cur][nx];
+        }
+        __syncthreads();
+    }
+    if (S.d[cur][0] != (uint32_t)m || S.nx[cur][0] != K) {  // not one cycle over all rows
+        if (t == 0) M.status = DEC_BAD_WALK;
+        return;
+    }
+    for (int k = t; k < K; k += 1024) rec[kWalkPos + k] = m - (int)S.d[cur][k];
+}
+
+__global__ void __launch_bounds__(256) dec_emit_kernel(const DecMeta *__restrict__ meta, const uint32_t *__restrict__ P_all,
+                                                       const int32_t *__restrict__ rec_all, uint8_t *__restrict__ blk_all) {
+    const int b = blockIdx.y, k = blockIdx.x * 256 + (int)threadIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    const int m = M.m, K = (m + kWalkStep - 1) / kWalkStep + 1;
+    if (k >= K) return;
+    const uint32_t *P = P_all + (size_t)b * kBlockCap;
+    const int32_t *rec = rec_all + (size_t)b * kBlockCap;
+    uint8_t *blk = blk_all + (size_t)b * kBlockCap;
+    const int len = rec[kWalkLen + k];
+    int r = walk_start(k, M.orig);
+    int at = m - rec[kWalkPos + k];  // bytes go to at - 1, at - 2, ...
+    uint64_t acc = 0;
+    int n = 0;  // bytes of the 8-byte word being filled, from its end
+    for (int s = 0; s < len; s++) {
+        const uint32_t p = P[r];
+        r = (int)(p & kRowMask);
+        at--;
+        acc |= (uint64_t)(p >> 20) << (8 * (at & 7));
+        n++;
+        if ((at & 7) == 0) {
+            if (n == 8) *reinterpret_cast<uint64_t *>(blk + at) = acc;
+            else
+                for (int q = 0; q < n; q++) blk[at + q] = (uint8_t)(acc >> (8 * q));
+            acc = 0;
+            n = 0;
+        }
+    }
+    for (int q = 0; q < n; q++) blk[at + q] = (uint8_t)(acc >> (8 * ((at & 7) + q)));
+}
+
+// ----------------------------------------------------- 7. inverse RLE1
+// A position q is a sync point when bytes q-2 and q-1 differ and bytes q-5 ..
+// q-2 are not all equal: byte q-1 is then a literal (a count byte follows
+// four equal literals) that starts a run, so decoding can start at q from
+// (run 1, last = byte q-1). A thread starts at the first sync point of its 16
+// bytes (the block's first thread at 0, fresh) and stops at the first one
+// past them.
+constexpr int kUnThreads = 256;
+constexpr int kUnStage = 3 * kTile;  // output bytes of a tile staged in shared memory
+
+__device__ __forceinline__ bool rle_sync(const uint8_t *blk, int q) {
+    const uint8_t b1 = blk[q - 1], b2 = blk[q - 2];
+    return b1 != b2 && !(blk[q - 5] == b2 && blk[q - 4] == b2 && blk[q - 3] == b2);
+}
+
+// Walks the thread's bytes; put(byte, count) takes each literal (count 1) and
+// repeat. Returns the output bytes, or -1 for a missing count byte.
+template <typename Put>
+__device__ __forceinline__ int rle_walk(const uint8_t *blk, int m, int a, Put put) {
+    const int e = min(m, a + 16);
+    int p = a;
+    if (a > 0) {
+        for (p = max(a, 5); p < e && !rle_sync(blk, p); p++) {}
+        if (p >= e) return 0;
+    }
+    int o = 0, same = p == 0 ? 0 : 1, last = p == 0 ? -1 : (int)blk[p - 1];
+    for (int i = p; i < m; i++) {
+        if (i >= max(a + 16, 5) && rle_sync(blk, i)) break;
+        const uint8_t v = blk[i];
+        put(v, 1, o);
+        o++;
+        same = (int)v == last ? same + 1 : 1;
+        last = v;
+        if (same == 4) {
+            if (i + 1 >= m) return -1;
+            const int extra = blk[++i];
+            put(v, extra, o);
+            o += extra;
+            same = 0;
+            last = -1;
+        }
+    }
+    return o;
+}
+
+__global__ void __launch_bounds__(kUnThreads) dec_unrle_count_kernel(DecMeta *__restrict__ meta, const uint8_t *__restrict__ blk_all,
+                                                                     int32_t *__restrict__ aux_all) {
+    __shared__ int sh[33];
+    const int b = blockIdx.y, tile = blockIdx.x;
+    DecMeta &M = meta[b];
+    if (__syncthreads_or(M.status != DEC_OK) || tile * kTile >= M.m) return;  // one answer for the CTA, as above
+    const int a = tile * kTile + 16 * (int)threadIdx.x;
+    int n = a < M.m ? rle_walk(blk_all + (size_t)b * kBlockCap, M.m, a, [](uint8_t, int, int) {}) : 0;
+    if (__syncthreads_or(n < 0)) {
+        if (threadIdx.x == 0) M.status = DEC_BAD_DATA;
+        n = 0;
+    }
+    int total;
+    block_excl_sum<int>(n, sh, &total);
+    if (threadIdx.x == 0) aux_all[((size_t)b * kTilesPerBlock + tile) * 4] = total;
+}
+
+__global__ void __launch_bounds__(256) dec_unrle_scan_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
+                                                             int32_t *__restrict__ aux_all) {
+    __shared__ int sh[33];
+    const int b = blockIdx.x, t = threadIdx.x;
+    DecMeta &M = meta[b];
+    if (M.status != DEC_OK) return;
+    const int nt = (M.m + kTile - 1) / kTile;  // <= 220
+    int32_t *aux = aux_all + (size_t)b * kTilesPerBlock * 4;
+    int total;
+    const int off = block_excl_sum<int>(t < nt ? aux[t * 4] : 0, sh, &total);
+    if (t < nt) aux[t * 4 + 1] = off;
+    if (t == 0 && total != blocks[b].expect) M.status = DEC_BAD_LEN;
+}
+
+__global__ void __launch_bounds__(kUnThreads) dec_unrle_write_kernel(const DecBlock *__restrict__ blocks, const DecMeta *__restrict__ meta,
+                                                                     const uint8_t *__restrict__ blk_all,
+                                                                     const int32_t *__restrict__ aux_all) {
+    __shared__ int sh[33];
+    __shared__ uint8_t ob[kUnStage];
+    const int b = blockIdx.y, tile = blockIdx.x;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK || tile * kTile >= M.m) return;
+    const uint8_t *blk = blk_all + (size_t)b * kBlockCap;
+    const int a = tile * kTile + 16 * (int)threadIdx.x;
+    const int n = a < M.m ? rle_walk(blk, M.m, a, [](uint8_t, int, int) {}) : 0;
+    int total;
+    const int o = block_excl_sum<int>(n, sh, &total);
+    uint8_t *dst = blocks[b].dst + aux_all[((size_t)b * kTilesPerBlock + tile) * 4 + 1];
+    const bool staged = total <= kUnStage;
+    uint8_t *to = (staged ? ob : dst) + o;  // the scan checked the block's total against the promised length
+    if (n)
+        rle_walk(blk, M.m, a, [&](uint8_t v, int cnt, int at) {
+            for (int k = 0; k < cnt; k++) to[at + k] = v;
+        });
+    if (!staged) return;
+    __syncthreads();
+    for (int k = threadIdx.x; k < total; k += kUnThreads) dst[k] = ob[k];
+}
+
+// Final status per block: what failed, or the CRC check.
+__global__ void dec_status_kernel(const DecMeta *__restrict__ meta, int nblocks, int32_t *__restrict__ status) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= nblocks) return;
+    const DecMeta &M = meta[b];
+    status[b] = M.status != DEC_OK ? M.status : (M.crc == M.stored_crc ? DEC_OK : DEC_BAD_CRC);
+}
+
+cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const void *d_blocks, int nblocks, const uint8_t *d_crc,
+                                const CrcRun &crc, int32_t *d_status) {
+    Workspace &ws = P->ws;
+    cudaStream_t s = P->stream;
+    const DecBlock *blocks = reinterpret_cast<const DecBlock *>(d_blocks);
+    DecMeta *meta = reinterpret_cast<DecMeta *>(ws.bstate);
+    DecTab *tabs = reinterpret_cast<DecTab *>(ws.act2);
+    const size_t ts = sizeof(int32_t) * (size_t)kBlockCap;
+    uint8_t *segs = reinterpret_cast<uint8_t *>(ws.act);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(ws.val);  // the group offsets' slot, free once the symbols are out
+    uint32_t *rows = reinterpret_cast<uint32_t *>(ws.sa);
+    const size_t list_smem = (size_t)256 * kSegThreadsM;
+    cudaError_t e = cudaFuncSetAttribute(dec_chase_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ChaseSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(dec_jump_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(JumpSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(dec_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankSmem));
+    if (e != cudaSuccess) return e;
+    int64_t max_bits = 0;
+    for (int b = 0; b < nblocks; b++)
+        if (h_blocks[b].src_len * 8 > max_bits) max_bits = h_blocks[b].src_len * 8;
+    dec_header_kernel<<<nblocks, kHdrThreads, 0, s>>>(blocks, meta, tabs, ts, ws.sel, ws.val);
+    int launches = 14;
+    for (int64_t r0 = 0; r0 < max_bits; r0 += kJRange, launches += 2) {
+        const int64_t n = max_bits - r0 < kJRange ? max_bits - r0 : kJRange;
+        dec_jump_kernel<<<dim3((unsigned)((n + kJTile - 1) / kJTile), nblocks), kJThreads, sizeof(JumpSmem), s>>>(
+            blocks, meta, tabs, ts, r0, ws.keys, ws.keys2);
+        dec_chase_kernel<<<nblocks, kChaseThreads, sizeof(ChaseSmem), s>>>(blocks, meta, tabs, ts, r0, ws.keys, ws.keys2, ws.sel, ws.val);
+    }
+    dec_symbols_kernel<<<dim3((kMaxSelectors + kSymGroups - 1) / kSymGroups, nblocks), kSymGroups, 0, s>>>(blocks, meta, tabs, ts, ws.sel,
+                                                                                                          ws.val, ws.sym);
+    const dim3 seg_grid(kSegs / kSegThreadsM, nblocks), tiles(kTilesPerBlock, nblocks), walkers((kWalkMax + 255) / 256, nblocks);
+    dec_mtf_kernel<0><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
+    dec_chain_kernel<<<nblocks, 256, 0, s>>>(meta, tabs, ts, segs);
+    dec_mtf_kernel<1><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
+    dec_lf_count_kernel<<<tiles, kLfThreads, 0, s>>>(meta, ws.bwt, hist);
+    dec_lf_scan_kernel<<<nblocks, 256, 0, s>>>(meta, hist);
+    dec_lf_map_kernel<<<tiles, kLfThreads, 0, s>>>(meta, ws.bwt, hist, rows);
+    dec_walk_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2);
+    dec_rank_kernel<<<nblocks, 1024, sizeof(RankSmem), s>>>(meta, ws.sa2);
+    dec_emit_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2, ws.rle);
+    dec_unrle_count_kernel<<<tiles, kUnThreads, 0, s>>>(meta, ws.rle, ws.tileaux);
+    dec_unrle_scan_kernel<<<nblocks, 256, 0, s>>>(blocks, meta, ws.tileaux);
+    dec_unrle_write_kernel<<<tiles, kUnThreads, 0, s>>>(blocks, meta, ws.rle, ws.tileaux);
+    e = launch_crc(P, d_crc, crc, &meta[0].crc, (int)(sizeof(DecMeta) / 4));
+    if (e != cudaSuccess) return e;
+    dec_status_kernel<<<(nblocks + 127) / 128, 128, 0, s>>>(meta, nblocks, d_status);
+    count_launches(P, launches);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------ inverse predictor
@@ -757,13 +1170,6 @@ __device__ __forceinline__ int32_t gp(int f, int row, int col, int32_t A, int32_
     return jp(f, A, B, C);
 }
 
-struct InvFrame {
-    const uint16_t *Z;      // symbol stream (stream order)
-    const uint16_t *prev;   // previous raw frame or nullptr
-    uint16_t *X;            // output frame
-    int32_t *E;             // int32 scratch field (W*H)
-    int32_t W, H, p, id;
-};
 
 __device__ __forceinline__ size_t stream_index(const InvFrame &F, int y, int x) {
     if (!((F.id >> 6) & 1)) return (size_t)y * F.W + x;
@@ -773,7 +1179,8 @@ __device__ __forceinline__ size_t stream_index(const InvFrame &F, int y, int x) 
 }
 
 // Residual field e at every pixel (raw for f == 0 without temporal).
-__global__ void inv_residual_kernel(InvFrame F) {
+__global__ void inv_residual_kernel(const InvFrame *__restrict__ frames) {
+    const InvFrame F = frames[blockIdx.y];
     const int64_t n = (int64_t)F.W * F.H;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int y = (int)(k / F.W), x = (int)(k % F.W);
@@ -790,35 +1197,65 @@ __global__ void inv_residual_kernel(InvFrame F) {
 // Inter-lenslet inverse over the view grid of every (u, v): one CTA per
 // view restores its Ny x Nx grid by anti-diagonals (cell (t, s) needs the
 // cells left, above and above-left, all on the two previous diagonals), one
-// thread per cell of a diagonal. signed_out: keep the result as signed
-// 16-bit (phase stage / temporal fields).
-__global__ void __launch_bounds__(128) inv_inter_kernel(InvFrame F, int signed_field) {
+// thread per cell of a diagonal. The result stays a signed 16-bit field for
+// the phase stage and temporal frames. The grid is staged in shared memory
+// (its cells are p pixels apart in memory, and a diagonal is one dependent
+// step: 60 against 600 cycles); one that does not fit is restored in place.
+constexpr int kInterThreads = 256;
+
+__global__ void __launch_bounds__(kInterThreads) inv_inter_kernel(const InvFrame *__restrict__ frames, int smem_cells) {
+    extern __shared__ __align__(16) uint16_t cells[];
+    const InvFrame F = frames[blockIdx.y];
     const int p = F.p, Nx = F.W / p, Ny = F.H / p;
     const int view = blockIdx.x;
+    const int f = id_f(F.id), dom = id_dom(F.id);
+    if (f == 0 || dom == 0 || view >= p * p) return;
+    const bool signed_field = dom == 2 || id_tmp(F.id);
     const int v = view / p, u = view % p;
-    const int f = id_f(F.id);
-    for (int d = 0; d < Nx + Ny - 1; d++) {
-        const int t_lo = max(0, d - (Nx - 1)), t_hi = min(Ny - 1, d);
-        for (int t = t_lo + (int)threadIdx.x; t <= t_hi; t += blockDim.x) {
-            const int s = d - t;
-            const size_t k = (size_t)(t * p + v) * F.W + s * p + u;
-            const int32_t A = s > 0 ? F.E[k - p] : 0;
-            const int32_t B = t > 0 ? F.E[k - (size_t)p * F.W] : 0;
-            const int32_t C = (s > 0 && t > 0) ? F.E[k - (size_t)p * F.W - p] : 0;
-            const uint32_t val = ((uint32_t)F.E[k] + (uint32_t)gp(f, t, s, A, B, C)) & 0xFFFFu;
-            F.E[k] = signed_field ? as_s16(val) : (int32_t)val;
+    int32_t *E = F.E + (size_t)v * F.W + u;
+    const size_t row = (size_t)p * F.W;
+    const bool staged = Nx * Ny <= smem_cells;
+    if (staged) {
+        for (int q = threadIdx.x; q < Nx * Ny; q += kInterThreads) {
+            const int t = q / Nx, s = q - t * Nx;
+            cells[q] = (uint16_t)E[t * row + (size_t)s * p];
         }
         __syncthreads();
     }
+    auto get = [&](int t, int s) -> int32_t {
+        if (!staged) return E[t * row + (size_t)s * p];
+        const uint32_t x = cells[t * Nx + s];
+        return signed_field ? as_s16(x) : (int32_t)x;
+    };
+    for (int d = 0; d < Nx + Ny - 1; d++) {
+        const int t_lo = max(0, d - (Nx - 1)), t_hi = min(Ny - 1, d);
+        for (int t = t_lo + (int)threadIdx.x; t <= t_hi; t += kInterThreads) {
+            const int s = d - t;
+            const int32_t A = s > 0 ? get(t, s - 1) : 0;
+            const int32_t B = t > 0 ? get(t - 1, s) : 0;
+            const int32_t C = (s > 0 && t > 0) ? get(t - 1, s - 1) : 0;
+            const uint32_t val = ((uint32_t)get(t, s) + (uint32_t)gp(f, t, s, A, B, C)) & 0xFFFFu;
+            if (staged) cells[t * Nx + s] = (uint16_t)val;
+            else E[t * row + (size_t)s * p] = signed_field ? as_s16(val) : (int32_t)val;
+        }
+        __syncthreads();
+    }
+    if (staged)
+        for (int q = threadIdx.x; q < Nx * Ny; q += kInterThreads) {
+            const int t = q / Nx, s = q - t * Nx;
+            E[t * row + (size_t)s * p] = get(t, s);
+        }
 }
 
 // Intra-lenslet inverse: one thread per lenslet, raster order inside it.
-__global__ void inv_intra_kernel(InvFrame F, int signed_field) {
+__global__ void inv_intra_kernel(const InvFrame *__restrict__ frames) {
+    const InvFrame F = frames[blockIdx.y];
     const int p = F.p, Nx = F.W / p, Ny = F.H / p;
     const int lens = blockIdx.x * blockDim.x + threadIdx.x;
-    if (lens >= Nx * Ny) return;
-    const int t = lens / Nx, s = lens % Nx;
     const int f = id_f(F.id);
+    if (f == 0 || id_dom(F.id) == 1 || lens >= Nx * Ny) return;
+    const bool signed_field = id_tmp(F.id);
+    const int t = lens / Nx, s = lens % Nx;
     for (int v = 0; v < p; v++) {
         for (int u = 0; u < p; u++) {
             const size_t k = (size_t)(t * p + v) * F.W + s * p + u;
@@ -832,7 +1269,8 @@ __global__ void inv_intra_kernel(InvFrame F, int signed_field) {
 }
 
 // Base field -> raw counts (adds the previous frame for temporal ids).
-__global__ void inv_finish_kernel(InvFrame F) {
+__global__ void inv_finish_kernel(const InvFrame *__restrict__ frame) {
+    const InvFrame F = *frame;
     const int64_t n = (int64_t)F.W * F.H;
     const bool tmp = (F.id >> 7) & 1;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -842,43 +1280,31 @@ __global__ void inv_finish_kernel(InvFrame F) {
     }
 }
 
-size_t decode_smem_bytes() { return sizeof(DecShared); }
-
-cudaError_t launch_bzip2_decode(lfc_plan P, const void *d_blocks, int nblocks, int32_t *d_status) {
-    Workspace &ws = P->ws;
-    const size_t smem = sizeof(DecShared);
-    cudaError_t e = cudaFuncSetAttribute(bzip2_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    bzip2_decode_kernel<<<nblocks, kDecThreads, smem, P->stream>>>(reinterpret_cast<const DecBlock *>(d_blocks), d_status,
-                                                                  ws.sel, ws.bwt, ws.sa, ws.sa2, ws.rle);
-    count_launches(P, 1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_inverse_predict(lfc_plan P, const uint16_t *Z, const uint16_t *prev, uint16_t *X, int32_t *E,
-                                   int W, int H, int p, int id) {
-    InvFrame F{Z, prev, X, E, W, H, p, id};
+// The frames of a call at once: residual fields, then the inverse
+// predictors of the frames that have each stage. The last step runs frame by
+// frame, as a temporal frame may need the one before.
+cudaError_t launch_inverse_predict(lfc_plan P, const InvFrame *h_frames, const InvFrame *d_frames, int n) {
     cudaStream_t s = P->stream;
-    const int f = id_f(id), dom = id_dom(id);
-    const bool tmp = id_tmp(id);
-    inv_residual_kernel<<<1216, 256, 0, s>>>(F);
-    int launches = 2;
-    if (f != 0) {
-        const int nl = (W / p) * (H / p), nv = p * p;
-        if (dom == 0) {
-            inv_intra_kernel<<<(nl + 127) / 128, 128, 0, s>>>(F, tmp ? 1 : 0);
-            launches++;
-        } else if (dom == 1) {
-            inv_inter_kernel<<<nv, 128, 0, s>>>(F, tmp ? 1 : 0);
-            launches++;
-        } else {
-            inv_inter_kernel<<<nv, 128, 0, s>>>(F, 1);
-            inv_intra_kernel<<<(nl + 127) / 128, 128, 0, s>>>(F, tmp ? 1 : 0);
-            launches += 2;
-        }
+    int lenslets = 0, views = 0, cells = 0;
+    constexpr int kCellsMax = 100 * 1024;  // 16-bit cells of a view's grid in shared memory
+    bool inter = false, intra = false;
+    for (int i = 0; i < n; i++) {
+        const InvFrame &F = h_frames[i];
+        const int f = id_f(F.id), dom = id_dom(F.id);
+        inter |= f != 0 && dom != 0;
+        intra |= f != 0 && dom != 1;
+        const int nl = (F.W / F.p) * (F.H / F.p), nv = F.p * F.p;
+        lenslets = nl > lenslets ? nl : lenslets;
+        views = nv > views ? nv : views;
+        if (nl <= kCellsMax && nl > cells) cells = nl;
     }
-    inv_finish_kernel<<<1216, 256, 0, s>>>(F);
-    count_launches(P, launches);
+    const cudaError_t e = cudaFuncSetAttribute(inv_inter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCellsMax * 2);
+    if (e != cudaSuccess) return e;
+    inv_residual_kernel<<<dim3(1216, n), 256, 0, s>>>(d_frames);
+    if (inter) inv_inter_kernel<<<dim3(views, n), kInterThreads, 2 * (size_t)cells, s>>>(d_frames, cells);
+    if (intra) inv_intra_kernel<<<dim3((lenslets + 127) / 128, n), 128, 0, s>>>(d_frames);
+    for (int i = 0; i < n; i++) inv_finish_kernel<<<1216, 256, 0, s>>>(d_frames + i);
+    count_launches(P, 1 + inter + intra + n);
     return cudaGetLastError();
 }
 

@@ -358,9 +358,6 @@ size_t crc_table_bytes(int nchunks, int n);
 void crc_build_tables(const uint8_t *const *ptr, const int64_t *len, int n, uint8_t *out, CrcRun *run);
 cudaError_t launch_crc(lfc_plan P, const uint8_t *d_tables, const CrcRun &run, uint32_t *out, int out_stride_words,
                        cudaStream_t stream = nullptr, uint32_t *part = nullptr);
-cudaError_t launch_block_crc(lfc_plan P, const BlockDesc *h_blocks, int nblocks, BlockState *d_state);
-cudaError_t launch_range_crc(lfc_plan P, const uint8_t *const *h_ptr, const int64_t *h_len, int n,
-                             uint32_t *d_out);
 
 // bwt.cu
 cudaError_t launch_rle1(lfc_plan P, int nblocks, const BlockDesc *d_blocks);
@@ -392,8 +389,16 @@ struct DecBlockHost {
     int32_t expect;
     int32_t pad;
 };
-cudaError_t launch_bzip2_decode(lfc_plan P, const void *d_blocks, int nblocks, int32_t *d_status);
-cudaError_t launch_inverse_predict(lfc_plan P, const uint16_t *Z, const uint16_t *prev, uint16_t *X, int32_t *E,
-                                   int W, int H, int p, int id);
+// d_crc / crc: a CRC run over the blocks' output ranges, laid out by the caller
+cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const void *d_blocks, int nblocks, const uint8_t *d_crc,
+                                const CrcRun &crc, int32_t *d_status);
+struct InvFrame {
+    const uint16_t *Z;      // symbol stream (stream order)
+    const uint16_t *prev;   // previous raw frame or nullptr
+    uint16_t *X;            // output frame
+    int32_t *E;             // int32 scratch field (W*H)
+    int32_t W, H, p, id;
+};
+cudaError_t launch_inverse_predict(lfc_plan P, const InvFrame *h_frames, const InvFrame *d_frames, int n);
 
 }  // namespace lfc
