@@ -60,14 +60,14 @@ __device__ __forceinline__ void build_tables(uint32_t (*T)[256]) {
 
 // One CTA per chunk, seen as front-padded with zeros to kCrcChunk bytes
 // (leading zeros leave a zero register unchanged): thread t reduces the
-// 256-byte piece t four bytes at a time, then the warps merge their pieces
-// in a shuffle tree (level j shifts the left half by x^(8 * 256 * 2^j)), the
-// warps are merged in order, and the chunk remainder is shifted by the bytes
-// of its range that follow it.
+// 256-byte piece t four bytes at a time, then the pieces are merged in a
+// shuffle tree (level j shifts the left half by x^(8 * 256 * 2^j)), and the
+// chunk remainder is shifted by the bytes of its range that follow it.
 constexpr int kCrcPiece = kCrcChunk / 256;
-// shuffle-tree level j merges halves of 2^j pieces; level 5 merges warps
-__constant__ uint32_t c_crc_pow[6] = {x_pow_8k(kCrcPiece),      x_pow_8k(kCrcPiece * 2),  x_pow_8k(kCrcPiece * 4),
-                                      x_pow_8k(kCrcPiece * 8),  x_pow_8k(kCrcPiece * 16), x_pow_8k(kCrcPiece * 32)};
+// tree level j merges halves of 2^j pieces: 0 .. 4 inside a warp, 5 .. 7 the warps
+__constant__ uint32_t c_crc_pow[8] = {x_pow_8k(kCrcPiece),      x_pow_8k(kCrcPiece * 2),  x_pow_8k(kCrcPiece * 4),
+                                      x_pow_8k(kCrcPiece * 8),  x_pow_8k(kCrcPiece * 16), x_pow_8k(kCrcPiece * 32),
+                                      x_pow_8k(kCrcPiece * 64), x_pow_8k(kCrcPiece * 128)};
 
 __global__ void __launch_bounds__(256) crc_chunk_kernel(const CrcChunk *__restrict__ chunks, uint32_t *__restrict__ part) {
     __shared__ uint32_t T[4][256];
@@ -78,20 +78,38 @@ __global__ void __launch_bounds__(256) crc_chunk_kernel(const CrcChunk *__restri
     const int start = (int)threadIdx.x * kCrcPiece - pad;  // real offset of the piece
     uint32_t r = 0;
     if (start + kCrcPiece > 0) {
-        const bool fast = start >= 0 && (((uintptr_t)(c.src + start)) & 3) == 0;
-        for (int i = 0; i < kCrcPiece; i += 4) {
-            uint32_t w;
-            if (fast) {
-                w = __byte_perm(__ldg(reinterpret_cast<const uint32_t *>(c.src + start + i)), 0u, 0x0123);
-            } else {
-                w = 0;
+        // a piece takes as long as its loads do, so several are in flight: 16
+        // bytes each where they are aligned, else aligned words joined by a
+        // funnel shift (byte loads one after the other took 19 us). Words
+        // that hold a byte of the piece are read whole.
+        const uintptr_t at = (uintptr_t)(c.src + start);
+        if (start >= 0 && (at & 15) == 0) {
+            const uint4 *in = reinterpret_cast<const uint4 *>(at);
+#pragma unroll 4
+            for (int i = 0; i < kCrcPiece / 16; i++) {
+                const uint4 v = __ldg(in + i);
+                const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
                 for (int q = 0; q < 4; q++) {
-                    const int o = start + i + q;
-                    w = (w << 8) | (o >= 0 ? (uint32_t)c.src[o] : 0u);
+                    r ^= __byte_perm(w4[q], 0u, 0x0123);
+                    r = T[3][r >> 24] ^ T[2][(r >> 16) & 255u] ^ T[1][(r >> 8) & 255u] ^ T[0][r & 255u];
                 }
             }
-            r ^= w;
-            r = T[3][r >> 24] ^ T[2][(r >> 16) & 255u] ^ T[1][(r >> 8) & 255u] ^ T[0][r & 255u];
+        } else {
+            const uint32_t *in = reinterpret_cast<const uint32_t *>(at & ~(uintptr_t)3);
+            const int sh = 8 * (int)(at & 3);
+#pragma unroll 8
+            for (int i = 0; i < kCrcPiece / 4; i++) {
+                const int o = start + 4 * i;  // of the word's first byte; the range begins at 0
+                uint32_t w = 0;
+                if (o + 3 >= 0) {
+                    const uint32_t a = __ldg(in + i), b = sh ? __ldg(in + i + 1) : 0u;
+                    w = __byte_perm(__funnelshift_r(a, b, sh), 0u, 0x0123);
+                    if (o < 0) w &= 0xFFFFFFFFu >> (-8 * o);
+                }
+                r ^= w;
+                r = T[3][r >> 24] ^ T[2][(r >> 16) & 255u] ^ T[1][(r >> 8) & 255u] ^ T[0][r & 255u];
+            }
         }
     }
     const int lane = threadIdx.x & 31;
@@ -103,10 +121,15 @@ __global__ void __launch_bounds__(256) crc_chunk_kernel(const CrcChunk *__restri
     }
     if (lane == 0) red[threadIdx.x >> 5] = r;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t t = red[0];
-        for (int i = 1; i < (int)(blockDim.x >> 5); i++) t = gf_mulmod(t, c_crc_pow[5]) ^ red[i];
-        part[blockIdx.x] = gf_mulmod(t, c.shift);
+    if (threadIdx.x < 8) {  // the eight warps' remainders in the same tree
+        uint32_t t = red[threadIdx.x];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const uint32_t tp = __shfl_xor_sync(0xFFu, t, 1 << j);
+            const bool right = (threadIdx.x >> j) & 1;
+            t = gf_mulmod(right ? tp : t, c_crc_pow[5 + j]) ^ (right ? t : tp);
+        }
+        if (threadIdx.x == 0) part[blockIdx.x] = gf_mulmod(t, c.shift);
     }
 }
 

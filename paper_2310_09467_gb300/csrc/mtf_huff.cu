@@ -392,6 +392,7 @@ struct HuffScratch {
     uint32_t lw[kMaxAlpha];          // leaf weights in (weight, symbol) order
     uint32_t nw[kMaxAlpha];          // joined-node weights
     uint16_t order[kMaxAlpha];       // leaves sorted by (w, symbol)
+    uint16_t lpar[kMaxAlpha];        // parents of the leaves in that order
     uint16_t par[2 * kMaxAlpha];     // parent of a node (leaves, then joined nodes)
     uint16_t dist[2 * kMaxAlpha];    // pointer-jumping distance to par
 };
@@ -433,36 +434,43 @@ __device__ void huff_lengths_warp(const uint32_t *freq, int alpha, int max_len, 
         __syncwarp();
         if (lane == 0) {
             // two-queue merge: the two smallest (weight, key) nodes, a leaf
-            // before a joined node of equal weight (its key is smaller)
-            int la = 0, lb = 0, nb = 0;
-            uint32_t ha = S.lw[0], hb = 0;
+            // before a joined node of equal weight (its key is smaller). The
+            // heads of both queues sit in registers kAhead deep, so that no
+            // pick waits for a load (a pick is a few dependent instructions;
+            // with the loads on the chain a table took 42 us instead of 13).
+            constexpr uint32_t kEmpty = 0xFFFFFFFFu;
+            uint32_t a0 = S.lw[0], a1 = 1 < alpha ? S.lw[1] : kEmpty, a2 = 2 < alpha ? S.lw[2] : kEmpty, a3 = 3 < alpha ? S.lw[3] : kEmpty;
+            uint32_t b0 = kEmpty, b1 = kEmpty, b2 = kEmpty, b3 = kEmpty;
+            int la = 0, lb = 0;  // queue heads; joined nodes made so far: k
             for (int k = 0; k < alpha - 1; k++) {
-                int pick[2];
-                uint32_t pw[2];
+                uint32_t sum = 0;
 #pragma unroll
                 for (int q = 0; q < 2; q++) {
-                    const bool takeA = lb >= nb || (la < alpha && ha <= hb);
-                    if (takeA) {
-                        pick[q] = S.order[la];
-                        pw[q] = ha;
+                    if (a0 <= b0) {  // never both empty
+                        sum += a0;
+                        S.lpar[la] = (uint16_t)(alpha + k);
+                        a0 = a1; a1 = a2; a2 = a3;
+                        a3 = la + 4 < alpha ? S.lw[la + 4] : kEmpty;
                         la++;
-                        ha = la < alpha ? S.lw[la] : 0u;
                     } else {
-                        pick[q] = alpha + lb;
-                        pw[q] = hb;
+                        sum += b0;
+                        S.par[alpha + lb] = (uint16_t)(alpha + k);
+                        b0 = b1; b1 = b2; b2 = b3;
+                        b3 = lb + 4 < k ? S.nw[lb + 4] : kEmpty;
                         lb++;
-                        hb = lb < nb ? S.nw[lb] : 0u;
                     }
                 }
-                const uint32_t sw = pw[0] + pw[1];
-                S.par[pick[0]] = (uint16_t)(alpha + k);
-                S.par[pick[1]] = (uint16_t)(alpha + k);
-                S.nw[nb] = sw;
-                if (lb == nb) hb = sw;  // the joined queue was empty
-                nb++;
+                S.nw[k] = sum;
+                const int n = k - lb;  // joined nodes waiting before this one
+                if (n == 0) b0 = sum;
+                else if (n == 1) b1 = sum;
+                else if (n == 2) b2 = sum;
+                else if (n == 3) b3 = sum;
             }
             S.par[root] = (uint16_t)root;
         }
+        __syncwarp();
+        for (int i = lane; i < alpha; i += 32) S.par[S.order[i]] = S.lpar[i];
         __syncwarp();
         uint16_t pn[kN], dn[kN];
 #pragma unroll
@@ -524,26 +532,29 @@ __device__ __forceinline__ int stage_tile_syms(const uint16_t *sym, int tile, in
 // partition by cumulative frequency (init); four refinement passes, each
 // "every 50-symbol group picks the cheapest table, ties to the lower" over
 // many CTAs (select) followed by "every table is rebuilt from its groups'
-// counts with a 17-bit limit" (build); canonical codes (codes).
+// counts with a 17-bit limit" (build), the last of them with the canonical
+// codes.
 constexpr int kHuffBuildThreads = 32 * kMaxGroups;
 
-__global__ void __launch_bounds__(256) huff_init_kernel(BlockState *__restrict__ st, const uint32_t *__restrict__ freq_all,
-                                                        uint8_t *__restrict__ lens_all, uint32_t *__restrict__ rfreq_all) {
-    const int b = blockIdx.x;
+constexpr int kHuffInitThreads = 288;
+static_assert(kHuffInitThreads >= kMaxAlpha, "a thread per symbol");
+
+__global__ void __launch_bounds__(kHuffInitThreads) huff_init_kernel(BlockState *__restrict__ st, const uint32_t *__restrict__ freq_all,
+                                                                     uint8_t *__restrict__ lens_all, uint32_t *__restrict__ rfreq_all) {
+    __shared__ uint32_t sh[33];
+    const int b = blockIdx.x, v = threadIdx.x;
     const int n_mtf = st[b].n_mtf;
     const int alpha = st[b].n_in_use + 2;
     const int ng = n_mtf < 200 ? 2 : n_mtf < 600 ? 3 : n_mtf < 1200 ? 4 : n_mtf < 2400 ? 5 : 6;
-    for (int i = threadIdx.x; i < kMaxGroups * kMaxAlpha; i += blockDim.x) rfreq_all[(size_t)b * kMaxGroups * kMaxAlpha + i] = 0;
-    if (threadIdx.x == 0) {
-        const uint32_t *freq = freq_all + (size_t)b * kMaxAlpha;
+    for (int i = v; i < kMaxGroups * kMaxAlpha; i += blockDim.x) rfreq_all[(size_t)b * kMaxGroups * kMaxAlpha + i] = 0;
+    const uint32_t f = v < alpha ? freq_all[(size_t)b * kMaxAlpha + v] : 0u;
+    const uint32_t cum = block_excl_sum<uint32_t>(f, sh, nullptr);  // cum * ng < 2^23
+    if (v < alpha) {
+        const int gsel = min((int)(cum * (uint32_t)ng / (uint32_t)n_mtf), ng - 1);
         uint8_t *len = lens_all + (size_t)b * kMaxGroups * kMaxAlpha;
-        int64_t cum = 0;
-        for (int v = 0; v < alpha; v++) {
-            int64_t gsel = cum * ng / n_mtf;
-            if (gsel > ng - 1) gsel = ng - 1;
-            for (int t = 0; t < ng; t++) len[t * kMaxAlpha + v] = (uint8_t)(t == gsel ? 0 : 15);
-            cum += freq[v];
-        }
+        for (int t = 0; t < ng; t++) len[t * kMaxAlpha + v] = (uint8_t)(t == gsel ? 0 : 15);
+    }
+    if (v == 0) {
         st[b].n_groups = ng;
         st[b].n_sel = (n_mtf + 49) / 50;
     }
@@ -606,13 +617,17 @@ __global__ void __launch_bounds__(kPackGroups) huff_select_kernel(const BlockSta
 }
 
 // Warp per table: code lengths from the pass's counts, which are then
-// cleared for the next pass.
+// cleared for the next pass. The last pass also writes the canonical codes
+// (by length, then symbol): 32 symbols at a time, equal lengths ranked by a
+// match and a running count per length.
 __global__ void __launch_bounds__(kHuffBuildThreads) huff_build_kernel(const BlockState *__restrict__ st,
                                                                        uint32_t *__restrict__ rfreq_all,
-                                                                       uint8_t *__restrict__ lens_all) {
+                                                                       uint8_t *__restrict__ lens_all, uint32_t *__restrict__ codes_all,
+                                                                       int last) {
     __shared__ uint32_t cnt[kMaxGroups][kMaxAlpha];
     __shared__ uint8_t lo[kMaxGroups][kMaxAlpha];
     __shared__ HuffScratch scratch[kMaxGroups];
+    __shared__ uint32_t next[kMaxGroups][32];
     const int b = blockIdx.x;
     const int ng = st[b].n_groups, alpha = st[b].n_in_use + 2;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -626,25 +641,28 @@ __global__ void __launch_bounds__(kHuffBuildThreads) huff_build_kernel(const Blo
     huff_lengths_warp(cnt[w], alpha, 17, lo[w], scratch[w]);
     uint8_t *len = lens_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
     for (int v = lane; v < alpha; v += 32) len[v] = lo[w][v];
-}
-
-// Canonical codes: by length, then symbol (lane 0 of the table's warp).
-__global__ void __launch_bounds__(kHuffBuildThreads) huff_codes_kernel(const BlockState *__restrict__ st,
-                                                                       const uint8_t *__restrict__ lens_all,
-                                                                       uint32_t *__restrict__ codes_all) {
-    const int b = blockIdx.x;
-    const int ng = st[b].n_groups, alpha = st[b].n_in_use + 2;
-    const int w = threadIdx.x >> 5;
-    if (w >= ng || (threadIdx.x & 31) != 0) return;
-    const uint8_t *len = lens_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
-    uint32_t next[22];
-    uint32_t cnt[22];
-    for (int l = 0; l < 22; l++) cnt[l] = 0;
-    for (int v = 0; v < alpha; v++) cnt[len[v]]++;
-    uint32_t c = 0;
-    for (int l = 1; l <= 20; l++) { next[l] = c; c = (c + cnt[l]) << 1; }
+    if (!last) return;
+    uint32_t n = 0;  // codes of length `lane`
+    for (int v = 0; v < alpha; v++) n += lo[w][v] == lane;
+    uint32_t c = 0, mine = 0;  // first code of each length
+    for (int l = 1; l <= 20; l++) {
+        if (lane == l) mine = c;
+        c = (c + __shfl_sync(LFC_FULL, n, l)) << 1;
+    }
+    next[w][lane] = mine;
+    __syncwarp();
     uint32_t *codes = codes_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
-    for (int v = 0; v < alpha; v++) codes[v] = next[len[v]]++;
+    for (int v0 = 0; v0 < alpha; v0 += 32) {
+        const int v = v0 + lane;
+        const bool in = v < alpha;
+        const uint32_t l = in ? lo[w][v] : 0u;
+        const uint32_t same = __match_any_sync(LFC_FULL, in ? l : 32u + lane);
+        const uint32_t first = in ? next[w][l] : 0u;
+        __syncwarp();
+        if (in) codes[v] = first + __popc(same & lanemask_lt());
+        if (in && (same & lanemask_gt()) == 0) next[w][l] = first + __popc(same);
+        __syncwarp();
+    }
 }
 
 // ------------------------------------------------------------ bit packing
@@ -929,14 +947,13 @@ cudaError_t launch_mtf_rle2(lfc_plan P, int nblocks) {
 cudaError_t launch_huffman(lfc_plan P, int nblocks) {
     Workspace &ws = P->ws;
     cudaStream_t s = P->stream;
-    huff_init_kernel<<<nblocks, 256, 0, s>>>(ws.bstate, ws.freq, ws.lens, ws.rfreq);
+    huff_init_kernel<<<nblocks, kHuffInitThreads, 0, s>>>(ws.bstate, ws.freq, ws.lens, ws.rfreq);
     const dim3 grid(kPackTiles, nblocks);
     for (int iter = 0; iter < 4; iter++) {
         huff_select_kernel<<<grid, kPackGroups, 0, s>>>(ws.bstate, ws.sym, ws.lens, ws.sel, ws.rfreq);
-        huff_build_kernel<<<nblocks, kHuffBuildThreads, 0, s>>>(ws.bstate, ws.rfreq, ws.lens);
+        huff_build_kernel<<<nblocks, kHuffBuildThreads, 0, s>>>(ws.bstate, ws.rfreq, ws.lens, ws.codes, iter == 3);
     }
-    huff_codes_kernel<<<nblocks, kHuffBuildThreads, 0, s>>>(ws.bstate, ws.lens, ws.codes);
-    count_launches(P, 10);
+    count_launches(P, 9);
     return cudaGetLastError();
 }
 
