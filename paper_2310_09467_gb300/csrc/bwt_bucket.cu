@@ -50,7 +50,7 @@ __device__ constexpr int kBucketCap[kBucketClasses] = {4096, 8192, 24576};
 constexpr int kBucketThreads[kBucketClasses] = {512, 512, 1024};
 constexpr int kBucketCtas[kBucketClasses] = {2, 2, 1};
 constexpr int kSubBins = 8192;  // 16-bit counters
-constexpr int kSubBig = 64;     // words of a sub-bin that are still ranked by counting
+constexpr int kSubCost = 256;    // words a word is compared with, on average, up to which counting beats the merge network
 constexpr int kTieGroup = 32;   // longest group ordered by further keys (a warp's lanes)
 constexpr int kTieShort = 4;    // longest one that a single thread orders
 constexpr int kTieRounds = 24;
@@ -113,8 +113,8 @@ __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState
     for (int i = t; i < kPlanHistWords / 4; i += kPlanThreads) reinterpret_cast<uint4 *>(h16)[i] = make_uint4(0, 0, 0, 0);
     for (int i = t; i < kBuckets; i += kPlanThreads) bcount[(size_t)b * kBuckets + i] = 0;
     __syncthreads();
-    // byte sample: at most 2047 16-byte pieces spread over the block
-    const int nv = m >> 4, vstep = max(1, nv >> 10);
+    // byte sample: at most 1024 16-byte pieces spread over the block
+    const int nv = m >> 4, vstep = (nv + kPlanThreads - 1) / kPlanThreads;
     for (int q = t; q * vstep < nv; q += kPlanThreads) {
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(rle) + (size_t)q * vstep);
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -142,23 +142,43 @@ __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState
         C.code[t] = (uint16_t)((code[t] >> 16 << 12) | (code[t] & 0xFFFu));
     }
     __syncthreads();
-    // prefix sample
+    // prefix sample: one rotation of every step, at a scrambled place (a fixed
+    // one would follow the (lo, hi) alternation of the stream). The first 12
+    // bytes of four rotations are loaded together.
     const int step = max(1, m >> 14), ns = (m + step - 1) / step;
-    for (int q = t; q < ns; q += kPlanThreads) {
-        // one rotation of every step, at a scrambled place: a fixed one would
-        // follow the (lo, hi) alternation of the stream
-        int pos = min(m - 1, q * step + (int)(((uint32_t)q * 2654435761u >> 8) % (uint32_t)step)), bits = 0;
-        uint32_t acc = 0, tab = kFirst;
-        while (bits < kPrefixBits) {
-            const uint32_t x = rle[pos], c = code[tab + x];
-            const int l = (int)(c >> 16);
-            acc = (acc << l) | (c & 0xFFFFu);
-            bits += l;
-            tab = x ? 256u : 0u;
-            if (++pos == m) pos = 0;
+    for (int q0 = t; q0 < ns; q0 += 4 * kPlanThreads) {
+        int at[4];
+        uint32_t w[4][3];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int q = q0 + i * kPlanThreads;
+            at[i] = q < ns ? min(m - 1, q * step + (int)(((uint32_t)q * 2654435761u >> 8) % (uint32_t)step)) : -1;
+            const int a4 = at[i] & ~3;
+            const bool in = at[i] >= 0 && a4 + 12 <= m;
+#pragma unroll
+            for (int k = 0; k < 3; k++) w[i][k] = in ? __ldg(reinterpret_cast<const uint32_t *>(rle + a4) + k) : 0u;
+            if (at[i] >= 0 && !in)  // the block's end: the bytes one by one, cyclic
+                for (int k = 0; k < 12; k++) w[i][k >> 2] |= (uint32_t)rle[(a4 + k) % m] << (8 * (k & 3));
         }
-        const uint32_t p = acc >> (bits - kPrefixBits), w = p >> 1;
-        atomicAdd(&h16[w + (w >> 5)], 1u << (16 * (p & 1)));
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            if (at[i] < 0) continue;
+            int k = at[i] & 3, bits = 0;
+            uint32_t acc = 0, tab = kFirst;
+            while (bits < kPrefixBits) {
+                uint32_t x;
+                if (k < 12) x = ((k < 4 ? w[i][0] : k < 8 ? w[i][1] : w[i][2]) >> (8 * (k & 3))) & 255u;
+                else x = rle[((at[i] & ~3) + k) % m];
+                const uint32_t c = code[tab + x];
+                const int l = (int)(c >> 16);
+                acc = (acc << l) | (c & 0xFFFFu);
+                bits += l;
+                tab = x ? 256u : 0u;
+                k++;
+            }
+            const uint32_t p = acc >> (bits - kPrefixBits), h = p >> 1;
+            atomicAdd(&h16[h + (h >> 5)], 1u << (16 * (p & 1)));
+        }
     }
     __syncthreads();
     // thread t: prefixes 64 t .. 64 t + 63 (words 33 t .. 33 t + 31). A bucket
@@ -171,28 +191,30 @@ __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState
     const uint32_t ex = block_excl_sum<uint32_t>(sum, shu, nullptr);
     const uint32_t target = max(1u, (uint32_t)(kBucketTarget / step));
     const uint32_t before = t > 0 ? h16[33 * t - 2] >> 16 : 0u;  // the count of prefix 64 t - 1
-    int base = 0, total = 0;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; pass++) {
+    uint64_t flags = t == 0 ? 1u : 0u;
+    {
         uint32_t cumc = ex, prev = before;
         uint32_t next = ((ex - before) / target + 1) * target;  // the multiple the running count crosses next
-        int id = base;
-#pragma unroll 1
+#pragma unroll 4
         for (int i = 0; i < 64; i++) {
             const uint32_t c = (hw[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
-            const bool cross = cumc >= next;
-            const bool flag = (t == 0 && i == 0) || c > target || prev > target || cross;
-            if (cross) next = (cumc / target + 1) * target;
-            if (flag) {
-                if (pass && id < kBuckets) C.split[id] = (uint16_t)(64 * t + i);
-                id++;
+            bool flag = max(c, prev) > target;
+            if (cumc >= next) {
+                flag = true;
+                next = (cumc / target + 1) * target;
             }
-            if (pass && (i & 15) == 0) C.base12[4 * t + (i >> 4)] = (uint16_t)min(id - 1, kBuckets - 1);
+            flags |= (uint64_t)flag << i;
             prev = c;
             cumc += c;
         }
-        if (pass == 0) base = block_excl_sum<int>(id, shi, &total);
     }
+    int total;
+    const int base = block_excl_sum<int>(__popcll(flags), shi, &total);
+#pragma unroll
+    for (int i = 0; i < 64; i += 16)
+        C.base12[4 * t + (i >> 4)] = (uint16_t)min(base + __popcll(flags & ((2ull << i) - 1)) - 1, kBuckets - 1);
+    for (int id = base; flags; flags &= flags - 1, id++)
+        if (id < kBuckets) C.split[id] = (uint16_t)(64 * t + __ffsll((long long)flags) - 1);
     if (t == 0) {
         const int nb = min(total, kBuckets);
         C.nb = nb;
@@ -568,7 +590,7 @@ struct BucketSmem {
     __align__(16) uint32_t cnt[2][kSubBins / 2 + 4];  // this bucket's and the next one's
     uint32_t sh[33];
     BucketItem item[3];
-    int big;
+    uint32_t cost;  // sum over the sub-bins of their words squared
 };
 
 // Persistent CTAs take buckets from the list of their size class. While a
@@ -638,12 +660,11 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
             const uint32_t sub = (uint32_t)(d >> (low - 1)), sh = 16 * (sub & 1);
             pr[r] = (sub << 16) | ((atomicAdd(&cnt[sub >> 1], 1u << sh) >> sh) & 0xFFFFu);
         }
-        if (t == 0) S.big = 0;
+        if (t == 0) S.cost = 0;
         __syncthreads();  // also: every thread is done with the previous bucket's words
         {
             constexpr int SP = kSubBins / 2 / TH;  // consecutive counter pairs per thread
-            uint32_t c[SP], sum = 0;
-            bool gbig = false;
+            uint32_t c[SP], sum = 0, cost = 0;
 #pragma unroll
             for (int i = 0; i < SP; i += 4) {
                 const uint4 v = reinterpret_cast<const uint4 *>(cnt)[(t * SP + i) / 4];
@@ -655,7 +676,7 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
 #pragma unroll
             for (int i = 0; i < SP; i++) {
                 const uint32_t x = c[i] & 0xFFFFu, y = c[i] >> 16;
-                gbig |= x > (uint32_t)kSubBig || y > (uint32_t)kSubBig;
+                cost += x * x + y * y;
                 c[i] = ex | ((ex + x) << 16);
                 ex += x + y;
             }
@@ -663,7 +684,8 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
             for (int i = 0; i < SP; i += 4)
                 reinterpret_cast<uint4 *>(cnt)[(t * SP + i) / 4] = make_uint4(c[i], c[i + 1], c[i + 2], c[i + 3]);
             if (t == 0) cnt[kSubBins / 2] = (uint32_t)n;
-            if (gbig) S.big = 1;
+            cost = warp_sum(cost);
+            if ((t & 31) == 0) atomicAdd(&S.cost, cost);
         }
         __syncthreads();
 #pragma unroll
@@ -674,10 +696,10 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
                 S.hi[at] = hi[r];
             }
         // the next bucket's counters (last read before this bucket's first
-        // barrier) are cleared, and S.big read, before the barrier: behind it
+        // barrier) are cleared, and S.cost read, before the barrier: behind it
         // threads run ahead into the next bucket
         for (int i = t; i < kSubBins / 8 + 1; i += TH) reinterpret_cast<uint4 *>(S.cnt[(it + 1) & 1])[i] = make_uint4(0, 0, 0, 0);
-        const bool big = S.big != 0;
+        const bool big = S.cost > (uint32_t)kSubCost * (uint32_t)n;
         __syncthreads();
         if (PRE && S.item[(it + 1) % 3].b >= 0) load_words(S.item[(it + 1) % 3]);
         if (t == 0) S.item[(it + 2) % 3] = look_up();
