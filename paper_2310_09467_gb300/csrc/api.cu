@@ -256,7 +256,7 @@ extern "C" int lfc_plan_block_capacity(lfc_plan P) { return P ? P->block_cap : 0
 static void free_ws(Workspace &w) {
     void *ptrs[] = {w.hist, w.summ, w.chain_first, w.scores, w.choice, w.jframes, w.cand, w.l2tab, w.stream, w.blocks, w.bstate,
                     w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.bcode, w.bcount, w.bcursor, w.bstart, w.bitems, w.bflag, w.tileaux, w.bwt,
-                    w.mtfidx, w.mtflists, w.mtfrec, w.mtfreclen, w.sym, w.freq, w.rfreq, w.sel, w.lens, w.codes, w.packed, w.cstream, w.masks, w.class_ids,
+                    w.mtfidx, w.mtflists, w.mtfrec, w.mtfreclen, w.mtfpres, w.mtfgrec, w.mtfgpres, w.mtfglen, w.sym, w.freq, w.rfreq, w.sel, w.lens, w.codes, w.packed, w.cstream, w.masks, w.class_ids,
                     w.act_total, w.block_dst, w.frame_crc, w.crc_part, w.crc_part2, w.chunk_desc, w.dec_tt,
                     w.hx_frames, w.hx_prev, w.hx_out, w.hx_choice, w.hx_sizes};
     for (void *p : ptrs)
@@ -365,9 +365,13 @@ extern "C" int lfc_plan_create(const lfc_config *cfg, void *cuda_stream, lfc_pla
     AL(tileaux, (size_t)BC * kTilesPerBlock * 4);
     AL(bwt, (size_t)BC * kBlockCap);
     AL(mtfidx, (size_t)BC * kBlockCap);
-    AL(mtflists, (size_t)BC * kTilesPerBlock * 256);
-    AL(mtfrec, (size_t)BC * kTilesPerBlock * 256);
-    AL(mtfreclen, (size_t)BC * kTilesPerBlock);
+    AL(mtflists, (size_t)BC * kMtfSegs * 256);
+    AL(mtfrec, (size_t)BC * kMtfSegs * 256);
+    AL(mtfreclen, (size_t)BC * kMtfSegs);
+    AL(mtfpres, (size_t)BC * kMtfSegs * 8);
+    AL(mtfgrec, (size_t)BC * (kMtfSegs / 16) * 256);
+    AL(mtfgpres, (size_t)BC * (kMtfSegs / 16) * 8);
+    AL(mtfglen, (size_t)BC * (kMtfSegs / 16));
     AL(sym, (size_t)BC * (kBlockCap + 64));
     AL(freq, (size_t)BC * kMaxAlpha);
     AL(rfreq, (size_t)BC * kMaxGroups * kMaxAlpha);
@@ -649,14 +653,14 @@ int run_pass(lfc_plan P, const CoderPass &cp, const uint8_t *d_arena) {
     CK(launch_bwt(P, nb, cp.max_m));
     if (P->bwt_timed_out) return fail(P, LFC_ERR_TIMEOUT, "suffix sort: a bounded look-back wait gave up");
     stage_begin(P, LFC_STAGE_MTF);
-    CK(launch_mtf_rle2(P, nb));
+    CK(launch_mtf_rle2(P, nb, cp.max_m));
     stage_end(P, LFC_STAGE_MTF);
     stage_begin(P, LFC_STAGE_HUFFMAN);
-    CK(launch_huffman(P, nb));
+    CK(launch_huffman(P, nb, cp.max_m));
     stage_end(P, LFC_STAGE_HUFFMAN);
     CK(cudaStreamWaitEvent(P->stream, P->side_join, 0));
     stage_begin(P, LFC_STAGE_PACK);
-    CK(launch_pack(P, nb));
+    CK(launch_pack(P, nb, cp.max_m));
     stage_end(P, LFC_STAGE_PACK);
     return LFC_OK;
 }

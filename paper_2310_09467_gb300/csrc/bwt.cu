@@ -977,25 +977,30 @@ __global__ void round_end_kernel(int32_t *rs, int max_m, cudaGraphConditionalHan
 
 // Bytes in use, and for flagged blocks L[j] = block[(SA[j] - 1) mod m] and
 // origPtr = j with SA[j] = 0 (the bucket sort has written both for the others).
-// Each CTA also writes the MTF summary of its 4096-byte segment of L: the
-// distinct bytes ordered by last occurrence, latest first. Thread = 16
-// consecutive positions; the last position of each byte value comes from one
-// shared-memory max per distinct value of a thread's run; each value is then
-// marked at its last position and the marks are compacted from the top.
+// Each CTA also writes the MTF records of its SEGS segments of L (1 of 4096
+// bytes or 4 of 1024): the distinct bytes ordered by last occurrence, latest
+// first, and their bitmap. Thread = 16 consecutive positions; the last
+// position of each byte value comes from one shared-memory max per distinct
+// value of a thread's run; each value is then marked at its last position and
+// the marks are compacted from the top.
 // After an aborted sort a flagged block's suffix array is incomplete: the
 // kernel then takes the identity order instead, so that every later stage still reads
 // in-range values (the call reports LFC_ERR_TIMEOUT and its output is void).
+template <int SEGS>
 __global__ void __launch_bounds__(kSortThreads) bwt_output_kernel(BlockState *__restrict__ st, const int32_t *__restrict__ sa_all,
                                                                   const uint8_t *__restrict__ rle_all, uint8_t *__restrict__ L_all,
                                                                   uint8_t *__restrict__ rec_all, int32_t *__restrict__ reclen_all,
-                                                                  const int32_t *__restrict__ rs, const int32_t *__restrict__ bflag) {
-    __shared__ int32_t lastpos[256];
+                                                                  uint32_t *__restrict__ pres_all, const int32_t *__restrict__ rs,
+                                                                  const int32_t *__restrict__ bflag) {
+    constexpr int TS = kSortThreads / SEGS;  // threads of a segment
+    __shared__ int32_t lastpos[SEGS][256];
     __shared__ uint16_t mark[kTile];  // value + 1 at its last position, 0 elsewhere
-    __shared__ int sh[33];
+    __shared__ int sh[33], base[SEGS];
     const int b = blockIdx.y, tile = blockIdx.x;
     const int m = st[b].m;
     if (tile * kTile >= m) return;
-    lastpos[threadIdx.x] = -1;
+#pragma unroll
+    for (int g = 0; g < SEGS; g++) lastpos[g][threadIdx.x] = -1;
     for (int i = threadIdx.x; i < kTile; i += kSortThreads) mark[i] = 0;
     __syncthreads();
     const size_t bo = (size_t)b * kBlockCap;
@@ -1027,29 +1032,40 @@ __global__ void __launch_bounds__(kSortThreads) bwt_output_kernel(BlockState *__
         bool seen = false;
 #pragma unroll
         for (int r = q + 1; r < kPerThread; r++) seen |= (j0 + r < m) && c[r] == c[q];
-        if (!seen) atomicMax(&lastpos[c[q]], jl + q);
+        if (!seen) atomicMax(&lastpos[threadIdx.x / TS][c[q]], jl + q);
     }
     __syncthreads();
     const int x = threadIdx.x;
-    const int lp = lastpos[x];
-    if (lp >= 0) mark[lp] = (uint16_t)(x + 1);
-    const uint32_t present = __ballot_sync(LFC_FULL, lp >= 0);  // values 32 w .. 32 w + 31
-    if ((threadIdx.x & 31) == 0 && present) atomicOr(&st[b].in_use[threadIdx.x >> 5], present);
+    const size_t seg0 = (size_t)b * kMtfSegs + (size_t)tile * SEGS;
+    uint32_t any = 0;
+#pragma unroll
+    for (int g = 0; g < SEGS; g++) {
+        const int lp = lastpos[g][x];
+        if (lp >= 0) mark[lp] = (uint16_t)(x + 1);
+        const uint32_t present = __ballot_sync(LFC_FULL, lp >= 0);  // values 32 w .. 32 w + 31
+        if ((x & 31) == 0 && tile * kTile + g * (kTile / SEGS) < m) pres_all[(seg0 + g) * 8 + (x >> 5)] = present;
+        any |= present;
+    }
+    if ((x & 31) == 0 && any) atomicOr(&st[b].in_use[x >> 5], any);
     __syncthreads();
     // compaction, highest positions first: thread t takes positions 4095 - 16 t - q
-    const int top = kTile - 1 - jl;
+    const int top = kTile - 1 - jl, g = SEGS - 1 - x / TS;
     int cnt = 0;
 #pragma unroll
     for (int q = 0; q < kPerThread; q++) cnt += mark[top - q] != 0;
     int total;
     int o = block_excl_sum<int>(cnt, sh, &total);
-    uint8_t *rec = rec_all + ((size_t)b * kTilesPerBlock + tile) * 256;
+    if (x % TS == 0) base[x / TS] = o;
+    __syncthreads();
+    o -= base[x / TS];
+    if (tile * kTile + g * (kTile / SEGS) >= m) return;
+    uint8_t *rec = rec_all + (seg0 + g) * 256;
 #pragma unroll
     for (int q = 0; q < kPerThread; q++) {
         const uint16_t mv = mark[top - q];
         if (mv) rec[o++] = (uint8_t)(mv - 1);
     }
-    if (threadIdx.x == 0) reclen_all[(size_t)b * kTilesPerBlock + tile] = total;
+    if (x % TS == TS - 1) reclen_all[seg0 + g] = o;
 }
 
 // Copies every block's last column out (lfc_bwt_blocks): stride bytes per
@@ -1257,8 +1273,9 @@ cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m) {
     }
     stage_end(P, LFC_STAGE_BWT_REFINE);
     stage_begin(P, LFC_STAGE_BWT_OUT);
-    bwt_output_kernel<<<dim3(tiles, nblocks), kSortThreads, 0, s>>>(ws.bstate, ws.sa, ws.rle, ws.bwt, ws.mtfrec, ws.mtfreclen,
-                                                                    ws.act_total, ws.bflag);
+    auto output = mtf_seg_log2(P, nblocks, max_m) == 12 ? bwt_output_kernel<1> : bwt_output_kernel<4>;
+    output<<<dim3(tiles, nblocks), kSortThreads, 0, s>>>(ws.bstate, ws.sa, ws.rle, ws.bwt, ws.mtfrec, ws.mtfreclen, ws.mtfpres,
+                                                         ws.act_total, ws.bflag);
     stage_end(P, LFC_STAGE_BWT_OUT);
     count_launches(P, 1);
     return cudaGetLastError();

@@ -24,6 +24,7 @@ constexpr int kMaxAlpha = 258;                       // bzip2 symbols: 256 MTF +
 constexpr int kMaxGroups = 6;
 constexpr int kMaxSelectors = 18002;
 constexpr int kHistBins = 65536;
+constexpr int kMtfSegs = kBlockCap / 1024;           // most MTF segments of a block
 constexpr int kMaxCand = 104;                        // candidates per frame: 26 default ids x 2 byte layouts x 2 (temporal)
 
 // Sort state in device memory (rs): tied elements after a round, their
@@ -247,9 +248,13 @@ struct Workspace {
     int32_t *tileaux = nullptr;    // block_cap * kTilesPerBlock * 4
     uint8_t *bwt = nullptr;        // L column
     uint8_t *mtfidx = nullptr;
-    uint8_t *mtflists = nullptr;   // block_cap * kTilesPerBlock * 256
-    uint8_t *mtfrec = nullptr;     // recency lists, same shape
-    int32_t *mtfreclen = nullptr;  // block_cap * kTilesPerBlock
+    uint8_t *mtflists = nullptr;   // starting list per MTF segment, block_cap * kMtfSegs * 256
+    uint8_t *mtfrec = nullptr;     // recency records, same shape
+    int32_t *mtfreclen = nullptr;  // block_cap * kMtfSegs
+    uint32_t *mtfpres = nullptr;   // bytes of a record as a bitmap, block_cap * kMtfSegs * 8
+    uint8_t *mtfgrec = nullptr;    // records, then starting lists, of groups of segments (a sixteenth of the segments)
+    uint32_t *mtfgpres = nullptr;
+    int32_t *mtfglen = nullptr;
     uint16_t *sym = nullptr;       // block_cap * (kBlockCap + 1)
     uint32_t *freq = nullptr;      // block_cap * kMaxAlpha
     uint32_t *rfreq = nullptr;     // block_cap * kMaxGroups * kMaxAlpha, counts of a refinement pass
@@ -367,9 +372,18 @@ cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph);
 cudaError_t launch_copy_bwt(lfc_plan P, int nblocks, uint8_t *d_L, size_t stride, uint32_t *d_len, uint32_t *d_orig);
 
 // mtf_huff.cu
-cudaError_t launch_mtf_rle2(lfc_plan P, int nblocks);
-cudaError_t launch_huffman(lfc_plan P, int nblocks);
-cudaError_t launch_pack(lfc_plan P, int nblocks);
+// max_m: the largest RLE1 length a block of the pass can have
+cudaError_t launch_mtf_rle2(lfc_plan P, int nblocks, int max_m);
+cudaError_t launch_huffman(lfc_plan P, int nblocks, int max_m);
+cudaError_t launch_pack(lfc_plan P, int nblocks, int max_m);
+
+// MTF segment length (log2) of a pass. A segment is one warp's serial work
+// (112 us for 4096 bytes), so a pass that cannot fill the SMs with 32 warps
+// twice over takes segments of 1024 bytes (30 us); a larger one is bound by
+// issue and keeps 4096 (fewer starting lists).
+inline int mtf_seg_log2(lfc_plan P, int nblocks, int max_m) {
+    return (int64_t)nblocks * ((max_m + 4095) / 4096) < (int64_t)64 * P->sm_count ? 10 : 12;
+}
 
 // container.cu
 struct FrameOut {

@@ -2,11 +2,12 @@
 // packing of every bzip2 block (Sec. 2.1.3; public bzip2 block format).
 //
 // MTF is sequential per block, so each block's BWT output is cut into
-// 4096-byte segments handled by one warp each. A segment's effect on the MTF
-// list is "its distinct symbols by most recent use, then the old list
-// without them"; one warp per block composes these summaries in order to get
-// every segment's starting list, then every segment replays MTF from its
-// list with the 256-entry list held in registers (8 entries per lane).
+// segments handled by one warp each. A segment's effect on the MTF list is
+// "its distinct bytes by most recent use, then the old list without them".
+// These records compose, and composing is associative: the records of groups
+// of segments are composed in parallel, one CTA per block chains the groups'
+// starting lists, and every group's CTA steps through its segments for
+// theirs. Lists hold byte values; only the bytes in use stand in them.
 #include <climits>
 
 #include "lfc_common.cuh"
@@ -15,60 +16,127 @@ namespace lfc {
 
 constexpr int kSymStride = kBlockCap + 64;  // uint16 symbols per block slot
 
-// Sequence index of byte c among the bytes in use (ascending byte order).
-__device__ __forceinline__ void build_seq_table(const uint32_t *in_use, uint8_t *seq) {
-    for (int c = threadIdx.x; c < 256; c += blockDim.x) {
-        int cnt = 0;
-        const int w = c >> 5;
-        for (int i = 0; i < w; i++) cnt += __popc(in_use[i]);
-        cnt += __popc(in_use[w] & ((1u << (c & 31)) - 1u));
-        seq[c] = (uint8_t)cnt;
+// ---------------------------------------------------- MTF: segment lists
+// The records (distinct bytes of a segment of L by last use, latest first,
+// and the bitmap of these bytes) come from the BWT output kernel.
+constexpr int kMtfGroup = 32;  // most segments of a group
+constexpr int kMtfGroupsMax = (kMtfSegs + 15) / 16;
+
+// Applies a record (length rl, this thread's byte r, bitmap pres) to the list
+// cur of n bytes, a byte per thread (256 threads); returns the new length.
+// wc: 8 words. Two barriers.
+__device__ __forceinline__ int list_apply(uint8_t (*lst)[256], int cur, int n, int rl, uint8_t r, const uint32_t *pres, int *wc) {
+    const int t = threadIdx.x, w = t >> 5;
+    const uint8_t x = lst[cur][t];
+    const bool keep = t < n && !((pres[x >> 5] >> (x & 31)) & 1u);
+    const uint32_t kept = __ballot_sync(LFC_FULL, keep);
+    if ((t & 31) == 0) wc[w] = __popc(kept);
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        before += i < w ? wc[i] : 0;
+        total += wc[i];
+    }
+    if (keep) lst[cur ^ 1][rl + before + __popc(kept & lanemask_lt())] = x;
+    if (t < rl) lst[cur ^ 1][t] = r;
+    __syncthreads();
+    return rl + total;
+}
+
+struct MtfGroupSmem {
+    __align__(16) uint8_t rec[kMtfGroup][256];
+    uint32_t pres[kMtfGroup][8];
+    int32_t len[kMtfGroup];
+    uint8_t lst[2][256];
+    int wc[8];
+};
+
+// The records of segments [s0, s0 + n) of block b into shared memory.
+__device__ __forceinline__ void load_records(MtfGroupSmem &S, int b, int s0, int n, const uint8_t *rec_all, const uint32_t *pres_all,
+                                             const int32_t *len_all) {
+    const size_t seg0 = (size_t)b * kMtfSegs + s0;
+    for (int i = threadIdx.x; i < n * 16; i += 256)
+        reinterpret_cast<uint4 *>(&S.rec[0][0])[i] = __ldg(reinterpret_cast<const uint4 *>(rec_all + seg0 * 256) + i);
+    for (int i = threadIdx.x; i < n * 8; i += 256) (&S.pres[0][0])[i] = pres_all[seg0 * 8 + i];
+    for (int i = threadIdx.x; i < n; i += 256) S.len[i] = len_all[seg0 + i];
+    __syncthreads();
+}
+
+// (1) one CTA per group: its segments' records composed.
+__global__ void __launch_bounds__(256) mtf_group_kernel(const BlockState *__restrict__ st, int seg_log2, int group,
+                                                        const uint8_t *__restrict__ rec_all, const uint32_t *__restrict__ pres_all,
+                                                        const int32_t *__restrict__ len_all, uint8_t *__restrict__ grec_all,
+                                                        uint32_t *__restrict__ gpres_all, int32_t *__restrict__ glen_all) {
+    __shared__ MtfGroupSmem S;
+    const int b = blockIdx.y, g = blockIdx.x, t = threadIdx.x;
+    const int nseg = (st[b].m + (1 << seg_log2) - 1) >> seg_log2, s0 = g * group, n = min(group, nseg - s0);
+    if (n <= 0) return;
+    load_records(S, b, s0, n, rec_all, pres_all, len_all);
+    int cur = 0, len = 0;
+    for (int i = 0; i < n; i++, cur ^= 1) len = list_apply(S.lst, cur, len, S.len[i], S.rec[i][t], S.pres[i], S.wc);
+    const size_t go = (size_t)b * kMtfGroupsMax + g;
+    grec_all[go * 256 + t] = S.lst[cur][t];
+    if (t < 8) {
+        uint32_t p = 0;
+        for (int i = 0; i < n; i++) p |= S.pres[i][t];
+        gpres_all[go * 8 + t] = p;
+    }
+    if (t == 0) glen_all[go] = len;
+}
+
+// (2) one CTA per block: the list at every group's start (in place of the
+// group's record), from the bytes in use in ascending order.
+__global__ void __launch_bounds__(256) mtf_chain_kernel(const BlockState *__restrict__ st, int seg_log2, int group,
+                                                        uint8_t *__restrict__ grec_all, const uint32_t *__restrict__ gpres_all,
+                                                        const int32_t *__restrict__ glen_all) {
+    __shared__ uint8_t lst[2][256];
+    __shared__ uint32_t pres[kMtfGroupsMax][8];
+    __shared__ int32_t lens[kMtfGroupsMax];
+    __shared__ int wc[8];
+    const int b = blockIdx.x, t = threadIdx.x;
+    const int nseg = (st[b].m + (1 << seg_log2) - 1) >> seg_log2, ng = (nseg + group - 1) / group;
+    uint8_t *grec = grec_all + (size_t)b * kMtfGroupsMax * 256;
+    for (int i = t; i < ng * 8; i += 256) (&pres[0][0])[i] = gpres_all[(size_t)b * kMtfGroupsMax * 8 + i];
+    for (int i = t; i < ng; i += 256) lens[i] = glen_all[(size_t)b * kMtfGroupsMax + i];
+    int n = 0, at = 0;  // bytes in use, those below t
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        const uint32_t w = st[b].in_use[i];
+        at += i < (t >> 5) ? __popc(w) : (i == (t >> 5) ? __popc(w & lanemask_lt()) : 0);
+        n += __popc(w);
+    }
+    if ((st[b].in_use[t >> 5] >> (t & 31)) & 1u) lst[0][at] = (uint8_t)t;
+    uint8_t r = ng > 0 ? grec[t] : (uint8_t)0;
+    __syncthreads();
+    int cur = 0;
+    for (int g = 0; g < ng; g++, cur ^= 1) {
+        const uint8_t next = g + 1 < ng ? grec[(g + 1) * 256 + t] : (uint8_t)0;
+        grec[g * 256 + t] = lst[cur][t];
+        list_apply(lst, cur, n, lens[g], r, pres[g], wc);
+        r = next;
     }
 }
 
-// ---------------------------------------------------- MTF: segment summaries
-// The summaries (distinct bytes of each 4096-byte segment of L by last use,
-// latest first) come from the BWT output kernel, as byte values.
-// One CTA per block: starting list of every segment, one list entry per
-// thread. Composing a segment's summary: its record first, then the old
-// list without the record's symbols (kept entries compacted by a scan).
-__global__ void __launch_bounds__(256) mtf_compose_kernel(const BlockState *__restrict__ st, const uint8_t *__restrict__ rec_all,
-                                                          const int32_t *__restrict__ reclen_all, uint8_t *__restrict__ lists_all) {
-    __shared__ uint8_t lst[256];
-    __shared__ uint8_t inr[256];
-    __shared__ uint8_t seq[256];
-    __shared__ uint32_t iush[8];
-    __shared__ int32_t rl_s[kTilesPerBlock];
-    __shared__ int sh[33];
-    const int b = blockIdx.x, t = threadIdx.x;
-    const int m = st[b].m;
-    if (t < 8) iush[t] = st[b].in_use[t];
-    __syncthreads();
-    build_seq_table(iush, seq);  // records hold byte values; lists hold their indices
-    int n_in_use = 0;
-    for (int i = 0; i < 8; i++) n_in_use += __popc(iush[i]);
-    const int ng = (m + kTile - 1) / kTile;
-    for (int g = t; g < ng; g += 256) rl_s[g] = reclen_all[(size_t)b * kTilesPerBlock + g];
-    lst[t] = t < n_in_use ? (uint8_t)t : (uint8_t)0xFF;
-    const uint8_t *recb = rec_all + (size_t)b * kTilesPerBlock * 256;
-    uint8_t r_next = ng > 0 ? recb[t] : 0;
-    __syncthreads();
-    r_next = seq[r_next];
-    for (int g = 0; g < ng; g++) {
-        lists_all[((size_t)b * kTilesPerBlock + g) * 256 + t] = lst[t];
-        const int rl = rl_s[g];
-        const uint8_t r = r_next;
-        if (g + 1 < ng) r_next = seq[recb[(size_t)(g + 1) * 256 + t]];
-        inr[t] = 0;
-        __syncthreads();
-        if (t < rl) inr[r] = 1;
-        __syncthreads();
-        const uint8_t x = lst[t];
-        const bool keep = t < n_in_use && !inr[x];
-        const int pos = rl + block_excl_sum<int>(keep ? 1 : 0, sh, nullptr);  // syncs: all of lst is read
-        if (keep) lst[pos] = x;
-        if (t < rl) lst[t] = r;
-        __syncthreads();
+// (3) one CTA per group: the list at every segment's start.
+__global__ void __launch_bounds__(256) mtf_lists_kernel(const BlockState *__restrict__ st, int seg_log2, int group,
+                                                        const uint8_t *__restrict__ rec_all, const uint32_t *__restrict__ pres_all,
+                                                        const int32_t *__restrict__ len_all, const uint8_t *__restrict__ grec_all,
+                                                        uint8_t *__restrict__ lists_all) {
+    __shared__ MtfGroupSmem S;
+    const int b = blockIdx.y, g = blockIdx.x, t = threadIdx.x;
+    const int nseg = (st[b].m + (1 << seg_log2) - 1) >> seg_log2, s0 = g * group, n = min(group, nseg - s0);
+    if (n <= 0) return;
+    int in_use = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) in_use += __popc(st[b].in_use[i]);
+    S.lst[0][t] = grec_all[((size_t)b * kMtfGroupsMax + g) * 256 + t];
+    load_records(S, b, s0, n, rec_all, pres_all, len_all);
+    uint8_t *lists = lists_all + ((size_t)b * kMtfSegs + s0) * 256;
+    int cur = 0;
+    for (int i = 0; i < n; i++, cur ^= 1) {
+        lists[i * 256 + t] = S.lst[cur][t];
+        if (i + 1 < n) list_apply(S.lst, cur, in_use, S.len[i], S.rec[i][t], S.pres[i], S.wc);
     }
 }
 
@@ -86,19 +154,18 @@ __global__ void __launch_bounds__(256) mtf_compose_kernel(const BlockState *__re
 // bit-sliced over ballots of the values' bits. The list then becomes the
 // window's symbols by last use, then the old list without them; entries
 // behind the deepest window symbol keep their places.
-__global__ void __launch_bounds__(32) mtf_encode_kernel(const BlockState *__restrict__ st, const uint8_t *__restrict__ L_all,
-                                                        const uint8_t *__restrict__ lists_all, uint8_t *__restrict__ idx_all) {
-    __shared__ uint8_t seq[256];
-    __shared__ uint32_t iush[8];
-    __shared__ uint8_t lst[256];
+__global__ void __launch_bounds__(32) mtf_encode_kernel(const BlockState *__restrict__ st, int seg_log2,
+                                                        const uint8_t *__restrict__ L_all, const uint8_t *__restrict__ lists_all,
+                                                        uint8_t *__restrict__ idx_all) {
+    __shared__ __align__(8) uint8_t lst[256];
     __shared__ uint8_t posof[256];
     __shared__ uint32_t WP[8];
     __shared__ __align__(16) uint8_t seg[kTile];  // the segment's bytes, loaded at once
     const int b = blockIdx.y, g = blockIdx.x;
     const int m = st[b].m;
-    const int s0 = g * kTile;
+    const int s0 = g << seg_log2;
     if (s0 >= m) return;
-    const int s1 = min(m, s0 + kTile);
+    const int s1 = min(m, s0 + (1 << seg_log2));
     const int lane = threadIdx.x;
     {
         const uint8_t *Lb = L_all + (size_t)b * kBlockCap + s0;  // 16-byte aligned (block slots and tiles are)
@@ -107,13 +174,11 @@ __global__ void __launch_bounds__(32) mtf_encode_kernel(const BlockState *__rest
             reinterpret_cast<uint4 *>(seg)[q] = __ldg(reinterpret_cast<const uint4 *>(Lb) + q);
         for (int q = (nb & ~15) + lane; q < nb; q += 32) seg[q] = Lb[q];
     }
-    if (lane < 8) iush[lane] = st[b].in_use[lane];
-    __syncwarp();
-    build_seq_table(iush, seq);
     int n_in_use = 0;
-    for (int i = 0; i < 8; i++) n_in_use += __popc(iush[i]);
-    const uint8_t *start = lists_all + ((size_t)b * kTilesPerBlock + g) * 256;
-    for (int q = lane; q < 256; q += 32) lst[q] = start[q];
+#pragma unroll
+    for (int i = 0; i < 8; i++) n_in_use += __popc(st[b].in_use[i]);
+    const uint64_t *start = reinterpret_cast<const uint64_t *>(lists_all + ((size_t)b * kMtfSegs + g) * 256);
+    reinterpret_cast<uint64_t *>(lst)[lane] = start[lane];
     __syncwarp();
     for (int q = lane; q < n_in_use; q += 32) posof[lst[q]] = (uint8_t)q;
     __syncwarp();
@@ -122,7 +187,7 @@ __global__ void __launch_bounds__(32) mtf_encode_kernel(const BlockState *__rest
     for (int w0 = s0; w0 < s1; w0 += 32) {
         const int i = w0 + lane;
         const bool valid = i < s1;
-        const uint32_t s = valid ? (uint32_t)seq[seg[i - s0]] : 256u + lane;
+        const uint32_t s = valid ? (uint32_t)seg[i - s0] : 256u + lane;
         const uint32_t grp = __match_any_sync(LFC_FULL, s);
         const uint32_t lower = grp & lt;
         const bool fo = valid && lower == 0;
@@ -382,133 +447,145 @@ __global__ void __launch_bounds__(kRle2Threads) rle2_write_kernel(const BlockSta
 }
 
 // --------------------------------------------------------------- Huffman
-// Code lengths of one table by one warp: weights max(freq, 1); the two nodes
-// with the smallest (weight, key) are joined (leaf key = symbol, k-th joined
-// node key = alpha + k; the two-queue method reproduces that order because
-// leaves are pre-sorted by (weight, symbol) and joined nodes appear in
-// non-decreasing weight); over-long codes halve the weights (1 + w/2).
+// Code lengths of one table by one CTA (a thread per symbol): weights
+// max(freq, 1); the two nodes with the smallest (weight, key) are joined (leaf
+// key = symbol, k-th joined node key = alpha + k; the two-queue method
+// reproduces that order because leaves are pre-sorted by (weight, symbol) and
+// joined nodes appear in non-decreasing weight); over-long codes halve the
+// weights (1 + w/2).
+constexpr int kHuffThreads = 288;
+static_assert(kHuffThreads >= kMaxAlpha, "a thread per symbol");
+
 struct HuffScratch {
-    uint32_t w[kMaxAlpha];
+    uint32_t w[kHuffThreads];
     uint32_t lw[kMaxAlpha];          // leaf weights in (weight, symbol) order
     uint32_t nw[kMaxAlpha];          // joined-node weights
+    uint32_t pair[kMaxAlpha];        // weights of a round's items in order
     uint16_t order[kMaxAlpha];       // leaves sorted by (w, symbol)
-    uint16_t lpar[kMaxAlpha];        // parents of the leaves in that order
     uint16_t par[2 * kMaxAlpha];     // parent of a node (leaves, then joined nodes)
     uint16_t dist[2 * kMaxAlpha];    // pointer-jumping distance to par
+    int longest;
 };
 
-// Keys (w << 9 | symbol) are distinct, so a key's rank is the count of
-// smaller keys; w < 2^21 (counts of one block), so the key fits 30 bits.
-// Node depths by pointer jumping: after r rounds par[n] is n's 2^r-th
-// ancestor (capped at the root) and dist[n] the distance to it; 9 rounds
-// cover depths up to 511 >= alpha - 1.
-__device__ void huff_lengths_warp(const uint32_t *freq, int alpha, int max_len, uint8_t *len_out, HuffScratch &S) {
-    constexpr int kQ = (kMaxAlpha + 31) / 32;       // leaves per lane
-    constexpr int kN = (2 * kMaxAlpha + 31) / 32;   // nodes per lane
+// Two-queue merge by one warp, in rounds: the pair of the two smallest
+// (weight, key) items makes a node of weight n0, and every item at hand of
+// weight <= n0 comes before it (a leaf before a joined node of equal weight, a
+// joined node before a later one: the keys), so all of them pair up in order
+// at once. An item's place among them is its index plus the count of the
+// other queue's items before it. About 20 rounds for the counts of one table
+// instead of 257 dependent steps.
+__device__ void huff_merge(int alpha, HuffScratch &S) {
+    constexpr uint32_t kEmpty = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
-    for (int i = lane; i < alpha; i += 32) S.w[i] = freq[i] ? freq[i] : 1u;
-    __syncwarp();
-    const int nodes = 2 * alpha - 1, root = 2 * alpha - 2;
-    int longest = 0;
-    for (;;) {
-        uint32_t myk[kQ], rk[kQ];
-#pragma unroll
-        for (int q = 0; q < kQ; q++) {
-            const int i = lane + 32 * q;
-            myk[q] = i < alpha ? ((S.w[i] << 9) | (uint32_t)i) : 0xFFFFFFFFu;
-            rk[q] = 0;
+    int la = 0, lb = 0, k = 0;  // queue heads, joined nodes made
+    while (k < alpha - 1) {
+        const uint32_t a0 = la < alpha ? S.lw[la] : kEmpty, a1 = la + 1 < alpha ? S.lw[la + 1] : kEmpty;
+        const uint32_t b0 = lb < k ? S.nw[lb] : kEmpty, b1 = lb + 1 < k ? S.nw[lb + 1] : kEmpty;
+        const uint32_t n0 = a0 <= b0 ? a0 + min(a1, b0) : b0 + min(a0, b1);
+        int ca = 0, cb = 0;  // items of weight <= n0 (the queues ascend)
+        for (uint32_t more = LFC_FULL; more == LFC_FULL;) {
+            const int i = la + ca + lane;
+            more = __ballot_sync(LFC_FULL, i < alpha && S.lw[i] <= n0);
+            ca += __popc(more);
         }
-        for (int j = 0; j < alpha; j++) {
-            const uint32_t kj = (S.w[j] << 9) | (uint32_t)j;
-#pragma unroll
-            for (int q = 0; q < kQ; q++) rk[q] += kj < myk[q];
+        for (uint32_t more = LFC_FULL; more == LFC_FULL;) {
+            const int i = lb + cb + lane;
+            more = __ballot_sync(LFC_FULL, i < k && S.nw[i] <= n0);
+            cb += __popc(more);
         }
-#pragma unroll
-        for (int q = 0; q < kQ; q++) {
-            const int i = lane + 32 * q;
-            if (i < alpha) {
-                S.order[rk[q]] = (uint16_t)i;
-                S.lw[rk[q]] = S.w[i];
-            }
-        }
-        __syncwarp();
-        if (lane == 0) {
-            // two-queue merge: the two smallest (weight, key) nodes, a leaf
-            // before a joined node of equal weight (its key is smaller). The
-            // heads of both queues sit in registers kAhead deep, so that no
-            // pick waits for a load (a pick is a few dependent instructions;
-            // with the loads on the chain a table took 42 us instead of 13).
-            constexpr uint32_t kEmpty = 0xFFFFFFFFu;
-            uint32_t a0 = S.lw[0], a1 = 1 < alpha ? S.lw[1] : kEmpty, a2 = 2 < alpha ? S.lw[2] : kEmpty, a3 = 3 < alpha ? S.lw[3] : kEmpty;
-            uint32_t b0 = kEmpty, b1 = kEmpty, b2 = kEmpty, b3 = kEmpty;
-            int la = 0, lb = 0;  // queue heads; joined nodes made so far: k
-            for (int k = 0; k < alpha - 1; k++) {
-                uint32_t sum = 0;
-#pragma unroll
-                for (int q = 0; q < 2; q++) {
-                    if (a0 <= b0) {  // never both empty
-                        sum += a0;
-                        S.lpar[la] = (uint16_t)(alpha + k);
-                        a0 = a1; a1 = a2; a2 = a3;
-                        a3 = la + 4 < alpha ? S.lw[la + 4] : kEmpty;
-                        la++;
-                    } else {
-                        sum += b0;
-                        S.par[alpha + lb] = (uint16_t)(alpha + k);
-                        b0 = b1; b1 = b2; b2 = b3;
-                        b3 = lb + 4 < k ? S.nw[lb + 4] : kEmpty;
-                        lb++;
-                    }
+        const int n = (ca + cb) & ~1;  // items that pair up; an odd last one waits
+        int used = 0;                  // leaves among them
+        for (int i0 = 0; i0 < ca; i0 += 32) {
+            const int i = i0 + lane;
+            bool mine = false;
+            if (i < ca) {
+                const uint32_t x = S.lw[la + i];
+                int lo = 0, hi = cb;  // joined nodes below x
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (S.nw[lb + mid] < x) lo = mid + 1; else hi = mid;
                 }
-                S.nw[k] = sum;
-                const int n = k - lb;  // joined nodes waiting before this one
-                if (n == 0) b0 = sum;
-                else if (n == 1) b1 = sum;
-                else if (n == 2) b2 = sum;
-                else if (n == 3) b3 = sum;
-            }
-            S.par[root] = (uint16_t)root;
-        }
-        __syncwarp();
-        for (int i = lane; i < alpha; i += 32) S.par[S.order[i]] = S.lpar[i];
-        __syncwarp();
-        uint16_t pn[kN], dn[kN];
-#pragma unroll
-        for (int q = 0; q < kN; q++) {
-            const int n = lane + 32 * q;
-            if (n < nodes) S.dist[n] = n == root ? 0 : 1;
-        }
-        __syncwarp();
-        for (int round = 0; round < 9; round++) {
-#pragma unroll
-            for (int q = 0; q < kN; q++) {
-                const int n = lane + 32 * q;
-                if (n < nodes) {
-                    const int pp = S.par[n];
-                    dn[q] = (uint16_t)(S.dist[n] + S.dist[pp]);
-                    pn[q] = S.par[pp];
+                mine = i + lo < n;
+                if (mine) {
+                    S.pair[i + lo] = x;
+                    S.par[S.order[la + i]] = (uint16_t)(alpha + k + ((i + lo) >> 1));
                 }
             }
-            __syncwarp();
-#pragma unroll
-            for (int q = 0; q < kN; q++) {
-                const int n = lane + 32 * q;
-                if (n < nodes) {
-                    S.dist[n] = dn[q];
-                    S.par[n] = pn[q];
-                }
-            }
-            __syncwarp();
+            used += __popc(__ballot_sync(LFC_FULL, mine));
         }
-        int mx = 0;
-        for (int i = lane; i < alpha; i += 32) mx = max(mx, (int)S.dist[i]);
-        longest = __reduce_max_sync(LFC_FULL, (unsigned)mx);
-        if (longest <= max_len) break;
-        for (int i = lane; i < alpha; i += 32) S.w[i] = 1u + S.w[i] / 2u;
+        for (int i = lane; i < cb; i += 32) {
+            const uint32_t x = S.nw[lb + i];
+            int lo = 0, hi = ca;  // leaves up to x
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (S.lw[la + mid] <= x) lo = mid + 1; else hi = mid;
+            }
+            if (i + lo < n) {
+                S.pair[i + lo] = x;
+                S.par[alpha + lb + i] = (uint16_t)(alpha + k + ((i + lo) >> 1));
+            }
+        }
         __syncwarp();
+        for (int i = lane; i < n / 2; i += 32) S.nw[k + i] = S.pair[2 * i] + S.pair[2 * i + 1];
+        __syncwarp();
+        la += used;
+        lb += n - used;
+        k += n / 2;
     }
-    for (int i = lane; i < alpha; i += 32) len_out[i] = (uint8_t)S.dist[i];
-    __syncwarp();
+}
+
+// The length of symbol threadIdx.x (w: its weight). Keys (w << 9 | symbol)
+// are distinct, so a key's rank is the count of smaller keys; w < 2^21
+// (counts of one block), so the key fits 30 bits. Node depths by pointer
+// jumping: after r rounds par[n] is n's 2^r-th ancestor (capped at the root)
+// and dist[n] the distance to it.
+__device__ int huff_length(uint32_t w, int alpha, int max_len, HuffScratch &S) {
+    const int v = threadIdx.x;
+    const int nodes = 2 * alpha - 1, root = 2 * alpha - 2;
+    for (;;) {
+        S.w[v] = w;
+        if (v == 0) S.longest = 0;
+        __syncthreads();
+        if (v < alpha) {
+            const uint32_t key = (w << 9) | (uint32_t)v;
+            int r = 0;
+#pragma unroll 8
+            for (int j = 0; j < alpha; j++) r += ((S.w[j] << 9) | (uint32_t)j) < key;
+            S.order[r] = (uint16_t)v;
+            S.lw[r] = w;
+        }
+        __syncthreads();
+        if (v < 32) huff_merge(alpha, S);
+        if (v == 0) S.par[root] = (uint16_t)root;
+        const int n0 = v, n1 = v + kHuffThreads;
+        if (n0 < nodes) S.dist[n0] = n0 == root ? 0 : 1;
+        if (n1 < nodes) S.dist[n1] = n1 == root ? 0 : 1;
+        __syncthreads();
+        for (int span = 1; span < alpha; span <<= 1) {
+            int p0 = 0, d0 = 0, p1 = 0, d1 = 0;
+            if (n0 < nodes) {
+                const int p = S.par[n0];
+                d0 = S.dist[n0] + S.dist[p];
+                p0 = S.par[p];
+            }
+            if (n1 < nodes) {
+                const int p = S.par[n1];
+                d1 = S.dist[n1] + S.dist[p];
+                p1 = S.par[p];
+            }
+            __syncthreads();
+            if (n0 < nodes) { S.dist[n0] = (uint16_t)d0; S.par[n0] = (uint16_t)p0; }
+            if (n1 < nodes) { S.dist[n1] = (uint16_t)d1; S.par[n1] = (uint16_t)p1; }
+            __syncthreads();
+        }
+        const int len = v < alpha ? S.dist[v] : 0;
+        const int longest = __reduce_max_sync(LFC_FULL, (unsigned)len);
+        if ((v & 31) == 0) atomicMax(&S.longest, longest);
+        __syncthreads();
+        if (S.longest <= max_len) return len;
+        w = 1u + w / 2u;
+        __syncthreads();
+    }
 }
 
 constexpr int kPackGroups = 128;                                           // selector groups per tile = threads
@@ -534,12 +611,7 @@ __device__ __forceinline__ int stage_tile_syms(const uint16_t *sym, int tile, in
 // many CTAs (select) followed by "every table is rebuilt from its groups'
 // counts with a 17-bit limit" (build), the last of them with the canonical
 // codes.
-constexpr int kHuffBuildThreads = 32 * kMaxGroups;
-
-constexpr int kHuffInitThreads = 288;
-static_assert(kHuffInitThreads >= kMaxAlpha, "a thread per symbol");
-
-__global__ void __launch_bounds__(kHuffInitThreads) huff_init_kernel(BlockState *__restrict__ st, const uint32_t *__restrict__ freq_all,
+__global__ void __launch_bounds__(kHuffThreads) huff_init_kernel(BlockState *__restrict__ st, const uint32_t *__restrict__ freq_all,
                                                                      uint8_t *__restrict__ lens_all, uint32_t *__restrict__ rfreq_all) {
     __shared__ uint32_t sh[33];
     const int b = blockIdx.x, v = threadIdx.x;
@@ -616,52 +688,47 @@ __global__ void __launch_bounds__(kPackGroups) huff_select_kernel(const BlockSta
     }
 }
 
-// Warp per table: code lengths from the pass's counts, which are then
-// cleared for the next pass. The last pass also writes the canonical codes
-// (by length, then symbol): 32 symbols at a time, equal lengths ranked by a
-// match and a running count per length.
-__global__ void __launch_bounds__(kHuffBuildThreads) huff_build_kernel(const BlockState *__restrict__ st,
-                                                                       uint32_t *__restrict__ rfreq_all,
-                                                                       uint8_t *__restrict__ lens_all, uint32_t *__restrict__ codes_all,
-                                                                       int last) {
-    __shared__ uint32_t cnt[kMaxGroups][kMaxAlpha];
-    __shared__ uint8_t lo[kMaxGroups][kMaxAlpha];
-    __shared__ HuffScratch scratch[kMaxGroups];
-    __shared__ uint32_t next[kMaxGroups][32];
-    const int b = blockIdx.x;
-    const int ng = st[b].n_groups, alpha = st[b].n_in_use + 2;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w >= ng) return;
-    uint32_t *rfreq = rfreq_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
-    for (int v = lane; v < alpha; v += 32) {
-        cnt[w][v] = rfreq[v];
-        rfreq[v] = 0;
+// CTA per table: code lengths from the pass's counts, which are then cleared
+// for the next pass. The last pass also writes the canonical codes (by
+// length, then symbol): a symbol's code is its length's first one plus the
+// symbols before it of the same length.
+__global__ void __launch_bounds__(kHuffThreads) huff_build_kernel(const BlockState *__restrict__ st, uint32_t *__restrict__ rfreq_all,
+                                                                  uint8_t *__restrict__ lens_all, uint32_t *__restrict__ codes_all,
+                                                                  int last) {
+    __shared__ HuffScratch S;
+    __shared__ uint8_t ls[kHuffThreads];
+    __shared__ uint32_t first[32];
+    const int b = blockIdx.y, g = blockIdx.x, v = threadIdx.x;
+    if (g >= st[b].n_groups) return;
+    const int alpha = st[b].n_in_use + 2;
+    const size_t at = ((size_t)b * kMaxGroups + g) * kMaxAlpha + v;
+    uint32_t w = 0xFFFFFFFFu >> 9;
+    if (v < alpha) {
+        w = max(rfreq_all[at], 1u);
+        rfreq_all[at] = 0;
     }
-    __syncwarp();
-    huff_lengths_warp(cnt[w], alpha, 17, lo[w], scratch[w]);
-    uint8_t *len = lens_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
-    for (int v = lane; v < alpha; v += 32) len[v] = lo[w][v];
+    const int len = huff_length(w, alpha, 17, S);
+    if (v < alpha) lens_all[at] = (uint8_t)len;
     if (!last) return;
-    uint32_t n = 0;  // codes of length `lane`
-    for (int v = 0; v < alpha; v++) n += lo[w][v] == lane;
-    uint32_t c = 0, mine = 0;  // first code of each length
-    for (int l = 1; l <= 20; l++) {
-        if (lane == l) mine = c;
-        c = (c + __shfl_sync(LFC_FULL, n, l)) << 1;
+    ls[v] = (uint8_t)len;
+    if (v < 32) first[v] = 0;
+    __syncthreads();
+    if (v < alpha) atomicAdd(&first[len], 1u);
+    __syncthreads();
+    if (v == 0) {
+        uint32_t c = 0;
+        for (int l = 1; l <= 20; l++) {
+            const uint32_t n = first[l];
+            first[l] = c;
+            c = (c + n) << 1;
+        }
     }
-    next[w][lane] = mine;
-    __syncwarp();
-    uint32_t *codes = codes_all + ((size_t)b * kMaxGroups + w) * kMaxAlpha;
-    for (int v0 = 0; v0 < alpha; v0 += 32) {
-        const int v = v0 + lane;
-        const bool in = v < alpha;
-        const uint32_t l = in ? lo[w][v] : 0u;
-        const uint32_t same = __match_any_sync(LFC_FULL, in ? l : 32u + lane);
-        const uint32_t first = in ? next[w][l] : 0u;
-        __syncwarp();
-        if (in) codes[v] = first + __popc(same & lanemask_lt());
-        if (in && (same & lanemask_gt()) == 0) next[w][l] = first + __popc(same);
-        __syncwarp();
+    __syncthreads();
+    if (v < alpha) {
+        uint32_t r = first[len];
+#pragma unroll 8
+        for (int j = 0; j < v; j++) r += ls[j] == len;
+        codes_all[at] = r;
     }
 }
 
@@ -930,38 +997,48 @@ __global__ void __launch_bounds__(kPackGroups) pack_data_kernel(const BlockState
     if (nacc > 0) atomicOr(&words[wpos >> 5], bswap32((uint32_t)(acc >> 32)));  // shared with the next
 }
 
-cudaError_t launch_mtf_rle2(lfc_plan P, int nblocks) {
+cudaError_t launch_mtf_rle2(lfc_plan P, int nblocks, int max_m) {
     Workspace &ws = P->ws;
     cudaStream_t s = P->stream;
-    dim3 grid(kTilesPerBlock, nblocks);
-    mtf_compose_kernel<<<nblocks, 256, 0, s>>>(ws.bstate, ws.mtfrec, ws.mtfreclen, ws.mtflists);
-    mtf_encode_kernel<<<grid, 32, 0, s>>>(ws.bstate, ws.bwt, ws.mtflists, ws.mtfidx);
-    const dim3 g2(kTilesPerBlock, nblocks);  // RLE1 output <= 900000 = 220 tiles
+    const int seg_log2 = mtf_seg_log2(P, nblocks, max_m);
+    const int segs = (max_m + (1 << seg_log2) - 1) >> seg_log2;
+    const int group = seg_log2 == 12 ? 16 : kMtfGroup, groups = (segs + group - 1) / group;
+    const dim3 ggrid(groups, nblocks);
+    mtf_group_kernel<<<ggrid, 256, 0, s>>>(ws.bstate, seg_log2, group, ws.mtfrec, ws.mtfpres, ws.mtfreclen, ws.mtfgrec, ws.mtfgpres,
+                                           ws.mtfglen);
+    mtf_chain_kernel<<<nblocks, 256, 0, s>>>(ws.bstate, seg_log2, group, ws.mtfgrec, ws.mtfgpres, ws.mtfglen);
+    mtf_lists_kernel<<<ggrid, 256, 0, s>>>(ws.bstate, seg_log2, group, ws.mtfrec, ws.mtfpres, ws.mtfreclen, ws.mtfgrec, ws.mtflists);
+    mtf_encode_kernel<<<dim3(segs, nblocks), 32, 0, s>>>(ws.bstate, seg_log2, ws.bwt, ws.mtflists, ws.mtfidx);
+    const dim3 g2((max_m + kRle2Tile - 1) / kRle2Tile, nblocks);
     rle2_tile_kernel<<<g2, kRle2Threads, 0, s>>>(ws.bstate, ws.mtfidx, ws.tileaux);
     rle2_scan_kernel<<<nblocks, 32, 0, s>>>(ws.bstate, ws.tileaux, ws.sym, ws.freq);
     rle2_write_kernel<<<g2, kRle2Threads, 0, s>>>(ws.bstate, ws.mtfidx, ws.tileaux, ws.sym, ws.freq);
-    count_launches(P, 5);
+    count_launches(P, 7);
     return cudaGetLastError();
 }
 
-cudaError_t launch_huffman(lfc_plan P, int nblocks) {
+// Tiles of selector groups of a block with max_m positions: at most a symbol
+// per position and EOB.
+static int pack_tiles(int max_m) { return (max_m + 1 + kTileSyms - 1) / kTileSyms; }
+
+cudaError_t launch_huffman(lfc_plan P, int nblocks, int max_m) {
     Workspace &ws = P->ws;
     cudaStream_t s = P->stream;
-    huff_init_kernel<<<nblocks, kHuffInitThreads, 0, s>>>(ws.bstate, ws.freq, ws.lens, ws.rfreq);
-    const dim3 grid(kPackTiles, nblocks);
+    huff_init_kernel<<<nblocks, kHuffThreads, 0, s>>>(ws.bstate, ws.freq, ws.lens, ws.rfreq);
+    const dim3 grid(pack_tiles(max_m), nblocks);
     for (int iter = 0; iter < 4; iter++) {
         huff_select_kernel<<<grid, kPackGroups, 0, s>>>(ws.bstate, ws.sym, ws.lens, ws.sel, ws.rfreq);
-        huff_build_kernel<<<nblocks, kHuffBuildThreads, 0, s>>>(ws.bstate, ws.rfreq, ws.lens, ws.codes, iter == 3);
+        huff_build_kernel<<<dim3(kMaxGroups, nblocks), kHuffThreads, 0, s>>>(ws.bstate, ws.rfreq, ws.lens, ws.codes, iter == 3);
     }
     count_launches(P, 9);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack(lfc_plan P, int nblocks) {
+cudaError_t launch_pack(lfc_plan P, int nblocks, int max_m) {
     Workspace &ws = P->ws;
     // group bit lengths live in the MTF index slots, free once RLE2 has run
     uint16_t *gbits = reinterpret_cast<uint16_t *>(ws.mtfidx);
-    const dim3 grid(kPackTiles, nblocks);
+    const dim3 grid(pack_tiles(max_m), nblocks);
     pack_bits_kernel<<<grid, kPackGroups, 0, P->stream>>>(ws.bstate, ws.sym, ws.sel, ws.lens, gbits, ws.tileaux);
     pack_layout_kernel<<<nblocks, kLayoutThreads, 0, P->stream>>>(ws.bstate, ws.sel, ws.lens, ws.tileaux, ws.packed,
                                                                   ws.stream_words);
