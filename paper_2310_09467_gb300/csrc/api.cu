@@ -15,6 +15,7 @@ constexpr int kJudgeFramesCap = 16;
 // the decoder never reads a stream past its 18002 selectors, six tables and
 // 18002 groups of 50 codes of at most 20 bits
 constexpr int64_t kMaxStreamRead = 3000000;
+constexpr int kChainRangeMin = 1024;  // bytes a chain warp walks at least
 constexpr int kDefaultWaitMs = 1000;  // bounded device waits give up after this long
 
 int fail(lfc_plan P, int code, const std::string &what, cudaError_t e = cudaSuccess) {
@@ -319,7 +320,8 @@ extern "C" int lfc_plan_create(const lfc_config *cfg, void *cuda_stream, lfc_pla
     const int JF = P->judge_frames_cap, BC = P->block_cap;
     const int64_t seg_min = chain_seg_bytes(16384);  // smallest tunable segment
     const int64_t segs_max = (n_max + seg_min - 1) / seg_min;
-    ws.summ_cap = (int64_t)JF * K * segs_max;
+    // shorter ranges are taken as long as their summaries fit (one wave's do)
+    ws.summ_cap = std::max<int64_t>((int64_t)JF * K * segs_max, P->sm_count);
     ws.cstream_kmax = K;
     ws.cstream_slot = (n_max + 255) & ~(int64_t)255;
     ws.stream_slot = (n_max + 255) & ~(int64_t)255;
@@ -488,7 +490,10 @@ bool capturing(lfc_plan P) {
 // range r gives sum_f K_f ceil(n_f / seg(r)) CTAs; its cost is taken as the
 // waves those need times (r + a fixed per-CTA share of 8 KB). Candidates: the
 // equal splits of the largest stream into s >= s0 segments (s0 the count at
-// the tuned range), at most 2 s0, a multiple of 512 bytes, >= 16 KB.
+// the tuned range), a multiple of 512 bytes: at most 2 s0 when those already
+// make two waves, else up to 32 more, down to 1 KB as long as the segments'
+// summaries fit (one 195 x 195 frame: 26 streams of 76 KB on one warp each took 427
+// us, cut over all SMs 60).
 int chain_range_for(lfc_plan P, const lfc_frame *frames, int nf) {
     const int tuned = P->tune.chain_range_bytes;
     int64_t n_max = 0;
@@ -499,17 +504,21 @@ int chain_range_for(lfc_plan P, const lfc_frame *frames, int nf) {
     const int64_t s0 = std::max<int64_t>(1, (n_max + w * tuned - 1) / (w * tuned));
     int best = tuned;
     double best_cost = -1.0;
-    for (int64_t s = s0; s <= 2 * s0; s++) {
+    int64_t s_end = 2 * s0;
+    for (int64_t s = s0; s <= s_end; s++) {
         int64_t r = (n_max + w * s - 1) / (w * s);
         r = (r + 511) / 512 * 512;
-        if (r > tuned || r < 16384) continue;
+        if (r > tuned) continue;
+        if (r < kChainRangeMin) break;
         int64_t ctas = 0;
         for (int i = 0; i < nf; i++) {
             const int64_t nb = 2LL * frames[i].width * frames[i].height;
             const int K = (frames[i].prev != nullptr && !P->ids_temporal.empty()) ? k_all : k_spatial;
             ctas += (int64_t)K * ((nb + w * r - 1) / (w * r));
         }
+        if (s == s0 && ctas < 2 * P->sm_count) s_end += 32;
         const int64_t waves = (ctas + P->sm_count - 1) / P->sm_count;
+        if (ctas > P->ws.summ_cap) break;
         const double cost = (double)waves * (double)(r + 8192);
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
