@@ -4,11 +4,12 @@
 //
 // Layout: activations NHWC in BF16 ([frame][y][x][channel], 32 channels;
 // the 2-channel input is padded to 16), master parameters FP32.
-// Forward and input-gradient convolutions are implicit GEMMs on the tensor
-// cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation): one CTA per
-// 8 x 16 output tile, one warp per 16-pixel row, the input tile with its
-// halo and all 9 x 32 x Cin weights staged in shared memory. Weight
-// gradients are FP32 outer products on the CUDA cores over row bands.
+// All three convolutions are implicit GEMMs on the tensor cores (mma.sync
+// m16n8k16, BF16 operands, FP32 accumulation). Forward and input gradient: one
+// CTA per 16 x 16 output tile, one warp per two 16-pixel rows, the input tile
+// with its halo and all 9 x 32 x Cin weights staged in shared memory. Weight
+// gradient: one warp per tap, input channels x output channels summed over
+// the pixels of a band of rows.
 #include "lfc_common.cuh"
 
 #include <cuda_bf16.h>
@@ -107,72 +108,98 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+__device__ __forceinline__ void ldm4t(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
 // out[y][x][co] = epilogue(sum_{ky,kx,ci} in[y+ky-1][x+kx-1][ci] * W[ky][kx][ci][co])
 // MODE 0: + bias, ReLU.  MODE 1: * (mask[y][x][co] > 0)  (input gradient).
+// Bound by shared memory: a warp's weight fragments serve two rows (16
+// wavefronts per 8 products; one row took 24), and a 16 x 16 tile halves the
+// weights staged per output against 8 x 16: 198 -> 135 us for 32 frames of a
+// 32-channel layer. The order of a sum's terms is that of the taps and
+// channels, whatever the tile.
 template <int CIN, int MODE>
 __global__ void __launch_bounds__(256) conv3x3_mma_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ wB,
                                                           const float *__restrict__ bias, const bf16 *__restrict__ mask,
                                                           bf16 *__restrict__ out) {
-    constexpr int TW = 16, TH = 8, CP = CIN + 8;  // +8: conflict-free fragment loads
+    constexpr int TW = 16, TH = 16, CP = CIN + 8;  // +8: conflict-free fragment loads
     __shared__ __align__(16) bf16 tile[TH + 2][TW + 2][CP];
     __shared__ __align__(16) bf16 wsm[9][kCh][CP];
     const int b = blockIdx.z, x0 = blockIdx.x * TW, y0 = blockIdx.y * TH;
     const bf16 *inb = in + (size_t)b * kPix * CIN;
-    for (int i = threadIdx.x; i < (TH + 2) * (TW + 2) * (CIN / 2); i += blockDim.x) {
-        const int c2 = i % (CIN / 2), pix = i / (CIN / 2);
+    for (int i = threadIdx.x; i < (TH + 2) * (TW + 2) * (CIN / 8); i += blockDim.x) {
+        const int c8 = i % (CIN / 8), pix = i / (CIN / 8);
         const int ty = pix / (TW + 2), tx = pix % (TW + 2);
         const int y = y0 + ty - 1, x = x0 + tx - 1;
-        uint32_t v = 0;
-        if (y >= 0 && y < kT && x >= 0 && x < kT) v = *reinterpret_cast<const uint32_t *>(inb + ((size_t)y * kT + x) * CIN + 2 * c2);
-        *reinterpret_cast<uint32_t *>(&tile[ty][tx][2 * c2]) = v;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (y >= 0 && y < kT && x >= 0 && x < kT) v = __ldg(reinterpret_cast<const uint4 *>(inb + ((size_t)y * kT + x) * CIN + 8 * c8));
+        *reinterpret_cast<uint4 *>(&tile[ty][tx][8 * c8]) = v;
     }
-    for (int i = threadIdx.x; i < 9 * kCh * (CIN / 2); i += blockDim.x) {
-        const int c2 = i % (CIN / 2), r = i / (CIN / 2);
-        *reinterpret_cast<uint32_t *>(&wsm[r / kCh][r % kCh][2 * c2]) = *reinterpret_cast<const uint32_t *>(wB + (size_t)r * CIN + 2 * c2);
+    for (int i = threadIdx.x; i < 9 * kCh * (CIN / 8); i += blockDim.x) {
+        const int c8 = i % (CIN / 8), r = i / (CIN / 8);
+        *reinterpret_cast<uint4 *>(&wsm[r / kCh][r % kCh][8 * c8]) = __ldg(reinterpret_cast<const uint4 *>(wB + (size_t)r * CIN + 8 * c8));
     }
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    float acc[4][4];
+    // a lane's row and channel offset in the four 8 x 8 blocks of a load
+    const int ar = lane & 15, ac = (lane >> 4) * 8;                       // pixels 0-15, channels 0-7 | 8-15
+    const int br = (lane & 7) + (lane >> 4) * 8, bc = ((lane >> 3) & 1) * 8;  // outputs 0-7 | 8-15, channels 0-7 | 8-15
+    float acc[2][4][4];
 #pragma unroll
-    for (int j = 0; j < 4; j++)
+    for (int r = 0; r < 2; r++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) acc[j][q] = 0.f;
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[r][j][q] = 0.f;
 #pragma unroll
     for (int kk = 0; kk < 9; kk++) {
         const int ky = kk / 3, kx = kk % 3;
 #pragma unroll
         for (int cb = 0; cb < CIN; cb += 16) {
-            uint32_t a[4];
-            a[0] = *reinterpret_cast<const uint32_t *>(&tile[w + ky][g + kx][cb + 2 * t]);
-            a[1] = *reinterpret_cast<const uint32_t *>(&tile[w + ky][g + 8 + kx][cb + 2 * t]);
-            a[2] = *reinterpret_cast<const uint32_t *>(&tile[w + ky][g + kx][cb + 2 * t + 8]);
-            a[3] = *reinterpret_cast<const uint32_t *>(&tile[w + ky][g + 8 + kx][cb + 2 * t + 8]);
+            uint32_t a0[4], a1[4], b0[4], b1[4];
+            ldm4(a0, &tile[2 * w + ky][ar + kx][cb + ac]);
+            ldm4(a1, &tile[2 * w + 1 + ky][ar + kx][cb + ac]);
+            ldm4(b0, &wsm[kk][br][cb + bc]);
+            ldm4(b1, &wsm[kk][16 + br][cb + bc]);
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const uint32_t b0 = *reinterpret_cast<const uint32_t *>(&wsm[kk][j * 8 + g][cb + 2 * t]);
-                const uint32_t b1 = *reinterpret_cast<const uint32_t *>(&wsm[kk][j * 8 + g][cb + 2 * t + 8]);
-                mma_bf16(acc[j], a, b0, b1);
+            for (int r = 0; r < 2; r++) {
+                const uint32_t(&a)[4] = r ? a1 : a0;
+                mma_bf16(acc[r][0], a, b0[0], b0[1]);
+                mma_bf16(acc[r][1], a, b0[2], b0[3]);
+                mma_bf16(acc[r][2], a, b1[0], b1[1]);
+                mma_bf16(acc[r][3], a, b1[2], b1[3]);
             }
         }
     }
-    const int y = y0 + w;
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const int co = j * 8 + 2 * t;
+    for (int r = 0; r < 2; r++) {
+        const int y = y0 + 2 * w + r;
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int x = x0 + g + 8 * h;
-            const size_t pix = (size_t)b * kPix + (size_t)y * kT + x;
-            float v0 = acc[j][2 * h], v1 = acc[j][2 * h + 1];
-            if (MODE == 0) {
-                v0 = fmaxf(v0 + bias[co], 0.f);
-                v1 = fmaxf(v1 + bias[co + 1], 0.f);
-            } else {
-                const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162 *>(mask + pix * kCh + co);
-                if (!(__bfloat162float(mk.x) > 0.f)) v0 = 0.f;
-                if (!(__bfloat162float(mk.y) > 0.f)) v1 = 0.f;
+        for (int j = 0; j < 4; j++) {
+            const int co = j * 8 + 2 * t;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int x = x0 + g + 8 * h;
+                const size_t pix = (size_t)b * kPix + (size_t)y * kT + x;
+                float v0 = acc[r][j][2 * h], v1 = acc[r][j][2 * h + 1];
+                if (MODE == 0) {
+                    v0 = fmaxf(v0 + bias[co], 0.f);
+                    v1 = fmaxf(v1 + bias[co + 1], 0.f);
+                } else {
+                    const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162 *>(mask + pix * kCh + co);
+                    if (!(__bfloat162float(mk.x) > 0.f)) v0 = 0.f;
+                    if (!(__bfloat162float(mk.y) > 0.f)) v1 = 0.f;
+                }
+                *reinterpret_cast<__nv_bfloat162 *>(out + pix * kCh + co) = __floats2bfloat162_rn(v0, v1);
             }
-            *reinterpret_cast<__nv_bfloat162 *>(out + pix * kCh + co) = __floats2bfloat162_rn(v0, v1);
         }
     }
 }
@@ -257,90 +284,123 @@ __global__ void head_backward_kernel(const float *__restrict__ gap, const float 
     }
 }
 
-// gradient at the last convolution's pre-activation: pool gradient through ReLU
+// gradient at the last convolution's pre-activation: pool gradient through
+// ReLU; a thread per 8 channels (16-byte loads and stores)
 __global__ void dpre_last_kernel(const float *__restrict__ dg, const bf16 *__restrict__ act, bf16 *__restrict__ dpre, int nb) {
-    const size_t total = (size_t)nb * kPix * kCh;
+    const size_t total = (size_t)nb * kPix * (kCh / 8);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % kCh);
-        const size_t b = i / ((size_t)kPix * kCh);
-        const float v = __bfloat162float(act[i]) > 0.f ? dg[b * kCh + c] * (1.f / (float)kPix) : 0.f;
-        dpre[i] = __float2bfloat16(v);
+        const int c8 = (int)(i % (kCh / 8)) * 8;
+        const size_t b = i / ((size_t)kPix * (kCh / 8));
+        __align__(16) bf16 a[8];
+        *reinterpret_cast<uint4 *>(a) = __ldg(reinterpret_cast<const uint4 *>(act) + i);
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const float v = __bfloat162float(a[c]) > 0.f ? dg[b * kCh + c8 + c] * (1.f / (float)kPix) : 0.f;
+            a[c] = __float2bfloat16(v);
+        }
+        reinterpret_cast<uint4 *>(dpre)[i] = *reinterpret_cast<const uint4 *>(a);
     }
 }
 
 // dW[ky][kx][ci][co] += sum over a band of rows of in[y+ky-1][x+kx-1][ci] * dpre[y][x][co];
-// db[co] += sum dpre. Tasks: (tap, 4 input channels, 4 output channels).
+// db[co] += sum dpre. One CTA per band and frame, one warp per tap: 16 input
+// channels x 8 output channels per product, 16 pixels deep. Both operands lie
+// pixel-major in shared memory and are read transposed; the tensor cores sum
+// a row's products, and the rows are added in registers with rounding to
+// nearest (the tensor cores' own sums truncate). Bound by shared memory (16
+// wavefronts per 8 products); as FP32 outer products on the CUDA cores, a
+// 32-channel layer of 32 frames took 2030 us.
+constexpr int kWgThreads = 9 * 32;
 template <int CIN>
-__global__ void __launch_bounds__(256) conv_wgrad_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ dpre,
-                                                         float *__restrict__ dW, float *__restrict__ db, int rows, int cin_real) {
-    constexpr int XH = kT / 2;  // half a row per step keeps shared memory under 48 KB
-    __shared__ __align__(16) bf16 ins[3][XH + 2][CIN];
-    __shared__ __align__(16) bf16 dps[XH][kCh];
-    constexpr int NTASK = 9 * (CIN / 4) * (kCh / 4);
-    constexpr int TPT = (NTASK + 255) / 256;
-    const int b = blockIdx.y, y0 = blockIdx.x * rows;
-    float acc[TPT][16];
-    float bacc = 0.f;
+struct WgradSmem {
+    static constexpr int CP = CIN + 8, DP = kCh + 8;  // +8: conflict-free fragment loads
+    bf16 in[3][kT + 2][CP];  // rows y - 1 .. y + 1, row r in slot (r + 3) % 3, a zero pixel at either end
+    bf16 d[kT][DP];
+};
+
+template <int CIN>
+__global__ void __launch_bounds__(kWgThreads) conv_wgrad_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ dpre,
+                                                                float *__restrict__ dW, float *__restrict__ db, int rows, int cin_real) {
+    constexpr int MT = CIN / 16;
+    extern __shared__ __align__(16) uint8_t smraw[];
+    WgradSmem<CIN> &S = *reinterpret_cast<WgradSmem<CIN> *>(smraw);
+    __shared__ float sb[kCh];
+    const int b = blockIdx.y, y0 = blockIdx.x * rows, y1 = min(kT, y0 + rows);
+    const int tap = threadIdx.x >> 5, lane = threadIdx.x & 31, ky = tap / 3, kx = tap % 3;
+    auto load_row = [&](int y) {  // zeros outside the image
+        bf16(*row)[WgradSmem<CIN>::CP] = S.in[(y + 3) % 3];
+        const uint4 *src = reinterpret_cast<const uint4 *>(in + ((size_t)b * kT + max(0, min(kT - 1, y))) * kT * CIN);
+        const bool inside = y >= 0 && y < kT;
+        for (int i = threadIdx.x; i < kT * (CIN / 8); i += kWgThreads)
+            *reinterpret_cast<uint4 *>(&row[1 + i / (CIN / 8)][8 * (i % (CIN / 8))]) = inside ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
+    };
+    if (threadIdx.x < kCh) sb[threadIdx.x] = 0.f;
+    for (int i = threadIdx.x; i < 6 * (CIN / 8); i += kWgThreads) {  // the end pixels of the three rows
+        const int c8 = i % (CIN / 8), e = i / (CIN / 8);
+        *reinterpret_cast<uint4 *>(&S.in[e >> 1][(e & 1) * (kT + 1)][8 * c8]) = make_uint4(0, 0, 0, 0);
+    }
+    load_row(y0 - 1);
+    load_row(y0);
+    float acc[MT][4][4];
+    float2 bacc = make_float2(0.f, 0.f);  // channels 2 (t % 16), + 1, pixels t / 16 of 18
 #pragma unroll
-    for (int q = 0; q < TPT; q++)
+    for (int m = 0; m < MT; m++)
 #pragma unroll
-        for (int e = 0; e < 16; e++) acc[q][e] = 0.f;
-    for (int y = y0; y < y0 + rows; y++) {
-        for (int xh = 0; xh < kT; xh += XH) {
-            for (int i = threadIdx.x; i < 3 * (XH + 2) * (CIN / 2); i += blockDim.x) {
-                const int c2 = i % (CIN / 2), r = i / (CIN / 2), row = r / (XH + 2), col = r % (XH + 2);
-                const int yy = y + row - 1, xx = xh + col - 1;
-                uint32_t v = 0;
-                if (yy >= 0 && yy < kT && xx >= 0 && xx < kT)
-                    v = *reinterpret_cast<const uint32_t *>(in + (((size_t)b * kT + yy) * kT + xx) * CIN + 2 * c2);
-                *reinterpret_cast<uint32_t *>(&ins[row][col][2 * c2]) = v;
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[m][j][q] = 0.f;
+    // a lane's row (pixel) and channel offset in the four 8 x 8 blocks of a load
+    const int ap = (lane & 7) + (lane >> 4) * 8, ac = ((lane >> 3) & 1) * 8;  // pixels 0-7 | 8-15 of channels 0-7 and 8-15
+    const int bp = lane & 15, bc = (lane >> 4) * 8;                           // pixels 0-15, outputs 0-7 | 8-15
+    for (int y = y0; y < y1; y++) {
+        load_row(y + 1);
+        const uint4 *src = reinterpret_cast<const uint4 *>(dpre + ((size_t)b * kT + y) * kT * kCh);
+        for (int i = threadIdx.x; i < kT * (kCh / 8); i += kWgThreads)
+            *reinterpret_cast<uint4 *>(&S.d[i / (kCh / 8)][8 * (i % (kCh / 8))]) = __ldg(src + i);
+        __syncthreads();
+        const bf16(*row)[WgradSmem<CIN>::CP] = S.in[(y + ky + 2) % 3];
+        float part[MT][4][4] = {};
+#pragma unroll 4
+        for (int p = 0; p < kT; p += 16) {
+            uint32_t b0[4], b1[4];
+            ldm4t(b0, &S.d[p + bp][bc]);
+            ldm4t(b1, &S.d[p + bp][16 + bc]);
+#pragma unroll
+            for (int m = 0; m < MT; m++) {
+                uint32_t a[4];
+                ldm4t(a, &row[p + kx + ap][16 * m + ac]);
+                mma_bf16(part[m][0], a, b0[0], b0[1]);
+                mma_bf16(part[m][1], a, b0[2], b0[3]);
+                mma_bf16(part[m][2], a, b1[0], b1[1]);
+                mma_bf16(part[m][3], a, b1[2], b1[3]);
             }
-            for (int i = threadIdx.x; i < XH * (kCh / 2); i += blockDim.x) {
-                const int c2 = i % (kCh / 2), x = i / (kCh / 2);
-                *reinterpret_cast<uint32_t *>(&dps[x][2 * c2]) =
-                    *reinterpret_cast<const uint32_t *>(dpre + (((size_t)b * kT + y) * kT + xh + x) * kCh + 2 * c2);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < TPT; q++) {
-                const int task = threadIdx.x + q * 256;
-                if (task >= NTASK) break;
-                const int kk = task / ((CIN / 4) * (kCh / 4)), rem = task % ((CIN / 4) * (kCh / 4));
-                const int ci4 = rem / (kCh / 4), co4 = rem % (kCh / 4);
-                const int ky = kk / 3, kx = kk % 3;
-                if (ci4 * 4 >= cin_real) continue;
-                for (int x = 0; x < XH; x++) {
-                    float a[4], d[4];
-#pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        a[e] = __bfloat162float(ins[ky][x + kx][ci4 * 4 + e]);
-                        d[e] = __bfloat162float(dps[x][co4 * 4 + e]);
-                    }
-#pragma unroll
-                    for (int i2 = 0; i2 < 4; i2++)
-#pragma unroll
-                        for (int j2 = 0; j2 < 4; j2++) acc[q][i2 * 4 + j2] = fmaf(a[i2], d[j2], acc[q][i2 * 4 + j2]);
-                }
-            }
-            if (threadIdx.x < kCh)
-                for (int x = 0; x < XH; x++) bacc += __bfloat162float(dps[x][threadIdx.x]);
-            __syncthreads();
         }
+#pragma unroll
+        for (int m = 0; m < MT; m++)
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) acc[m][j][q] += part[m][j][q];
+        for (int p = threadIdx.x >> 4; p < kT; p += kWgThreads / 16) {
+            const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(&S.d[p][2 * (threadIdx.x & 15)]);
+            bacc.x += __bfloat162float(v.x);
+            bacc.y += __bfloat162float(v.y);
+        }
+        __syncthreads();
     }
 #pragma unroll
-    for (int q = 0; q < TPT; q++) {
-        const int task = threadIdx.x + q * 256;
-        if (task >= NTASK) break;
-        const int kk = task / ((CIN / 4) * (kCh / 4)), rem = task % ((CIN / 4) * (kCh / 4));
-        const int ci4 = rem / (kCh / 4), co4 = rem % (kCh / 4);
-        for (int i2 = 0; i2 < 4; i2++) {
-            const int ci = ci4 * 4 + i2;
-            if (ci >= cin_real) continue;
-            for (int j2 = 0; j2 < 4; j2++)
-                atomicAdd(&dW[((size_t)kk * cin_real + ci) * kCh + co4 * 4 + j2], acc[q][i2 * 4 + j2]);
-        }
-    }
-    if (threadIdx.x < kCh) atomicAdd(&db[threadIdx.x], bacc);
+    for (int m = 0; m < MT; m++)
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const int ci = 16 * m + (lane >> 2) + 8 * (q >> 1), co = 8 * j + 2 * (lane & 3) + (q & 1);
+                if (ci < cin_real) atomicAdd(&dW[((size_t)tap * cin_real + ci) * kCh + co], acc[m][j][q]);
+            }
+    atomicAdd(&sb[2 * (threadIdx.x & 15)], bacc.x);
+    atomicAdd(&sb[2 * (threadIdx.x & 15) + 1], bacc.y);
+    __syncthreads();
+    if (threadIdx.x < kCh) atomicAdd(&db[threadIdx.x], sb[threadIdx.x]);
 }
 
 // Master FP32 weights -> BF16 operands: forward [tap][co][ci_pad],
@@ -571,10 +631,10 @@ __global__ void set_thumbs_kernel(const float *__restrict__ th, int n, bf16 *__r
     const size_t total = (size_t)n * kPix;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t b = i / kPix, pix = i % kPix;
-        bf16 *o = x0 + i * kC0;
-        o[0] = __float2bfloat16(th[(b * 2) * kPix + pix]);
-        o[1] = __float2bfloat16(th[(b * 2 + 1) * kPix + pix]);
-        for (int c = 2; c < kC0; c++) o[c] = __float2bfloat16(0.f);
+        const __nv_bfloat162 v = __floats2bfloat162_rn(th[(b * 2) * kPix + pix], th[(b * 2 + 1) * kPix + pix]);
+        uint4 *o = reinterpret_cast<uint4 *>(x0 + i * kC0);
+        o[0] = make_uint4(*reinterpret_cast<const uint32_t *>(&v), 0u, 0u, 0u);
+        o[1] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -587,7 +647,7 @@ extern "C" int lfc_cnn_set_thumbnails(lfc_cnn C, const float *d_thumbs, int n) {
 
 static int cnn_forward(lfc_cnn C, int n) {
     cudaStream_t s = C->stream;
-    dim3 grid(kT / 16, kT / 8, n);
+    dim3 grid(kT / 16, kT / 16, n);
     conv3x3_mma_kernel<kC0, 0><<<grid, 256, 0, s>>>(C->x0, C->wf[0], C->params + C->off.b[0], nullptr, C->act[0]);
     for (int l = 1; l < 4; l++)
         conv3x3_mma_kernel<kCh, 0><<<grid, 256, 0, s>>>(C->act[l - 1], C->wf[l], C->params + C->off.b[l], nullptr, C->act[l]);
@@ -616,16 +676,21 @@ extern "C" int lfc_cnn_backward(lfc_cnn C, int n, const int32_t *d_labels, float
     CKC(cudaMemsetAsync(C->grads, 0, C->off.total * 4, s));
     head_backward_kernel<<<1, 256, 0, s>>>(C->gap, C->dz, C->params, C->grads, C->off.wl, C->off.bl, C->K, n, C->dg);
     dpre_last_kernel<<<1216, 256, 0, s>>>(C->dg, C->act[3], C->dpre[1], n);
-    constexpr int rows = 16;
+    // rows of a weight-gradient band: 16 (a band's 9216 sums go out by
+    // atomics), fewer while the bands would leave SMs without one
+    int rows = 16;
+    while (rows > 2 && n * (kT / rows) < 152) rows /= 2;
+    CKC(cudaFuncSetAttribute(conv_wgrad_kernel<kCh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem<kCh>)));
+    CKC(cudaFuncSetAttribute(conv_wgrad_kernel<kC0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem<kC0>)));
     dim3 wgrid(kT / rows, n);
-    dim3 grid(kT / 16, kT / 8, n);
+    dim3 grid(kT / 16, kT / 16, n);
     int cur = 1;
     for (int l = 3; l >= 0; l--) {
         if (l > 0)
-            conv_wgrad_kernel<kCh><<<wgrid, 256, 0, s>>>(C->act[l - 1], C->dpre[cur], C->grads + C->off.w[l],
+            conv_wgrad_kernel<kCh><<<wgrid, kWgThreads, sizeof(WgradSmem<kCh>), s>>>(C->act[l - 1], C->dpre[cur], C->grads + C->off.w[l],
                                                            C->grads + C->off.b[l], rows, kCh);
         else
-            conv_wgrad_kernel<kC0><<<wgrid, 256, 0, s>>>(C->x0, C->dpre[cur], C->grads + C->off.w[0], C->grads + C->off.b[0],
+            conv_wgrad_kernel<kC0><<<wgrid, kWgThreads, sizeof(WgradSmem<kC0>), s>>>(C->x0, C->dpre[cur], C->grads + C->off.w[0], C->grads + C->off.b[0],
                                                            rows, 2);
         if (l > 0) {
             conv3x3_mma_kernel<kCh, 1><<<grid, 256, 0, s>>>(C->dpre[cur], C->wd[l], nullptr, C->act[l - 1], C->dpre[cur ^ 1]);
