@@ -57,11 +57,11 @@ struct DecMeta {
 };
 static_assert(sizeof(DecMeta) == sizeof(BlockState), "the decoder's block records live in the coder's");
 
-constexpr int kJBits = 13;  // prefix bits of the length table
+constexpr int kJBits = 12;  // prefix bits of the length table
 struct DecTab {
-    uint16_t jlut[kMaxGroups][1 << kJBits];  // bits of the first code | bits of the first two << 5 (0: do not fit)
+    uint2 jlut[1 << kJBits];                 // a byte per table: bits of the code (0: longer)
     uint16_t lut[kMaxGroups][1 << 10];       // symbol << 5 | code length, 0: longer code
-    int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];
+    int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];  // laid out as Canon
     uint16_t perm[kMaxGroups][kMaxAlpha];    // symbols by code
     uint8_t seq_to_unseq[256];
 };
@@ -138,19 +138,21 @@ struct BitReader {
     }
 };
 
+// Canonical tables, per code length.
+struct Canon {
+    int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];
+};
+
 // One Huffman symbol with table t: the 10-bit lookup, else the canonical
 // search from 11 bits; -1 for a code that is not in the table or a stream
 // that ends first (br.err).
-__device__ __forceinline__ int huff_symbol(BitReader &br, const uint16_t *lut, const DecTab &T, int t) {
-    const uint32_t e = lut[br.peek(10)];
+__device__ __forceinline__ int huff_symbol(BitReader &br, const uint16_t *lut, const Canon &C, const DecTab &T, int t) {
+    if (br.bcnt < 20) br.refill();
+    const uint32_t v = (uint32_t)(br.buf >> 44), e = lut[v >> 10];
     if (e) return br.skip(e & 31) ? (int)(e >> 5) : -1;
-    int32_t c = (int32_t)br.peek(10);
-    if (!br.skip(10)) return -1;
     for (int l = 11; l <= 20; l++) {
-        c = (c << 1) | (int32_t)br.get(1);
-        if (br.err) return -1;
-        const uint32_t d = (uint32_t)(c - T.first[t][l]);
-        if (d < (uint32_t)T.count[t][l]) return T.perm[t][T.pidx[t][l] + (int)d];
+        const uint32_t d = (uint32_t)((int32_t)(v >> (20 - l)) - C.first[t][l]);
+        if (d < (uint32_t)C.count[t][l]) return br.skip(l) ? T.perm[t][C.pidx[t][l] + (int)d] : -1;
     }
     return -1;
 }
@@ -176,6 +178,7 @@ __global__ void __launch_bounds__(kHdrThreads) dec_header_kernel(const DecBlock 
                                                                  uint8_t *__restrict__ sel_all, int32_t *__restrict__ zpos_all) {
     __shared__ uint8_t len[kMaxGroups][kMaxAlpha];
     __shared__ int32_t first[kMaxGroups][22], count[kMaxGroups][22], pidx[kMaxGroups][22];
+    __shared__ uint16_t perm[kMaxGroups][kMaxAlpha];
     __shared__ int sh[33];
     __shared__ uint32_t wlist[kHdrThreads / 32];
     __shared__ int s_status, s_alpha, s_ng, s_nsel, s_bit;
@@ -334,36 +337,33 @@ __global__ void __launch_bounds__(kHdrThreads) dec_header_kernel(const DecBlock 
         const int g = i / alpha, v = i - g * alpha, k = len[g][v];
         int r = 0;
         for (int x = 0; x < v; x++) r += len[g][x] == k;
-        T.perm[g][pidx[g][k] + r] = (uint16_t)v;
+        perm[g][pidx[g][k] + r] = (uint16_t)v;
     }
+    __syncthreads();
+    for (int i = t; i < kMaxGroups * kMaxAlpha; i += kHdrThreads) (&T.perm[0][0])[i] = (&perm[0][0])[i];
     for (int i = t; i < kMaxGroups * 22; i += kHdrThreads) {
         (&T.first[0][0])[i] = (&first[0][0])[i];
         (&T.count[0][0])[i] = (&count[0][0])[i];
         (&T.pidx[0][0])[i] = (&pidx[0][0])[i];
     }
-    for (int i = t; i < ng << kJBits; i += kHdrThreads) {  // length of the first code of a prefix
-        const int g = i >> kJBits, x = i & ((1 << kJBits) - 1);
-        uint16_t v = 0;
-        for (int k = 1; k <= kJBits; k++)
-            if ((uint32_t)((x >> (kJBits - k)) - first[g][k]) < (uint32_t)count[g][k]) { v = (uint16_t)k; break; }
-        T.jlut[g][x] = v;
-    }
-    __syncthreads();
-    for (int i = t; i < ng << kJBits; i += kHdrThreads) {  // and of the second one, if the prefix holds it
-        const int g = i >> kJBits, x = i & ((1 << kJBits) - 1);
-        const int k = T.jlut[g][x] & 31;
-        if (!k) continue;
-        const int k2 = T.jlut[g][(x << k) & ((1 << kJBits) - 1)] & 31;
-        if (k2 && k + k2 <= kJBits) T.jlut[g][x] = (uint16_t)(k | ((k + k2) << 5));
+    // length of the code that x, n bits, begins with; 0 if it is longer
+    auto code_len = [&](int g, uint32_t x, int n) {
+        for (int k = 1; k <= n; k++)
+            if ((uint32_t)((int32_t)(x >> (n - k)) - first[g][k]) < (uint32_t)count[g][k]) return k;
+        return 0;
+    };
+    for (int x = t; x < 1 << kJBits; x += kHdrThreads) {
+        uint32_t k[8] = {};
+#pragma unroll
+        for (int g = 0; g < kMaxGroups; g++)
+            if (g < ng) k[g] = code_len(g, x, kJBits);
+        T.jlut[x] = make_uint2(k[0] | (k[1] << 8) | (k[2] << 16) | (k[3] << 24), k[4] | (k[5] << 8));
     }
     for (int i = t; i < ng << 10; i += kHdrThreads) {
-        const int g = i >> 10, x = i & 1023;
-        uint16_t v = 0;
-        for (int k = 1; k <= 10; k++) {
-            const uint32_t d = (uint32_t)((x >> (10 - k)) - first[g][k]);
-            if (d < (uint32_t)count[g][k]) { v = (uint16_t)((T.perm[g][pidx[g][k] + (int)d] << 5) | k); break; }
-        }
-        T.lut[g][x] = v;
+        const int g = i >> 10;
+        const uint32_t x = i & 1023;
+        const int k = code_len(g, x, 10);
+        T.lut[g][x] = k ? (uint16_t)((perm[g][pidx[g][k] + ((int32_t)(x >> (10 - k)) - first[g][k])] << 5) | k) : (uint16_t)0;
     }
     if (t == 0) {
         M.group = 0;
@@ -377,42 +377,39 @@ __global__ void __launch_bounds__(kHdrThreads) dec_header_kernel(const DecBlock 
 // ------------------------------------------------------ 2. group offsets
 // Lengths of 50 codes from every bit of a stretch of kJRange bits, for every
 // table: a tile of kJTile bits per CTA with the bits its groups reach into.
-// A tile holds, per bit, the bit a number of codes further (kJSpan: none), so
-// a doubling is one gather: out[i] = in[in[i]]. Bound by issue: about 40
-// instructions per bit and table, two bits per load and store.
+// One 8-byte lookup gives a bit position's code length in all six tables;
+// lengths of 2, 4, 8 and 16 codes are bytes (0: there are none, or they are
+// too long; such a group is decoded on the chase), four positions a thread:
+// one load and one store of a word, four byte gathers and byte-wise sums a
+// doubling. Bound by shared memory, about 10 accesses per bit and table.
 constexpr int kJTile = 8192;
-constexpr int kJHalo = 1024;                  // 50 codes of at most 20 bits
+constexpr int kJHalo = 1024;                  // 2 + 16 + 16 + 16 codes: at most 40 + 3 * 254 bits, and the last code's 20
 constexpr int kJSpan = kJTile + kJHalo;
 constexpr int kJRange = (kBlockCap * 4 / 3) / kJTile * kJTile;  // bits per round: three tables fill a slot of 8-byte words
-constexpr int kJThreads = 512;
+constexpr int kJThreads = 768;                // three words each
 static_assert((size_t)kJRange * 3 * 2 <= (size_t)kBlockCap * 8, "three tables of one round fit a key slot");
+static_assert(kJSpan % (4 * kJThreads) == 0, "whole words per thread");
 
 struct JumpSmem {
+    uint2 lut[1 << kJBits];
+    __align__(16) uint8_t one[kMaxGroups][kJSpan + 256];             // 256 zeros behind every span
+    __align__(16) uint8_t b[kJSpan + 256], c[kJSpan + 256];
+    int32_t first[kMaxGroups][20 - kJBits], count[kMaxGroups][20 - kJBits];  // codes longer than the lookup's
     uint32_t bits[kJSpan / 32 + 4];
-    __align__(16) uint16_t lut[1 << kJBits];
-    __align__(4) uint16_t a[kJSpan + 2], b[kJSpan + 2], c[kJSpan + 2];
 };
 
-// Bits of two codes from bit p of the span, by the canonical tables (codes
-// longer than the lookup prefix); 0 if there are none.
-__device__ __noinline__ int two_codes(const uint32_t *bits, int p, const DecTab &T, int t) {
-    int total = 0;
-    for (int n = 0; n < 2; n++) {
-        const int q = p + total;
-        if (q + 20 > kJSpan + 64) return 0;
-        const uint32_t v = __funnelshift_l(bits[(q >> 5) + 1], bits[q >> 5], q & 31);
-        int l = 1;
-        for (; l <= 20; l++)
-            if ((uint32_t)((int32_t)(v >> (32 - l)) - T.first[t][l]) < (uint32_t)T.count[t][l]) break;
-        if (l > 20) return 0;
-        total += l;
-    }
-    return total;
+// 0xff for every byte of x whose top bit is set
+__device__ __forceinline__ uint32_t top_bytes(uint32_t x) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, 0xba98;" : "=r"(r) : "r"(x));
+    return r;
 }
+// 0xff for every byte of x, all below 128, that is not 0
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) { return top_bytes(x + 0x7f7f7f7fu); }
 
-__global__ void __launch_bounds__(kJThreads) dec_jump_kernel(const DecBlock *__restrict__ blocks, const DecMeta *__restrict__ meta,
-                                                             const DecTab *__restrict__ tabs, size_t tab_stride, int64_t range0,
-                                                             uint64_t *__restrict__ j0_all, uint64_t *__restrict__ j1_all) {
+__global__ void __launch_bounds__(kJThreads, 2) dec_jump_kernel(const DecBlock *__restrict__ blocks, const DecMeta *__restrict__ meta,
+                                                                const DecTab *__restrict__ tabs, size_t tab_stride, int64_t range0,
+                                                                uint64_t *__restrict__ j0_all, uint64_t *__restrict__ j1_all) {
     extern __shared__ __align__(16) uint8_t smraw[];
     JumpSmem &S = *reinterpret_cast<JumpSmem *>(smraw);
     const int b = blockIdx.y, t = threadIdx.x;
@@ -423,48 +420,92 @@ __global__ void __launch_bounds__(kJThreads) dec_jump_kernel(const DecBlock *__r
     const int64_t w0 = range0 + (int64_t)blockIdx.x * kJTile;
     if (w0 >= nbits || w0 + kJTile <= M.bit) return;
     const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
+    const int ng = M.n_groups;
+    for (int i = t; i < (1 << kJBits) / 2; i += kJThreads)
+        reinterpret_cast<uint4 *>(S.lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.jlut) + i);
     for (int i = t; i < kJSpan / 32 + 4; i += kJThreads) S.bits[i] = stream_bits32(D.src, D.src_len, w0 + 32 * i);
-    for (int g = 0; g < M.n_groups; g++) {
-        for (int i = t; i < (1 << kJBits) / 8; i += kJThreads)
-            reinterpret_cast<uint4 *>(S.lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.jlut[g]) + i);
-        __syncthreads();
-        auto two = [&](int i) -> uint32_t {  // the bit two codes after bit i
-            const uint32_t v = __funnelshift_l(S.bits[(i >> 5) + 1], S.bits[i >> 5], i & 31);
-            const uint32_t e = S.lut[v >> (32 - kJBits)];
-            int l = (int)(e >> 5);
-            if (!l) {
-                const int k = (int)(e & 31), q = i + k;
-                const uint32_t v2 = __funnelshift_l(S.bits[(q >> 5) + 1], S.bits[q >> 5], q & 31);
-                const int k2 = k ? (int)(S.lut[v2 >> (32 - kJBits)] & 31u) : 0;
-                l = k2 ? k + k2 : two_codes(S.bits, i, T, g);
+    for (int i = t; i < kMaxGroups * (20 - kJBits); i += kJThreads) {
+        const int g = i / (20 - kJBits), l = kJBits + 1 + i % (20 - kJBits);
+        (&S.first[0][0])[i] = T.first[g][l];
+        (&S.count[0][0])[i] = g < ng ? T.count[g][l] : 0;
+    }
+    if (t < 64 * (kMaxGroups + 2)) {
+        const int r = t >> 6;
+        reinterpret_cast<uint32_t *>((r < kMaxGroups ? S.one[r] : r == kMaxGroups ? S.b : S.c) + kJSpan)[t & 63] = 0;
+    }
+    __syncthreads();
+    for (int i = 4 * t; i < kJSpan; i += 4 * kJThreads) {  // single codes, all tables
+        const uint32_t v0 = S.bits[i >> 5], v1 = S.bits[(i >> 5) + 1];
+        const uint32_t v = __funnelshift_l(v1, v0, i & 31);  // 20 + 3 bits are looked at
+        uint2 e[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) e[k] = S.lut[(v << k) >> (32 - kJBits)];
+        uint32_t x[kMaxGroups];
+        {
+            const uint32_t p = __byte_perm(e[0].x, e[1].x, 0x5140), q = __byte_perm(e[2].x, e[3].x, 0x5140);
+            const uint32_t r = __byte_perm(e[0].x, e[1].x, 0x7362), u = __byte_perm(e[2].x, e[3].x, 0x7362);
+            x[0] = __byte_perm(p, q, 0x5410);
+            x[1] = __byte_perm(p, q, 0x7632);
+            x[2] = __byte_perm(r, u, 0x5410);
+            x[3] = __byte_perm(r, u, 0x7632);
+            const uint32_t f = __byte_perm(e[0].y, e[1].y, 0x5140), h = __byte_perm(e[2].y, e[3].y, 0x5140);
+            x[4] = __byte_perm(f, h, 0x5410);
+            x[5] = __byte_perm(f, h, 0x7632);
+        }
+#pragma unroll
+        for (int g = 0; g < kMaxGroups; g++) {
+            if (g >= ng) break;
+            uint32_t z = ~nonzero_bytes(x[g]) & 0x01010101u;
+            while (z) {  // a longer code, or none
+                const int sh = __ffs(z) - 1;
+                z &= z - 1;
+                const uint32_t y = v << (sh >> 3);
+                for (int l = kJBits + 1; l <= 20; l++)
+                    if ((uint32_t)((int32_t)(y >> (32 - l)) - S.first[g][l - kJBits - 1]) < (uint32_t)S.count[g][l - kJBits - 1]) {
+                        x[g] |= (uint32_t)l << sh;
+                        break;
+                    }
             }
-            return (uint32_t)(l ? min(i + l, kJSpan) : kJSpan);
-        };
-        for (int i = 2 * t; i < kJSpan; i += 2 * kJThreads)
-            *reinterpret_cast<uint32_t *>(&S.a[i]) = two(i) | (two(i + 1) << 16);
-        if (t == 0) S.a[kJSpan] = S.b[kJSpan] = S.c[kJSpan] = (uint16_t)kJSpan;
+            *reinterpret_cast<uint32_t *>(S.one[g] + i) = x[g];
+        }
+    }
+    __syncthreads();
+    auto twice = [&](const uint8_t *in, uint8_t *out, bool cap) {
+#pragma unroll
+        for (int r = 0; r < kJSpan / (4 * kJThreads); r++) {
+            const int i = 4 * (t + r * kJThreads);
+            const uint32_t x = *reinterpret_cast<const uint32_t *>(in + i);
+            const uint32_t y0 = in[__dp4a(x, 0x1u, (uint32_t)i)], y1 = in[__dp4a(x, 0x100u, (uint32_t)i) + 1];
+            const uint32_t y2 = in[__dp4a(x, 0x10000u, (uint32_t)i) + 2], y3 = in[__dp4a(x, 0x1000000u, (uint32_t)i) + 3];
+            const uint32_t y = __byte_perm(__byte_perm(y0, y1, 0x0040), __byte_perm(y2, y3, 0x0040), 0x5410);
+            uint32_t v = (x + y) & nonzero_bytes(y);  // x is 0 where y is read at its own place
+            if (cap) v &= ~top_bytes(v);  // eight codes of more than 127 bits
+            *reinterpret_cast<uint32_t *>(out + i) = v;
+        }
         __syncthreads();
-        auto twice = [&](const uint16_t *in, uint16_t *out) {
-#pragma unroll 3
-            for (int i = 2 * t; i < kJSpan; i += 2 * kJThreads) {
-                const uint32_t x = *reinterpret_cast<const uint32_t *>(&in[i]);
-                *reinterpret_cast<uint32_t *>(&out[i]) = (uint32_t)in[x & 0xFFFFu] | ((uint32_t)in[x >> 16] << 16);
-            }
-            __syncthreads();
-        };
-        twice(S.a, S.b);  // 4
-        twice(S.b, S.c);  // 8
-        twice(S.c, S.b);  // 16
+    };
+    for (int g = 0; g < ng; g++) {
+        twice(S.one[g], S.b, false);  // 2: at most 40 bits
+        twice(S.b, S.c, false);       // 4: at most 80
+        twice(S.c, S.one[g], true);   // 8: at most 127
+        twice(S.one[g], S.c, false);  // 16: at most 254
         uint16_t *out = reinterpret_cast<uint16_t *>((g < 3 ? j0_all : j1_all) + (size_t)b * kBlockCap) + (size_t)(g % 3) * kJRange +
                         (size_t)blockIdx.x * kJTile;
-        auto fifty = [&](uint32_t at16, int i) -> uint32_t {  // 16 + 16 + 16 + 2
-            const uint32_t j = S.a[S.b[S.b[at16]]];
-            return j == (uint32_t)kJSpan ? 0u : j - (uint32_t)i;
-        };
-#pragma unroll 2
-        for (int i = 2 * t; i < kJTile; i += 2 * kJThreads) {
-            const uint32_t x = *reinterpret_cast<const uint32_t *>(&S.b[i]);
-            *reinterpret_cast<uint32_t *>(&out[i]) = fifty(x & 0xFFFFu, i) | (fifty(x >> 16, i + 1) << 16);
+#pragma unroll
+        for (int r = 0; r < kJSpan / (4 * kJThreads); r++) {  // 2 + 16 + 16 + 16
+            const int i = 4 * (t + r * kJThreads);
+            if (i >= kJTile) break;
+            const uint32_t x = *reinterpret_cast<const uint32_t *>(S.b + i);
+            uint32_t v[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                uint32_t j = __dp4a(x, 1u << (8 * k), (uint32_t)i) + k;  // a walk that meets a 0 stands still on it
+                j += S.c[j];
+                j += S.c[j];
+                const uint32_t d = S.c[j];
+                v[k] = d ? j + d - (i + k) : 0u;
+            }
+            *reinterpret_cast<uint2 *>(out + i) = make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
         }
         __syncthreads();
     }
@@ -474,8 +515,8 @@ __global__ void __launch_bounds__(kJThreads) dec_jump_kernel(const DecBlock *__r
 // fetch the next window of them. After the last round also the last group,
 // up to EOB.
 constexpr int kChaseThreads = 256;
-constexpr int kChaseWin = 4096;  // bits of a window
-constexpr int kChaseBufs = 3;    // one in use, two on their way
+constexpr int kChaseWin = 8192;  // bits of a window: long enough that its barriers and copies hide behind 56 groups' adds
+constexpr int kChaseBufs = 2;    // one in use, one on its way
 struct ChaseSmem {
     __align__(16) uint16_t j[kChaseBufs][kMaxGroups][kChaseWin];
     uint8_t sel[kMaxSelectors + 14];
@@ -524,12 +565,11 @@ __global__ void __launch_bounds__(kChaseThreads) dec_chase_kernel(const DecBlock
     if (S.p < range1 && S.g < last) {
         int64_t w = range0 + (S.p - range0) / kChaseWin * kChaseWin;
         fetch(w, 0);
-        fetch(w + kChaseWin, 1);
-        for (int buf = 0; w < range1; w += kChaseWin, buf = buf == kChaseBufs - 1 ? 0 : buf + 1) {
+        for (int buf = 0; w < range1; w += kChaseWin, buf ^= 1) {
             bool stop = false;
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
             __syncthreads();  // the window is there, and the one before is done with
-            fetch(w + 2 * kChaseWin, buf == 0 ? 2 : buf - 1);
+            fetch(w + kChaseWin, buf ^ 1);
             if (t == 0) {
                 int g = S.g;
                 int q = (int)(S.p - w);
@@ -545,7 +585,7 @@ __global__ void __launch_bounds__(kChaseThreads) dec_chase_kernel(const DecBlock
                         br.init(D.src, D.src_len);
                         br.seek(w + q);
                         for (int k = 0; k < 50; k++)
-                            if (huff_symbol(br, T.lut[tb], T, tb) < 0) { S.status = br.err ? DEC_TRUNC : DEC_BAD_DATA; break; }
+                            if (huff_symbol(br, T.lut[tb], *reinterpret_cast<const Canon *>(T.first), T, tb) < 0) { S.status = br.err ? DEC_TRUNC : DEC_BAD_DATA; break; }
                         d = (int)(br.tell() - (w + q));
                         if (S.status != DEC_OK) { g = last; break; }
                     }
@@ -577,7 +617,7 @@ __global__ void __launch_bounds__(kChaseThreads) dec_chase_kernel(const DecBlock
     const int tb = S.sel[last], alpha = M.alpha;
     gofs[last] = (int32_t)S.p;
     for (int k = 0; k < 50; k++) {
-        const int sym = huff_symbol(br, T.lut[tb], T, tb);
+        const int sym = huff_symbol(br, T.lut[tb], *reinterpret_cast<const Canon *>(T.first), T, tb);
         if (sym < 0) { M.status = br.err ? DEC_TRUNC : DEC_BAD_DATA; return; }
         if (sym == alpha - 1) {
             M.nsym = last * 50 + k + 1;
@@ -597,6 +637,7 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
                                                                  uint16_t *__restrict__ sym_all) {
     __shared__ __align__(16) uint16_t lut[kMaxGroups][1 << 10];
     __shared__ __align__(16) uint16_t out[kSymGroups * 50];
+    __shared__ Canon C;
     const int b = blockIdx.y, t = threadIdx.x;
     DecMeta &M = meta[b];
     if (__syncthreads_or(M.status != DEC_OK)) return;  // one answer for the CTA: another one may set it meanwhile
@@ -606,6 +647,7 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
     const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
     for (int i = t; i < M.n_groups * 128; i += kSymGroups)
         reinterpret_cast<uint4 *>(lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.lut) + i);
+    for (int i = t; i < 3 * kMaxGroups * 22; i += kSymGroups) (&C.first[0][0])[i] = (&T.first[0][0])[i];
     __syncthreads();
     const int g = g0 + t;
     if (g * 50 < ns) {
@@ -615,7 +657,7 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
         const int tb = sel_all[(size_t)b * kMaxSelectors + g], cnt = min(50, ns - g * 50);
         bool bad = false;
         for (int k = 0; k < cnt; k++) {
-            const int sym = huff_symbol(br, lut[tb], T, tb);
+            const int sym = huff_symbol(br, lut[tb], C, T, tb);
             bad |= sym < 0 || (sym == eob) != (g * 50 + k == ns - 1);  // EOB is the last symbol, and only that
             out[t * 50 + k] = (uint16_t)sym;
         }
@@ -634,14 +676,16 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
 // word i of thread t at [i][t]; moving entry j to the front shifts the words
 // below it by a byte.
 constexpr int kSegThreadsM = 128;
-constexpr int kSegs = 6 * kSegThreadsM;
+constexpr int kSegs = 24 * kSegThreadsM;
+constexpr int kSegGroup = 48, kSegGroups = kSegs / kSegGroup;  // 64 groups
 
 struct SegInfo {
     int32_t len, status, off;
 };
 // a block's slot in the segment buffer: permutations, start lists, records
-constexpr size_t kSegPerm = 0, kSegList = (size_t)kSegs * 256, kSegInfo = 2 * (size_t)kSegs * 256;
-static_assert(kSegInfo + kSegs * sizeof(SegInfo) <= sizeof(int32_t) * (size_t)kBlockCap, "segment records fit a block's slot");
+constexpr size_t kSegPerm = 0, kSegList = (size_t)kSegs * 256, kSegInfo = 2 * (size_t)kSegs * 256,
+                 kGroupPerm = kSegInfo + kSegs * sizeof(SegInfo);
+static_assert(kGroupPerm + kSegGroups * 256 <= sizeof(int32_t) * (size_t)kBlockCap, "segment records fit a block's slot");
 
 // PASS 0: the permutation of list positions and the output length; PASS 1:
 // the output bytes from the segment's starting list.
@@ -741,13 +785,34 @@ __global__ void __launch_bounds__(kSegThreadsM) dec_mtf_kernel(DecMeta *__restri
     }
 }
 
-// One CTA per block: the list at every segment's start (byte values) and the
-// output offsets.
-__global__ void __launch_bounds__(256) dec_chain_kernel(DecMeta *__restrict__ meta, const DecTab *__restrict__ tabs, size_t tab_stride,
-                                                        uint8_t *__restrict__ seg_all) {
-    constexpr int kAhead = 32, PER = kSegs / 256;
-    __shared__ __align__(16) uint8_t perm[2][kAhead * 256];
-    __shared__ uint8_t list[2][256];
+// The lists at the segments' starts. A segment takes the list entry at
+// position perm[q] to position q, so the segments compose as gathers: per
+// group of 48 the whole group's permutation, per block the list at every
+// group's start (and the segments' output offsets), per group the list at
+// every segment's start. One after the other over 3072 segments it would be
+// 0.2 ms.
+__global__ void __launch_bounds__(256) dec_seg_group_kernel(const DecMeta *__restrict__ meta, uint8_t *__restrict__ seg_all) {
+    __shared__ __align__(16) uint8_t perm[kSegGroup * 256];
+    __shared__ uint8_t cur[2][256];
+    const int b = blockIdx.y, g = blockIdx.x, t = threadIdx.x;
+    if (meta[b].status != DEC_OK) return;
+    uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
+    const uint4 *in = reinterpret_cast<const uint4 *>(slot + kSegPerm + (size_t)g * kSegGroup * 256);
+    for (int i = t; i < kSegGroup * 16; i += 256) reinterpret_cast<uint4 *>(perm)[i] = in[i];
+    cur[0][t] = (uint8_t)t;
+    __syncthreads();
+    for (int k = 0; k < kSegGroup; k++) {
+        cur[(k & 1) ^ 1][t] = cur[k & 1][perm[k * 256 + t]];
+        __syncthreads();
+    }
+    slot[kGroupPerm + g * 256 + t] = cur[kSegGroup & 1][t];
+}
+
+__global__ void __launch_bounds__(256) dec_seg_chain_kernel(DecMeta *__restrict__ meta, const DecTab *__restrict__ tabs,
+                                                            size_t tab_stride, uint8_t *__restrict__ seg_all) {
+    constexpr int PER = kSegs / 256;
+    __shared__ __align__(16) uint8_t perm[kSegGroups * 256];
+    __shared__ uint8_t cur[2][256];
     __shared__ int sh[33];
     const int b = blockIdx.x, t = threadIdx.x;
     DecMeta &M = meta[b];
@@ -755,43 +820,55 @@ __global__ void __launch_bounds__(256) dec_chain_kernel(DecMeta *__restrict__ me
     const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
     uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
     SegInfo *info = reinterpret_cast<SegInfo *>(slot + kSegInfo);
-    const uint4 *in = reinterpret_cast<const uint4 *>(slot + kSegPerm);
-    uint8_t *lists = slot + kSegList;
-    // output offsets
-    int c[PER], sum = 0, st = DEC_OK;
+    uint4 *groups = reinterpret_cast<uint4 *>(slot + kGroupPerm);
+    for (int i = t; i < kSegGroups * 16; i += 256) reinterpret_cast<uint4 *>(perm)[i] = groups[i];
+    // output offsets; a segment has at most block_max bytes, so the sum of
+    // 3072 lengths fits 32 bits unsigned
+    uint32_t c[PER], sum = 0;
+    bool bad = false;
 #pragma unroll
     for (int i = 0; i < PER; i++) {
         const SegInfo I = info[t * PER + i];
-        c[i] = I.len;
-        sum += min(I.len, kBlockCap);  // at most 768 x 2^20: no overflow
-        if (I.status != DEC_OK) st = I.status;
+        c[i] = (uint32_t)I.len;
+        sum += c[i];
+        bad |= I.status != DEC_OK;
     }
-    int total;
-    int off = block_excl_sum<int>(sum, sh, &total);
-#pragma unroll
-    for (int i = 0; i < PER; i++) {
-        info[t * PER + i].off = off;
-        off += c[i];
-    }
-    const int bad = __syncthreads_or(st != DEC_OK);
-    if (bad || total > M.block_max || total > kBlockCap || M.orig >= total) {
-        if (t == 0) M.status = bad ? DEC_BAD_DATA : M.orig >= total && total <= M.block_max ? DEC_BAD_ORIG : DEC_OVERFLOW;
+    uint32_t total;
+    uint32_t off = block_excl_sum<uint32_t>(sum, reinterpret_cast<uint32_t *>(sh), &total);
+    if (__syncthreads_or(bad) || total > (uint32_t)M.block_max || total > (uint32_t)kBlockCap || (uint32_t)M.orig >= total) {
+        if (t == 0) M.status = total <= (uint32_t)M.block_max && (uint32_t)M.orig >= total ? DEC_BAD_ORIG : DEC_BAD_DATA;
         return;
     }
-    if (t == 0) M.m = total;
-    list[0][t] = t < M.n_in_use ? T.seq_to_unseq[t] : (uint8_t)0;
-    for (int i = t; i < kAhead * 16; i += 256) reinterpret_cast<uint4 *>(perm[0])[i] = in[i];
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        info[t * PER + i].off = (int32_t)off;
+        off += c[i];
+    }
+    if (t == 0) M.m = (int32_t)total;
+    cur[0][t] = t < M.n_in_use ? T.seq_to_unseq[t] : (uint8_t)0;
     __syncthreads();
-    for (int s0 = 0; s0 < kSegs; s0 += kAhead) {
-        const int buf = (s0 / kAhead) & 1;
-        if (s0 + kAhead < kSegs)
-            for (int i = t; i < kAhead * 16; i += 256) reinterpret_cast<uint4 *>(perm[buf ^ 1])[i] = in[(s0 + kAhead) * 16 + i];
-        for (int k = 0; k < kAhead; k++) {
-            const uint8_t v = list[k & 1][t];
-            lists[(size_t)(s0 + k) * 256 + t] = v;
-            list[(k & 1) ^ 1][t] = list[k & 1][perm[buf][k * 256 + t]];
-            __syncthreads();
-        }
+    for (int k = 0; k < kSegGroups; k++) {
+        slot[kGroupPerm + k * 256 + t] = cur[k & 1][t];  // the group's permutation is in shared memory
+        cur[(k & 1) ^ 1][t] = cur[k & 1][perm[k * 256 + t]];
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) dec_seg_lists_kernel(const DecMeta *__restrict__ meta, uint8_t *__restrict__ seg_all) {
+    __shared__ __align__(16) uint8_t perm[kSegGroup * 256];
+    __shared__ uint8_t cur[2][256];
+    const int b = blockIdx.y, g = blockIdx.x, t = threadIdx.x;
+    if (meta[b].status != DEC_OK) return;
+    uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
+    const uint4 *in = reinterpret_cast<const uint4 *>(slot + kSegPerm + (size_t)g * kSegGroup * 256);
+    for (int i = t; i < kSegGroup * 16; i += 256) reinterpret_cast<uint4 *>(perm)[i] = in[i];
+    cur[0][t] = slot[kGroupPerm + g * 256 + t];
+    __syncthreads();
+    uint8_t *lists = slot + kSegList + (size_t)g * kSegGroup * 256;
+    for (int k = 0; k < kSegGroup; k++) {
+        lists[k * 256 + t] = cur[k & 1][t];
+        cur[(k & 1) ^ 1][t] = cur[k & 1][perm[k * 256 + t]];
+        __syncthreads();
     }
 }
 
@@ -1119,7 +1196,7 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
     for (int b = 0; b < nblocks; b++)
         if (h_blocks[b].src_len * 8 > max_bits) max_bits = h_blocks[b].src_len * 8;
     dec_header_kernel<<<nblocks, kHdrThreads, 0, s>>>(blocks, meta, tabs, ts, ws.sel, ws.val);
-    int launches = 14;
+    int launches = 16;
     for (int64_t r0 = 0; r0 < max_bits; r0 += kJRange, launches += 2) {
         const int64_t n = max_bits - r0 < kJRange ? max_bits - r0 : kJRange;
         dec_jump_kernel<<<dim3((unsigned)((n + kJTile - 1) / kJTile), nblocks), kJThreads, sizeof(JumpSmem), s>>>(
@@ -1130,7 +1207,9 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
                                                                                                           ws.val, ws.sym);
     const dim3 seg_grid(kSegs / kSegThreadsM, nblocks), tiles(kTilesPerBlock, nblocks), walkers((kWalkMax + 255) / 256, nblocks);
     dec_mtf_kernel<0><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
-    dec_chain_kernel<<<nblocks, 256, 0, s>>>(meta, tabs, ts, segs);
+    dec_seg_group_kernel<<<dim3(kSegGroups, nblocks), 256, 0, s>>>(meta, segs);
+    dec_seg_chain_kernel<<<nblocks, 256, 0, s>>>(meta, tabs, ts, segs);
+    dec_seg_lists_kernel<<<dim3(kSegGroups, nblocks), 256, 0, s>>>(meta, segs);
     dec_mtf_kernel<1><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
     dec_lf_count_kernel<<<tiles, kLfThreads, 0, s>>>(meta, ws.bwt, hist);
     dec_lf_scan_kernel<<<nblocks, 256, 0, s>>>(meta, hist);
