@@ -34,14 +34,23 @@ __device__ __forceinline__ int32_t jf_pred(int f, int32_t A, int32_t B, int32_t 
     default: return 0;
     }
 }
-__device__ __forceinline__ int32_t g_pred(int f, int row, int col, int32_t A, int32_t B, int32_t C) {
-    if (row == 0) return col == 0 ? 0 : A;
-    if (col == 0) return B;
-    return jf_pred(f, A, B, C);
+// The 2-D grid rule (origin 0, first row from the left, first column from the
+// top) without a case per function: with equal neighbours every function
+// gives their value.
+__device__ __forceinline__ void grid_edges(bool top, bool left, int32_t &A, int32_t &B, int32_t &C) {
+    if (left) A = C = top ? 0 : B;
+    if (top) B = C = A;
 }
 __device__ __forceinline__ uint16_t zz16(int32_t e) {
     const int32_t s = (int32_t)(int16_t)(uint16_t)(uint32_t)e;
     return (uint16_t)(((s << 1) ^ (s >> 31)) & 0xFFFF);
+}
+
+// Two 16-bit residuals to their zigzag symbols.
+__device__ __forceinline__ uint32_t zz16x2(uint32_t w) {
+    uint32_t m;
+    asm("prmt.b32 %0, %1, 0, 0xbb99;" : "=r"(m) : "r"(w));  // 0xffff for a negative one
+    return ((w << 1) & 0xfffefffeu) ^ m;
 }
 
 // Division by a per-CTA constant d (1 <= d < 2^16) as a multiply-high by
@@ -56,26 +65,51 @@ struct DivU16 {
     __device__ __forceinline__ uint32_t mod(uint32_t n) const { return n - div(n) * d; }
 };
 
+// The tile in shared memory: 2p rows of tc cells, the halo lenslet's columns
+// and then, from cell pad, those of the tile's ts lenslets. pad, tc and the
+// symbol planes' rows of out_tc cells are multiples of 8 cells, so that 8
+// symbols of a row are one 16-byte load.
+struct EmitTile {
+    int pad, tc, out_tc;
+    __host__ __device__ EmitTile(int p, int ts) : pad((p + 7) & ~7), tc(pad + ((ts * p + 7) & ~7)), out_tc((ts * p + 7) & ~7) {}
+};
+
+static size_t emit_smem(int p, int ts, int nslots, int tc, int out_tc) {
+    const size_t cells = (size_t)(2 * p) * (size_t)tc, outpx = (size_t)p * (size_t)out_tc;
+    return cells * 2 * (size_t)(1 + nslots) + outpx * 2 * (size_t)(nslots > 0 ? nslots : 1) + 256;
+}
+// The tile without its padding, which the choice of the tile's width goes by.
 // nslots bounds both the residual fields (f with an intra or phase-space
 // candidate) and the symbol planes (f with an inter or phase-space candidate).
-size_t emit_all_smem_bytes(int p, int ts, int nslots) {
-    const size_t cells = (size_t)(2 * p) * (size_t)((ts + 1) * p);
-    const size_t outpx = (size_t)p * (size_t)(ts * p);
-    return cells * 2 * (size_t)(1 + nslots) + outpx * 2 * (size_t)(nslots > 0 ? nslots : 1) + 256;
+// What fits 200 KB fits 220 KB with the padding, for every pitch, width and
+// nslots.
+size_t emit_all_smem_bytes(int p, int ts, int nslots) { return emit_smem(p, ts, nslots, (ts + 1) * p, ts * p); }
+
+// body(on) with on(f) telling whether f is in the set; for the default
+// functions 4..7 a compile-time answer (a test per pixel and function else).
+template <class Body>
+__device__ __forceinline__ void with_functions(uint32_t set, Body body) {
+    if (set == 0xF0u) body([](int f) { return f >= 4; });
+    else body([set](int f) { return ((set >> f) & 1u) != 0u; });
 }
 
 // grid (tiles, frames, kind); kind 0 = raw base field, 1 = temporal difference.
 // Symbols do not depend on the ordering, only their positions do: per
-// predictor function f, the intra / inter / phase-space symbols of the
+// predictor function f, the intra / inter / phase-space residuals of the
 // tile's pixels are computed once into shared memory (thread = pixel column,
 // p rows each), then every candidate of that f is written from there in
 // its ordering, consecutive threads on consecutive output positions.
+// Bound by instructions, 26 candidates a pixel: edges without a case per
+// function, the default functions without a test each, 8 cells a load and
+// two symbols a zigzag took 12 2040 x 2040 frames from 1835 to 1482 us and a
+// 195 x 195 one from 41 to 35 us (more threads a CTA are slower: fewer CTAs
+// fit).
 // PL: the candidate set holds planar-layout ids (otherwise their stores
 // compile away).
 template <int kind, bool PL>
 __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ frames, const uint8_t *__restrict__ cand,
                                               uint8_t *__restrict__ cstream, int64_t cslot, int kmax, int TS,
-                                              uint8_t *esm, int16_t (*slot_of)[3][2][2], int8_t *eslot_of) {
+                                              uint8_t *esm, int16_t (*slot_of)[3][2][2]) {
     const int fi = blockIdx.y;
     const JudgeFrame &J = frames[fi];
     const FrameDev F = J.F;
@@ -84,9 +118,10 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
     const int tiles_s = (Nx + TS - 1) / TS;
     if ((int)blockIdx.x >= Ny * tiles_s) return;
     const int t = blockIdx.x / tiles_s, s0 = (blockIdx.x % tiles_s) * TS, ns = min(TS, Nx - s0);
-    const int TR = 2 * p, TC = (TS + 1) * p, ncols = (ns + 1) * p;
-    const int cells = TR * TC;
-    const int nco = ns * p, npx = p * nco;  // output columns and pixels of the tile
+    const EmitTile tile(p, TS);
+    const int TR = 2 * p, TC = tile.tc, PC = tile.pad, OC = tile.out_tc, ncols = (ns + 1) * p;
+    const int cells = TR * TC, lx0 = PC - p;  // cell of the halo's first column
+    const int nco = ns * p, npx = p * OC;     // output columns of the tile, cells of a symbol plane
     uint32_t fset = 0, fany = 0;
     int nc = 0;
     for (int k = 0; k < J.K; k++) {
@@ -104,7 +139,6 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
     uint16_t *Sy = reinterpret_cast<uint16_t *>(E + (size_t)nslots * cells);  // [3][npx]
     if (threadIdx.x == 0) {
         for (int i = 0; i < 96; i++) (&slot_of[0][0][0][0])[i] = -1;
-        for (int f = 0; f < 8; f++) eslot_of[f] = (int8_t)__popc(fset & ((1u << f) - 1u));
         for (int k = 0; k < J.K; k++) {
             const int id = cand[J.cand_off + k];
             if (((id >> 7) & 1) != kind || !cand_on(J, id)) continue;
@@ -136,7 +170,7 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
                 if (lx < 0 || lx >= ncols) continue;
                 uint32_t v = (aw[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
                 if (kind) v = (v - ((bw[j >> 1] >> (16 * (j & 1))) & 0xFFFFu)) & 0xFFFFu;
-                Fb[ly * TC + lx] = (uint16_t)v;
+                Fb[ly * TC + lx0 + lx] = (uint16_t)v;
             }
         }
     } else {
@@ -150,27 +184,33 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
                     v = __ldg(F.X + k);
                     if (kind) v = (v - (uint32_t)__ldg(F.prev + k)) & 0xFFFFu;
                 }
-                Fb[ly * TC + lx] = (uint16_t)v;
+                Fb[ly * TC + lx0 + lx] = (uint16_t)v;
             }
         }
     }
     __syncthreads();
 #define FVAL(idx) (kind ? (int32_t)(int16_t)Fb[idx] : (int32_t)Fb[idx])  // kind is a template constant
-    // intra residual fields (signed 16-bit) for every f in use
-    for (int lx = threadIdx.x; lx < ncols; lx += blockDim.x) {
-        const int u = (int)div_p.mod((uint32_t)lx);
-        for (int ly = 0; ly < TR; ly++) {
-            const int v = ly < p ? ly : ly - p;  // TR = 2p rows
-            const int idx = ly * TC + lx;
-            const int32_t Xv = FVAL(idx);
-            const int32_t A = u > 0 ? FVAL(idx - 1) : 0;
-            const int32_t B = v > 0 ? FVAL(idx - TC) : 0;
-            const int32_t C = (u > 0 && v > 0) ? FVAL(idx - TC - 1) : 0;
+    int e_of[8];  // first cell of f's residual field
 #pragma unroll
-            for (int f = 1; f < 8; f++)
-                if (fset & (1u << f)) E[(size_t)eslot_of[f] * cells + idx] = (int16_t)(Xv - g_pred(f, v, u, A, B, C));
+    for (int f = 0; f < 8; f++) e_of[f] = __popc(fset & ((1u << f) - 1u)) * cells;
+    // intra residual fields (signed 16-bit) for every f in use
+    with_functions(fset, [&](auto on) {
+        for (int lx = threadIdx.x; lx < ncols; lx += blockDim.x) {
+            const int u = (int)div_p.mod((uint32_t)lx);
+            for (int ly = 0; ly < TR; ly++) {
+                const int v = ly < p ? ly : ly - p;  // TR = 2p rows
+                const int idx = ly * TC + lx0 + lx;
+                const int32_t Xv = FVAL(idx);
+                int32_t A = u > 0 ? FVAL(idx - 1) : 0;
+                int32_t B = v > 0 ? FVAL(idx - TC) : 0;
+                int32_t C = (u > 0 && v > 0) ? FVAL(idx - TC - 1) : 0;
+                grid_edges(v == 0, u == 0, A, B, C);
+#pragma unroll
+                for (int f = 1; f < 8; f++)
+                    if (on(f)) E[e_of[f] + idx] = (int16_t)(Xv - jf_pred(f, A, B, C));
+            }
         }
-    }
+    });
     __syncthreads();
     uint8_t *base8 = cstream + (size_t)fi * kmax * (size_t)cslot;
     uint16_t *base = reinterpret_cast<uint16_t *>(base8);
@@ -195,12 +235,14 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
         hi[0] = (uint8_t)(v >> 8);
         hi[nsym] = (uint8_t)v;
     };
-    // Writes the symbols get(r, c) of the tile's output pixels (row r of the
-    // lenslet row, column c) in raw order to candidate k0 ((lo, hi) layout)
-    // and k0p (planar layout), and in view-major order (view v = r, u = c mod
-    // p, lenslet s0 + c / p) to k1 and k1p; consecutive threads on
-    // consecutive output positions, every symbol computed once.
-    auto write_both = [&](int k0, int k1, int k0p, int k1p, auto get) {
+    // Writes the symbols of the tile's output pixels (row r of the lenslet
+    // row, column c; fin(two of the values at src + r * pitch + c, packed))
+    // in raw order to candidate k0 ((lo, hi) layout) and k0p (planar layout),
+    // and in view-major order (view v = r, u = c mod p, lenslet s0 + c / p)
+    // to k1 and k1p; consecutive threads on consecutive output positions.
+    auto write_both = [&](int k0, int k1, int k0p, int k1p, const uint16_t *src, int pitch, auto fin) {
+        auto cell = [&](int r, int c) -> uint32_t { return src[r * pitch + c]; };
+        auto get = [&](int r, int c) -> uint32_t { return fin(cell(r, c)) & 0xFFFFu; };
         if (k0 >= 0 || k0p >= 0) {
             const size_t i0 = (size_t)(t * p) * W + (size_t)s0 * p;  // symbol index of the tile's first pixel
             uint16_t *dst = k0 >= 0 ? base + (size_t)k0 * cslot16 + i0 : nullptr;
@@ -209,11 +251,8 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
                 const int h = nco >> 3;
                 for (int q = threadIdx.x; q < p * h; q += blockDim.x) {
                     const int r = (int)div_h8.div((uint32_t)q), c8 = 8 * (q - r * h);
-                    uint4 o;
-                    o.x = (uint32_t)get(r, c8) | ((uint32_t)get(r, c8 + 1) << 16);
-                    o.y = (uint32_t)get(r, c8 + 2) | ((uint32_t)get(r, c8 + 3) << 16);
-                    o.z = (uint32_t)get(r, c8 + 4) | ((uint32_t)get(r, c8 + 5) << 16);
-                    o.w = (uint32_t)get(r, c8 + 6) | ((uint32_t)get(r, c8 + 7) << 16);
+                    uint4 o = *reinterpret_cast<const uint4 *>(src + r * pitch + c8);
+                    o = make_uint4(fin(o.x), fin(o.y), fin(o.z), fin(o.w));
                     if (dst) *reinterpret_cast<uint4 *>(dst + (size_t)r * W + c8) = o;
                     if (dsp) put8(dsp + (size_t)r * W + c8, o);
                 }
@@ -248,10 +287,10 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
                     const int v = (int)div_p.div((uint32_t)vu), u = vu - v * p;
                     const int c = 8 * hh * p + u;
                     uint4 o;
-                    o.x = (uint32_t)get(v, c) | ((uint32_t)get(v, c + p) << 16);
-                    o.y = (uint32_t)get(v, c + 2 * p) | ((uint32_t)get(v, c + 3 * p) << 16);
-                    o.z = (uint32_t)get(v, c + 4 * p) | ((uint32_t)get(v, c + 5 * p) << 16);
-                    o.w = (uint32_t)get(v, c + 6 * p) | ((uint32_t)get(v, c + 7 * p) << 16);
+                    o.x = fin(cell(v, c) | (cell(v, c + p) << 16));
+                    o.y = fin(cell(v, c + 2 * p) | (cell(v, c + 3 * p) << 16));
+                    o.z = fin(cell(v, c + 4 * p) | (cell(v, c + 5 * p) << 16));
+                    o.w = fin(cell(v, c + 6 * p) | (cell(v, c + 7 * p) << 16));
                     const size_t e = (size_t)v * Ny * W + (size_t)u * Nx + 8 * hh;
                     if (dst) *reinterpret_cast<uint4 *>(dst + e) = o;
                     if (dsp) put8(dsp + e, o);
@@ -278,23 +317,17 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
     };
     // raw candidates (no predictor) and intra-lenslet candidates straight from
     // the staged frame and the residual fields
-    if (fany & 1u)
-        write_both(slot_of[0][0][0][0], slot_of[0][0][1][0], slot_of[0][0][0][1], slot_of[0][0][1][1], [&](int r, int c) -> uint16_t {
-            const int32_t Xv = FVAL((p + r) * TC + p + c);
-            return kind ? zz16(Xv) : (uint16_t)Xv;
-        });
-#pragma unroll
-    for (int f = 1; f < 8; f++) {
-        if (!((fset >> f) & 1u) || (slot_of[f][0][0][0] < 0 && slot_of[f][0][1][0] < 0 && slot_of[f][0][0][1] < 0 &&
-                                    slot_of[f][0][1][1] < 0))
-            continue;
-        const int16_t *Ef = E + (size_t)eslot_of[f] * cells;
-        write_both(slot_of[f][0][0][0], slot_of[f][0][1][0], slot_of[f][0][0][1], slot_of[f][0][1][1],
-                   [&](int r, int c) -> uint16_t { return zz16(Ef[(p + r) * TC + p + c]); });
+    auto as_is = [](uint32_t w) { return w; };
+    auto zigzag = [](uint32_t w) { return zz16x2(w); };
+    const int out0 = p * TC + PC;  // cell of the first output pixel
+    if (fany & 1u) {
+        if (kind) write_both(slot_of[0][0][0][0], slot_of[0][0][1][0], slot_of[0][0][0][1], slot_of[0][0][1][1], Fb + out0, TC, zigzag);
+        else write_both(slot_of[0][0][0][0], slot_of[0][0][1][0], slot_of[0][0][0][1], slot_of[0][0][1][1], Fb + out0, TC, as_is);
     }
-    // inter-lenslet candidates of every f in one pass over the pixels, then
-    // the phase-space ones: symbols into planes of Sy, then written out
-    for (int dom = 1; dom <= 2; dom++) {
+    // then per domain the candidates of every f: the intra ones straight from
+    // the residual fields, the inter and phase-space ones by way of symbol
+    // planes, formed in one pass over the pixels
+    for (int dom = 0; dom <= 2; dom++) {
         uint32_t fm = 0;
         int plane[8];
         int np = 0;
@@ -308,42 +341,46 @@ __device__ __forceinline__ void emit_all_body(const JudgeFrame *__restrict__ fra
             }
         }
         if (!fm) continue;
-        for (int c = threadIdx.x; c < nco; c += blockDim.x) {
-            const int sc = (int)div_p.div((uint32_t)c);
-            const int lx = p + c, s = s0 + sc;
-            for (int r = 0; r < p; r++) {
-                const int idx = (p + r) * TC + lx, q = r * nco + c;
-                if (dom == 1) {
-                    const int32_t Xv = FVAL(idx);
-                    const int32_t XA = s > 0 ? FVAL(idx - p) : 0;
-                    const int32_t XB = t > 0 ? FVAL(idx - p * TC) : 0;
-                    const int32_t XC = (s > 0 && t > 0) ? FVAL(idx - p * TC - p) : 0;
+        if (dom) with_functions(fm, [&](auto on) {
+            for (int c = threadIdx.x; c < nco; c += blockDim.x) {
+                const int sc = (int)div_p.div((uint32_t)c);
+                const int lx = PC + c, s = s0 + sc;
+                for (int r = 0; r < p; r++) {
+                    const int idx = (p + r) * TC + lx, q = r * OC + c;
+                    if (dom == 1) {
+                        const int32_t Xv = FVAL(idx);
+                        int32_t XA = s > 0 ? FVAL(idx - p) : 0;
+                        int32_t XB = t > 0 ? FVAL(idx - p * TC) : 0;
+                        int32_t XC = (s > 0 && t > 0) ? FVAL(idx - p * TC - p) : 0;
+                        grid_edges(t == 0, s == 0, XA, XB, XC);
 #pragma unroll
-                    for (int f = 1; f < 8; f++)
-                        if ((fm >> f) & 1u) Sy[(size_t)plane[f] * npx + q] = zz16(Xv - g_pred(f, t, s, XA, XB, XC));
-                } else {
+                        for (int f = 1; f < 8; f++)
+                            if (on(f)) Sy[plane[f] * npx + q] = (uint16_t)(Xv - jf_pred(f, XA, XB, XC));
+                    } else {
 #pragma unroll
-                    for (int f = 1; f < 8; f++) {
-                        if (!((fm >> f) & 1u)) continue;
-                        const int16_t *Ef = E + (size_t)eslot_of[f] * cells;
-                        const int32_t e = Ef[idx];
-                        const int32_t eA = s > 0 ? Ef[idx - p] : 0;
-                        const int32_t eB = t > 0 ? Ef[idx - p * TC] : 0;
-                        const int32_t eC = (s > 0 && t > 0) ? Ef[idx - p * TC - p] : 0;
-                        Sy[(size_t)plane[f] * npx + q] = zz16(e - g_pred(f, t, s, eA, eB, eC));
+                        for (int f = 1; f < 8; f++) {
+                            if (!on(f)) continue;
+                            const int16_t *Ef = E + e_of[f];
+                            const int32_t e = Ef[idx];
+                            int32_t eA = s > 0 ? Ef[idx - p] : 0;
+                            int32_t eB = t > 0 ? Ef[idx - p * TC] : 0;
+                            int32_t eC = (s > 0 && t > 0) ? Ef[idx - p * TC - p] : 0;
+                            grid_edges(t == 0, s == 0, eA, eB, eC);
+                            Sy[plane[f] * npx + q] = (uint16_t)(e - jf_pred(f, eA, eB, eC));
+                        }
                     }
                 }
             }
-        }
-        __syncthreads();
-#pragma unroll
+        });
+        if (dom) __syncthreads();
+        const uint16_t *src = dom ? Sy : reinterpret_cast<const uint16_t *>(E) + out0;
         for (int f = 1; f < 8; f++) {
-            if (!((fm >> f) & 1u)) continue;
-            const uint16_t *src = Sy + (size_t)plane[f] * npx;
-            write_both(slot_of[f][dom][0][0], slot_of[f][dom][1][0], slot_of[f][dom][0][1], slot_of[f][dom][1][1],
-                       [&](int r, int c) -> uint16_t { return src[r * nco + c]; });
+            if ((fm >> f) & 1u)
+                write_both(slot_of[f][dom][0][0], slot_of[f][dom][1][0], slot_of[f][dom][0][1], slot_of[f][dom][1][1], src, dom ? OC : TC,
+                           zigzag);
+            if (dom ? (fm >> f) & 1u : (fset >> f) & 1u) src += dom ? npx : cells;  // the next plane or field
         }
-        __syncthreads();
+        if (dom) __syncthreads();
     }
 #undef FVAL
 }
@@ -354,9 +391,8 @@ __global__ void __launch_bounds__(kEmitThreads) emit_all_kernel(const JudgeFrame
                                                                 int64_t cslot, int kmax, int TS) {
     extern __shared__ __align__(16) uint8_t esm[];
     __shared__ int16_t slot_of[8][3][2][2];  // candidate index for (f, domain, ordering, layout), -1 if absent
-    __shared__ int8_t eslot_of[8];        // intra residual field of f
-    if (blockIdx.z == 0) emit_all_body<0, PL>(frames, cand, cstream, cslot, kmax, TS, esm, slot_of, eslot_of);
-    else emit_all_body<1, PL>(frames, cand, cstream, cslot, kmax, TS, esm, slot_of, eslot_of);
+    if (blockIdx.z == 0) emit_all_body<0, PL>(frames, cand, cstream, cslot, kmax, TS, esm, slot_of);
+    else emit_all_body<1, PL>(frames, cand, cstream, cslot, kmax, TS, esm, slot_of);
 }
 
 // ------------------------------------------------------ pair-chain histogram
@@ -615,7 +651,8 @@ chain_hist_kernel(const JudgeFrame *__restrict__ frames, int nframes, const uint
 
 cudaError_t launch_emit_all(lfc_plan P, const JudgeFrame *d_frames, int nframes, const uint8_t *d_cand, int max_tiles,
                             int TS, int nslots_max, int any_temporal, int max_p) {
-    const size_t smem = emit_all_smem_bytes(max_p, TS, nslots_max);
+    const EmitTile tile(max_p, TS);
+    const size_t smem = emit_smem(max_p, TS, nslots_max, tile.tc, tile.out_tc);
     bool planar = false;
     for (uint8_t id : P->ids_spatial) planar |= id_planar(id) != 0;
     for (uint8_t id : P->ids_temporal) planar |= id_planar(id) != 0;
