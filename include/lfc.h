@@ -161,8 +161,8 @@ size_t lfc_max_compressed_bytes(int32_t width, int32_t height, int32_t block_byt
  * bytes(W_j, H_j, block_bytes); its size goes to d_out_sizes[i].
  *   d_choice    device n ids to use, or NULL to run lfc_judge first.
  *   out_cap     bytes available at d_out; CAPACITY if below the slot sum.
- * The call blocks the host until the stream has finished the BWT rounds
- * (it reads per-round active counts). Errors: INVALID_ARG, CAPACITY, CUDA,
+ * The call blocks the host until the stream has sorted the blocks' rotations
+ * (it reads which blocks are left for passes and doubling rounds). Errors: INVALID_ARG, CAPACITY, CUDA,
  * TIMEOUT (a bounded wait of the suffix sort gave up; see wait_budget_ms). */
 int lfc_compress(lfc_plan plan, const lfc_frame *h_frames, int n, const uint8_t *d_choice,
                  uint8_t *d_out, size_t out_cap, uint64_t *d_out_sizes);
@@ -258,10 +258,12 @@ int lfc_decompress(lfc_plan plan, const uint8_t *const *h_in, const uint64_t *h_
  *   wait_budget_ms          how long one bounded device wait may last
  *                           before the kernel gives up and the call returns
  *                           LFC_ERR_TIMEOUT, 1 .. 60000 (default 1000). The
- *                           suffix sort's radix passes wait on each other
- *                           (every tile waits for the digit counts of the
- *                           block's earlier tiles); such waits always end in
- *                           a correct run, so the budget only bounds a fault.
+ *                           suffix sort's radix passes (only blocks with
+ *                           more equal prefixes than a bucket holds take
+ *                           them) wait on each other: every tile waits for
+ *                           the digit counts of the block's earlier tiles.
+ *                           Such waits always end in a correct run, so the
+ *                           budget only bounds a fault.
  * Errors: INVALID_ARG for values outside these sets. */
 typedef struct {
     int32_t emit_tile_lenslets;
@@ -281,7 +283,8 @@ int lfc_plan_get_tuning(lfc_plan plan, lfc_tuning *tuning);
 int lfc_plan_device_status(lfc_plan plan);
 
 /* Fault injection for tests of the bounded waits (host side: nothing on the
- * GPU faults). LFC_FAULT_SORT_WITHHOLD: in the next suffix sort the first
+ * GPU faults). LFC_FAULT_SORT_WITHHOLD: the next suffix sort sends its first
+ * block to the radix passes, whose first
  * tile of the first block sorts its elements but never publishes its digit
  * counts, so the block's later tiles wait for a flag that nothing sets, give
  * up after the plan's wait budget and the call returns LFC_ERR_TIMEOUT
@@ -304,15 +307,15 @@ enum {
     LFC_STAGE_EMIT,           /* chosen symbol streams */
     LFC_STAGE_CRC,            /* raw-frame and block CRCs */
     LFC_STAGE_RLE1,
-    LFC_STAGE_BWT_SORT8,      /* 8-byte prefix radix sort: the 8 LSD passes */
-    LFC_STAGE_BWT_REFINE,     /* prefix-doubling rounds */
+    LFC_STAGE_BWT_SORT8,      /* rotations scattered into buckets, buckets sorted, ties */
+    LFC_STAGE_BWT_REFINE,     /* flagged blocks only: LSD passes, prefix-doubling rounds */
     LFC_STAGE_BWT_OUT,        /* last column, origin, bytes in use */
     LFC_STAGE_MTF,            /* MTF and RUNA/RUNB coding */
     LFC_STAGE_HUFFMAN,
     LFC_STAGE_PACK,
     LFC_STAGE_CONTAINER,
     LFC_STAGE_JUDGE_EMIT,     /* every candidate stream of the judged frames */
-    LFC_STAGE_BWT_KEYS,       /* prefix keys, byte histograms, sort work items */
+    LFC_STAGE_BWT_KEYS,       /* codes and splitters of every block, bucket counts and starts */
     LFC_NUM_STAGES
 };
 int lfc_plan_set_timing(lfc_plan plan, int enable);

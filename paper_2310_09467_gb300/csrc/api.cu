@@ -258,7 +258,7 @@ static void free_ws(Workspace &w) {
     void *ptrs[] = {w.hist, w.summ, w.chain_first, w.scores, w.choice, w.jframes, w.cand, w.l2tab, w.stream, w.blocks, w.bstate,
                     w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.bcode, w.bcount, w.bcursor, w.bstart, w.bitems, w.bflag, w.tileaux, w.bwt,
                     w.mtfidx, w.mtflists, w.mtfrec, w.mtfreclen, w.mtfpres, w.mtfgrec, w.mtfgpres, w.mtfglen, w.sym, w.freq, w.rfreq, w.sel, w.lens, w.codes, w.packed, w.cstream, w.masks, w.class_ids,
-                    w.act_total, w.block_dst, w.frame_crc, w.crc_part, w.crc_part2, w.chunk_desc, w.dec_tt,
+                    w.act_total, w.block_dst, w.frame_crc, w.crc_part, w.crc_part2, w.chunk_desc,
                     w.hx_frames, w.hx_prev, w.hx_out, w.hx_choice, w.hx_sizes};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -493,7 +493,7 @@ bool capturing(lfc_plan P) {
 // the tuned range), a multiple of 512 bytes: at most 2 s0 when those already
 // make two waves, else up to 32 more, down to 1 KB as long as the segments'
 // summaries fit (one 195 x 195 frame: 26 streams of 76 KB on one warp each took 427
-// us, cut over all SMs 60).
+// us, cut over all SMs 52).
 int chain_range_for(lfc_plan P, const lfc_frame *frames, int nf) {
     const int tuned = P->tune.chain_range_bytes;
     int64_t n_max = 0;

@@ -24,7 +24,9 @@
 // What bounds it: two reads of the bytes, 8 B written and read per rotation
 // and one byte gathered per rotation (L2); against the 8 LSD passes over
 // 12-byte pairs it replaces (192 B per rotation), a rank scatter and two
-// doubling rounds.
+// doubling rounds. 12 2040 x 2040 frames (139 blocks, 99 M rotations): plan
+// 0.04, counts 0.47, scatter 0.73, buckets 1.45 ms and few ties, where keys,
+// passes and rounds took 8.5 ms; one 195 x 195 frame 0.09 ms against 0.26.
 //
 // Blocks this cannot finish are flagged for bwt.cu: a bucket above the
 // largest class's words (kFlagOver: all its words take LSD passes), or groups
@@ -361,6 +363,9 @@ __device__ __forceinline__ uint64_t key_bits(BitWindow &W, const uint4 &v4, cons
 }
 
 // ------------------------------------------------------- count, offsets
+// Words per bucket, a tile per CTA (0.47 ms for 99 M rotations: every
+// position's 16 prefix bits are looked up as the scatter does again; keeping
+// them would cost 2 B written and read per rotation).
 __global__ void __launch_bounds__(kEncThreads) bwt_count_kernel(const BlockState *__restrict__ st, const uint8_t *__restrict__ rle_all,
                                                                 const BwtCode *__restrict__ codes, uint32_t *__restrict__ bcount) {
     __shared__ EncTile E;

@@ -123,7 +123,7 @@ __device__ __forceinline__ void ldm4t(uint32_t (&r)[4], const void *p) {
 // MODE 0: + bias, ReLU.  MODE 1: * (mask[y][x][co] > 0)  (input gradient).
 // Bound by shared memory: a warp's weight fragments serve two rows (16
 // wavefronts per 8 products; one row took 24), and a 16 x 16 tile halves the
-// weights staged per output against 8 x 16: 198 -> 135 us for 32 frames of a
+// weights staged per output against 8 x 16: 198 -> 124 us for 32 frames of a
 // 32-channel layer. The order of a sum's terms is that of the taps and
 // channels, whatever the tile.
 template <int CIN, int MODE>

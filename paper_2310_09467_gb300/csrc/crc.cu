@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(256) crc_chunk_kernel(const CrcChunk *__restri
         // a piece takes as long as its loads do, so several are in flight: 16
         // bytes each where they are aligned, else aligned words joined by a
         // funnel shift (byte loads one after the other took 19 us). Words
-        // that hold a byte of the piece are read whole.
+        // that hold a byte of the range are read whole.
         const uintptr_t at = (uintptr_t)(c.src + start);
         if (start >= 0 && (at & 15) == 0) {
             const uint4 *in = reinterpret_cast<const uint4 *>(at);
@@ -103,7 +103,8 @@ __global__ void __launch_bounds__(256) crc_chunk_kernel(const CrcChunk *__restri
                 const int o = start + 4 * i;  // of the word's first byte; the range begins at 0
                 uint32_t w = 0;
                 if (o + 3 >= 0) {
-                    const uint32_t a = __ldg(in + i), b = sh ? __ldg(in + i + 1) : 0u;
+                    // a word all before the range is not read: it may be another allocation's, or none's
+                    const uint32_t a = o - (int)(at & 3) + 3 >= 0 ? __ldg(in + i) : 0u, b = sh ? __ldg(in + i + 1) : 0u;
                     w = __byte_perm(__funnelshift_r(a, b, sh), 0u, 0x0123);
                     if (o < 0) w &= 0xFFFFFFFFu >> (-8 * o);
                 }

@@ -27,6 +27,8 @@
 //     the rows until it meets another walker's start; the pieces are ranked
 //     along their list by pointer doubling; every walker writes its piece.
 //  7. Inverse RLE1 by tiles from sync points; block CRCs (crc.cu).
+// One 1300 x 1300 frame (5 blocks) takes 2.2 ms, 12 frames of 2040 x 2040
+// (139 blocks) 10.5 ms; with one CTA per block it was 47 and 58 ms.
 #include <climits>
 
 #include "lfc_common.cuh"
@@ -158,6 +160,9 @@ __device__ __forceinline__ int huff_symbol(BitReader &br, const uint16_t *lut, c
 }
 
 // ------------------------------------------------------------- 1. header
+// A CTA per block, 0.17 ms for one frame and 0.20 ms for 139 blocks: bound by
+// the one thread that reads the code lengths, a chain of a few instructions
+// per bit.
 constexpr int kHdrThreads = 512;
 
 // Lists of six tables as nibbles, entry k in bits 4k .. 4k + 3.
@@ -381,7 +386,9 @@ __global__ void __launch_bounds__(kHdrThreads) dec_header_kernel(const DecBlock 
 // lengths of 2, 4, 8 and 16 codes are bytes (0: there are none, or they are
 // too long; such a group is decoded on the chase), four positions a thread:
 // one load and one store of a word, four byte gathers and byte-wise sums a
-// doubling. Bound by shared memory, about 10 accesses per bit and table.
+// doubling. Bound by shared memory, about 10 accesses per bit and table: 139
+// blocks take 3.06 ms (16-bit lengths, two positions a thread and a lookup per
+// table: 6.04), one 1300 x 1300 frame 0.17 ms (0.42).
 constexpr int kJTile = 8192;
 constexpr int kJHalo = 1024;                  // 2 + 16 + 16 + 16 codes: at most 40 + 3 * 254 bits, and the last code's 20
 constexpr int kJSpan = kJTile + kJHalo;
@@ -513,7 +520,9 @@ __global__ void __launch_bounds__(kJThreads, 2) dec_jump_kernel(const DecBlock *
 
 // One CTA per block: thread 0 adds up the groups' lengths, the other warps
 // fetch the next window of them. After the last round also the last group,
-// up to EOB.
+// up to EOB. Bound by that chain and by what one SM can fetch (96 KB a
+// window): 0.73 ms for one 1300 x 1300 frame and 0.94 ms for 139 blocks (with
+// windows of 4096 bits 0.91 and 1.10).
 constexpr int kChaseThreads = 256;
 constexpr int kChaseWin = 8192;  // bits of a window: long enough that its barriers and copies hide behind 56 groups' adds
 constexpr int kChaseBufs = 2;    // one in use, one on its way
@@ -629,6 +638,7 @@ __global__ void __launch_bounds__(kChaseThreads) dec_chase_kernel(const DecBlock
 }
 
 // ---------------------------------------------------------- 3. symbols
+// 0.03 ms for one frame, 0.22 ms for 139 blocks.
 constexpr int kSymGroups = 128;
 
 __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
@@ -688,7 +698,10 @@ constexpr size_t kSegPerm = 0, kSegList = (size_t)kSegs * 256, kSegInfo = 2 * (s
 static_assert(kGroupPerm + kSegGroups * 256 <= sizeof(int32_t) * (size_t)kBlockCap, "segment records fit a block's slot");
 
 // PASS 0: the permutation of list positions and the output length; PASS 1:
-// the output bytes from the segment's starting list.
+// the output bytes from the segment's starting list. One 1300 x 1300 frame
+// takes 0.13 and 0.27 ms, 139 blocks 0.68 and 0.90: a serial chain of shared
+// memory accesses per symbol, so the segments are short (768 of them, one
+// after the other in the chaining, took 0.49 and 1.02, 0.77 and 1.31).
 template <int PASS>
 __global__ void __launch_bounds__(kSegThreadsM) dec_mtf_kernel(DecMeta *__restrict__ meta, const uint16_t *__restrict__ sym_all,
                                                                uint8_t *__restrict__ seg_all, uint8_t *__restrict__ L_all) {
@@ -965,6 +978,9 @@ __global__ void __launch_bounds__(kLfThreads) dec_lf_map_kernel(const DecMeta *_
 }
 
 // ------------------------------------------------------- 6. inverse BWT
+// Bound by the latency of dependent 4-byte gathers from L2, 64 a walker and
+// two walks (the bytes can only be placed once the pieces are ranked): 0.12 +
+// 0.14 ms for one 1300 x 1300 frame, 0.66 + 0.84 ms for 139 blocks.
 constexpr int kWalkStep = 64;                             // rows between walkers
 constexpr int kWalkMax = kBlockCap / kWalkStep + 2;       // walkers of a block
 constexpr uint32_t kRowMask = (1u << 20) - 1u;

@@ -274,7 +274,6 @@ struct Workspace {
     void *chunk_desc = nullptr;        // descriptor staging (CRC chunks, frame tables)
     size_t chunk_desc_bytes = 0;
     // decode
-    uint8_t *dec_tt = nullptr;
 };
 
 }  // namespace lfc
