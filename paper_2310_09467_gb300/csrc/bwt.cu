@@ -390,20 +390,26 @@ __global__ void __launch_bounds__(1024) sort_items_kernel(int32_t *__restrict__ 
 
 // After the radix passes of the kFlagOver blocks: suffix array with the
 // non-head mark (an element whose key equals its predecessor's) in bit 31.
-__global__ void __launch_bounds__(kSortThreads) over_heads_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
+__global__ void __launch_bounds__(kSortThreads) over_heads_kernel(int32_t *__restrict__ rs, const BlockState *__restrict__ st,
                                                                   const uint64_t *__restrict__ K_all, const int32_t *__restrict__ bflag,
+                                                                  const uint8_t *__restrict__ rle_all, const BwtCode *__restrict__ codes,
                                                                   int32_t *__restrict__ sa_all) {
     const int b = blockIdx.y;
     if (rs[kRsAbort] || !(bflag[b] & kFlagOver)) return;
     const int m = st[b].m;
     const uint64_t *K = K_all + (size_t)b * kBlockCap;
+    int depth = kBlockCap;  // bytes the groups' members share at least
     for (int r = 0; r < kPerThread; r++) {
         const int k = blockIdx.x * kTile + r * kSortThreads + threadIdx.x;
-        if (k >= m) return;
+        if (k >= m) break;
         const uint64_t w = K[k];
         const bool tied = k > 0 && (K[k - 1] >> 20) == (w >> 20);
         sa_all[(size_t)b * kBlockCap + k] = (int32_t)(w & kElemMask) | (tied ? (int32_t)0x80000000 : 0);
+        if (tied && (k == 1 || (K[k - 2] >> 20) != (w >> 20)))
+            depth = min(depth, key_depth(rle_all + (size_t)b * kBlockCap, m, codes[b].code, (int)(w & kElemMask)));
     }
+    depth = __reduce_min_sync(LFC_FULL, (unsigned)depth);
+    if ((threadIdx.x & 31) == 0 && depth < kBlockCap) atomicMin(&rs[kRsH], depth);
 }
 
 // Segmented sort of a doubling round. The tied elements of a block are
@@ -734,7 +740,7 @@ radix_sweep_kernel(int pass, int nblocks, int32_t *__restrict__ rs, const BlockS
 // Pass A: per tile, the largest head position and the number of elements
 // that stay tied. Head flags go to flags[] for pass B.
 template <int MODE>
-__global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(const int32_t *__restrict__ rs, const BlockState *__restrict__ st,
+__global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(int32_t *__restrict__ rs, const BlockState *__restrict__ st,
                                                                   const int32_t *__restrict__ bflag,
                                                                   const uint64_t *__restrict__ keys_all, const int32_t *__restrict__ sa_all,
                                                                   const int32_t *__restrict__ actA, const int32_t *__restrict__ actB,
@@ -793,6 +799,14 @@ __global__ void __launch_bounds__(kSortThreads) heads_tile_kernel(const int32_t 
     if (threadIdx.x == 0) {
         int mx = -1, tt = 0;
         for (int i = 0; i < kSortThreads / 32; i++) { mx = max(mx, wm[i]); tt += wt[i]; }
+        // with a head in every half tile no group is longer than a tile, so
+        // the next round's segmented sort takes them all
+        int lower = -1, upper = -1;
+        for (int i = 0; i < kSortThreads / 64; i++) {
+            lower = max(lower, wm[i]);
+            upper = max(upper, wm[kSortThreads / 64 + i]);
+        }
+        if ((tile * kTile + kTile / 2 <= n && lower < 0) || (tile * kTile + kTile <= n && upper < 0)) rs[kRsLongGroup] = 1;
         int32_t *aux = aux_all + ((size_t)b * kTilesPerBlock + tile) * 4;
         aux[0] = mx;
         aux[1] = tt;
@@ -951,6 +965,8 @@ __global__ void commit_round_kernel(BlockState *st, int nblocks) {
 }
 
 __global__ void round_start_kernel(int32_t *rs) {
+    rs[kRsEnter] = rs[kRsTied];
+    rs[kRsLongGroup] = 0;
     rs[kRsTied] = 0;
     rs[kRsTiedMax] = 0;
 }
@@ -1117,7 +1133,7 @@ static void bwt_over(lfc_plan P, cudaStream_t st, int nblocks, int tiles) {
         if (pass & 1) sweep_pass<0>(P, st, nblocks, ctas, pass, ws.keys, ws.keys2);
         else sweep_pass<0>(P, st, nblocks, ctas, pass, ws.keys2, ws.keys);
     }
-    over_heads_kernel<<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys2, ws.bflag, ws.sa);
+    over_heads_kernel<<<grid, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys2, ws.bflag, ws.rle, ws.bcode, ws.sa);
     count_launches(P, 4);
 }
 
@@ -1136,27 +1152,31 @@ static void bwt_heads(lfc_plan P, cudaStream_t st, int nblocks, int tiles) {
 
 // One prefix-doubling round over the tied elements (h and the parity of the
 // active lists come from the round state in device memory).
+// passes: a group may be too long for the segmented sort.
 static void bwt_round(lfc_plan P, cudaStream_t st, int nblocks, int tiles, int max_m, cudaGraphConditionalHandle cond,
-                      int set_cond) {
+                      int set_cond, bool passes) {
     Workspace &ws = P->ws;
     round_start_kernel<<<1, 1, 0, st>>>(ws.act_total);
-    const size_t nd = (size_t)nblocks * kSweepPasses * 256;
-    zero_u32_kernel<<<(unsigned)std::min<size_t>(64, (nd + 255) / 256), 256, 0, st>>>(ws.dhist, nd);
     dim3 g1(tiles, nblocks);
     key40_kernel<<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.val, ws.rank, ws.keys, ws.segbig);
     // groups within their windows: keys -> keys2 directly; blocks with a
     // longer group are flagged and take the 5 LSD passes over bits 20..59 of
     // the words instead: keys -> keys2 -> ... -> keys2
     segsort_kernel<<<g1, kSegThreads, kSegSmem, st>>>(ws.act_total, ws.bstate, ws.keys, ws.keys2, ws.segbig);
-    sweep_digits_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys, ws.dhist, ws.segbig, ws.lbstat,
-                                                        ws.lbstat_words);
-    sort_items_kernel<1><<<1, 1024, 0, st>>>(ws.act_total, ws.bstate, nblocks, ws.segbig);
-    count_launches(P, 6);
-    const int ctas = sweep_ctas(P, nblocks, tiles);
-    for (int pass = 0; pass < 5; pass++) {
-        if (pass & 1) sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys2, ws.keys);
-        else sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys, ws.keys2);
+    if (passes) {
+        const size_t nd = (size_t)nblocks * kSweepPasses * 256;
+        zero_u32_kernel<<<(unsigned)std::min<size_t>(64, (nd + 255) / 256), 256, 0, st>>>(ws.dhist, nd);
+        sweep_digits_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.keys, ws.dhist, ws.segbig, ws.lbstat,
+                                                            ws.lbstat_words);
+        sort_items_kernel<1><<<1, 1024, 0, st>>>(ws.act_total, ws.bstate, nblocks, ws.segbig);
+        const int ctas = sweep_ctas(P, nblocks, tiles);
+        for (int pass = 0; pass < 5; pass++) {
+            if (pass & 1) sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys2, ws.keys);
+            else sweep_pass<1>(P, st, nblocks, ctas, pass, ws.keys, ws.keys2);
+        }
+        count_launches(P, 3);
     }
+    count_launches(P, 3);
     heads_tile_kernel<1><<<g1, kSortThreads, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.keys2, ws.sa, ws.act, ws.act2,
                                                       ws.bwt, ws.tileaux);
     heads_scan_kernel<1><<<nblocks, 256, 0, st>>>(ws.act_total, ws.bstate, ws.bflag, ws.tileaux);
@@ -1243,7 +1263,7 @@ cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m) {
         rounds_cond_kernel<<<1, 1, 0, s>>>(ws.act_total, max_m, rounds);
         e = begin_cond(P, s, rounds, cudaGraphCondTypeWhile, &node, &body);
         if (e != cudaSuccess) return e;
-        bwt_round(P, P->aux_stream, nblocks, tiles, max_m, rounds, 1);
+        bwt_round(P, P->aux_stream, nblocks, tiles, max_m, rounds, 1, true);
         e = end_cond(P, s, &node, &body);
         if (e != cudaSuccess) return e;
         count_launches(P, 2);
@@ -1258,15 +1278,20 @@ cudaError_t launch_bwt(lfc_plan P, int nblocks, int max_m) {
         if (h[kRsFlagged] > 0) {
             if (h[kRsOver] > 0) bwt_over(P, s, nblocks, tiles);
             bwt_heads(P, s, nblocks, tiles);
-            e = read_state();
-            if (e != cudaSuccess) return e;
-            for (int round = 0; h[kRsAbort] == 0 && h[kRsTied] > 0 && h[kRsH] < max_m; round++) {
-                P->bwt_rounds++;
-                P->bwt_tied_total += h[kRsTied];
-                if (round < 32) P->bwt_round_tied[round] += h[kRsTied];
-                bwt_round(P, s, nblocks, (h[kRsTiedMax] + kTile - 1) / kTile, max_m, cudaGraphConditionalHandle{}, 0);
+            // the first round right behind the heads, over every tile (it
+            // does nothing where nothing is tied)
+            int round_tiles = tiles;
+            for (int round = 0;; round++) {
+                bwt_round(P, s, nblocks, round_tiles, max_m, cudaGraphConditionalHandle{}, 0, round == 0 || h[kRsLongGroup] != 0);
                 e = read_state();
                 if (e != cudaSuccess) return e;
+                if (h[kRsAbort] == 0 && h[kRsEnter] > 0 && h[kRsH] / 2 < max_m) {  // round_end doubled h
+                    P->bwt_rounds++;
+                    P->bwt_tied_total += h[kRsEnter];
+                    if (round < 32) P->bwt_round_tied[round] += h[kRsEnter];
+                }
+                if (h[kRsAbort] != 0 || h[kRsTied] == 0 || h[kRsH] >= max_m) break;
+                round_tiles = (h[kRsTiedMax] + kTile - 1) / kTile;
             }
             if (h[kRsAbort] != 0) P->bwt_timed_out = true;
         }

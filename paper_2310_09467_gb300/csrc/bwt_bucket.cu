@@ -53,6 +53,7 @@ constexpr int kBucketThreads[kBucketClasses] = {512, 512, 1024};
 constexpr int kBucketCtas[kBucketClasses] = {2, 2, 1};
 constexpr int kSubBins = 8192;  // 16-bit counters
 constexpr int kSubCost = 256;    // words a word is compared with, on average, up to which counting beats the merge network
+constexpr int64_t kSmallPass = 4 << 20;  // words of a pass below which 8 LSD passes take less than 0.23 ms
 constexpr int kTieGroup = 32;   // longest group ordered by further keys (a warp's lanes)
 constexpr int kTieShort = 4;    // longest one that a single thread orders
 constexpr int kTieRounds = 24;
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState
     if (b == 0 && t == 0) {  // a new suffix sort: no wait has given up, nothing is flagged or queued
         rs[kRsTied] = rs[kRsTiedMax] = rs[kRsAbort] = 0;
         rs[kRsH] = kBlockCap;  // the least depth of the groups left tied, see leave_tied
-        rs[kRsRound] = 0;
+        rs[kRsRound] = rs[kRsLongGroup] = 0;
         rs[kRsFlagged] = rs[kRsOver] = rs[kRsTies] = rs[kRsTiesLong] = 0;
         for (int i = 0; i < kBucketClasses; i++) rs[kRsBucketQueue + i] = rs[kRsBucketItems + i] = 0;
         if (clear_sticky) rs[kRsSticky] = 0;
@@ -394,12 +395,13 @@ __global__ void __launch_bounds__(kEncThreads) bwt_count_kernel(const BlockState
 }
 
 // One CTA per block: bucket starts, scatter cursors, the sort's work lists
-// (one per size class). The pending fault of the test hook sends block 0 to
+// (one per size class); a block with a bucket of more than limit words takes
+// the LSD passes. The pending fault of the test hook sends block 0 to
 // the LSD passes, whose waits it breaks.
 __global__ void __launch_bounds__(256) bwt_offsets_kernel(const BwtCode *__restrict__ codes, const uint32_t *__restrict__ bcount,
                                                           uint32_t *__restrict__ bstart, uint32_t *__restrict__ cursor,
                                                           uint32_t *__restrict__ items_all, size_t items_cap,
-                                                          int32_t *__restrict__ bflag, int32_t *__restrict__ rs) {
+                                                          int32_t *__restrict__ bflag, int32_t *__restrict__ rs, uint32_t limit) {
     constexpr int PER = (kBuckets + 255) / 256;
     __shared__ uint32_t shu[33];
     __shared__ int s_base[kBucketClasses];
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(256) bwt_offsets_kernel(const BwtCode *__restr
         const int k = t * PER + i;
         c[i] = k < nb ? bcount[(size_t)b * kBuckets + k] : 0u;
         sum += c[i];
-        over |= c[i] > (uint32_t)kBucketCap[kBucketClasses - 1];
+        over |= c[i] > limit;
     }
     uint32_t total;
     uint32_t ex = block_excl_sum<uint32_t>(sum, shu, &total);
@@ -429,7 +431,6 @@ __global__ void __launch_bounds__(256) bwt_offsets_kernel(const BwtCode *__restr
     if (__syncthreads_or(over)) {
         if (t == 0) {
             bflag[b] = kFlagOver;
-            atomicMin(&rs[kRsH], kMinDepth);
             atomicAdd(&rs[kRsFlagged], 1);
             atomicAdd(&rs[kRsOver], 1);
         }
@@ -558,20 +559,6 @@ __device__ __forceinline__ uint64_t next_key(const uint8_t *rle, int m, const ui
         if (++pos == m) pos = 0;
     }
     return acc >> (used - kKeyBits);
-}
-
-// Whole codes (bytes) in the key of a rotation.
-__device__ __noinline__ int key_depth(const uint8_t *rle, int m, const uint16_t *code, int idx) {
-    int pos = idx, used = 0, depth = 0;
-    uint32_t tab = kFirst;
-    for (;;) {
-        const uint32_t x = rle[pos];
-        used += (int)(code[tab + x] >> 12);
-        if (used > kKeyBits) return depth;
-        depth++;
-        tab = x ? 256u : 0u;
-        if (++pos == m) pos = 0;
-    }
 }
 
 // Leaves a group of block b tied after depth equal bytes: prefix doubling
@@ -922,13 +909,18 @@ cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph) {
         e = cudaFuncSetAttribute(bwt_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ScatterSmem));
     if (e != cudaSuccess) return e;
     const dim3 grid((max_m + kEncTile - 1) / kEncTile, nblocks);
+    // A bucket of the largest class is 0.23 ms of one CTA (repetitive text has
+    // such buckets); a small pass is sooner done when the blocks with one take
+    // the LSD passes (6 blocks of text of up to 400 000 bytes: 1775 us a call
+    // against 1590; 30 of up to 700 000: 4.4 ms with the class).
+    const int classes = (int64_t)nblocks * max_m < kSmallPass ? 2 : kBucketClasses;
     stage_begin(P, LFC_STAGE_BWT_KEYS);
     // outside graphs the call itself reports a wait that gave up
     bwt_plan_kernel<<<nblocks, kPlanThreads, kPlanSmem, s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcount, ws.bflag, ws.act_total,
                                                              graph ? 0 : 1);
     bwt_count_kernel<<<grid, kEncThreads, 0, s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcount);
     bwt_offsets_kernel<<<nblocks, 256, 0, s>>>(ws.bcode, ws.bcount, ws.bstart, ws.bcursor, ws.bitems, ws.bitems_cap, ws.bflag,
-                                               ws.act_total);
+                                               ws.act_total, (uint32_t)kBucketCap[classes - 1]);
     stage_end(P, LFC_STAGE_BWT_KEYS);
     stage_begin(P, LFC_STAGE_BWT_SORT8);
     bwt_scatter_kernel<<<grid, kEncThreads, sizeof(ScatterSmem), s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcursor, ws.keys2);
@@ -937,12 +929,13 @@ cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph) {
     if (e == cudaSuccess) e = launch_class<0>(P, most);
     // a bucket of a larger class needs a block of more words than the class below holds
     if (e == cudaSuccess && max_m > kBucketCap[0]) e = launch_class<1>(P, most);
-    if (e == cudaSuccess && max_m > kBucketCap[1]) e = launch_class<2>(P, most);
+    if (e == cudaSuccess && max_m > kBucketCap[1] && classes > 2) e = launch_class<2>(P, most);
+    if (e != cudaSuccess) return e;
     bwt_tie_kernel<<<8 * P->sm_count, kTieThreads, 0, s>>>(ws.bstate, ws.rle, ws.bcode, ws.keys,
                                                            (size_t)P->block_cap * kBlockCap, ws.sa, ws.bwt, ws.bflag, ws.act_total);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = cudaGetLastError();
     stage_end(P, LFC_STAGE_BWT_SORT8);
-    count_launches(P, 5 + 1 + (max_m > kBucketCap[0]) + (max_m > kBucketCap[1]));
+    count_launches(P, 5 + 1 + (max_m > kBucketCap[0]) + (max_m > kBucketCap[1] && classes > 2));
     return e;
 }
 

@@ -39,14 +39,14 @@ enum : int {
     kRsTied = 0, kRsTiedMax = 1, kRsH = 2, kRsRound = 3, kRsAbort = 4, kRsFault = 5, kRsQueue = 6, kRsItems = 8,
     kRsSticky = 9, kRsFlagged = 10, kRsOver = 11, kRsBucketQueue = 12, kRsBucketClasses = 3,
     kRsBucketItems = kRsBucketQueue + kRsBucketClasses, kRsTies = kRsBucketItems + kRsBucketClasses,
-    kRsTiesLong = kRsTies + 1, kRsTileOff = kRsTiesLong + 1
+    kRsTiesLong = kRsTies + 1, kRsEnter = kRsTiesLong + 1,
+    kRsLongGroup = kRsEnter + 1, kRsTileOff = kRsLongGroup + 1
 };
 constexpr int kSortCtlHead = kRsTileOff;             // sort state words before the per-block tile counts
-constexpr int kFlagTied = 1, kFlagOver = 2;          // block flags of the bucket sort (bwt_bucket.cu)
+constexpr int kFlagTied = 1, kFlagOver = 2;  // block flags of the bucket sort (bwt_bucket.cu)
 constexpr uint64_t kElemMask = (1u << 20) - 1u;      // rotation start in a sort word, below its key
 constexpr int kCodeMax = 12;                         // longest code of the order-preserving byte code
 constexpr int kKeyBits = 44;                         // code bits in a sort word
-constexpr int kMinDepth = kKeyBits / kCodeMax;       // bytes that rotations with equal keys share at least
 constexpr int kBuckets = 1408;                       // most buckets of a block
 constexpr int kBucketRow = kBuckets + 8;             // bucket starts of a block (one more than buckets)
 
@@ -61,6 +61,20 @@ struct BwtCode {
     uint16_t split[kBuckets];
     int32_t nb, pad[3];
 };
+
+// Whole codes (bytes) in the key of a rotation.
+static __device__ __noinline__ int key_depth(const uint8_t *rle, int m, const uint16_t *code, int idx) {
+    int pos = idx, used = 0, depth = 0;
+    uint32_t tab = 512;  // the first byte's table
+    for (;;) {
+        const uint32_t x = rle[pos];
+        used += (int)(code[tab + x] >> 12);
+        if (used > kKeyBits) return depth;
+        depth++;
+        tab = x ? 256u : 0u;
+        if (++pos == m) pos = 0;
+    }
+}
 static_assert(sizeof(BwtCode) % 16 == 0, "BwtCode rows stay 16-byte aligned");
 
 // ------------------------------------------------------------ warp helpers
