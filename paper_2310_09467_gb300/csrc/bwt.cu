@@ -6,7 +6,8 @@
 // start index, over all blocks of a pass at once. The bucket sort of
 // bwt_bucket.cu finishes almost every block; this file has what is left for
 // the blocks it flags (repetitive data):
-//  1. kFlagOver blocks (a bucket too large for shared memory): their words
+//  1. kFlagOver blocks (a bucket too large for shared memory, or for a small
+//     pass to wait for): their words
 //     (44 key bits above the 20-bit start) take 8 stable LSD passes of 8-bit
 //     digits. A radix pass is one persistent kernel whose CTAs take
 //     4096-element tiles from a device work queue, tile-major over the blocks

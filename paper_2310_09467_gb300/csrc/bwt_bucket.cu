@@ -29,7 +29,8 @@
 // passes and rounds took 8.5 ms; one 195 x 195 frame 0.09 ms against 0.26.
 //
 // Blocks this cannot finish are flagged for bwt.cu: a bucket above the
-// largest class's words (kFlagOver: all its words take LSD passes), or groups
+// largest class's words, in a small pass above the one below (kFlagOver: all
+// its words take LSD passes), or groups
 // longer than kTieGroup or still tied after kTieRounds more keys (kFlagTied:
 // prefix doubling from the bytes the groups share).
 #include <algorithm>

@@ -91,3 +91,35 @@ def test_flagged_blocks_in_a_graph(lfc):
         assert batch.to_bytes() == refs
     batch.close()
     plan.close()
+
+
+def _check(lfc, blocks):
+    import torch
+    plan = lfc.Plan(195, 195, 13, max_frames=24)
+    data = torch.from_numpy(np.frombuffer(b"".join(blocks), dtype=np.uint8).copy()).cuda()
+    sizes = [len(b) for b in blocks]
+    L, ln, orig = plan.bwt_blocks(data, np.cumsum([0] + sizes)[:-1], sizes)
+    L, ln, orig = L.cpu().numpy(), ln.cpu().numpy(), orig.cpu().numpy()
+    for i, b in enumerate(blocks):
+        r = oracle.rle1(b)
+        ref, ref_row = oracle.bwt(r)
+        assert int(ln[i]) == r.size and int(orig[i]) == ref_row, i
+        assert np.array_equal(L[i, :r.size], ref), i
+    plan.close()
+
+
+def test_largest_class_in_a_large_pass(lfc):
+    """24 blocks of at most 195 000 bytes are more than 4 M words, so the
+    bucket of 15 000 words is sorted as one (a small pass takes LSD passes)."""
+    rng = np.random.default_rng(7)
+    _check(lfc, _inputs("class_24576") + [bytes(rng.integers(0, 30, 500 + i, dtype=np.uint8)) for i in range(22)])
+
+
+@pytest.mark.parametrize("copies", [1500, 2100, 4000, 4200, 9000])
+def test_group_lengths_of_the_rounds(lfc, copies):
+    """Groups that stay together for several doubling rounds, around half a
+    tile, a tile and the segmented sort's window: a round takes its radix
+    passes only when a half tile holds no group head."""
+    rng = np.random.default_rng(copies)
+    word = bytes(rng.integers(97, 123, 60, dtype=np.uint8))
+    _check(lfc, [_repeats(rng, word, 3, 63 * copies), bytes(rng.integers(0, 4, 20000, dtype=np.uint8))])
