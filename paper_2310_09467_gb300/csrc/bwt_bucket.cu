@@ -783,7 +783,11 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
 
 // The listed groups: members ordered by further keys, equal ones by start;
 // the pieces still tied are taken up to kTieRounds keys deep. Identical
-// rotations (the whole block agrees) stay in start order. One thread orders a
+// rotations (the whole block agrees) stay in start order; they are marked as
+// tied without a call for prefix doubling, for where a block takes it on
+// account of other groups, rotations that differ only by such a piece have to
+// find it undivided (ordered by the starts of the piece's members, they could
+// come out of start order themselves). One thread orders a
 // group of up to kTieShort members (almost all: pairs), one warp a longer one
 // (a lane per member: the walks over the bytes are the time it takes). The
 // list holds the short groups from its front, the long ones from its end.
@@ -818,7 +822,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
             pend = false;
             for (int p0 = 0; p0 < len;) {
                 const int pl = piece[p0];
-                if (pl == 1) { p0++; continue; }
+                if (pl == 1 || dep[p0] >= m) { p0 += pl; continue; }
                 int d = 0;
                 for (int k = p0; k < p0 + pl; k++) {
                     d = dep[p0];
@@ -831,20 +835,16 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
                 for (int k = p0; k < p0 + pl;) {
                     int q = k + 1;
                     while (q < p0 + pl && (w[q] >> 20) == (w[k] >> 20)) q++;
-                    if (q - k == 1 || d >= m) {
-                        for (int z = k; z < q; z++) piece[z] = 1;
-                    } else {
-                        piece[k] = q - k;
-                        dep[k] = d;
-                        pend = true;
-                    }
+                    piece[k] = q - k;
+                    dep[k] = d;
+                    pend |= q - k > 1 && d < m;
                     k = q;
                 }
                 p0 += pl;
             }
         }
         for (int p0 = 0; p0 < len; p0 += piece[p0]) {
-            if (piece[p0] > 1) leave_tied(bflag, rs, b, dep[p0]);
+            if (piece[p0] > 1 && dep[p0] < m) leave_tied(bflag, rs, b, dep[p0]);
             for (int k = p0; k < p0 + piece[p0]; k++) out(b, m, rle, at + k, w[k], k > p0);
         }
     }
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
         uint64_t w = in ? (uint64_t)(uint32_t)sa_all[(size_t)b * kBlockCap + at + lane] : ~0ull;
         int p0 = in ? 0 : lane, p1 = in ? len : lane + 1, dep = 0;  // the member's piece, the bytes it shares
         for (int round = 0; round < kTieRounds; round++) {
-            const bool act = p1 - p0 > 1;
+            const bool act = p1 - p0 > 1 && dep < m;
             if (!__any_sync(LFC_FULL, act)) break;
             if (act) {
                 const uint32_t idx = (uint32_t)(w & kElemMask);
@@ -873,7 +873,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
             sw[warp][to] = w;
             __syncwarp();
             w = sw[warp][lane];  // a piece's members share dep, wherever they stand
-            const bool head = !act || lane == p0 || (sw[warp][lane - 1] >> 20) != (w >> 20) || dep >= m;
+            const bool head = lane == p0 || (act && (sw[warp][lane - 1] >> 20) != (w >> 20));
             const uint32_t heads = __ballot_sync(LFC_FULL, head);
             if (act) {
                 const uint32_t above = heads & lanemask_gt();
@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
             __syncwarp();
         }
         if (in) {
-            if (p1 - p0 > 1 && lane == p0) leave_tied(bflag, rs, b, dep);
+            if (p1 - p0 > 1 && lane == p0 && dep < m) leave_tied(bflag, rs, b, dep);
             out(b, m, rle, at + lane, w, lane > p0);
         }
     }
