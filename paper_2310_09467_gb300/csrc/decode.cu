@@ -25,7 +25,9 @@
 //     the next row and the row's byte.
 //  6. Inverse BWT: a walker per kWalkStep rows (and one at the origin) follows
 //     the rows until it meets another walker's start; the pieces are ranked
-//     along their list by pointer doubling; every walker writes its piece.
+//     along their list by pointer doubling; every walker writes its piece. The
+//     rows of a block that repeats a shorter string form one cycle per copy:
+//     the origin's is the string, and the block is filled with it.
 //  7. Inverse RLE1 by tiles from sync points; block CRCs (crc.cu).
 // One 1300 x 1300 frame (5 blocks) takes 2.2 ms, 12 frames of 2040 x 2040
 // (139 blocks) 10.5 ms; with one CTA per block it was 47 and 58 ms.
@@ -54,8 +56,9 @@ struct DecMeta {
     int32_t group, bit;   // next group and its bit offset (group chase)
     int32_t nsym;         // symbols up to and including EOB
     int32_t m;            // bytes of the last column
+    int32_t period;       // rows of the origin's cycle: m, or less in a block that repeats a shorter string
     uint32_t stored_crc, crc;
-    int32_t pad[7];
+    int32_t pad[6];
 };
 static_assert(sizeof(DecMeta) == sizeof(BlockState), "the decoder's block records live in the coder's");
 
@@ -1014,7 +1017,11 @@ __global__ void __launch_bounds__(256) dec_walk_kernel(const DecMeta *__restrict
 }
 
 // One CTA per block: where each walker's piece goes, from its distance to
-// the end of the list (walker 0 first, ended by the return to it).
+// the end of the list (walker 0 first, ended by the return to it). The list
+// holds the rows of the origin's cycle. Identical rotations are neighbouring
+// rows in the same order everywhere, so in a block of r copies of a string
+// every copy has a cycle of its own, of m / r rows; a cycle whose length does
+// not divide m is no encoder's. Walkers off the list write nothing.
 struct RankSmem {
     uint32_t d[2][kWalkMax + 1];
     uint16_t nx[2][kWalkMax + 1];
@@ -1042,11 +1049,16 @@ __global__ void __launch_bounds__(1024) dec_rank_kernel(DecMeta *__restrict__ me
         }
         __syncthreads();
     }
-    if (S.d[cur][0] != (uint32_t)m || S.nx[cur][0] != K) {  // not one cycle over all rows
+    const int period = (int)S.d[cur][0];
+    if (S.nx[cur][0] != K || m % period != 0) {
         if (t == 0) M.status = DEC_BAD_WALK;
         return;
     }
-    for (int k = t; k < K; k += 1024) rec[kWalkPos + k] = m - (int)S.d[cur][k];
+    if (t == 0) M.period = period;
+    for (int k = t; k < K; k += 1024) {
+        if (S.nx[cur][k] == K) rec[kWalkPos + k] = period - (int)S.d[cur][k];
+        else rec[kWalkLen + k] = 0;
+    }
 }
 
 __global__ void __launch_bounds__(256) dec_emit_kernel(const DecMeta *__restrict__ meta, const uint32_t *__restrict__ P_all,
@@ -1079,6 +1091,18 @@ __global__ void __launch_bounds__(256) dec_emit_kernel(const DecMeta *__restrict
         }
     }
     for (int q = 0; q < n; q++) blk[at + q] = (uint8_t)(acc >> (8 * ((at & 7) + q)));
+}
+
+// The bytes before the last period of a block that repeats it (any other
+// block is left at once).
+__global__ void __launch_bounds__(256) dec_repeat_kernel(const DecMeta *__restrict__ meta, uint8_t *__restrict__ blk_all) {
+    const int b = blockIdx.y;
+    const DecMeta &M = meta[b];
+    if (M.status != DEC_OK || M.period == M.m) return;
+    const int period = M.period, start = M.m - period;
+    uint8_t *blk = blk_all + (size_t)b * kBlockCap;
+    const int e = min(start, ((int)blockIdx.x + 1) * kTile);
+    for (int i = blockIdx.x * kTile + threadIdx.x; i < e; i += 256) blk[i] = blk[start + i % period];
 }
 
 // ----------------------------------------------------- 7. inverse RLE1
@@ -1212,7 +1236,7 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
     for (int b = 0; b < nblocks; b++)
         if (h_blocks[b].src_len * 8 > max_bits) max_bits = h_blocks[b].src_len * 8;
     dec_header_kernel<<<nblocks, kHdrThreads, 0, s>>>(blocks, meta, tabs, ts, ws.sel, ws.val);
-    int launches = 16;
+    int launches = 17;
     for (int64_t r0 = 0; r0 < max_bits; r0 += kJRange, launches += 2) {
         const int64_t n = max_bits - r0 < kJRange ? max_bits - r0 : kJRange;
         dec_jump_kernel<<<dim3((unsigned)((n + kJTile - 1) / kJTile), nblocks), kJThreads, sizeof(JumpSmem), s>>>(
@@ -1233,6 +1257,7 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
     dec_walk_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2);
     dec_rank_kernel<<<nblocks, 1024, sizeof(RankSmem), s>>>(meta, ws.sa2);
     dec_emit_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2, ws.rle);
+    dec_repeat_kernel<<<tiles, 256, 0, s>>>(meta, ws.rle);
     dec_unrle_count_kernel<<<tiles, kUnThreads, 0, s>>>(meta, ws.rle, ws.tileaux);
     dec_unrle_scan_kernel<<<nblocks, 256, 0, s>>>(blocks, meta, ws.tileaux);
     dec_unrle_write_kernel<<<tiles, kUnThreads, 0, s>>>(blocks, meta, ws.rle, ws.tileaux);

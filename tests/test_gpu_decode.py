@@ -155,6 +155,7 @@ def _content(name):
 
 # Not "runs" in blocks of 900 bytes: a block that repeats a shorter string
 # (here two bytes) is refused, its rows form several cycles.
+# (It was refused when this was written; test_gpu_repeats.py decodes such blocks.)
 @pytest.mark.gpu
 @pytest.mark.parametrize("name,block_bytes", [("one_lenslet", 900), ("one_lenslet", 720000), ("constant", 900),
                                               ("constant", 720000), ("noise", 900), ("noise", 720000), ("runs", 720000),
