@@ -1,5 +1,6 @@
-"""Blocks that repeat a shorter string: the origin row among identical
-rotations, and decoding blocks whose rows form several cycles."""
+"""Blocks that repeat a shorter string, or nearly do: the origin row among
+identical rotations, decoding blocks whose rows form several cycles, and the
+pieces of the inverse BWT where a row keeps its place among 64 k rows."""
 import bz2
 
 import numpy as np
@@ -136,3 +137,32 @@ def test_repeated_blocks_damaged(lfc):
             continue
         assert np.array_equal(got, fr), bit
     plan.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(64, 1406), (256, 1020)])
+def test_nearly_repeated_blocks_are_not_serial(lfc, shape):
+    """One row over and over with one pixel changed: as fast as noise of the
+    same size, give or take (a piece of 100 000 rows and more, walked by one
+    thread, took over 20 times as long)."""
+    import torch
+    rng = np.random.default_rng(29)
+    near = np.tile(rng.integers(0, 4096, shape[1]).astype(np.uint16), (shape[0], 1))
+    near[-1, -1] ^= 1
+    ms = []
+    plan = lfc.Plan(shape[1], shape[0], 2)
+    for fr in (near, rng.integers(0, 4096, shape).astype(np.uint16)):
+        blob = torch.from_numpy(np.frombuffer(oracle.compress_id(fr, 2, 0), dtype=np.uint8).copy()).cuda()
+        out = torch.zeros(shape, dtype=torch.int16, device="cuda")
+        best = float("inf")
+        for _ in range(3):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            plan.decompress([blob], [out])
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        assert np.array_equal(lfc.from_device_frame(out), fr)
+        ms.append(best)
+    plan.close()
+    assert ms[0] < 4 * ms[1], ms
