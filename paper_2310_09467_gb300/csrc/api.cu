@@ -256,7 +256,7 @@ extern "C" int lfc_plan_block_capacity(lfc_plan P) { return P ? P->block_cap : 0
 
 static void free_ws(Workspace &w) {
     void *ptrs[] = {w.hist, w.summ, w.chain_first, w.scores, w.choice, w.jframes, w.cand, w.l2tab, w.stream, w.blocks, w.bstate,
-                    w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.bcode, w.bcount, w.bcursor, w.bstart, w.bitems, w.bflag, w.tileaux, w.bwt,
+                    w.rle, w.sa, w.sa2, w.rank, w.act, w.act2, w.val, w.keys, w.keys2, w.lbstat, w.dhist, w.segbig, w.bcode, w.bcount, w.bcursor, w.bstart, w.bitems, w.bflag, w.bdeep, w.tileaux, w.bwt,
                     w.mtfidx, w.mtflists, w.mtfrec, w.mtfreclen, w.mtfpres, w.mtfgrec, w.mtfgpres, w.mtfglen, w.sym, w.freq, w.rfreq, w.sel, w.lens, w.codes, w.packed, w.cstream, w.masks, w.class_ids,
                     w.act_total, w.block_dst, w.frame_crc, w.crc_part, w.crc_part2, w.chunk_desc,
                     w.hx_frames, w.hx_prev, w.hx_out, w.hx_choice, w.hx_sizes};
@@ -364,6 +364,7 @@ extern "C" int lfc_plan_create(const lfc_config *cfg, void *cuda_stream, lfc_pla
     ws.bitems_cap = (size_t)BC * kBuckets;
     AL(bitems, kRsBucketClasses * ws.bitems_cap);
     AL(bflag, (size_t)BC);
+    AL(bdeep, (size_t)BC);
     AL(tileaux, (size_t)BC * kTilesPerBlock * 4);
     AL(bwt, (size_t)BC * kBlockCap);
     AL(mtfidx, (size_t)BC * kBlockCap);

@@ -31,9 +31,11 @@
 // Blocks this cannot finish are flagged for bwt.cu: a bucket above the
 // largest class's words, in a small pass above the one below (kFlagOver: all
 // its words take LSD passes), or groups
-// longer than kTieGroup or still tied after kTieRounds more keys (kFlagTied:
-// prefix doubling from the bytes the groups share).
+// longer than kTieGroup, still tied after kTieRounds more keys, or of a block
+// with many that are still tied after a few (kFlagTied: prefix doubling from
+// the bytes the groups share).
 #include <algorithm>
+#include <climits>
 
 #include "lfc_common.cuh"
 
@@ -58,6 +60,9 @@ constexpr int64_t kSmallPass = 4 << 20;  // words of a pass below which 8 LSD pa
 constexpr int kTieGroup = 32;   // longest group ordered by further keys (a warp's lanes)
 constexpr int kTieShort = 4;    // longest one that a single thread orders
 constexpr int kTieRounds = 24;
+constexpr int kTieFew = 4;      // keys after which the groups still tied are counted, per block
+constexpr int kTieMany = 64, kTieShare = 256;  // most of them: kTieMany, or one per kTieShare rotations
+constexpr int kTieWaves = 4;    // long groups per warp up to which none is given up
 constexpr int kTables = 3;      // codes: after a zero byte, after another byte, first byte of a key
 constexpr int kFirst = 512;     // where the last one starts
 static_assert(kEncLook >= kKeyBits, "a key reaches at most one byte per bit");
@@ -94,8 +99,8 @@ __device__ __forceinline__ uint32_t alphabetic_code(const uint32_t *cum, int s) 
 
 __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState *__restrict__ st, const uint8_t *__restrict__ rle_all,
                                                                 BwtCode *__restrict__ codes, uint32_t *__restrict__ bcount,
-                                                                int32_t *__restrict__ bflag, int32_t *__restrict__ rs,
-                                                                int clear_sticky) {
+                                                                int32_t *__restrict__ bflag, int32_t *__restrict__ bdeep,
+                                                                int32_t *__restrict__ rs, int clear_sticky) {
     extern __shared__ __align__(16) uint32_t h16[];
     __shared__ uint32_t hist[512], cum[kTables * 256 + 1], code[kTables * 256];
     __shared__ uint32_t shu[33];
@@ -112,7 +117,7 @@ __global__ void __launch_bounds__(kPlanThreads) bwt_plan_kernel(const BlockState
         for (int i = 0; i < kBucketClasses; i++) rs[kRsBucketQueue + i] = rs[kRsBucketItems + i] = 0;
         if (clear_sticky) rs[kRsSticky] = 0;
     }
-    if (t == 0) bflag[b] = 0;
+    if (t == 0) bflag[b] = bdeep[b] = 0;
     if (t < 512) hist[t] = 0;
     for (int i = t; i < kPlanHistWords / 4; i += kPlanThreads) reinterpret_cast<uint4 *>(h16)[i] = make_uint4(0, 0, 0, 0);
     for (int i = t; i < kBuckets; i += kPlanThreads) bcount[(size_t)b * kBuckets + i] = 0;
@@ -564,9 +569,10 @@ __device__ __forceinline__ uint64_t next_key(const uint8_t *rle, int m, const ui
 
 // Leaves a group of block b tied after depth equal bytes: prefix doubling
 // takes the block, from the least depth of any such group.
+__device__ __forceinline__ int ld_flag(const int32_t *p) { return *reinterpret_cast<const volatile int32_t *>(p); }
 __device__ __forceinline__ void leave_tied(int32_t *bflag, int32_t *rs, int b, int depth) {
-    atomicMin(&rs[kRsH], depth);
-    if (atomicOr(&bflag[b], kFlagTied) == 0) atomicAdd(&rs[kRsFlagged], 1);
+    if (ld_flag(rs + kRsH) > depth) atomicMin(&rs[kRsH], depth);
+    if ((ld_flag(bflag + b) & kFlagTied) == 0 && atomicOr(&bflag[b], kFlagTied) == 0) atomicAdd(&rs[kRsFlagged], 1);
 }
 
 struct BucketItem {
@@ -787,16 +793,27 @@ bwt_bucket_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_a
 // tied without a call for prefix doubling, for where a block takes it on
 // account of other groups, rotations that differ only by such a piece have to
 // find it undivided (ordered by the starts of the piece's members, they could
-// come out of start order themselves). One thread orders a
-// group of up to kTieShort members (almost all: pairs), one warp a longer one
-// (a lane per member: the walks over the bytes are the time it takes). The
-// list holds the short groups from its front, the long ones from its end.
+// come out of start order themselves). One thread orders a group of up to
+// kTieShort members (almost all: pairs), one warp a longer one (a lane per
+// member: the walks over the bytes are the time it takes). The list holds the
+// short groups from its front, the long ones from its end.
+// A block with a long repeat takes prefix doubling whatever the number of
+// keys, so its groups are not walked far: groups still tied after kTieFew keys
+// (streams of frames have next to none) are counted per block, and from the
+// count most() on its other groups are left as they are (the long ones by a
+// lane each) and those on their way stop at their next key. 24 blocks of
+// 100 000 bytes take 2.1 ms a call with 8 copies of a string each and 2.4 with
+// 2; with every group walked to kTieRounds it was 7.7 and 4.2. When the whole
+// list is few groups a warp, the walks cost less than the doubling rounds they
+// may save, and none is given up (300 000 bytes of 200-byte strings twice each
+// 0.67 ms, 0.84 without that).
 constexpr int kTieThreads = 128;
 
 __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__restrict__ st, const uint8_t *__restrict__ rle_all,
                                                               const BwtCode *__restrict__ codes, const uint64_t *__restrict__ ties,
                                                               size_t ties_cap, int32_t *__restrict__ sa_all, uint8_t *__restrict__ L_all,
-                                                              int32_t *__restrict__ bflag, int32_t *__restrict__ rs) {
+                                                              int32_t *__restrict__ bflag, int32_t *__restrict__ bdeep,
+                                                              int32_t *__restrict__ rs) {
     __shared__ uint64_t sw[kTieThreads / 32][32];
     const int total = rs[kRsTies], total_long = rs[kRsTiesLong];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -806,8 +823,26 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
         L_all[(size_t)b * kBlockCap + at] = rle[idx == 0 ? m - 1 : idx - 1];
         if (idx == 0) st[b].orig_ptr = at;
     };
+    const int warps = gridDim.x * (kTieThreads / 32), chunk = min(32, (total_long + warps - 1) / warps);
+    const bool few = total <= warps * 32 && total_long <= kTieWaves * warps;
+    auto most = [few](int m) { return few ? INT_MAX : max(kTieMany, m / kTieShare); };
+    auto given_up = [&](uint64_t e) { return ld_flag(bdeep + (e >> 32)) >= most(st[e >> 32].m); };
+    auto leave = [&](uint64_t e) {  // the group stays as it is, tied (one thread)
+        const int b = (int)(e >> 32), len = (int)((e >> 24) & 255u);
+        int32_t *sa = sa_all + (size_t)b * kBlockCap + (e & 0xFFFFFFu);
+        leave_tied(bflag, rs, b, key_depth(rle_all + (size_t)b * kBlockCap, st[b].m, codes[b].code, sa[0]));
+        for (int k = 1; k < len; k++) sa[k] |= (int32_t)(1u << 31);
+    };
+    auto go_on = [&](int b, int m, int round) {  // whether a group is compared by one more key
+        if (!few && round == kTieFew) return ld_flag(bdeep + b) < most(m) && atomicAdd(&bdeep[b], 1) < most(m);
+        return round < kTieRounds && (few || round < kTieFew || (ld_flag(bflag + b) & kFlagTied) == 0);
+    };
     for (int g = blockIdx.x * kTieThreads + threadIdx.x; g < total; g += gridDim.x * kTieThreads) {
         const uint64_t e = ties[g];
+        if (given_up(e)) {
+            leave(e);
+            continue;
+        }
         const int b = (int)(e >> 32), len = (int)((e >> 24) & 255u), at = (int)(e & 0xFFFFFFu);
         const int m = st[b].m;
         const uint8_t *rle = rle_all + (size_t)b * kBlockCap;
@@ -818,7 +853,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
         piece[0] = len;
         dep[0] = 0;
         bool pend = true;
-        for (int round = 0; pend && round < kTieRounds; round++) {
+        for (int round = 0; pend && go_on(b, m, round); round++) {
             pend = false;
             for (int p0 = 0; p0 < len;) {
                 const int pl = piece[p0];
@@ -848,44 +883,54 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
             for (int k = p0; k < p0 + piece[p0]; k++) out(b, m, rle, at + k, w[k], k > p0);
         }
     }
-    for (int g = blockIdx.x * (kTieThreads / 32) + warp; g < total_long; g += gridDim.x * (kTieThreads / 32)) {
-        const uint64_t e = ties[ties_cap - 1 - (size_t)g];
-        const int b = (int)(e >> 32), len = (int)((e >> 24) & 255u), at = (int)(e & 0xFFFFFFu);
-        const int m = st[b].m;
-        const uint8_t *rle = rle_all + (size_t)b * kBlockCap;
-        const uint16_t *code = codes[b].code;
-        const bool in = lane < len;
-        uint64_t w = in ? (uint64_t)(uint32_t)sa_all[(size_t)b * kBlockCap + at + lane] : ~0ull;
-        int p0 = in ? 0 : lane, p1 = in ? len : lane + 1, dep = 0;  // the member's piece, the bytes it shares
-        for (int round = 0; round < kTieRounds; round++) {
-            const bool act = p1 - p0 > 1 && dep < m;
-            if (!__any_sync(LFC_FULL, act)) break;
-            if (act) {
-                const uint32_t idx = (uint32_t)(w & kElemMask);
-                w = (next_key(rle, m, code, (int)idx, dep) << 20) | (uint64_t)idx;
+    for (int g0 = (blockIdx.x * (kTieThreads / 32) + warp) * chunk; g0 < total_long; g0 += warps * chunk) {
+        const int gn = min(chunk, total_long - g0);
+        const uint64_t mine = lane < gn ? ties[ties_cap - 1 - (size_t)(g0 + lane)] : 0ull;
+        for (uint32_t todo = LFC_FULL >> (32 - gn); todo;) {
+            const bool drop = ((todo >> lane) & 1u) && given_up(mine);  // a lane for each of these
+            if (drop) leave(mine);
+            todo &= ~__ballot_sync(LFC_FULL, drop);
+            if (!todo) break;
+            const uint64_t e = __shfl_sync(LFC_FULL, mine, __ffs(todo) - 1);
+            todo &= todo - 1;
+            const int b = (int)(e >> 32), len = (int)((e >> 24) & 255u), at = (int)(e & 0xFFFFFFu);
+            const int m = st[b].m;
+            const uint8_t *rle = rle_all + (size_t)b * kBlockCap;
+            const uint16_t *code = codes[b].code;
+            const bool in = lane < len;
+            uint64_t w = in ? (uint64_t)(uint32_t)sa_all[(size_t)b * kBlockCap + at + lane] : ~0ull;
+            int p0 = in ? 0 : lane, p1 = in ? len : lane + 1, dep = 0;  // the member's piece, the bytes it shares
+            for (int round = 0;; round++) {
+                const bool act = p1 - p0 > 1 && dep < m;
+                if (!__any_sync(LFC_FULL, act)) break;
+                if (!__any_sync(LFC_FULL, lane == 0 && go_on(b, m, round))) break;
+                if (act) {
+                    const uint32_t idx = (uint32_t)(w & kElemMask);
+                    w = (next_key(rle, m, code, (int)idx, dep) << 20) | (uint64_t)idx;
+                }
+                __syncwarp();
+                int to = act ? p0 : lane;
+                for (int j = 0; j < len; j++) {
+                    const uint64_t x = __shfl_sync(LFC_FULL, w, j);
+                    to += act && j >= p0 && j < p1 && x < w;
+                }
+                sw[warp][to] = w;
+                __syncwarp();
+                w = sw[warp][lane];  // a piece's members share dep, wherever they stand
+                const bool head = lane == p0 || (act && (sw[warp][lane - 1] >> 20) != (w >> 20));
+                const uint32_t heads = __ballot_sync(LFC_FULL, head);
+                if (act) {
+                    const uint32_t above = heads & lanemask_gt();
+                    p0 = 31 - __clz(heads & (lanemask_lt() | (1u << lane)));
+                    p1 = above ? __ffs(above) - 1 : 32;
+                    p1 = min(p1, len);
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            int to = act ? p0 : lane;
-            for (int j = 0; j < len; j++) {
-                const uint64_t x = __shfl_sync(LFC_FULL, w, j);
-                to += act && j >= p0 && j < p1 && x < w;
+            if (in) {
+                if (p1 - p0 > 1 && lane == p0 && dep < m) leave_tied(bflag, rs, b, dep);
+                out(b, m, rle, at + lane, w, lane > p0);
             }
-            sw[warp][to] = w;
-            __syncwarp();
-            w = sw[warp][lane];  // a piece's members share dep, wherever they stand
-            const bool head = lane == p0 || (act && (sw[warp][lane - 1] >> 20) != (w >> 20));
-            const uint32_t heads = __ballot_sync(LFC_FULL, head);
-            if (act) {
-                const uint32_t above = heads & lanemask_gt();
-                p0 = 31 - __clz(heads & (lanemask_lt() | (1u << lane)));
-                p1 = above ? __ffs(above) - 1 : 32;
-                p1 = min(p1, len);
-            }
-            __syncwarp();
-        }
-        if (in) {
-            if (p1 - p0 > 1 && lane == p0 && dep < m) leave_tied(bflag, rs, b, dep);
-            out(b, m, rle, at + lane, w, lane > p0);
         }
     }
 }
@@ -917,8 +962,8 @@ cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph) {
     const int classes = (int64_t)nblocks * max_m < kSmallPass ? 2 : kBucketClasses;
     stage_begin(P, LFC_STAGE_BWT_KEYS);
     // outside graphs the call itself reports a wait that gave up
-    bwt_plan_kernel<<<nblocks, kPlanThreads, kPlanSmem, s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcount, ws.bflag, ws.act_total,
-                                                             graph ? 0 : 1);
+    bwt_plan_kernel<<<nblocks, kPlanThreads, kPlanSmem, s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcount, ws.bflag, ws.bdeep,
+                                                             ws.act_total, graph ? 0 : 1);
     bwt_count_kernel<<<grid, kEncThreads, 0, s>>>(ws.bstate, ws.rle, ws.bcode, ws.bcount);
     bwt_offsets_kernel<<<nblocks, 256, 0, s>>>(ws.bcode, ws.bcount, ws.bstart, ws.bcursor, ws.bitems, ws.bitems_cap, ws.bflag,
                                                ws.act_total, (uint32_t)kBucketCap[classes - 1]);
@@ -933,7 +978,8 @@ cudaError_t launch_bucket_sort(lfc_plan P, int nblocks, int max_m, bool graph) {
     if (e == cudaSuccess && max_m > kBucketCap[1] && classes > 2) e = launch_class<2>(P, most);
     if (e != cudaSuccess) return e;
     bwt_tie_kernel<<<8 * P->sm_count, kTieThreads, 0, s>>>(ws.bstate, ws.rle, ws.bcode, ws.keys,
-                                                           (size_t)P->block_cap * kBlockCap, ws.sa, ws.bwt, ws.bflag, ws.act_total);
+                                                           (size_t)P->block_cap * kBlockCap, ws.sa, ws.bwt, ws.bflag, ws.bdeep,
+                                                           ws.act_total);
     e = cudaGetLastError();
     stage_end(P, LFC_STAGE_BWT_SORT8);
     count_launches(P, 5 + 1 + (max_m > kBucketCap[0]) + (max_m > kBucketCap[1] && classes > 2));

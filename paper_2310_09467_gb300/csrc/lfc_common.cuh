@@ -259,6 +259,7 @@ struct Workspace {
     uint32_t *bitems = nullptr;    // bucket work lists, one of bitems_cap entries per size class
     size_t bitems_cap = 0;
     int32_t *bflag = nullptr;      // kFlag* per block
+    int32_t *bdeep = nullptr;      // per block: groups still tied after some further keys (bwt_bucket.cu)
     int32_t *tileaux = nullptr;    // block_cap * kTilesPerBlock * 4
     uint8_t *bwt = nullptr;        // L column
     uint8_t *mtfidx = nullptr;

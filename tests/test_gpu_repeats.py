@@ -1,6 +1,7 @@
 """Blocks that repeat a shorter string, or nearly do: the origin row among
-identical rotations, decoding blocks whose rows form several cycles, and the
-pieces of the inverse BWT where a row keeps its place among 64 k rows."""
+identical rotations, decoding blocks whose rows form several cycles, the
+pieces of the inverse BWT where a row keeps its place among 64 k rows, and the
+suffix sort's time on long repeats."""
 import bz2
 
 import numpy as np
@@ -166,3 +167,42 @@ def test_nearly_repeated_blocks_are_not_serial(lfc, shape):
         ms.append(best)
     plan.close()
     assert ms[0] < 4 * ms[1], ms
+
+
+def _skewed(rng, n):
+    return np.minimum(rng.geometric(0.3, n), 255).astype(np.uint8).tobytes()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("copies", [2, 8, 32])
+def test_long_repeats_encode(lfc, copies):
+    """24 blocks of a string over and over (prefix doubling orders them) take
+    no more than 8 times as long as 24 plain ones, and give the oracle's
+    streams (walking every group of ties far took 14 times as long)."""
+    import torch
+    rng = np.random.default_rng(67)
+
+    def repeats():
+        w = _skewed(rng, 100000 // copies)
+        return b"".join(w + _skewed(rng, 20) for _ in range(copies))
+
+    plan = lfc.Plan(2040, 2040, 15, max_frames=2)
+    ms = []
+    for blocks in ([repeats() for _ in range(24)], [_skewed(rng, 100000) for _ in range(24)]):
+        sizes = [len(b) for b in blocks]
+        offs = [int(v) for v in np.cumsum([0] + sizes[:-1])]
+        data = torch.from_numpy(np.frombuffer(b"".join(blocks), dtype=np.uint8).copy()).cuda()
+        best = float("inf")
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            out, n, stride = plan.bzip2_encode(data, offs, sizes)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+        out, n = out.cpu().numpy(), n.cpu().numpy()
+        for i in (0, 11, 23):
+            assert out[i * stride:i * stride + int(n[i])].tobytes() == oracle.bz2_stream(blocks[i]), i
+    plan.close()
+    assert ms[0] < 8 * ms[1], ms
