@@ -16,7 +16,7 @@
 //     last group, as an encoder writes one selector per group it uses: a
 //     stream with more selectors is rejected as corrupt).
 //  3. Every group's symbols, a thread per group.
-//  4. Inverse RUNA/RUNB and MTF by kSegs segments, a thread each with its
+//  4. Inverse RUNA/RUNB and MTF by up to kSegs segments, a thread each with its
 //     256-byte list in shared memory: a segment's moves permute list
 //     positions whatever the list holds, so the permutations and output
 //     lengths come first, the segment-start lists and offsets are chained,
@@ -31,6 +31,7 @@
 //  7. Inverse RLE1 by tiles from sync points; block CRCs (crc.cu).
 // One 1300 x 1300 frame (5 blocks) takes 2.2 ms, 12 frames of 2040 x 2040
 // (139 blocks) 10.5 ms; with one CTA per block it was 47 and 58 ms.
+#include <algorithm>
 #include <climits>
 
 #include "lfc_common.cuh"
@@ -61,6 +62,12 @@ struct DecMeta {
     int32_t pad[6];
 };
 static_assert(sizeof(DecMeta) == sizeof(BlockState), "the decoder's block records live in the coder's");
+
+// Most bytes of the last column of a block that decodes to `expect` bytes:
+// five of them give at least four. A block has at most one symbol per byte and
+// EOB. What has more decodes to more than the container promises, and the
+// grids of the later steps are sized by it.
+__host__ __device__ inline int column_bound(int expect) { return expect + expect / 4; }
 
 constexpr int kJBits = 12;  // prefix bits of the length table
 struct DecTab {
@@ -657,6 +664,10 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
     const int g0 = blockIdx.x * kSymGroups, ns = M.nsym, eob = M.alpha - 1;
     if (g0 * 50 >= ns) return;
     const DecBlock D = blocks[b];
+    if (ns - 1 > column_bound(D.expect)) {
+        M.status = DEC_BAD_DATA;
+        return;
+    }
     const DecTab &T = *reinterpret_cast<const DecTab *>(reinterpret_cast<const uint8_t *>(tabs) + (size_t)b * tab_stride);
     for (int i = t; i < M.n_groups * 128; i += kSymGroups)
         reinterpret_cast<uint4 *>(lut)[i] = __ldg(reinterpret_cast<const uint4 *>(T.lut) + i);
@@ -689,8 +700,11 @@ __global__ void __launch_bounds__(kSymGroups) dec_symbols_kernel(const DecBlock 
 // word i of thread t at [i][t]; moving entry j to the front shifts the words
 // below it by a byte.
 constexpr int kSegThreadsM = 128;
-constexpr int kSegs = 24 * kSegThreadsM;
+constexpr int kSegs = 24 * kSegThreadsM;                       // most segments of a block
 constexpr int kSegGroup = 48, kSegGroups = kSegs / kSegGroup;  // 64 groups
+constexpr int kSegStep = 384;                                  // segment counts are multiples of 3 CTAs and 8 groups
+constexpr int kSegSyms = 32;  // symbols of a segment, at least, in the largest block there can be
+static_assert(kSegs % kSegStep == 0 && kSegStep % kSegThreadsM == 0 && kSegStep % kSegGroup == 0, "whole CTAs and groups");
 
 struct SegInfo {
     int32_t len, status, off;
@@ -707,7 +721,7 @@ static_assert(kGroupPerm + kSegGroups * 256 <= sizeof(int32_t) * (size_t)kBlockC
 // after the other in the chaining, took 0.49 and 1.02, 0.77 and 1.31).
 template <int PASS>
 __global__ void __launch_bounds__(kSegThreadsM) dec_mtf_kernel(DecMeta *__restrict__ meta, const uint16_t *__restrict__ sym_all,
-                                                               uint8_t *__restrict__ seg_all, uint8_t *__restrict__ L_all) {
+                                                               uint8_t *__restrict__ seg_all, uint8_t *__restrict__ L_all, int segs) {
     extern __shared__ __align__(16) uint64_t list_all[];
     const int b = blockIdx.y, t = threadIdx.x, s = blockIdx.x * kSegThreadsM + t;
     const DecMeta &M = meta[b];
@@ -717,7 +731,7 @@ __global__ void __launch_bounds__(kSegThreadsM) dec_mtf_kernel(DecMeta *__restri
     SegInfo *info = reinterpret_cast<SegInfo *>(slot + kSegInfo) + s;
     const uint16_t *sym = sym_all + (size_t)b * (kBlockCap + 64);
     const int ns = M.nsym, niu = M.n_in_use, alpha = M.alpha, block_max = M.block_max;
-    const int per = (ns + kSegs - 1) / kSegs, s0 = min(ns, s * per), e0 = min(ns, s0 + per);
+    const int per = (ns + segs - 1) / segs, s0 = min(ns, s * per), e0 = min(ns, s0 + per);
     int i = s0;
     if (s > 0)
         while (i < e0 && sym[i - 1] < 2) i++;
@@ -824,9 +838,11 @@ __global__ void __launch_bounds__(256) dec_seg_group_kernel(const DecMeta *__res
     slot[kGroupPerm + g * 256 + t] = cur[kSegGroup & 1][t];
 }
 
-__global__ void __launch_bounds__(256) dec_seg_chain_kernel(DecMeta *__restrict__ meta, const DecTab *__restrict__ tabs,
-                                                            size_t tab_stride, uint8_t *__restrict__ seg_all) {
+__global__ void __launch_bounds__(256) dec_seg_chain_kernel(const DecBlock *__restrict__ blocks, DecMeta *__restrict__ meta,
+                                                            const DecTab *__restrict__ tabs, size_t tab_stride,
+                                                            uint8_t *__restrict__ seg_all, int segs) {
     constexpr int PER = kSegs / 256;
+    const int groups_n = segs / kSegGroup;
     __shared__ __align__(16) uint8_t perm[kSegGroups * 256];
     __shared__ uint8_t cur[2][256];
     __shared__ int sh[33];
@@ -837,13 +853,15 @@ __global__ void __launch_bounds__(256) dec_seg_chain_kernel(DecMeta *__restrict_
     uint8_t *slot = seg_all + (size_t)b * kBlockCap * sizeof(int32_t);
     SegInfo *info = reinterpret_cast<SegInfo *>(slot + kSegInfo);
     uint4 *groups = reinterpret_cast<uint4 *>(slot + kGroupPerm);
-    for (int i = t; i < kSegGroups * 16; i += 256) reinterpret_cast<uint4 *>(perm)[i] = groups[i];
+    for (int i = t; i < groups_n * 16; i += 256) reinterpret_cast<uint4 *>(perm)[i] = groups[i];
     // output offsets; a segment has at most block_max bytes, so the sum of
     // 3072 lengths fits 32 bits unsigned
     uint32_t c[PER], sum = 0;
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < PER; i++) {
+        c[i] = 0;
+        if (t * PER + i >= segs) continue;
         const SegInfo I = info[t * PER + i];
         c[i] = (uint32_t)I.len;
         sum += c[i];
@@ -851,19 +869,20 @@ __global__ void __launch_bounds__(256) dec_seg_chain_kernel(DecMeta *__restrict_
     }
     uint32_t total;
     uint32_t off = block_excl_sum<uint32_t>(sum, reinterpret_cast<uint32_t *>(sh), &total);
-    if (__syncthreads_or(bad) || total > (uint32_t)M.block_max || total > (uint32_t)kBlockCap || (uint32_t)M.orig >= total) {
+    if (__syncthreads_or(bad) || total > (uint32_t)M.block_max || total > (uint32_t)column_bound(blocks[b].expect) ||
+        (uint32_t)M.orig >= total) {
         if (t == 0) M.status = total <= (uint32_t)M.block_max && (uint32_t)M.orig >= total ? DEC_BAD_ORIG : DEC_BAD_DATA;
         return;
     }
 #pragma unroll
     for (int i = 0; i < PER; i++) {
-        info[t * PER + i].off = (int32_t)off;
+        if (t * PER + i < segs) info[t * PER + i].off = (int32_t)off;
         off += c[i];
     }
     if (t == 0) M.m = (int32_t)total;
     cur[0][t] = t < M.n_in_use ? T.seq_to_unseq[t] : (uint8_t)0;
     __syncthreads();
-    for (int k = 0; k < kSegGroups; k++) {
+    for (int k = 0; k < groups_n; k++) {
         slot[kGroupPerm + k * 256 + t] = cur[k & 1][t];  // the group's permutation is in shared memory
         cur[(k & 1) ^ 1][t] = cur[k & 1][perm[k * 256 + t]];
         __syncthreads();
@@ -1229,7 +1248,7 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
     DecMeta *meta = reinterpret_cast<DecMeta *>(ws.bstate);
     DecTab *tabs = reinterpret_cast<DecTab *>(ws.act2);
     const size_t ts = sizeof(int32_t) * (size_t)kBlockCap;
-    uint8_t *segs = reinterpret_cast<uint8_t *>(ws.act);
+    uint8_t *seg_buf = reinterpret_cast<uint8_t *>(ws.act);
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws.val);  // the group offsets' slot, free once the symbols are out
     uint32_t *rows = reinterpret_cast<uint32_t *>(ws.sa);
     const size_t list_smem = (size_t)256 * kSegThreadsM;
@@ -1240,8 +1259,16 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
         e = cudaFuncSetAttribute(dec_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RankSmem));
     if (e != cudaSuccess) return e;
     int64_t max_bits = 0;
-    for (int b = 0; b < nblocks; b++)
+    int max_m = 0;  // of the last columns
+    for (int b = 0; b < nblocks; b++) {
         if (h_blocks[b].src_len * 8 > max_bits) max_bits = h_blocks[b].src_len * 8;
+        if (column_bound(h_blocks[b].expect) > max_m) max_m = column_bound(h_blocks[b].expect);
+    }
+    // Grids for the largest block there can be, not for the largest of the
+    // format: 338 blocks of 900 bytes took 1.3 ms with 3072 segments, 220
+    // tiles and 141 CTAs of groups each.
+    const int max_groups = (max_m + 1 + 49) / 50, max_tiles = (max_m + kTile - 1) / kTile;
+    const int segs = kSegStep * std::min(kSegs / kSegStep, (max_m + kSegStep * kSegSyms) / (kSegStep * kSegSyms));
     dec_header_kernel<<<nblocks, kHdrThreads, 0, s>>>(blocks, meta, tabs, ts, ws.sel, ws.val);
     int launches = 17;
     for (int64_t r0 = 0; r0 < max_bits; r0 += kJRange, launches += 2) {
@@ -1250,14 +1277,15 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
             blocks, meta, tabs, ts, r0, ws.keys, ws.keys2);
         dec_chase_kernel<<<nblocks, kChaseThreads, sizeof(ChaseSmem), s>>>(blocks, meta, tabs, ts, r0, ws.keys, ws.keys2, ws.sel, ws.val);
     }
-    dec_symbols_kernel<<<dim3((kMaxSelectors + kSymGroups - 1) / kSymGroups, nblocks), kSymGroups, 0, s>>>(blocks, meta, tabs, ts, ws.sel,
+    dec_symbols_kernel<<<dim3((max_groups + kSymGroups - 1) / kSymGroups, nblocks), kSymGroups, 0, s>>>(blocks, meta, tabs, ts, ws.sel,
                                                                                                           ws.val, ws.sym);
-    const dim3 seg_grid(kSegs / kSegThreadsM, nblocks), tiles(kTilesPerBlock, nblocks), walkers((kWalkMax + 255) / 256, nblocks);
-    dec_mtf_kernel<0><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
-    dec_seg_group_kernel<<<dim3(kSegGroups, nblocks), 256, 0, s>>>(meta, segs);
-    dec_seg_chain_kernel<<<nblocks, 256, 0, s>>>(meta, tabs, ts, segs);
-    dec_seg_lists_kernel<<<dim3(kSegGroups, nblocks), 256, 0, s>>>(meta, segs);
-    dec_mtf_kernel<1><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, segs, ws.bwt);
+    const dim3 seg_grid(segs / kSegThreadsM, nblocks), groups(segs / kSegGroup, nblocks), tiles(max_tiles, nblocks);
+    const dim3 walkers((max_m / kWalkStep + 2 + 255) / 256, nblocks);
+    dec_mtf_kernel<0><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, seg_buf, ws.bwt, segs);
+    dec_seg_group_kernel<<<groups, 256, 0, s>>>(meta, seg_buf);
+    dec_seg_chain_kernel<<<nblocks, 256, 0, s>>>(blocks, meta, tabs, ts, seg_buf, segs);
+    dec_seg_lists_kernel<<<groups, 256, 0, s>>>(meta, seg_buf);
+    dec_mtf_kernel<1><<<seg_grid, kSegThreadsM, list_smem, s>>>(meta, ws.sym, seg_buf, ws.bwt, segs);
     dec_lf_count_kernel<<<tiles, kLfThreads, 0, s>>>(meta, ws.bwt, hist);
     dec_lf_scan_kernel<<<nblocks, 256, 0, s>>>(meta, hist);
     dec_lf_map_kernel<<<tiles, kLfThreads, 0, s>>>(meta, ws.bwt, hist, rows);
