@@ -909,8 +909,24 @@ __global__ void __launch_bounds__(256) dec_seg_lists_kernel(const DecMeta *__res
 
 // -------------------------------------------------------- 5. LF mapping
 // next[j] = C[L[j]] + rank of j among equal bytes; a row's word holds it with
-// the row's byte above (bits 20 .. 27).
+// the row's byte above (bits 20 .. 27) and whether a walker of the inverse BWT
+// starts at the next row (bit 28).
 constexpr int kLfThreads = 256;
+constexpr int kRowStart = 28;
+constexpr int kWalkStep = 48;  // rows between walkers: as few as the ranking's shared memory allows
+
+// Walker 0 starts at the origin row, walker k > 0 in stretch k - 1 of kWalkStep
+// rows, at a scrambled place: in a block that nearly repeats a string n times
+// a row's next one has the same place among n rows throughout a copy, so with
+// a fixed place and n a multiple of kWalkStep a walk met no start for many
+// copies (64 copies of 2812 bytes, starts at every 64th row: one piece of 174 587
+// of 179 968 rows, 44 ms). A piece is as long as its walker's luck, and a call of
+// few blocks takes as long as its longest one: 550 to 750 rows of a 1300 x 1300
+// frame with 64 rows between walkers, whatever the multiplier; with 48 such a
+// frame takes 2.19 to 2.25 ms (2.22 to 2.27 with 64).
+__device__ __forceinline__ int walk_place(uint32_t stretch) { return (int)__umulhi(stretch * 0x85EBCA6Bu, kWalkStep); }
+__device__ __forceinline__ int walk_start(int k, int orig) { return k == 0 ? orig : (k - 1) * kWalkStep + walk_place(k - 1); }
+__device__ __forceinline__ bool is_walk_start(uint32_t r) { return r % kWalkStep == (uint32_t)walk_place(r / kWalkStep); }
 
 __global__ void __launch_bounds__(kLfThreads) dec_lf_count_kernel(const DecMeta *__restrict__ meta, const uint8_t *__restrict__ L_all,
                                                                   uint32_t *__restrict__ hist_all) {
@@ -962,7 +978,7 @@ __global__ void __launch_bounds__(kLfThreads) dec_lf_map_kernel(const DecMeta *_
     const int b = blockIdx.y, tile = blockIdx.x, t = threadIdx.x, w = t >> 5, lane = t & 31;
     const DecMeta &M = meta[b];
     if (M.status != DEC_OK || tile * kTile >= M.m) return;
-    const int cnt = min(kTile, M.m - tile * kTile);
+    const int cnt = min(kTile, M.m - tile * kTile), orig = M.orig;
     const uint8_t *L = L_all + (size_t)b * kBlockCap + (size_t)tile * kTile;
     reinterpret_cast<uint4 *>(by)[t] = *reinterpret_cast<const uint4 *>(L + 16 * t);  // the slot holds whole tiles
     for (int i = t; i < NW * 256; i += kLfThreads) (&wc[0][0])[i] = 0;
@@ -995,29 +1011,21 @@ __global__ void __launch_bounds__(kLfThreads) dec_lf_map_kernel(const DecMeta *_
 #pragma unroll
     for (int r = 0; r < kTile / kLfThreads; r++) {
         const int k = w * 512 + r * 32 + lane;
-        if (k < cnt) P[k] = (wc[w][by[k]] + rk[r]) | ((uint32_t)by[k] << 20);
+        if (k >= cnt) continue;
+        const uint32_t next = wc[w][by[k]] + rk[r];
+        const bool start = is_walk_start(next) || (int)next == orig;
+        P[k] = next | ((uint32_t)by[k] << 20) | ((uint32_t)start << kRowStart);
     }
 }
 
 // ------------------------------------------------------- 6. inverse BWT
-// Bound by the latency of dependent 4-byte gathers from L2, about 64 a walker
+// Bound by the latency of dependent 4-byte gathers from L2, about 48 a walker
 // and two walks (the bytes can only be placed once the pieces are ranked): 0.12 +
 // 0.14 ms for one 1300 x 1300 frame, 0.66 + 0.84 ms for 139 blocks.
-constexpr int kWalkStep = 64;                             // rows between walkers
 constexpr int kWalkMax = kBlockCap / kWalkStep + 2;       // walkers of a block
 constexpr uint32_t kRowMask = (1u << 20) - 1u;
 // walker records in a block's slot: length, next walker, output position
 constexpr size_t kWalkLen = 0, kWalkNext = kWalkMax, kWalkPos = 2 * (size_t)kWalkMax;
-
-// Walker 0 starts at the origin row, walker k > 0 in stretch k - 1 of kWalkStep
-// rows, at a scrambled place: in a block that nearly repeats a string n times
-// a row's next one has the same place among n rows throughout a copy, so with
-// a fixed place and n a multiple of kWalkStep a walk met no start for many
-// copies (64 copies of 2812 bytes: one piece of 174 587 of 179 968 rows, 44 ms).
-__device__ __forceinline__ int walk_place(uint32_t stretch) { return (int)(stretch * 2654435761u >> 26); }
-static_assert(kWalkStep == 64, "a place is 6 bits");
-__device__ __forceinline__ int walk_start(int k, int orig) { return k == 0 ? orig : (k - 1) * kWalkStep + walk_place(k - 1); }
-__device__ __forceinline__ bool is_walk_start(int r) { return (r & (kWalkStep - 1)) == walk_place((uint32_t)r / kWalkStep); }
 
 __global__ void __launch_bounds__(256) dec_walk_kernel(const DecMeta *__restrict__ meta, const uint32_t *__restrict__ P_all,
                                                        int32_t *__restrict__ rec_all) {
@@ -1034,10 +1042,12 @@ __global__ void __launch_bounds__(256) dec_walk_kernel(const DecMeta *__restrict
         rec[kWalkNext + k] = 0;
         return;
     }
+    uint32_t p;
     do {  // the rows form cycles, so a walk ends at its own row at the latest
-        r = (int)(P[r] & kRowMask);
+        p = P[r];
+        r = (int)(p & kRowMask);
         steps++;
-    } while (r != orig && !is_walk_start(r));
+    } while ((p >> kRowStart) == 0);
     rec[kWalkLen + k] = steps;
     rec[kWalkNext + k] = r == orig ? 0 : r / kWalkStep + 1;
 }
@@ -1106,7 +1116,7 @@ __global__ void __launch_bounds__(256) dec_emit_kernel(const DecMeta *__restrict
         const uint32_t p = P[r];
         r = (int)(p & kRowMask);
         at--;
-        acc |= (uint64_t)(p >> 20) << (8 * (at & 7));
+        acc |= (uint64_t)((p >> 20) & 255u) << (8 * (at & 7));
         n++;
         if ((at & 7) == 0) {
             if (n == 8) *reinterpret_cast<uint64_t *>(blk + at) = acc;
@@ -1120,15 +1130,15 @@ __global__ void __launch_bounds__(256) dec_emit_kernel(const DecMeta *__restrict
 }
 
 // The bytes before the last period of a block that repeats it (any other
-// block is left at once).
+// block is left at once, so the grid is small).
+constexpr int kRepeatCtas = 8;
 __global__ void __launch_bounds__(256) dec_repeat_kernel(const DecMeta *__restrict__ meta, uint8_t *__restrict__ blk_all) {
     const int b = blockIdx.y;
     const DecMeta &M = meta[b];
     if (M.status != DEC_OK || M.period == M.m) return;
     const int period = M.period, start = M.m - period;
     uint8_t *blk = blk_all + (size_t)b * kBlockCap;
-    const int e = min(start, ((int)blockIdx.x + 1) * kTile);
-    for (int i = blockIdx.x * kTile + threadIdx.x; i < e; i += 256) blk[i] = blk[start + i % period];
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < start; i += kRepeatCtas * 256) blk[i] = blk[start + i % period];
 }
 
 // ----------------------------------------------------- 7. inverse RLE1
@@ -1292,7 +1302,7 @@ cudaError_t launch_bzip2_decode(lfc_plan P, const DecBlockHost *h_blocks, const 
     dec_walk_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2);
     dec_rank_kernel<<<nblocks, 1024, sizeof(RankSmem), s>>>(meta, ws.sa2);
     dec_emit_kernel<<<walkers, 256, 0, s>>>(meta, rows, ws.sa2, ws.rle);
-    dec_repeat_kernel<<<tiles, 256, 0, s>>>(meta, ws.rle);
+    dec_repeat_kernel<<<dim3(kRepeatCtas, nblocks), 256, 0, s>>>(meta, ws.rle);
     dec_unrle_count_kernel<<<tiles, kUnThreads, 0, s>>>(meta, ws.rle, ws.tileaux);
     dec_unrle_scan_kernel<<<nblocks, 256, 0, s>>>(blocks, meta, ws.tileaux);
     dec_unrle_write_kernel<<<tiles, kUnThreads, 0, s>>>(blocks, meta, ws.rle, ws.tileaux);

@@ -1,6 +1,6 @@
 """Blocks that repeat a shorter string, or nearly do: the origin row among
 identical rotations, decoding blocks whose rows form several cycles, the
-pieces of the inverse BWT where a row keeps its place among 64 k rows, and the
+pieces of the inverse BWT where a row keeps its place among 48 k or 64 k rows, and the
 suffix sort's time on long repeats."""
 import bz2
 
@@ -141,7 +141,7 @@ def test_repeated_blocks_damaged(lfc):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("shape", [(64, 1406), (256, 1020)])
+@pytest.mark.parametrize("shape", [(64, 1406), (256, 1020), (96, 1406), (48, 2000)])
 def test_nearly_repeated_blocks_are_not_serial(lfc, shape):
     """One row over and over with one pixel changed: as fast as noise of the
     same size, give or take (a piece of 100 000 rows and more, walked by one
