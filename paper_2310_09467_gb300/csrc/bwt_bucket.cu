@@ -823,7 +823,8 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
         L_all[(size_t)b * kBlockCap + at] = rle[idx == 0 ? m - 1 : idx - 1];
         if (idx == 0) st[b].orig_ptr = at;
     };
-    const int warps = gridDim.x * (kTieThreads / 32), chunk = min(32, (total_long + warps - 1) / warps);
+    // long groups a warp takes at once: it asks for the block's count once a chunk
+    const int warps = gridDim.x * (kTieThreads / 32), chunk = min(8, (total_long + warps - 1) / warps);
     const bool few = total <= warps * 32 && total_long <= kTieWaves * warps;
     auto most = [few](int m) { return few ? INT_MAX : max(kTieMany, m / kTieShare); };
     auto given_up = [&](uint64_t e) { return ld_flag(bdeep + (e >> 32)) >= most(st[e >> 32].m); };
@@ -886,11 +887,14 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
     for (int g0 = (blockIdx.x * (kTieThreads / 32) + warp) * chunk; g0 < total_long; g0 += warps * chunk) {
         const int gn = min(chunk, total_long - g0);
         const uint64_t mine = lane < gn ? ties[ties_cap - 1 - (size_t)(g0 + lane)] : 0ull;
+        bool check = true;  // at first and after a group that went far
         for (uint32_t todo = LFC_FULL >> (32 - gn); todo;) {
-            const bool drop = ((todo >> lane) & 1u) && given_up(mine);  // a lane for each of these
-            if (drop) leave(mine);
-            todo &= ~__ballot_sync(LFC_FULL, drop);
-            if (!todo) break;
+            if (check) {
+                const bool drop = ((todo >> lane) & 1u) && given_up(mine);  // a lane for each of these
+                if (drop) leave(mine);
+                todo &= ~__ballot_sync(LFC_FULL, drop);
+                if (!todo) break;
+            }
             const uint64_t e = __shfl_sync(LFC_FULL, mine, __ffs(todo) - 1);
             todo &= todo - 1;
             const int b = (int)(e >> 32), len = (int)((e >> 24) & 255u), at = (int)(e & 0xFFFFFFu);
@@ -900,7 +904,8 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
             const bool in = lane < len;
             uint64_t w = in ? (uint64_t)(uint32_t)sa_all[(size_t)b * kBlockCap + at + lane] : ~0ull;
             int p0 = in ? 0 : lane, p1 = in ? len : lane + 1, dep = 0;  // the member's piece, the bytes it shares
-            for (int round = 0;; round++) {
+            int round = 0;
+            for (;; round++) {
                 const bool act = p1 - p0 > 1 && dep < m;
                 if (!__any_sync(LFC_FULL, act)) break;
                 if (!__any_sync(LFC_FULL, lane == 0 && go_on(b, m, round))) break;
@@ -931,6 +936,7 @@ __global__ void __launch_bounds__(kTieThreads) bwt_tie_kernel(BlockState *__rest
                 if (p1 - p0 > 1 && lane == p0 && dep < m) leave_tied(bflag, rs, b, dep);
                 out(b, m, rle, at + lane, w, lane > p0);
             }
+            check = round >= kTieFew;
         }
     }
 }
