@@ -50,7 +50,7 @@ static POff param_offsets(int K) {
 }  // namespace lfc
 
 struct lfc_cnn_s {
-    int K = 0, max_batch = 0;
+    int K = 0, max_batch = 0, sm_count = 1;
     cudaStream_t stream = nullptr;
     lfc::POff off;
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
@@ -532,6 +532,10 @@ extern "C" int lfc_cnn_create(int n_classes, int max_batch, uint64_t seed, void 
     C->K = n_classes;
     C->max_batch = max_batch;
     C->stream = reinterpret_cast<cudaStream_t>(cuda_stream);
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&C->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || C->sm_count <= 0)
+        C->sm_count = 1;
     C->off = param_offsets(n_classes);
     const size_t np = C->off.total, B = (size_t)max_batch;
     cudaError_t e = cudaSuccess;
@@ -679,7 +683,7 @@ extern "C" int lfc_cnn_backward(lfc_cnn C, int n, const int32_t *d_labels, float
     // rows of a weight-gradient band: 16 (a band's 9216 sums go out by
     // atomics), fewer while the bands would leave SMs without one
     int rows = 16;
-    while (rows > 2 && n * (kT / rows) < 152) rows /= 2;
+    while (rows > 2 && n * (kT / rows) < C->sm_count) rows /= 2;
     CKC(cudaFuncSetAttribute(conv_wgrad_kernel<kCh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem<kCh>)));
     CKC(cudaFuncSetAttribute(conv_wgrad_kernel<kC0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradSmem<kC0>)));
     dim3 wgrid(kT / rows, n);
