@@ -121,10 +121,11 @@ __device__ __forceinline__ void ldm4t(uint32_t (&r)[4], const void *p) {
 
 // out[y][x][co] = epilogue(sum_{ky,kx,ci} in[y+ky-1][x+kx-1][ci] * W[ky][kx][ci][co])
 // MODE 0: + bias, ReLU.  MODE 1: * (mask[y][x][co] > 0)  (input gradient).
-// Bound by shared memory: a warp's weight fragments serve two rows (16
-// wavefronts per 8 products; one row took 24), and a 16 x 16 tile halves the
-// weights staged per output against 8 x 16: 198 -> 124 us for 32 frames of a
-// 32-channel layer. The order of a sum's terms is that of the taps and
+// Bound by the shared-memory data pipe (ncu, 32 frames of a 32-channel layer:
+// 83 % of its peak forward, 68 % in the input gradient, tensor pipe 54 and 41 %):
+// a warp's weight fragments serve two rows (16 wavefronts per 8 products; one
+// row took 24), and a 16 x 16 tile halves the weights staged per output against
+// 8 x 16: 198 -> 124 us for that layer. The order of a sum's terms is that of the taps and
 // channels, whatever the tile.
 template <int CIN, int MODE>
 __global__ void __launch_bounds__(256) conv3x3_mma_kernel(const bf16 *__restrict__ in, const bf16 *__restrict__ wB,
@@ -307,9 +308,11 @@ __global__ void dpre_last_kernel(const float *__restrict__ dg, const bf16 *__res
 // channels x 8 output channels per product, 16 pixels deep. Both operands lie
 // pixel-major in shared memory and are read transposed; the tensor cores sum
 // a row's products, and the rows are added in registers with rounding to
-// nearest (the tensor cores' own sums truncate). Bound by shared memory (16
-// wavefronts per 8 products); as FP32 outer products on the CUDA cores, a
-// 32-channel layer of 32 frames took 2030 us.
+// nearest (the tensor cores' own sums truncate). Bound by the wait for a row's
+// loads between its two barriers, with two CTAs an SM (ncu, 32 frames of a
+// 32-channel layer, 222 us: about half of the stalls wait for global memory,
+// shared-memory data pipe 45 %, tensor pipe 32 % of peak); as FP32 outer
+// products on the CUDA cores that layer took 2030 us.
 constexpr int kWgThreads = 9 * 32;
 template <int CIN>
 struct WgradSmem {

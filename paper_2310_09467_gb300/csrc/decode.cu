@@ -30,7 +30,7 @@
 //     the origin's is the string, and the block is filled with it.
 //  7. Inverse RLE1 by tiles from sync points; block CRCs (crc.cu).
 // One 1300 x 1300 frame (5 blocks) takes 2.2 ms, 12 frames of 2040 x 2040
-// (139 blocks) 10.5 ms; with one CTA per block it was 47 and 58 ms.
+// (139 blocks) 10.2 ms; with one CTA per block it was 47 and 58 ms.
 #include <algorithm>
 #include <climits>
 
@@ -530,9 +530,10 @@ __global__ void __launch_bounds__(kJThreads, 2) dec_jump_kernel(const DecBlock *
 
 // One CTA per block: thread 0 adds up the groups' lengths, the other warps
 // fetch the next window of them. After the last round also the last group,
-// up to EOB. Bound by that chain and by what one SM can fetch (96 KB a
-// window): 0.73 ms for one 1300 x 1300 frame and 0.94 ms for 139 blocks (with
-// windows of 4096 bits 0.91 and 1.10).
+// up to EOB. Bound by that chain, about 80 cycles a group: the copying warps
+// wait four times as long at the barrier as for their loads (ncu, one frame's
+// five blocks). 0.73 ms for one 1300 x 1300 frame and 0.94 ms for 139 blocks
+// (with windows of 4096 bits 0.91 and 1.10).
 constexpr int kChaseThreads = 256;
 constexpr int kChaseWin = 8192;  // bits of a window: long enough that its barriers and copies hide behind 56 groups' adds
 constexpr int kChaseBufs = 2;    // one in use, one on its way
@@ -1020,8 +1021,8 @@ __global__ void __launch_bounds__(kLfThreads) dec_lf_map_kernel(const DecMeta *_
 
 // ------------------------------------------------------- 6. inverse BWT
 // Bound by the latency of dependent 4-byte gathers from L2, about 48 a walker
-// and two walks (the bytes can only be placed once the pieces are ranked): 0.12 +
-// 0.14 ms for one 1300 x 1300 frame, 0.66 + 0.84 ms for 139 blocks.
+// and two walks (the bytes can only be placed once the pieces are ranked): 0.10 +
+// 0.12 ms for one 1300 x 1300 frame, 0.50 + 0.67 ms for 139 blocks.
 constexpr int kWalkMax = kBlockCap / kWalkStep + 2;       // walkers of a block
 constexpr uint32_t kRowMask = (1u << 20) - 1u;
 // walker records in a block's slot: length, next walker, output position

@@ -99,7 +99,8 @@ __device__ __forceinline__ void with_functions(uint32_t set, Body body) {
 // tile's pixels are computed once into shared memory (thread = pixel column,
 // p rows each), then every candidate of that f is written from there in
 // its ordering, consecutive threads on consecutive output positions.
-// Bound by instructions, 26 candidates a pixel: edges without a case per
+// Bound by instructions at the 16 warps an SM that its shared memory leaves room
+// for (issue slots 62 % busy, 26 candidates a pixel): edges without a case per
 // function, the default functions without a test each, 8 cells a load and
 // two symbols a zigzag took 12 2040 x 2040 frames from 1835 to 1482 us and a
 // 195 x 195 one from 41 to 35 us (more threads a CTA are slower: fewer CTAs

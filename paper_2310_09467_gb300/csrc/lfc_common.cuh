@@ -61,6 +61,7 @@ struct BwtCode {
     uint16_t split[kBuckets];
     int32_t nb, pad[3];
 };
+static_assert(sizeof(BwtCode) % 16 == 0, "BwtCode rows stay 16-byte aligned");
 
 // Whole codes (bytes) in the key of a rotation.
 static __device__ __noinline__ int key_depth(const uint8_t *rle, int m, const uint16_t *code, int idx) {
@@ -75,7 +76,6 @@ static __device__ __noinline__ int key_depth(const uint8_t *rle, int m, const ui
         if (++pos == m) pos = 0;
     }
 }
-static_assert(sizeof(BwtCode) % 16 == 0, "BwtCode rows stay 16-byte aligned");
 
 // ------------------------------------------------------------ warp helpers
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
@@ -288,7 +288,6 @@ struct Workspace {
     int64_t crc_part_cap = 0;
     void *chunk_desc = nullptr;        // descriptor staging (CRC chunks, frame tables)
     size_t chunk_desc_bytes = 0;
-    // decode
 };
 
 }  // namespace lfc
